@@ -247,3 +247,90 @@ def tolerance(case):
     if case["kind"] == "decode":
         return {"rel": 4e-4, "max": 4e-3, "differ": 0.0}
     return {"rel": 8e-4, "max": 1.3e-2, "differ": 0.0}
+
+
+def _codes(x, scale, zero, qmax):
+    """The value a code stands for, in 64 bits: codes by the format's own 32-bit formula."""
+    code = (torch.round(x / torch.where(scale == 0, 1.0, scale)) + zero).clamp_(0, qmax)
+    return scale.double() * (code.double() - zero.double())
+
+
+def _pairs(mn, mx, qmax):
+    """(scale, zero) of groups with extremes mn, mx (infinite where a group has no member)."""
+    r = mx - mn
+    scale = torch.where(r == 0, torch.where(mn == 0, 1.0, mn.abs()), r / torch.full_like(r, qmax))   # a tensor: by a number it would be a product with 1 / qmax
+    zero = 0.0 - torch.round(mn / scale)
+    none = torch.isinf(mn)
+    return torch.where(none, 0.0, scale), torch.where(none, 0.0, zero)
+
+
+def _extremes(x, sink, dims):
+    return (x.masked_fill(sink, math.inf).amin(dims, keepdim=True), x.masked_fill(sink, -math.inf).amax(dims, keepdim=True))
+
+
+def _as_cached(case, K, V, sink, params):
+    """One sequence's keys and values [Hkv, n, D] as the cache holds them, in 64 bits; sink [n]."""
+    h, n, d = K.shape
+    qmax, G = float(2 ** case["bits"] - 1), case["group"]
+    gv, keep = min(G, d), sink[None, :, None]
+    k, v = K.float(), V.float()
+    by_group = lambda x: x.view(h, n, d // gv, gv)
+    token_pairs = lambda x: _pairs(*_extremes(by_group(x), keep[..., None], -1), qmax)
+    if case["scheme"] == "static":
+        kd = _codes(k, params["k"][0][:, None], params["k"][1][:, None], qmax)
+        vd = _codes(by_group(v), *(p[:, None, :, None] for p in params["v"]), qmax).view(h, n, d)
+    else:
+        vd = _codes(by_group(v), *token_pairs(v), qmax).view(h, n, d)
+        if case["scheme"] == "per_token":
+            kd = _codes(by_group(k), *token_pairs(k), qmax).view(h, n, d)
+        else:
+            kd, body = k.double(), n // G * G                    # the open group stays as it came
+            kg, sg = k[:, :body].view(h, body // G, G, d), sink[:body].view(1, body // G, G, 1)
+            kd[:, :body] = _codes(kg, *_pairs(*_extremes(kg, sg, 2), qmax), qmax).view(h, body, d)
+    return torch.where(keep, k.double(), kd), torch.where(keep, v.double(), vd)
+
+
+def exact(case, seed):
+    """Attention outputs in 64 bits over the values that the cache's codes, parameters and exact rows stand for."""
+    if case["kind"] in ("predict", "append"):
+        return None                                              # integers, codes and moved rows: compared bit by bit
+    g = _gen(seed)
+    B, hq, hkv, d, start, T = (case[k] for k in ("batch", "hq", "hkv", "dim", "start", "tokens"))
+    rep, decode = hq // hkv, case["kind"] == "decode"
+    prompt = start if decode else start + T
+    hidden, pos = _plant(B, prompt, case["topk"], NARROW, NARROW_CHANNELS, g)
+    score = hidden[:, :, list(NARROW_CHANNELS)].abs().amax(-1)
+    sinks = torch.zeros((B, start + T), dtype=torch.bool, device="cuda")
+    sinks.scatter_(1, score.sort(dim=1, descending=True, stable=True).indices[:, : case["topk"]], True)
+    sinks[:, :PFN] = True
+    del hidden
+    K, V = _keys_values(case, prompt, pos, g)
+    params = None
+    if case["scheme"] == "static":
+        ngv, keep = d // min(case["group"], d), sinks[:, None, :prompt, None]
+        ext = lambda x, s, dims: [f([e(x[b : b + 1].float(), s[b : b + 1], dims) for b in range(B)])
+                                  for e, f in ((lambda *a: _extremes(*a)[0], lambda m: torch.stack(m).amin(0)),
+                                               (lambda *a: _extremes(*a)[1], lambda m: torch.stack(m).amax(0)))]
+        qmax = float(2 ** case["bits"] - 1)
+        params = {"k": [p.view(hkv, d) for p in _pairs(*ext(K, keep, (0, 2)), qmax)],
+                  "v": [p.view(hkv, ngv) for p in _pairs(*ext(V.view(B, hkv, prompt, ngv, -1), keep[..., None], (0, 2, 4)), qmax)]}
+    if decode:
+        k1, v1 = _keys_values(case, 1, None, g)
+        q = _queries(case, 1, K[:, :, 0], g)
+    else:
+        q = _queries(case, T, K[:, :, 0], g)
+    out = torch.empty((B, hq, T, d), dtype=torch.float64, device="cuda")
+    lse = torch.empty((B, hq, T), dtype=torch.float64, device="cuda")
+    seen = torch.arange(start + T, device="cuda")[None] <= start + torch.arange(T, device="cuda")[:, None]
+    for b in range(B):
+        kb, vb = (torch.cat([K[b], k1[b]], 1), torch.cat([V[b], v1[b]], 1)) if decode else (K[b], V[b])
+        for h in range(hkv):
+            sub = {n: [p[h : h + 1] for p in x] for n, x in params.items()} if params else None
+            kd, vd = _as_cached(case, kb[h : h + 1], vb[h : h + 1], sinks[b], sub)
+            for i in range(h * rep, (h + 1) * rep):
+                s = (q[b, i].double() @ kd[0].T / math.sqrt(d)).masked_fill_(~seen, -math.inf)
+                lse[b, i] = s.logsumexp(-1)
+                out[b, i] = (s - lse[b, i][:, None]).exp_() @ vd[0]
+    if decode:
+        out, lse = out[:, :, 0], lse[:, :, 0]
+    return [out, lse] + [None] * 9
