@@ -174,6 +174,7 @@ extern "C" int kvsink_prefill_attention(const kvsink_config *cfg, const kvsink_c
     if (stride_t < p.D || (stride_t % 8) || (stride_h % 8) || (stride_b % 8) || stride_h < 0 || stride_b < 0) return KVSINK_ERR_BAD_ARG;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     const __half *qq = (const __half *)q;
+    if (prompt_takes(p, T)) return launch_prompt(p, *cache, qq, T, q_pos0, stride_b, stride_h, stride_t, out, lse, st);
     if (p.bits == 2) return launch_prefill_b2(p, *cache, qq, T, q_pos0, stride_b, stride_h, stride_t, out, lse, st);
     if (p.bits == 3) return launch_prefill_b3(p, *cache, qq, T, q_pos0, stride_b, stride_h, stride_t, out, lse, st);
     return launch_prefill_b4(p, *cache, qq, T, q_pos0, stride_b, stride_h, stride_t, out, lse, st);

@@ -158,6 +158,9 @@ int launch_prefill_b3(const Params &p, const kvsink_cache &c, const __half *q, i
                       float *lse, cudaStream_t st);
 int launch_prefill_b4(const Params &p, const kvsink_cache &c, const __half *q, int T, int q_pos0, int64_t sb, int64_t sh, int64_t stt, float *out,
                       float *lse, cudaStream_t st);
+bool prompt_takes(const Params &p, int T);
+int launch_prompt(const Params &p, const kvsink_cache &c, const __half *q, int T, int q_pos0, int64_t sb, int64_t sh, int64_t stt, float *out,
+                  float *lse, cudaStream_t st);
 int launch_calibrate(const Params &p, const __half *k, const __half *v, int T, int64_t sb, int64_t sh, int64_t stt, const uint32_t *bitmask,
                      const kvsink_static_params &sp, void *workspace, cudaStream_t st);
 int launch_quantize_calibrated(const Params &p, const kvsink_cache &c, const kvsink_static_params &sp, const __half *k_src, const __half *v_src,

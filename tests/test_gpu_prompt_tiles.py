@@ -1,0 +1,81 @@
+"""GPU parity of prompt attention on the 256-row tensor-core blocks (head size 128, many rows) against the CPU oracle:
+|gpu - oracle| <= 2e-3 + 1e-2 |oracle| for every query row, at the edges of row tiles, steps and key groups."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2508_04257_b200 as kv
+from paper_2508_04257_b200 import synth
+
+from parity_util import assert_close, configs, np16
+
+pytestmark = pytest.mark.gpu
+TINY = synth.WORKLOADS["tiny"]
+
+
+def _check(wl, T, pos0, shape_keys=None, shape_values=None, strided=False):
+    ocfg, gcfg = configs(wl)
+    H = synth.make_hidden(wl, "cuda")
+    K, V = synth.make_kv(wl, 0, "cuda")
+    if shape_keys:
+        shape_keys(K)
+    if shape_values:
+        shape_values(V)
+    gs = kv.SinkSet(gcfg)
+    kv.predict_sinks(gcfg, H, gs)
+    bm, pos, cnt = oracle.predict_sinks(ocfg, np16(H))
+    gc, oc = kv.KVCache(gcfg, gs), oracle.Cache(ocfg, bm, pos, cnt)
+    kv.quantize_append(gcfg, gc, K, V)
+    oracle.quantize_append(ocfg, oc, np16(K), np16(V))
+    g = torch.Generator("cuda").manual_seed(wl.seed + T)
+    q = torch.randn((wl.batch, wl.n_q_heads, T, wl.head_dim), device="cuda", generator=g).half()
+    if strided:     # [B, T, Hq, D] storage
+        q = q.permute(0, 2, 1, 3).contiguous().permute(0, 2, 1, 3)
+    out, lse = kv.prefill_attention(gcfg, gc, q, pos0)
+    ref, ref_lse = oracle.prefill_attention(ocfg, oc, np16(q), pos0)
+    torch.cuda.synchronize()
+    assert kv.read_status(gc) == 0
+    # an output is a mean of values with weights that carry 22 bits: its error goes with the largest value
+    top = float(V.abs().max())
+    assert_close(out.cpu().numpy(), ref, "prompt attention", atol=2e-3 * max(1.0, top / 6.0))
+    assert np.abs(lse.cpu().numpy() - ref_lse).max() <= 2e-3 + 1e-3 * np.abs(ref_lse).max()
+
+
+# rows of a unit: 64, 8 x 63, 8 x 129 (five blocks), 4 x 257, 3 x 171 = 513, 513; sequence ends inside a step, a tile, a group
+@pytest.mark.parametrize("bits,group,hq,hkv,batch,T,pos0", [
+    (2, 128, 16, 16, 8, 64, 0), (4, 64, 64, 8, 8, 63, 70), (3, 64, 32, 4, 8, 129, 0), (2, 32, 16, 4, 2, 257, 0),
+    (4, 144, 12, 4, 4, 171, 29), (2, 128, 4, 4, 4, 513, 0), (3, 128, 8, 8, 16, 256, 1), (4, 32, 8, 8, 8, 130, 190)])
+@pytest.mark.parametrize("topk", [3, 90])
+def test_tiles(bits, group, hq, hkv, batch, T, pos0, topk):
+    wl = TINY.scaled(bits=bits, head_dim=128, group=group, n_q_heads=hq, n_kv_heads=hkv, batch=batch, seq=pos0 + T, topk=min(topk, pos0 + T),
+                     pfn_n=2, seed=21000 + bits * 100 + group + T + topk)
+    _check(wl, T, pos0, strided=T % 2 == 1)
+
+
+def _wide(K):
+    n = K.shape[2]
+    K[:, :, :, 3] = 2.5
+    K[:, :, :, 4] = 0.0
+    K[:, :, :, 6] *= 300.0
+    K[:, :, :, 70] *= 1e-3
+    K[:, :, :, 8] = 300.0 + torch.arange(n, device="cuda").half() * 0.25
+    K[:, :, :, 100] = -40.0 + torch.randn(n, device="cuda", generator=torch.Generator("cuda").manual_seed(5)).half() * 0.01
+
+
+def _far(x):           # narrow ranges far from zero: zero points of some ten thousands
+    x[:, :, :, ::3] = 40.0 + x[:, :, :, ::3] * 0.02
+    x[:, :, :, 1::3] = -500.0 + x[:, :, :, 1::3] * 0.3
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("keys,values", [(_wide, None), (None, _far), (_far, _far), (lambda K: K.mul_(1e-3), lambda V: V.mul_(1e-4)),
+                                         (lambda K: K.mul_(8.0), lambda V: V.mul_(8000.0).clamp_(-60000, 60000))])
+def test_ranges(bits, keys, values):
+    wl = TINY.scaled(bits=bits, head_dim=128, group=32, n_q_heads=16, n_kv_heads=4, batch=2, seq=300, topk=6, pfn_n=1, seed=22000 + bits)
+    _check(wl, 300, 0, keys, values)
+
+
+def test_every_token_a_sink():
+    wl = TINY.scaled(bits=2, head_dim=128, group=64, n_q_heads=16, n_kv_heads=4, batch=2, seq=270, topk=270, pfn_n=0, seed=23000)
+    _check(wl, 270, 0)
