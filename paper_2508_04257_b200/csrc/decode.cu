@@ -75,6 +75,10 @@ int max_splits(const Params &p)
     return (int)(ns < 1 ? 1 : ns);
 }
 
+// Two and four bit: whole waves of resident blocks times the groups of a warp.  Three bit is bound by issue slots, so an SM's time
+// goes with the number of blocks it gets in all (four resident ones run at full rate, two at three quarters of it), each with the
+// groups of a warp and about one group's time for its prologue and epilogue: 16 x 32 units of 8101 tokens take two splits of
+// 512 blocks' work (7 blocks on the fullest SM instead of 4 of twice the size), 150 -> 129 us.
 int choose_splits(const Params &p, int n_groups)
 {
     const int qchunks = decode_qchunks(p);
@@ -83,10 +87,17 @@ int choose_splits(const Params &p, int n_groups)
     int best = 1;
     double best_cost = 1e300;
     for (int ns = 1; ns <= ns_max; ++ns) {
-        const long waves = (units * ns + DEC_SLOTS - 1) / DEC_SLOTS;
         const int per_block = (n_groups + ns - 1) / ns;
         const int per_warp = (per_block + DEC_WARPS - 1) / DEC_WARPS;
-        const double cost = (double)waves * (per_warp + 0.5);
+        double cost;
+        if (p.bits == 3) {
+            static const double rate[5] = {1.0, 0.4, 0.75, 0.93, 1.0};
+            const long on_sm = (units * ns + 147) / 148;
+            cost = (double)on_sm / rate[on_sm < 4 ? on_sm : 4] * ((double)per_block / DEC_WARPS + 0.93) + 0.02 * ns;   // the last term: one more record to merge
+        } else {
+            const long waves = (units * ns + DEC_SLOTS - 1) / DEC_SLOTS;
+            cost = (double)waves * (per_warp + 0.5);
+        }
         if (cost < best_cost - 1e-9) { best_cost = cost; best = ns; }
     }
     return best;

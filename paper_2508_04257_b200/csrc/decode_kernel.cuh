@@ -1222,8 +1222,14 @@ static int launch_decode_p(const Params &p, const kvsink_cache &c, const kvsink_
     pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     pdl[0].val.programmaticStreamSerializationAllowed = 1;
     // up to eight splits (the portable cluster size): the splits of a unit are launched as one thread-block cluster and
-    // merged inside the kernel through distributed shared memory; more splits go through the workspace and the merge kernel
-    bool cluster_merge = nsplit > 1 && nsplit <= 8;
+    // merged inside the kernel through distributed shared memory, which saves the merge kernel's 1 to 1.8 us (4 x 32 units of 2048
+    // tokens, 2 bit: 12.3 -> 10.5 us).  A cluster has to be placed as a whole, though, and where the grid fills the chip with
+    // long blocks the slots it leaves empty cost more: 18 x 8 units of 47328 tokens in four splits, 3 bit, 232 us as clusters and
+    // 181 us without, 11 x 8 units of 9068 in six, 4 bit, 29.2 and 26.6 us; pairs are better off alone from some 256 KB a block
+    // (25.1 against 26.6 us at 128 KB, 417 against 412 us at 512 KB)
+    const int64_t blocks = (int64_t)nsplit * p.Hkv * qchunks * p.B;
+    const int64_t block_bytes = (int64_t)gps * (PM != 0 ? CT * KVSINK_TILE : p.G) * 2 * p.row_bytes;
+    bool cluster_merge = nsplit > 1 && nsplit <= 8 && (blocks <= 2 * 148 || block_bytes < (nsplit == 2 ? 256 : 64) * 1024);
     for (;;) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(nsplit, p.Hkv * qchunks, p.B);
