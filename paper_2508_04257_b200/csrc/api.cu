@@ -38,10 +38,10 @@ static int derive(const kvsink_config *cfg, Params *p)
 
 // Whole groups: the streaming kernel where the shape has one, else the generic kernel.
 static int quantize_groups(const Params &p, const kvsink_cache &c, const __half *k, const __half *v, int first_token, int n_groups,
-                           int64_t sb, int64_t sh, int64_t stt, bool do_v_and_sinks, cudaStream_t st)
+                           int64_t sb, int64_t sh, int64_t stt, bool do_v_and_sinks, bool after_edges, cudaStream_t st)
 {
     int rc = KVSINK_ERR_UNSUPPORTED;
-    if (do_v_and_sinks) rc = launch_quantize_groups_bulk(p, c, k, v, first_token, n_groups, sb, sh, stt, st);
+    if (do_v_and_sinks) rc = launch_quantize_groups_bulk(p, c, k, v, first_token, n_groups, sb, sh, stt, after_edges, st);
     if (rc != KVSINK_ERR_UNSUPPORTED) return rc;
     rc = launch_quantize_groups_fast(p, c, k, v, first_token, n_groups, sb, sh, stt, do_v_and_sinks, st);
     if (rc != KVSINK_ERR_UNSUPPORTED) return rc;
@@ -117,8 +117,23 @@ extern "C" int kvsink_quantize_append(const kvsink_config *cfg, kvsink_cache *ca
     cudaStream_t st = (cudaStream_t)cuda_stream;
     const int S0 = cache->seq_len, G = p.G;
     const __half *k = (const __half *)k_new, *v = (const __half *)v_new;
-    // A chunk that starts inside an open group first completes (or extends) that group token by token; whole groups
-    // that follow take the bulk kernels; what is left goes to the tail token by token.
+    // A chunk that starts inside an open group first completes (or extends) that group; whole groups that follow take the
+    // bulk kernels; what is left goes to the tail.  Both ragged ends in one kernel, ahead of the whole groups', where a group is
+    // small enough for it, else token by token.
+    if (T > 1 && G <= 128) {
+        const int head = S0 % G == 0 ? 0 : (T < G - S0 % G ? T : G - S0 % G), n_groups = (T - head) / G, rem = T - head - n_groups * G;
+        if (head > 0 || rem > 0) {
+            rc = launch_append_edges(p, *cache, k, v, S0, head, T - rem, rem, stride_b, stride_h, stride_t, st);
+            if (rc) return rc;
+        }
+        if (n_groups > 0) {
+            rc = quantize_groups(p, *cache, k + (int64_t)head * stride_t, v + (int64_t)head * stride_t, S0 + head, n_groups, stride_b, stride_h,
+                                 stride_t, true, head > 0 || rem > 0, st);
+            if (rc) return rc;
+        }
+        cache->seq_len = S0 + T;
+        return KVSINK_OK;
+    }
     int done = 0;
     if (S0 % G != 0) {
         const int head = T < G - S0 % G ? T : G - S0 % G;
@@ -127,7 +142,7 @@ extern "C" int kvsink_quantize_append(const kvsink_config *cfg, kvsink_cache *ca
         if ((S0 + head) % G == 0) {
             // the open group is complete: quantize its keys per channel from the fp16 tail
             rc = quantize_groups(p, *cache, (const __half *)cache->k_tail, (const __half *)cache->k_tail, S0 + head - G, 1,
-                                 (int64_t)p.Hkv * G * p.D, (int64_t)G * p.D, p.D, false, st);
+                                 (int64_t)p.Hkv * G * p.D, (int64_t)G * p.D, p.D, false, false, st);
             if (rc) return rc;
         }
         done = head;
@@ -136,7 +151,7 @@ extern "C" int kvsink_quantize_append(const kvsink_config *cfg, kvsink_cache *ca
         const int n_groups = (T - done) / G;
         if (n_groups > 0) {
             rc = quantize_groups(p, *cache, k + (int64_t)done * stride_t, v + (int64_t)done * stride_t, S0 + done, n_groups, stride_b,
-                                 stride_h, stride_t, true, st);
+                                 stride_h, stride_t, true, false, st);
             if (rc) return rc;
         }
         rc = launch_quantize_tokens(p, *cache, k, v, done + n_groups * G, S0 + done + n_groups * G, T - done - n_groups * G, stride_b,

@@ -147,9 +147,11 @@ int launch_quantize_groups(const Params &p, const kvsink_cache &c, const __half 
 int launch_quantize_groups_fast(const Params &p, const kvsink_cache &c, const __half *k_src, const __half *v_src, int first_token,
                                 int n_groups, int64_t sb, int64_t sh, int64_t stt, bool do_v_and_sinks, cudaStream_t st);
 int launch_quantize_groups_bulk(const Params &p, const kvsink_cache &c, const __half *k_src, const __half *v_src, int first_token,
-                                int n_groups, int64_t sb, int64_t sh, int64_t stt, cudaStream_t st);
+                                int n_groups, int64_t sb, int64_t sh, int64_t stt, bool after_edges, cudaStream_t st);
 int launch_quantize_tokens(const Params &p, const kvsink_cache &c, const __half *k_src, const __half *v_src, int src_offset,
                            int first_token, int n_tokens, int64_t sb, int64_t sh, int64_t stt, cudaStream_t st);
+int launch_append_edges(const Params &p, const kvsink_cache &c, const __half *k_src, const __half *v_src, int head_first, int head_n, int rem_src,
+                        int rem_n, int64_t sb, int64_t sh, int64_t stt, cudaStream_t st);
 int launch_decode(const Params &p, const kvsink_cache &c, const kvsink_static_params *cal, int mode, const __half *q, float *out, float *lse, void *workspace,
                   size_t workspace_bytes, cudaStream_t st);
 int launch_prefill_b2(const Params &p, const kvsink_cache &c, const __half *q, int T, int q_pos0, int64_t sb, int64_t sh, int64_t stt, float *out,

@@ -351,6 +351,211 @@ append_one_kernel(Params p, kvsink_cache c, const __half *__restrict__ k_src, co
     }
 }
 
+// ---------------------------------------------------------------------------------------------------------
+// The ragged edges of a chunk in one kernel: the tokens that complete (or extend) an open group, the flush of that group's
+// keys, and the tokens behind the last whole group.  One block per (sequence, KV head, 64 channels) has the keys; one per tile
+// touched the values.  Latency bound (a few rows per block), so it is one launch instead of three that wait for one another: a 2779-token
+// chunk that starts inside a group, 5 x 8 units at 3 bit, had 12 us of head tokens and 7 us of flush before its whole groups.
+// ---------------------------------------------------------------------------------------------------------
+constexpr int QE_THREADS = 256, QE_CH = 64, QE_SHARE = QE_THREADS / QE_CH;
+
+struct EdgeShape {
+    int head_first, head_n, flush;             // tokens inside the open group; whether they complete it
+    int rem_first, rem_n, rem_src;             // tokens behind the last whole group (at a group boundary), offset of the first in the source
+    int head_tiles;                            // tiles the head tokens touch
+};
+
+__global__ void __launch_bounds__(QE_THREADS)
+append_edges_kernel(Params p, kvsink_cache c, const __half *__restrict__ k_src, const __half *__restrict__ v_src, EdgeShape e, int64_t sb, int64_t sh,
+                    int64_t stt)
+{
+    extern __shared__ __align__(16) unsigned char dyn[];
+    __shared__ float part[QE_SHARE][2][QE_CH]; // keys: extremes of the row quarters; then scale, zero
+    __shared__ uint8_t flag[128];              // keys: sink flags of the open group; values: tokens of the tile that are new
+    __shared__ uint8_t vcode[KVSINK_TILE * 128];
+    const int D = p.D, G = p.G, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int h = blockIdx.y, b = blockIdx.z;
+    const int64_t unit = (int64_t)b * p.Hkv + h, src0 = b * sb + h * sh;
+    const float qmax = (float)((1 << p.bits) - 1);
+    const uint32_t *bm = c.sink_bitmask + (size_t)b * p.mask_words;
+    const int32_t *sink_pos = c.sink_pos + (size_t)b * p.cap;
+    pdl_wait();
+    // what follows in the stream may start: the whole groups' kernel, which touches nothing this one writes, at once
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (!in_bounds(e.head_first >= 0 && e.head_first + e.head_n <= p.max_seq && (e.rem_n == 0 || e.rem_first + e.rem_n <= p.max_seq), c.status)) return;
+    const int count = min(c.sink_count[b], p.cap);
+
+    const int slices = D / QE_CH;
+    if ((int)blockIdx.x < slices) {            // ---- keys: a slice of 64 channels ----
+        constexpr int CHUNKS = QE_CH / 8, RS = QE_CH + 8;
+        const int c0 = (int)blockIdx.x * QE_CH, old = e.head_first % G;               // rows of the open group that the tail holds
+        __half *tail = (__half *)c.k_tail + (size_t)unit * G * D + c0;
+        const __half *src = k_src + src0 + c0;
+        if (e.flush) {
+            __half *Kt = (__half *)dyn;        // [G][RS]
+            uint8_t *code = (uint8_t *)(Kt + (size_t)G * RS);                         // [G][QE_CH]
+            const int g0 = e.head_first - old;
+            for (int idx = tid; idx < G * CHUNKS; idx += QE_THREADS) {
+                const int t = idx / CHUNKS, ch = (idx % CHUNKS) * 8;
+                const __half *row = t < old ? tail + (size_t)t * D : src + (int64_t)(t - old) * stt;
+                *(uint4 *)(Kt + (size_t)t * RS + ch) = *(const uint4 *)(row + ch);
+            }
+            for (int t = tid; t < G; t += QE_THREADS) flag[t] = mask_bit(bm, g0 + t) ? 1 : 0;
+            __syncthreads();
+            // extremes per channel: four threads with a share of the rows each, then one thread per channel
+            const int ch = tid % QE_CH, qt = tid / QE_CH;
+            float mn = INFINITY, mx = -INFINITY;
+            for (int t = qt; t < G; t += QE_SHARE)
+                if (!flag[t]) {
+                    const float x = __half2float(Kt[(size_t)t * RS + ch]);
+                    mn = fminf(mn, x);
+                    mx = fmaxf(mx, x);
+                }
+            part[qt][0][ch] = mn;
+            part[qt][1][ch] = mx;
+            __syncthreads();
+            if (tid < QE_CH) {
+                for (int i = 1; i < QE_SHARE; ++i) {
+                    mn = fminf(mn, part[i][0][tid]);
+                    mx = fmaxf(mx, part[i][1][tid]);
+                }
+                float s, z;
+                group_params(mn <= mx, mn, mx, qmax, &s, &z);                          // no member: +inf, -inf
+                part[0][0][tid] = s;
+                part[0][1][tid] = z;
+                const size_t o = ((size_t)unit * (p.max_seq / G) + g0 / G) * D + c0 + tid;
+                c.k_scale[o] = s;
+                c.k_zero[o] = z;
+            }
+            __syncthreads();
+            const float s = part[0][0][ch], z = part[0][1][ch];
+            for (int t = qt; t < G; t += QE_SHARE)
+                code[t * QE_CH + ch] = flag[t] ? 0 : (uint8_t)code_exact(__half2float(Kt[(size_t)t * RS + ch]), s, z, qmax);
+            __syncthreads();
+            // the slice's words: per tile and lane two words of a 2-bit section, four of a 4-bit one, one of the 3-bit high section
+            uint32_t *out = (uint32_t *)(c.k_codes + (size_t)unit * p.max_seq * p.row_bytes + (size_t)(g0 / KVSINK_TILE) * p.tile_bytes);
+            const int tile_words = p.tile_bytes / 4, per_lane = p.bits, fields = p.bits == 4 ? 4 : 8, lo_words = p.bits == 4 ? 4 : 2;
+            const int n_lo = D * (p.bits == 4 ? 4 : 2) / 64;
+            for (int idx = tid; idx < G / KVSINK_TILE * 32 * per_lane; idx += QE_THREADS) {
+                const int ln = idx % 32, i = idx / 32 % per_lane, tile = idx / (32 * per_lane);
+                const uint8_t *rows = code + tile * KVSINK_TILE * QE_CH;
+                uint32_t word = 0;
+                int m, row, col;
+                if (i < lo_words) {
+                    for (int k = 0; k < fields; ++k)
+                        for (int x = 0; x < 2; ++x) {
+                            slot_to_elem(ln, fields * i + k, x, &m, &row, &col);
+                            word |= (rows[row * QE_CH + 16 * m + col] & (p.bits == 4 ? 15u : 3u)) << (16 * x + (p.bits == 4 ? 4 : 2) * k);
+                        }
+                    out[tile * tile_words + section_word_offset(n_lo, ln, lo_words * (int)blockIdx.x + i)] = word;
+                } else {
+                    for (int k = 0; k < 16; ++k)
+                        for (int x = 0; x < 2; ++x) {
+                            slot_to_elem(ln, k, x, &m, &row, &col);
+                            const int w = k >> 3, f = k & 7;
+                            word |= (uint32_t)((rows[row * QE_CH + 16 * m + col] >> 2) & 1) << (16 * x + 4 * (f >> 1) + 2 * (1 - w) + (f & 1));
+                        }
+                    out[tile * tile_words + 32 * n_lo + section_word_offset(D / 64, ln, (int)blockIdx.x)] = word;
+                }
+            }
+        }
+        // rows to the tail, as if token by token: those behind the last whole group lie over a completed group's
+        for (int idx = tid; idx < e.head_n * CHUNKS; idx += QE_THREADS) {
+            const int t = idx / CHUNKS, ch = (idx % CHUNKS) * 8;
+            if (!e.flush || old + t >= e.rem_n) *(uint4 *)(tail + (size_t)(old + t) * D + ch) = __ldg((const uint4 *)(src + (int64_t)t * stt + ch));
+        }
+        for (int idx = tid; idx < e.rem_n * CHUNKS; idx += QE_THREADS) {
+            const int t = idx / CHUNKS, ch = (idx % CHUNKS) * 8;
+            *(uint4 *)(tail + (size_t)t * D + ch) = __ldg((const uint4 *)(src + (int64_t)(e.rem_src + t) * stt + ch));
+        }
+        for (int i = warp; i < e.head_n + e.rem_n; i += QE_THREADS / 32) {            // exact rows of sink tokens
+            const int pos = i < e.head_n ? e.head_first + i : e.rem_first + i - e.head_n;
+            if (!mask_bit(bm, pos)) continue;
+            const int slot = find_slot(sink_pos, count, pos);
+            if (slot < 0) continue;                                                   // the values' block reports it
+            const __half *row = src + (int64_t)(i < e.head_n ? i : e.rem_src + i - e.head_n) * stt;
+            __half *dk = (__half *)c.sink_k + ((size_t)unit * p.cap + slot) * D + c0;
+            if (lane < CHUNKS) *(uint4 *)(dk + lane * 8) = __ldg((const uint4 *)(row + lane * 8));
+        }
+        return;
+    }
+
+    // ---- values of one tile ----
+    const int vt = (int)blockIdx.x - slices;
+    const bool head = vt < e.head_tiles;
+    const int first = head ? e.head_first : e.rem_first, n = head ? e.head_n : e.rem_n, offset = head ? 0 : e.rem_src;
+    const int tile = first / KVSINK_TILE + vt - (head ? 0 : e.head_tiles);
+    const int t_lo = max(first, tile * KVSINK_TILE), t_hi = min(first + n, (tile + 1) * KVSINK_TILE);
+    if (tid < KVSINK_TILE) flag[tid] = (tile * KVSINK_TILE + tid >= t_lo && tile * KVSINK_TILE + tid < t_hi) ? 1 : 0;
+    const int cpl = D / 32;   // channels per lane (2 or 4)
+    for (int pos = t_lo + warp; pos < t_hi; pos += QE_THREADS / 32) {
+        const __half *row = v_src + src0 + (int64_t)(offset + pos - first) * stt + lane * cpl;
+        __half2 v2[2];
+        v2[0] = *(const __half2 *)row;
+        v2[1] = cpl == 4 ? *(const __half2 *)(row + 2) : v2[0];
+        const float2 lo = __half22float2(v2[0]), hi = __half22float2(v2[1]);
+        const float x[4] = {lo.x, lo.y, hi.x, hi.y};
+        const bool sink = mask_bit(bm, pos);
+        if (sink) {
+            const int slot = find_slot(sink_pos, count, pos);
+            if (slot < 0) {
+                if (lane == 0) atomicOr(c.status, KVSINK_STATUS_SINK_MISMATCH);
+            } else {
+                __half2 *dv = (__half2 *)((__half *)c.sink_v + ((size_t)unit * p.cap + slot) * D + lane * cpl);
+                dv[0] = v2[0];
+                if (cpl == 4) dv[1] = v2[1];
+            }
+        }
+        float mn = fminf(x[0], x[1]), mx = fmaxf(x[0], x[1]);
+        mn = fminf(mn, fminf(x[2], x[3]));
+        mx = fmaxf(mx, fmaxf(x[2], x[3]));
+        const int lanes_per_group = p.Gv / cpl;
+        for (int o = 1; o < lanes_per_group; o <<= 1) {
+            mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        }
+        float s, z;
+        group_params(!sink, mn, mx, qmax, &s, &z);
+        if (lane % lanes_per_group == 0) {
+            const size_t o = ((size_t)unit * p.max_seq + pos) * p.NGv + lane / lanes_per_group;
+            c.v_scale[o] = s;
+            c.v_zero[o] = z;
+        }
+        for (int i = 0; i < cpl; ++i) vcode[(pos % KVSINK_TILE) * D + lane * cpl + i] = sink ? 0 : (uint8_t)code_exact(x[i], s, z, qmax);
+    }
+    __syncthreads();
+    // the new tokens' fields; fields of other tokens keep their bits, a fresh tile is written whole
+    const int tile_words = p.tile_bytes / 4;
+    uint32_t *vout = (uint32_t *)(c.v_codes + (size_t)unit * p.max_seq * p.row_bytes + (size_t)tile * p.tile_bytes);
+    const bool fresh = t_lo % KVSINK_TILE == 0;
+    for (int word = tid; word < tile_words; word += QE_THREADS) {
+        const uint32_t keep = fresh ? 0u : vout[word];
+        uint32_t fieldmask;
+        const uint32_t newbits = assemble_word_masked(p.bits, D, word, [&](int m, int row, int col) {
+            return flag[col] ? (uint32_t)vcode[col * D + 16 * m + row] : 0x100u; }, &fieldmask);
+        if (fieldmask || fresh) vout[word] = (keep & ~fieldmask) | newbits;
+    }
+}
+
+// Groups of more than 128 tokens keep the kernels that go token by token (the group would not fit a block's shared memory).
+int launch_append_edges(const Params &p, const kvsink_cache &c, const __half *k_src, const __half *v_src, int head_first, int head_n, int rem_src,
+                        int rem_n, int64_t sb, int64_t sh, int64_t stt, cudaStream_t st)
+{
+    if (p.G > 128) return KVSINK_ERR_UNSUPPORTED;
+    auto tiles = [](int first, int n) { return n > 0 ? (first + n - 1) / KVSINK_TILE - first / KVSINK_TILE + 1 : 0; };
+    EdgeShape e;
+    e.head_first = head_first;
+    e.head_n = head_n;
+    e.flush = head_n > 0 && (head_first + head_n) % p.G == 0;
+    e.rem_first = head_first + rem_src;
+    e.rem_n = rem_n;
+    e.rem_src = rem_src;
+    e.head_tiles = tiles(head_first, head_n);
+    const dim3 grid(p.D / QE_CH + e.head_tiles + tiles(e.rem_first, rem_n), p.Hkv, p.B);
+    const size_t smem = e.flush ? (size_t)p.G * ((QE_CH + 8) * 2 + QE_CH) : 0;
+    return launch_pdl(append_edges_kernel, grid, dim3(QE_THREADS), smem, st, p, c, k_src, v_src, e, sb, sh, stt) == cudaSuccess ? KVSINK_OK : KVSINK_ERR_CUDA;
+}
+
 int launch_quantize_tokens(const Params &p, const kvsink_cache &c, const __half *k_src, const __half *v_src, int src_offset,
                            int first_token, int n_tokens, int64_t sb, int64_t sh, int64_t stt, cudaStream_t st)
 {

@@ -249,6 +249,7 @@ __device__ __forceinline__ void qb_pack_matrix(const uint32_t (&pc)[4], int m, u
 struct QbShape {
     int first_token, n_groups;
     unsigned n_items;
+    int after_edges;     // launched behind append_edges_kernel of the same call
 };
 
 template <int G, int BITS = 2>
@@ -374,7 +375,10 @@ quantize_bulk_kernel(Params p, kvsink_cache c, const __grid_constant__ CUtensorM
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();   // the only block-wide barrier
-    pdl_wait();        // nothing before this line touches global memory
+    // nothing before this line touches global memory.  Behind the kernel of the same chunk's ragged edges, which writes nothing
+    // that is read here and let this one start only once everything before it had completed, the wait comes at the end
+    // instead (so that what follows still finds the edges done)
+    if (!sh.after_edges) pdl_wait();
     if (!in_bounds(sh.first_token >= 0 && (long long)sh.first_token + (long long)sh.n_groups * G <= p.max_seq, c.status)) return;   // every thread alike
     if (smem_addr(smem) & 1023u) {   // the swizzle pattern of the stages assumes 1024-byte alignment
         if (tid == 0) atomicOr(c.status, KVSINK_STATUS_TIMEOUT);
@@ -831,6 +835,7 @@ quantize_bulk_kernel(Params p, kvsink_cache c, const __grid_constant__ CUtensorM
         nxt = nn;
         mw = mw_next;
     }
+    if (sh.after_edges) pdl_wait();
 }
 
 // ---- host side ----
@@ -870,7 +875,7 @@ bool make_map(CUtensorMap *tm, const __half *base, const Params &p, int T, int64
 
 template <int BITS, int G, int MODE = 0>
 int launch_bulk(const Params &p, const kvsink_cache &c, const kvsink_static_params &sp, const __half *k_src, const __half *v_src, int first_token,
-                int n_groups, int64_t sb, int64_t sh, int64_t stt, cudaStream_t st)
+                int n_groups, int64_t sb, int64_t sh, int64_t stt, cudaStream_t st, bool after_edges = false)
 {
     using Geo = QbGeo<G, BITS>;
     CUtensorMap tm_k, tm_v;
@@ -888,6 +893,7 @@ int launch_bulk(const Params &p, const kvsink_cache &c, const kvsink_static_para
     QbShape shp;
     shp.first_token = first_token;
     shp.n_groups = n_groups;
+    shp.after_edges = after_edges;
     const long n_items = (long)p.B * p.Hkv * n_groups * Geo::IPG;
     if (n_items >= (1L << 30)) return KVSINK_ERR_UNSUPPORTED;
     shp.n_items = (unsigned)n_items;
@@ -901,15 +907,15 @@ int launch_bulk(const Params &p, const kvsink_cache &c, const kvsink_static_para
 // Whole groups of a bulk append (keys, values and sink rows).  Returns KVSINK_ERR_UNSUPPORTED when the shape has no
 // kernel of this kind or the inputs cannot be described by a tensor map; the caller then uses another kernel.
 int launch_quantize_groups_bulk(const Params &p, const kvsink_cache &c, const __half *k_src, const __half *v_src, int first_token,
-                                int n_groups, int64_t sb, int64_t sh, int64_t stt, cudaStream_t st)
+                                int n_groups, int64_t sb, int64_t sh, int64_t stt, bool after_edges, cudaStream_t st)
 {
     if (p.D != QB_D || n_groups < 1) return KVSINK_ERR_UNSUPPORTED;
     const kvsink_static_params none = {nullptr, nullptr, nullptr, nullptr};
-    if (p.bits == 2 && p.G == 128) return launch_bulk<2, 128>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st);
-    if (p.bits == 2 && p.G == 64) return launch_bulk<2, 64>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st);
-    if (p.bits == 3 && p.G == 64) return launch_bulk<3, 64>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st);
-    if (p.bits == 4 && p.G == 128) return launch_bulk<4, 128>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st);
-    if (p.bits == 4 && p.G == 64) return launch_bulk<4, 64>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st);
+    if (p.bits == 2 && p.G == 128) return launch_bulk<2, 128>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, after_edges);
+    if (p.bits == 2 && p.G == 64) return launch_bulk<2, 64>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, after_edges);
+    if (p.bits == 3 && p.G == 64) return launch_bulk<3, 64>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, after_edges);
+    if (p.bits == 4 && p.G == 128) return launch_bulk<4, 128>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, after_edges);
+    if (p.bits == 4 && p.G == 64) return launch_bulk<4, 64>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, after_edges);
     return KVSINK_ERR_UNSUPPORTED;
 }
 

@@ -1,0 +1,42 @@
+"""GPU parity of appends whose ragged ends (tokens that extend or complete an open group, tokens behind the last whole group)
+go through one kernel ahead of the whole groups': every cache array bit for bit against the CPU oracle."""
+import pytest
+import torch
+
+import oracle
+import paper_2508_04257_b200 as kv
+from paper_2508_04257_b200 import synth
+
+from parity_util import CACHE_BUFFERS, SINK_BUFFERS, check_guards, compare_cache, configs, guard, np16
+
+pytestmark = pytest.mark.gpu
+TINY = synth.WORKLOADS["tiny"]
+
+
+# chunk ends: inside the open group, on its end, with whole groups behind, with a remainder shorter and longer than the head's slots
+@pytest.mark.parametrize("bits,d,group", [(2, 128, 128), (3, 128, 64), (4, 128, 64), (2, 128, 32), (3, 128, 128), (4, 64, 32), (2, 64, 64)])
+@pytest.mark.parametrize("cuts", [(0.3, 0.7), (0.9, 1.0), (0.4, 3.2), (0.6, 2.95), (1.0, 2.03), (0.02, 4.0)])
+def test_chunks(bits, d, group, cuts):
+    ends = [max(1, int(x * group)) for x in cuts] + [5 * group + 3]
+    seq = ends[-1]
+    wl = TINY.scaled(bits=bits, head_dim=d, group=group, n_q_heads=6, n_kv_heads=3, batch=2, seq=seq, topk=min(seq, 9 + group // 4), pfn_n=2,
+                     seed=31000 + bits * 1000 + d + group + ends[1])
+    ocfg, gcfg = configs(wl)
+    H = synth.make_hidden(wl, "cuda")
+    K, V = synth.make_kv(wl, 0, "cuda")
+    gs = guard(kv.SinkSet(gcfg), SINK_BUFFERS)
+    kv.predict_sinks(gcfg, H, gs)
+    gc = guard(kv.KVCache(gcfg, gs), CACHE_BUFFERS)
+    bm, pos, cnt = oracle.predict_sinks(ocfg, np16(H))
+    oc = oracle.Cache(ocfg, bm, pos, cnt)
+    at = 0
+    for end in ends:
+        # [B, T, Hkv, D] storage for every other chunk
+        k, v = (x[:, :, at:end] if at % 2 else x[:, :, at:end].permute(0, 2, 1, 3).contiguous().permute(0, 2, 1, 3) for x in (K, V))
+        kv.quantize_append(gcfg, gc, k, v)
+        oracle.quantize_append(ocfg, oc, np16(K[:, :, at:end]), np16(V[:, :, at:end]))
+        compare_cache(gc, oc, wl, f"after {end} tokens: ")
+        at = end
+    assert kv.read_status(gc) == 0
+    check_guards(gs)
+    check_guards(gc)
