@@ -30,9 +30,12 @@ class KvsinkError(RuntimeError):
         super().__init__(f"{what}: {strerror(code)} ({code})")
 
 
+_Channels = C.c_int32 * 8
+
+
 class _Cfg(C.Structure):
     _fields_ = [(n, C.c_int32) for n in ("batch", "n_q_heads", "n_kv_heads", "head_dim", "hidden", "bits", "group",
-                                         "max_seq", "topk", "pfn_n", "n_channels")] + [("channels", C.c_int32 * 8)]
+                                         "max_seq", "topk", "pfn_n", "n_channels")] + [("channels", _Channels)]
 
 
 class _Cache(C.Structure):
@@ -49,6 +52,26 @@ class _Sizes(C.Structure):
                [(n, C.c_int32) for n in ("sink_capacity", "v_group", "v_groups_per_row", "tile_bytes")]
 
 
+_P, _I, _L, _Z = C.c_void_p, C.c_int32, C.c_int64, C.c_size_t
+# argument types of the entry points, so that plain integers (addresses, sizes, strides) are converted by the foreign call itself
+_ARGS = {
+    "kvsink_cache_sizes": (_P, _P),
+    "kvsink_predict_sinks": (_P, _P, _I, _L, _L, _P, _P, _P, _P, _Z, _P),
+    "kvsink_quantize_append": (_P, _P, _P, _P, _I, _L, _L, _L, _P),
+    "kvsink_decode_attention": (_P, _P, _P, _P, _P, _P, _Z, _P),
+    "kvsink_decode_attention_static": (_P, _P, _P, _P, _P, _P),
+    "kvsink_prefill_attention": (_P, _P, _P, _I, _I, _L, _L, _L, _P, _P, _P),
+    "kvsink_calibrate": (_P, _P, _P, _I, _L, _L, _L, _P, _P, _P, _Z, _P),
+    "kvsink_quantize_append_calibrated": (_P, _P, _P, _P, _P, _I, _L, _L, _L, _P),
+    "kvsink_decode_attention_calibrated": (_P, _P, _P, _P, _P, _P, _P, _Z, _P),
+    "kvsink_quantize_append_pertoken": (_P, _P, _P, _P, _I, _L, _L, _L, _P),
+    "kvsink_decode_attention_pertoken": (_P, _P, _P, _P, _P, _P, _Z, _P),
+    "kvsink_channel_absmax": (_P, _I, _I, _I, _L, _L, _P, _P),
+    "kvsink_quant_error": (_P, _P, _I, _L, _L, _L, _I, _I, _P, _P, _P),
+    "kvsink_read_status": (_P, _P, _P),
+    "kvsink_launch_count": (),
+    "kvsink_strerror": (_I,),
+}
 _lib = None
 
 
@@ -58,11 +81,12 @@ def lib():
     if _lib is None:
         if not os.path.exists(_LIB_PATH):
             raise ImportError(f"{_LIB_PATH} is missing: build it with `python -m paper_2508_04257_b200.build`")
-        _lib = C.CDLL(_LIB_PATH)
-        _lib.kvsink_strerror.restype = C.c_char_p
-        _lib.kvsink_launch_count.restype = C.c_ulonglong
+        loaded = C.CDLL(_LIB_PATH)
+        loaded.kvsink_strerror.restype = C.c_char_p
+        loaded.kvsink_launch_count.restype = C.c_ulonglong
         for name in EXPORTS:
-            getattr(_lib, name)
+            getattr(loaded, name).argtypes = _ARGS[name]
+        _lib = loaded
     return _lib
 
 
@@ -85,7 +109,7 @@ class Config:
     channels: Sequence[int] = field(default_factory=tuple)
 
     def c(self) -> _Cfg:
-        ch = (C.c_int32 * 8)(*list(self.channels)[:8])
+        ch = _Channels(*tuple(self.channels)[:8])
         return _Cfg(self.batch, self.n_q_heads, self.n_kv_heads, self.head_dim, self.hidden, self.bits, self.group,
                     self.max_seq, self.topk, self.pfn_n, len(self.channels), ch)
 
@@ -98,12 +122,25 @@ def cache_sizes(cfg: Config) -> dict:
     return {n: getattr(s, n) for n, _ in _Sizes._fields_}
 
 
-def _stream() -> C.c_void_p:
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+_raw_stream, _device = torch._C._cuda_getCurrentRawStream, torch.cuda.current_device
 
 
-def _ptr(t: Optional[torch.Tensor]) -> C.c_void_p:
-    return C.c_void_p(0 if t is None else t.data_ptr())
+def _size(cfg: Config, name: str) -> int:
+    """One entry of cache_sizes(cfg)."""
+    s = _Sizes()
+    rc = lib().kvsink_cache_sizes(C.byref(cfg.c()), C.byref(s))
+    if rc:
+        raise KvsinkError(rc, "kvsink_cache_sizes")
+    return getattr(s, name)
+
+
+def _stream() -> int:
+    """The current stream of the current device, as torch.cuda.current_stream().cuda_stream gives it, without the object."""
+    return _raw_stream(_device())
+
+
+def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
+    return None if t is None else t.data_ptr()
 
 
 class SinkSet:
@@ -137,19 +174,19 @@ class KVCache:
 
     def c(self) -> _Cache:
         s = self.sinks
-        return _Cache(_ptr(self.k_codes), _ptr(self.v_codes), _ptr(self.k_scale), _ptr(self.k_zero), _ptr(self.v_scale),
-                      _ptr(self.v_zero), _ptr(self.k_tail), _ptr(self.sink_k), _ptr(self.sink_v), _ptr(s.bitmask), _ptr(s.pos),
-                      _ptr(s.count), _ptr(self.status), self.seq_len)
+        return _Cache(self.k_codes.data_ptr(), self.v_codes.data_ptr(), self.k_scale.data_ptr(), self.k_zero.data_ptr(), self.v_scale.data_ptr(),
+                      self.v_zero.data_ptr(), self.k_tail.data_ptr(), self.sink_k.data_ptr(), self.sink_v.data_ptr(), s.bitmask.data_ptr(),
+                      s.pos.data_ptr(), s.count.data_ptr(), self.status.data_ptr(), self.seq_len)
 
 
 def predict_sinks(cfg: Config, hidden: torch.Tensor, sinks: SinkSet, workspace: Optional[torch.Tensor] = None) -> SinkSet:
     """kvsink_predict_sinks: hidden fp16 [B, S, d] on the device (last axis contiguous)."""
     assert hidden.is_cuda and hidden.dtype == torch.float16 and hidden.dim() == 3 and hidden.stride(2) == 1
     if workspace is None:
-        workspace = torch.empty(cache_sizes(cfg)["predict_workspace_bytes"], dtype=torch.uint8, device=hidden.device)
-    rc = lib().kvsink_predict_sinks(C.byref(cfg.c()), _ptr(hidden), C.c_int32(hidden.shape[1]), C.c_int64(hidden.stride(0)),
-                                    C.c_int64(hidden.stride(1)), _ptr(sinks.bitmask), _ptr(sinks.pos), _ptr(sinks.count),
-                                    _ptr(workspace), C.c_size_t(workspace.numel()), _stream())
+        workspace = hidden.new_empty(_size(cfg, "predict_workspace_bytes"), dtype=torch.uint8)
+    rc = lib().kvsink_predict_sinks(C.byref(cfg.c()), _ptr(hidden), hidden.shape[1], hidden.stride(0),
+                                    hidden.stride(1), _ptr(sinks.bitmask), _ptr(sinks.pos), _ptr(sinks.count),
+                                    _ptr(workspace), workspace.numel(), _stream())
     if rc:
         raise KvsinkError(rc, "kvsink_predict_sinks")
     return sinks
@@ -160,8 +197,8 @@ def quantize_append(cfg: Config, cache: KVCache, k_new: torch.Tensor, v_new: tor
     assert k_new.is_cuda and k_new.dtype == torch.float16 and k_new.dim() == 4 and k_new.stride(3) == 1
     assert v_new.shape == k_new.shape and v_new.stride() == k_new.stride() and v_new.dtype == torch.float16
     cc = cache.c()
-    rc = lib().kvsink_quantize_append(C.byref(cfg.c()), C.byref(cc), _ptr(k_new), _ptr(v_new), C.c_int32(k_new.shape[2]),
-                                      C.c_int64(k_new.stride(0)), C.c_int64(k_new.stride(1)), C.c_int64(k_new.stride(2)), _stream())
+    rc = lib().kvsink_quantize_append(C.byref(cfg.c()), C.byref(cc), _ptr(k_new), _ptr(v_new), k_new.shape[2],
+                                      k_new.stride(0), k_new.stride(1), k_new.stride(2), _stream())
     if rc:
         raise KvsinkError(rc, "kvsink_quantize_append")
     cache.seq_len = cc.seq_len
@@ -172,14 +209,14 @@ def decode_attention(cfg: Config, cache: KVCache, q: torch.Tensor, out: Optional
     """kvsink_decode_attention: q fp16 [B, Hq, D] contiguous. Returns (out fp32 [B,Hq,D], lse fp32 [B,Hq] or None)."""
     assert q.is_cuda and q.dtype == torch.float16 and q.is_contiguous()
     if out is None:
-        out = torch.empty((cfg.batch, cfg.n_q_heads, cfg.head_dim), dtype=torch.float32, device=q.device)
+        out = q.new_empty((cfg.batch, cfg.n_q_heads, cfg.head_dim), dtype=torch.float32)
     if lse is None and want_lse:
-        lse = torch.empty((cfg.batch, cfg.n_q_heads), dtype=torch.float32, device=q.device)
+        lse = q.new_empty((cfg.batch, cfg.n_q_heads), dtype=torch.float32)
     if workspace is None:
-        workspace = torch.empty(cache.sizes["decode_workspace_bytes"], dtype=torch.uint8, device=q.device)
+        workspace = q.new_empty(cache.sizes["decode_workspace_bytes"], dtype=torch.uint8)
     cc = cache.c()
     rc = lib().kvsink_decode_attention(C.byref(cfg.c()), C.byref(cc), _ptr(q), _ptr(out), _ptr(lse), _ptr(workspace),
-                                       C.c_size_t(workspace.numel()), _stream())
+                                       workspace.numel(), _stream())
     if rc:
         raise KvsinkError(rc, "kvsink_decode_attention")
     return out, lse
@@ -192,12 +229,12 @@ def prefill_attention(cfg: Config, cache: KVCache, q: torch.Tensor, q_pos0: int,
     assert q.is_cuda and q.dtype == torch.float16 and q.dim() == 4 and q.stride(3) == 1
     T = q.shape[2]
     if out is None:
-        out = torch.empty((cfg.batch, cfg.n_q_heads, T, cfg.head_dim), dtype=torch.float32, device=q.device)
+        out = q.new_empty((cfg.batch, cfg.n_q_heads, T, cfg.head_dim), dtype=torch.float32)
     if lse is None and want_lse:
-        lse = torch.empty((cfg.batch, cfg.n_q_heads, T), dtype=torch.float32, device=q.device)
+        lse = q.new_empty((cfg.batch, cfg.n_q_heads, T), dtype=torch.float32)
     cc = cache.c()
-    rc = lib().kvsink_prefill_attention(C.byref(cfg.c()), C.byref(cc), _ptr(q), C.c_int32(T), C.c_int32(q_pos0), C.c_int64(q.stride(0)),
-                                        C.c_int64(q.stride(1)), C.c_int64(q.stride(2)), _ptr(out), _ptr(lse), _stream())
+    rc = lib().kvsink_prefill_attention(C.byref(cfg.c()), C.byref(cc), _ptr(q), T, q_pos0, q.stride(0),
+                                        q.stride(1), q.stride(2), _ptr(out), _ptr(lse), _stream())
     if rc:
         raise KvsinkError(rc, "kvsink_prefill_attention")
     return out, lse
@@ -243,11 +280,11 @@ def calibrate(cfg: Config, k_cal: torch.Tensor, v_cal: torch.Tensor, sinks: Sink
     assert v_cal.shape == k_cal.shape and v_cal.stride() == k_cal.stride() and v_cal.dtype == torch.float16
     if params is None:
         params = StaticParams(cfg, k_cal.device)
-    ws = torch.empty(cache_sizes(cfg)["calibrate_workspace_bytes"], dtype=torch.uint8, device=k_cal.device)
+    ws = k_cal.new_empty(_size(cfg, "calibrate_workspace_bytes"), dtype=torch.uint8)
     cs = params.c()
-    rc = lib().kvsink_calibrate(C.byref(cfg.c()), _ptr(k_cal), _ptr(v_cal), C.c_int32(k_cal.shape[2]), C.c_int64(k_cal.stride(0)),
-                                C.c_int64(k_cal.stride(1)), C.c_int64(k_cal.stride(2)), _ptr(sinks.bitmask), C.byref(cs), _ptr(ws),
-                                C.c_size_t(ws.numel()), _stream())
+    rc = lib().kvsink_calibrate(C.byref(cfg.c()), _ptr(k_cal), _ptr(v_cal), k_cal.shape[2], k_cal.stride(0),
+                                k_cal.stride(1), k_cal.stride(2), _ptr(sinks.bitmask), C.byref(cs), _ptr(ws),
+                                ws.numel(), _stream())
     if rc:
         raise KvsinkError(rc, "kvsink_calibrate")
     return params
@@ -258,8 +295,8 @@ def quantize_append_calibrated(cfg: Config, cache: KVCache, params: StaticParams
     assert k_new.is_cuda and k_new.dtype == torch.float16 and k_new.dim() == 4 and k_new.stride(3) == 1
     assert v_new.shape == k_new.shape and v_new.stride() == k_new.stride() and v_new.dtype == torch.float16
     cc, cs = cache.c(), params.c()
-    rc = lib().kvsink_quantize_append_calibrated(C.byref(cfg.c()), C.byref(cc), C.byref(cs), _ptr(k_new), _ptr(v_new), C.c_int32(k_new.shape[2]),
-                                                 C.c_int64(k_new.stride(0)), C.c_int64(k_new.stride(1)), C.c_int64(k_new.stride(2)), _stream())
+    rc = lib().kvsink_quantize_append_calibrated(C.byref(cfg.c()), C.byref(cc), C.byref(cs), _ptr(k_new), _ptr(v_new), k_new.shape[2],
+                                                 k_new.stride(0), k_new.stride(1), k_new.stride(2), _stream())
     if rc:
         raise KvsinkError(rc, "kvsink_quantize_append_calibrated")
     cache.seq_len = cc.seq_len
@@ -270,14 +307,14 @@ def decode_attention_calibrated(cfg: Config, cache: KVCache, params: StaticParam
     """kvsink_decode_attention_calibrated: q fp16 [B, Hq, D] contiguous. Returns (out fp32 [B,Hq,D], lse fp32 [B,Hq] or None)."""
     assert q.is_cuda and q.dtype == torch.float16 and q.is_contiguous()
     if out is None:
-        out = torch.empty((cfg.batch, cfg.n_q_heads, cfg.head_dim), dtype=torch.float32, device=q.device)
+        out = q.new_empty((cfg.batch, cfg.n_q_heads, cfg.head_dim), dtype=torch.float32)
     if lse is None and want_lse:
-        lse = torch.empty((cfg.batch, cfg.n_q_heads), dtype=torch.float32, device=q.device)
+        lse = q.new_empty((cfg.batch, cfg.n_q_heads), dtype=torch.float32)
     if workspace is None:
-        workspace = torch.empty(cache.sizes["decode_workspace_bytes"], dtype=torch.uint8, device=q.device)
+        workspace = q.new_empty(cache.sizes["decode_workspace_bytes"], dtype=torch.uint8)
     cc, cs = cache.c(), params.c()
     rc = lib().kvsink_decode_attention_calibrated(C.byref(cfg.c()), C.byref(cc), C.byref(cs), _ptr(q), _ptr(out), _ptr(lse), _ptr(workspace),
-                                                  C.c_size_t(workspace.numel()), _stream())
+                                                  workspace.numel(), _stream())
     if rc:
         raise KvsinkError(rc, "kvsink_decode_attention_calibrated")
     return out, lse
@@ -289,8 +326,8 @@ def quantize_append_pertoken(cfg: Config, cache: KVCache, k_new: torch.Tensor, v
     assert k_new.is_cuda and k_new.dtype == torch.float16 and k_new.dim() == 4 and k_new.stride(3) == 1
     assert v_new.shape == k_new.shape and v_new.stride() == k_new.stride() and v_new.dtype == torch.float16
     cc = cache.c()
-    rc = lib().kvsink_quantize_append_pertoken(C.byref(cfg.c()), C.byref(cc), _ptr(k_new), _ptr(v_new), C.c_int32(k_new.shape[2]),
-                                               C.c_int64(k_new.stride(0)), C.c_int64(k_new.stride(1)), C.c_int64(k_new.stride(2)), _stream())
+    rc = lib().kvsink_quantize_append_pertoken(C.byref(cfg.c()), C.byref(cc), _ptr(k_new), _ptr(v_new), k_new.shape[2],
+                                               k_new.stride(0), k_new.stride(1), k_new.stride(2), _stream())
     if rc:
         raise KvsinkError(rc, "kvsink_quantize_append_pertoken")
     cache.seq_len = cc.seq_len
@@ -302,14 +339,14 @@ def decode_attention_pertoken(cfg: Config, cache: KVCache, q: torch.Tensor, out:
     assert cache.per_token_keys, "the cache was not sized for per-token key parameters"
     assert q.is_cuda and q.dtype == torch.float16 and q.is_contiguous()
     if out is None:
-        out = torch.empty((cfg.batch, cfg.n_q_heads, cfg.head_dim), dtype=torch.float32, device=q.device)
+        out = q.new_empty((cfg.batch, cfg.n_q_heads, cfg.head_dim), dtype=torch.float32)
     if lse is None and want_lse:
-        lse = torch.empty((cfg.batch, cfg.n_q_heads), dtype=torch.float32, device=q.device)
+        lse = q.new_empty((cfg.batch, cfg.n_q_heads), dtype=torch.float32)
     if workspace is None:
-        workspace = torch.empty(cache.sizes["decode_workspace_bytes"], dtype=torch.uint8, device=q.device)
+        workspace = q.new_empty(cache.sizes["decode_workspace_bytes"], dtype=torch.uint8)
     cc = cache.c()
     rc = lib().kvsink_decode_attention_pertoken(C.byref(cfg.c()), C.byref(cc), _ptr(q), _ptr(out), _ptr(lse), _ptr(workspace),
-                                                C.c_size_t(workspace.numel()), _stream())
+                                                workspace.numel(), _stream())
     if rc:
         raise KvsinkError(rc, "kvsink_decode_attention_pertoken")
     return out, lse
@@ -320,8 +357,8 @@ def channel_absmax(hidden: torch.Tensor, out: Optional[torch.Tensor] = None) -> 
     assert hidden.is_cuda and hidden.dtype == torch.float16 and hidden.dim() == 3 and hidden.stride(2) == 1
     if out is None:
         out = torch.empty(hidden.shape[2], dtype=torch.float32, device=hidden.device)
-    rc = lib().kvsink_channel_absmax(_ptr(hidden), C.c_int32(hidden.shape[0]), C.c_int32(hidden.shape[1]), C.c_int32(hidden.shape[2]),
-                                     C.c_int64(hidden.stride(0)), C.c_int64(hidden.stride(1)), _ptr(out), _stream())
+    rc = lib().kvsink_channel_absmax(_ptr(hidden), hidden.shape[0], hidden.shape[1], hidden.shape[2],
+                                     hidden.stride(0), hidden.stride(1), _ptr(out), _stream())
     if rc:
         raise KvsinkError(rc, "kvsink_channel_absmax")
     return out
@@ -333,8 +370,8 @@ def quant_error(cfg: Config, x: torch.Tensor, sinks: SinkSet, per_channel: bool,
     assert x.is_cuda and x.dtype == torch.float16 and x.dim() == 4 and x.stride(3) == 1
     if out is None:
         out = torch.empty(4, dtype=torch.float64, device=x.device)
-    rc = lib().kvsink_quant_error(C.byref(cfg.c()), _ptr(x), C.c_int32(x.shape[2]), C.c_int64(x.stride(0)), C.c_int64(x.stride(1)),
-                                  C.c_int64(x.stride(2)), C.c_int32(int(per_channel)), C.c_int32(int(exclude_sinks)), _ptr(sinks.bitmask),
+    rc = lib().kvsink_quant_error(C.byref(cfg.c()), _ptr(x), x.shape[2], x.stride(0), x.stride(1),
+                                  x.stride(2), int(per_channel), int(exclude_sinks), _ptr(sinks.bitmask),
                                   _ptr(out), _stream())
     if rc:
         raise KvsinkError(rc, "kvsink_quant_error")

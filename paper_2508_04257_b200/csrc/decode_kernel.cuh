@@ -1217,7 +1217,8 @@ static int launch_decode_p(const Params &p, const kvsink_cache &c, const kvsink_
     if (qchunks * (I8 == 1 ? 1 : (PL ? 4 : 8)) < p.rep) return KVSINK_ERR_UNSUPPORTED;
     const size_t smem = DecodePlan<BITS, D, NGV, CT, I8 == 1 ? 1 : (PL ? 4 : 8), PM == 2>::BYTES;
     auto kern = decode_kernel<BITS, D, NGV, CT, PL, I8, PM>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return KVSINK_ERR_CUDA;
+    // up to 48 KB need no leave, which costs a call
+    if (smem > 48 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return KVSINK_ERR_CUDA;
     cudaLaunchAttribute pdl[2];
     pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     pdl[0].val.programmaticStreamSerializationAllowed = 1;
