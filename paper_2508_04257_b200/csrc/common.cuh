@@ -93,6 +93,9 @@ __device__ __forceinline__ uint32_t code_exact(float x, float scale, float zero,
 // may have touched.  pdl_wait() returns once every prerequisite grid has completed and its writes are visible (at once
 // when the kernel was launched the ordinary way).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// From here on the next kernel in the stream may be scheduled beside this one, up to its own wait.  Only after pdl_wait(), so
+// that a kernel that waits for this one has waited for everything before it too.
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Kernel launches made by the library since it was loaded (kvsink_launch_count).
 extern std::atomic<unsigned long long> g_launches;

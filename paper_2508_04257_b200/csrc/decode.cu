@@ -19,7 +19,8 @@ __global__ void decode_merge_kernel(const float *__restrict__ part_ws, int nspli
     const float *base = part_ws + oq * nsplit * PS;
     // launched with programmatic stream serialization: the blocks may start while the split kernel drains, and wait
     // here until all of it has completed and its records are visible
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    pdl_wait();
+    pdl_release();
     float M = M_INIT;
     for (int s = sl; s < nsplit; s += MERGE_SLICES) M = fmaxf(M, base[(size_t)s * PS + D]);
     float acc = 0.f, L = 0.f;

@@ -254,26 +254,6 @@ quantize_tokens_kernel(Params p, kvsink_cache c, const __half *__restrict__ k_sr
 // ---------------------------------------------------------------------------------------------------------
 constexpr int QA_WARPS = 4;
 
-// Word (index among the tile's 32-bit words) and bit position of the field of matrix element (m, row, col); for 3 bit
-// the low two bits, and through *hi_word / *hi_shift the high bit.
-__device__ __forceinline__ void field_place(int bits, int D, int m, int row, int col, int *word, int *shift, int *hi_word, int *hi_shift)
-{
-    const int lane = 4 * (row & 7) + ((col & 7) >> 1), e = col & 1;
-    const int s = 4 * m + (row >> 3) + 2 * (col >> 3);
-    if (bits == 3) {
-        const int nlo = D / 32, nhi = D / 64, i = s >> 3, k = s & 7;
-        *word = section_word_offset(nlo, lane, i);
-        *shift = 16 * e + 2 * k;
-        *hi_word = 32 * nlo + section_word_offset(nhi, lane, i >> 1);
-        *hi_shift = 16 * e + 4 * (k >> 1) + 2 * (1 - (i & 1)) + (k & 1);
-    } else {
-        const int n = D * bits / 64, fields = 16 / bits;
-        *word = section_word_offset(n, lane, s / fields);
-        *shift = 16 * e + bits * (s % fields);
-        *hi_word = *hi_shift = 0;
-    }
-}
-
 __global__ void __launch_bounds__(32 * QA_WARPS)
 append_one_kernel(Params p, kvsink_cache c, const __half *__restrict__ k_src, const __half *__restrict__ v_src, int src_token, int pos,
                   int64_t sb, int64_t sh, int64_t stt)
@@ -282,6 +262,7 @@ append_one_kernel(Params p, kvsink_cache c, const __half *__restrict__ k_src, co
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t unit = (int64_t)blockIdx.x * QA_WARPS + warp;
     pdl_wait();
+    pdl_release();
     if (unit >= (int64_t)p.B * p.Hkv) return;
     if (!in_bounds(pos >= 0 && pos < p.max_seq, c.status)) return;
     const int b = (int)(unit / p.Hkv), h = (int)(unit % p.Hkv);
@@ -338,16 +319,7 @@ append_one_kernel(Params p, kvsink_cache c, const __half *__restrict__ k_src, co
     }
     for (int e = 0; e < cpl; ++e) {
         const int ch = lane * cpl + e;
-        const uint32_t code = sink ? 0u : code_exact(x[e], s, z, qmax);
-        int word, shift, hi_word, hi_shift;
-        field_place(p.bits, D, ch >> 4, ch & 15, col, &word, &shift, &hi_word, &hi_shift);
-        const uint32_t lo_mask = p.bits == 3 ? 3u : (1u << p.bits) - 1u;
-        if (!fresh) atomicAnd(&vout[word], ~(lo_mask << shift));
-        if (code & lo_mask) atomicOr(&vout[word], (code & lo_mask) << shift);
-        if (p.bits == 3) {
-            if (!fresh) atomicAnd(&vout[hi_word], ~(1u << hi_shift));
-            if (code >> 2) atomicOr(&vout[hi_word], 1u << hi_shift);
-        }
+        set_field(vout, p.bits, D, ch >> 4, ch & 15, col, sink ? 0u : code_exact(x[e], s, z, qmax), fresh);
     }
 }
 
@@ -380,8 +352,7 @@ append_edges_kernel(Params p, kvsink_cache c, const __half *__restrict__ k_src, 
     const uint32_t *bm = c.sink_bitmask + (size_t)b * p.mask_words;
     const int32_t *sink_pos = c.sink_pos + (size_t)b * p.cap;
     pdl_wait();
-    // what follows in the stream may start: the whole groups' kernel, which touches nothing this one writes, at once
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    pdl_release();        // the whole groups' kernel of the same call, which touches nothing this one writes, does not even wait
     if (!in_bounds(e.head_first >= 0 && e.head_first + e.head_n <= p.max_seq && (e.rem_n == 0 || e.rem_first + e.rem_n <= p.max_seq), c.status)) return;
     const int count = min(c.sink_count[b], p.cap);
 

@@ -111,4 +111,39 @@ __device__ __forceinline__ uint32_t assemble_word_masked(int bits, int D, int wo
     return out;
 }
 
+// Word (index among the tile's 32-bit words) and bit position of the field of matrix element (m, row, col); for 3 bit
+// the low two bits, and through *hi_word / *hi_shift the high bit.
+__device__ __forceinline__ void field_place(int bits, int D, int m, int row, int col, int *word, int *shift, int *hi_word, int *hi_shift)
+{
+    const int lane = 4 * (row & 7) + ((col & 7) >> 1), e = col & 1;
+    const int s = 4 * m + (row >> 3) + 2 * (col >> 3);
+    if (bits == 3) {
+        const int nlo = D / 32, nhi = D / 64, i = s >> 3, k = s & 7;
+        *word = section_word_offset(nlo, lane, i);
+        *shift = 16 * e + 2 * k;
+        *hi_word = 32 * nlo + section_word_offset(nhi, lane, i >> 1);
+        *hi_shift = 16 * e + 4 * (k >> 1) + 2 * (1 - (i & 1)) + (k & 1);
+    } else {
+        const int n = D * bits / 64, fields = 16 / bits;
+        *word = section_word_offset(n, lane, s / fields);
+        *shift = 16 * e + bits * (s % fields);
+        *hi_word = *hi_shift = 0;
+    }
+}
+
+// Sets the field of matrix element (m, row, col) in a tile in memory with word atomics, so that nothing but it is touched; in a
+// fresh (zeroed) tile there is nothing to clear.
+__device__ __forceinline__ void set_field(uint32_t *tile, int bits, int D, int m, int row, int col, uint32_t code, bool fresh)
+{
+    int word, shift, hi_word, hi_shift;
+    field_place(bits, D, m, row, col, &word, &shift, &hi_word, &hi_shift);
+    const uint32_t lo_mask = bits == 3 ? 3u : (1u << bits) - 1u;
+    if (!fresh) atomicAnd(&tile[word], ~(lo_mask << shift));
+    if (code & lo_mask) atomicOr(&tile[word], (code & lo_mask) << shift);
+    if (bits == 3) {
+        if (!fresh) atomicAnd(&tile[hi_word], ~(1u << hi_shift));
+        if (code >> 2) atomicOr(&tile[hi_word], 1u << hi_shift);
+    }
+}
+
 }  // namespace kvsink

@@ -40,3 +40,16 @@ def test_chunks(bits, d, group, cuts):
     assert kv.read_status(gc) == 0
     check_guards(gs)
     check_guards(gc)
+
+
+# schemes without token groups (static pairs, per-token keys): chunks that start between group and tile boundaries send their whole
+# spans to the bulk kernel and whole tiles to the tile kernel; single tokens have a kernel of their own, on fresh and used tiles
+@pytest.mark.parametrize("scheme,bits,group", [("static", 2, 128), ("static", 3, 64), ("static", 4, 64), ("static", 3, 128), ("per_token", 2, 64),
+                                               ("per_token", 4, 128), ("per_token", 3, 128)])
+def test_flat_chunks(scheme, bits, group):
+    import test_gpu_calibrated
+    import test_gpu_pertoken
+    chunks = (1, 36, 2 * group + 50, 1, 2, 13, 1, group + 17, 15, 1, 1)
+    wl = TINY.scaled(bits=bits, head_dim=128, group=group, n_q_heads=3, n_kv_heads=3, batch=2, seq=sum(chunks), topk=40, pfn_n=1,
+                     seed=33000 + bits * 100 + group)
+    (test_gpu_calibrated if scheme == "static" else test_gpu_pertoken)._both(wl, chunks=chunks)
