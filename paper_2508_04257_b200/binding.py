@@ -174,9 +174,14 @@ class KVCache:
 
     def c(self) -> _Cache:
         s = self.sinks
-        return _Cache(self.k_codes.data_ptr(), self.v_codes.data_ptr(), self.k_scale.data_ptr(), self.k_zero.data_ptr(), self.v_scale.data_ptr(),
-                      self.v_zero.data_ptr(), self.k_tail.data_ptr(), self.sink_k.data_ptr(), self.sink_v.data_ptr(), s.bitmask.data_ptr(),
-                      s.pos.data_ptr(), s.count.data_ptr(), self.status.data_ptr(), self.seq_len)
+        try:
+            return _Cache(self.k_codes.data_ptr(), self.v_codes.data_ptr(), self.k_scale.data_ptr(), self.k_zero.data_ptr(), self.v_scale.data_ptr(),
+                          self.v_zero.data_ptr(), self.k_tail.data_ptr(), self.sink_k.data_ptr(), self.sink_v.data_ptr(), s.bitmask.data_ptr(),
+                          s.pos.data_ptr(), s.count.data_ptr(), self.status.data_ptr(), self.seq_len)
+        except AttributeError:      # a buffer that the scheme in use does not need may be None (the same record, a call more per buffer)
+            return _Cache(_ptr(self.k_codes), _ptr(self.v_codes), _ptr(self.k_scale), _ptr(self.k_zero), _ptr(self.v_scale), _ptr(self.v_zero),
+                          _ptr(self.k_tail), _ptr(self.sink_k), _ptr(self.sink_v), _ptr(s.bitmask), _ptr(s.pos), _ptr(s.count), _ptr(self.status),
+                          self.seq_len)
 
 
 def predict_sinks(cfg: Config, hidden: torch.Tensor, sinks: SinkSet, workspace: Optional[torch.Tensor] = None) -> SinkSet:
