@@ -122,7 +122,8 @@ def cache_sizes(cfg: Config) -> dict:
     return {n: getattr(s, n) for n, _ in _Sizes._fields_}
 
 
-_raw_stream, _device = torch._C._cuda_getCurrentRawStream, torch.cuda.current_device
+# a torch without this name (a build without CUDA has none) takes the public property, which costs an object more
+_raw_stream, _device = getattr(torch._C, "_cuda_getCurrentRawStream", None), torch.cuda.current_device
 
 
 def _size(cfg: Config, name: str) -> int:
@@ -136,7 +137,7 @@ def _size(cfg: Config, name: str) -> int:
 
 def _stream() -> int:
     """The current stream of the current device, as torch.cuda.current_stream().cuda_stream gives it, without the object."""
-    return _raw_stream(_device())
+    return _raw_stream(_device()) if _raw_stream else torch.cuda.current_stream().cuda_stream
 
 
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:

@@ -1,5 +1,8 @@
 """The binding's own work: records of device addresses (no GPU needed: the addresses are not followed)."""
 import ctypes as C
+import os
+import subprocess
+import sys
 
 import pytest
 import torch
@@ -47,3 +50,22 @@ def test_static_parameters_without_the_arrays_they_do_not_use():
         kv.quantize_append_calibrated(cfg, cache, params, K, V)
         got.append((*kv.decode_attention_calibrated(cfg, cache, params, q), cache.k_codes, cache.v_codes))
     assert all(torch.equal(a, b) for a, b in zip(*got))
+
+
+def test_a_torch_without_the_raw_stream_handle_imports():
+    script = ("import torch; del torch._C._cuda_getCurrentRawStream; import paper_2508_04257_b200 as kv; "
+              "print(kv.cache_sizes(kv.Config(1, 8, 8, 64, 512, 4, 32, 256, 2, 1, (1,)))['tile_bytes'])")
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", script], capture_output=True, text=True, cwd=root, timeout=300)
+    assert r.returncode == 0 and r.stdout.split() == ["512"], r.stderr[-2000:]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("raw", [True, False])
+def test_work_goes_to_the_current_stream(raw, monkeypatch):
+    if not raw:
+        monkeypatch.setattr(binding, "_raw_stream", None)
+    assert binding._stream() == torch.cuda.current_stream().cuda_stream
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        assert binding._stream() == side.cuda_stream != 0
