@@ -58,7 +58,7 @@ struct PromptSmem {
     int k_rank[2][64], v_rank[2][64];           // side buffer rows of the step's sink tokens, in token order
     uint64_t k_full[PR_KSTAGES], k_empty[PR_KSTAGES], v_full[PR_VSTAGES], v_empty[PR_VSTAGES];
     uint64_t kpar_full[2], kpar_empty[2], vpar_full[2], vpar_empty[2], v_hdr[PR_HDRS];
-    uint64_t s_full[PR_SBUFS], p_full[PR_SBUFS], o_done[PR_SBUFS], q_full[2], drained;
+    uint64_t s_full[PR_SBUFS], p_full[PR_SBUFS], o_done[PR_SBUFS], o_last[2], q_full[2], drained;
     uint32_t tmem;
     int failed;
 };
@@ -341,6 +341,7 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
                 bar_init(&sm.kpar_full[i], 1); bar_init(&sm.kpar_empty[i], 4);
                 bar_init(&sm.vpar_full[i], 1); bar_init(&sm.vpar_empty[i], 4);
                 bar_init(&sm.q_full[i], 4);
+                bar_init(&sm.o_last[i], 1);
             }
             for (int i = 0; i < PR_HDRS; ++i) bar_init(&sm.v_hdr[i], 1);
             bar_init(&sm.drained, 1);
@@ -397,8 +398,10 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
         // weights are 2^(score - M - e) with M the row's reference, moved only when a weight would leave fp16: the weights of a
         // step stay below 2^15 and the values below 2^15 in the step's units 2^-e, so that P V is in the units of 2^-M throughout
         float M = M_INIT, l = 0.f;
-        // items: steps of the tiles, in turn.  Barriers are per score buffer: an item's next user of the buffer comes three items on,
-        // after this item's outputs, so no barrier can run two phases ahead of a waiter
+        // items: steps of the tiles, in turn.  Barriers are per score buffer.  Inside the loop none can run two phases ahead of a waiter:
+        // the buffer's next user comes three items on, behind the same tile's next item, whose outputs need this warp's weights.
+        // Behind a tile's last item the other tile may have three more, which pass through the same buffers without it, so the
+        // end of a tile has a barrier of its own, completed once
         int item = i, before = 0;
 #pragma unroll 1
         for (int j = 0; j < steps; before = item, item += 1 + (j + i < (i ? n0 : n1)), ++j) {
@@ -482,7 +485,7 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
             __syncwarp();
             if (lane == 0) bar_arrive(&sm.p_full[sb]);
         }
-        if (ok && steps > 0 && bar_wait_warp(&sm.o_done[before % PR_SBUFS], (before / PR_SBUFS) & 1, &sm.failed)) {
+        if (ok && steps > 0 && bar_wait_warp(&sm.o_last[i], 0, &sm.failed)) {
             tc_fence_after();
             const float inv = l > 0.f ? 1.f / l : 0.f;
             const size_t oq = ((size_t)b * p.Hq + qh) * a.T + qt;
@@ -668,6 +671,7 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
                                    vj > 0 || part + x > 0);
                     tc_commit(&sm.o_done[vbuf]);
                     if (last) tc_commit(&sm.v_empty[vstage]);
+                    if (vj == (vi ? m1 : m0) - 1) tc_commit(&sm.o_last[vi]);
                 }
                 __syncwarp();
                 if (last) {

@@ -79,3 +79,28 @@ def test_ranges(bits, keys, values):
 def test_every_token_a_sink():
     wl = TINY.scaled(bits=2, head_dim=128, group=64, n_q_heads=16, n_kv_heads=4, batch=2, seq=270, topk=270, pfn_n=0, seed=23000)
     _check(wl, 270, 0)
+
+
+def _prompt(wl):
+    """A cache that holds a whole prompt, and queries for all of it."""
+    _, gcfg = configs(wl)
+    gs = kv.predict_sinks(gcfg, synth.make_hidden(wl, "cuda"), kv.SinkSet(gcfg))
+    K, V = synth.make_kv(wl, 0, "cuda")
+    gc = kv.KVCache(gcfg, gs)
+    kv.quantize_append(gcfg, gc, K, V)
+    q = torch.randn((wl.batch, wl.n_q_heads, wl.seq, wl.head_dim), device="cuda", generator=torch.Generator("cuda").manual_seed(wl.seed)).half()
+    return gcfg, gc, q
+
+
+# one query head per KV head: the second row tile of a block has two steps more than the first, which ends while the other's products go on
+@pytest.mark.parametrize("bits,T", [(2, 700), (3, 333), (4, 512)])
+def test_a_tile_that_ends_before_the_other(bits, T):
+    wl = TINY.scaled(bits=bits, head_dim=128, group=64, n_q_heads=16, n_kv_heads=16, batch=2, seq=T, topk=5, pfn_n=1, seed=24000 + bits)
+    _check(wl, T, 0)
+    gcfg, gc, q = _prompt(wl)
+    first = kv.prefill_attention(gcfg, gc, q, 0)
+    for _ in range(20):
+        out, lse = (torch.full_like(x, float("nan")) for x in first)
+        kv.prefill_attention(gcfg, gc, q, 0, out=out, lse=lse)
+        assert torch.equal(out, first[0]) and torch.equal(lse, first[1])
+    assert kv.read_status(gc) == 0
