@@ -10,8 +10,8 @@
 // and subtracting the zero-point terms afterwards) leaves no large terms to cancel.
 //
 // Warps: 0-3 / 4-7 softmax of row tile 0 / 1 (a thread owns a row), 8-11 expand keys and 12-15 values (a warp owns 32 channels),
-// 16 issues the matrix instructions, 17 and 18 prepare the steps' key and value parameter tables (19 only evens the warpgroup).  While one tile's scores are in the
-// softmax the tensor cores run the other tile's products.
+// 16 issues the outputs' and 19 the scores' matrix instructions, 17 and 18 prepare the steps' key and value parameter tables.  While one
+// tile's scores are in the softmax the tensor cores run the other tile's products.
 //
 // What bounds it: five matrix products of 128 x 64 x 128 per row tile and step are 2560 clocks for both tiles (2816 with tile 1's
 // queries in shared memory); measured are about 4400: issue slots (the softmax's ~320 instructions for 64 scores of a row, the
@@ -58,7 +58,7 @@ struct PromptSmem {
     int k_rank[2][64], v_rank[2][64];           // side buffer rows of the step's sink tokens, in token order
     uint64_t k_full[PR_KSTAGES], k_empty[PR_KSTAGES], v_full[PR_VSTAGES], v_empty[PR_VSTAGES];
     uint64_t kpar_full[2], kpar_empty[2], vpar_full[2], vpar_empty[2], v_hdr[PR_HDRS];
-    uint64_t s_full[PR_SBUFS], p_full[PR_SBUFS], o_done[PR_SBUFS], o_last[2], q_full[2], drained;
+    uint64_t s_full[PR_SBUFS], p_full[PR_SBUFS], o_done[PR_SBUFS], o_last[2], q_full[2], drained[2];
     uint32_t tmem;
     int failed;
 };
@@ -342,9 +342,9 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
                 bar_init(&sm.vpar_full[i], 1); bar_init(&sm.vpar_empty[i], 4);
                 bar_init(&sm.q_full[i], 4);
                 bar_init(&sm.o_last[i], 1);
+                bar_init(&sm.drained[i], 1);
             }
             for (int i = 0; i < PR_HDRS; ++i) bar_init(&sm.v_hdr[i], 1);
-            bar_init(&sm.drained, 1);
             sm.failed = 0;
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         }
@@ -642,57 +642,65 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
         }
     } else {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
-    if (warp == 16) {
-        // ---------------- matrix instructions ----------------
-        // Items (steps of the tiles, in turn: tile 0 of a step, tile 1 of it) get their scores three items before their outputs.
-        // After a wait that ran out the loop goes on (its waits return at once, nothing leaves the block's memory): its control
-        // must not depend on the waits, or descriptors leave the uniform registers.
+    if (warp == 16 || warp == 19) {
+        // ---------------- matrix instructions: warp 16 the outputs', warp 19 the scores' ----------------
+        // Items are the steps of the tiles, in turn: tile 0 of a step, tile 1 of it.  An item's scores go where the weights of the item
+        // three before were, so they wait for its outputs: only products on one accumulator are sure to run in the order they were
+        // issued.  With one warp for both kinds that wait also held up the next outputs (the two shapes above, with the append: 2887
+        // and 308 us; two warps: 2707 and 287).
+        // After a wait that ran out the loops go on (their waits return at once, nothing leaves the block's memory): their control
+        // does not depend on the waits.
+        const bool scores = warp == 19;
         const uint32_t kb = smem_addr(&sm.k[0][0][0]), vb = smem_addr(&sm.v[0][0][0]);
         const uint64_t qd = smem_desc(smem_addr(sm.q));
         const int m0 = __reduce_max_sync(0xffffffffu, n0), m1 = __reduce_max_sync(0xffffffffu, n1), items = m0 + m1;
-        int ki = 0, kj = 0, kstage = 0, kphase = 0, kbuf = 0, vi = 0, vj = 0, vstage = 0, vphase = 0, vbuf = 0, vbphase = 0;
-        bar_wait_warp(&sm.q_full[0], 0, &sm.failed);
-        if (m1 > 0) bar_wait_warp(&sm.q_full[1], 0, &sm.failed);
+        int i = 0, j = 0, stage = 0, phase = 0, buf = 0, bphase = 0;       // the item: tile, step; its step's stage, its score buffer
+        auto next = [&](bool last, int stages) {
+            if (last) {
+                ++j;
+                i = j < m0 ? 0 : 1;
+                if (++stage == stages) { stage = 0; phase ^= 1; }
+            } else {
+                i = 1;
+            }
+            if (++buf == PR_SBUFS) { buf = 0; bphase ^= 1; }
+        };
+        if (!scores) {
 #pragma unroll 1
-        for (int it = 0; it < items + PR_SBUFS; ++it) {
-            if (it >= PR_SBUFS) {                              // O += P_hi V_lo + P_lo V_hi + P_hi V_hi
-                if (vi == 0 || vj >= m0) bar_wait_warp(&sm.v_full[vstage], vphase, &sm.failed);
-                bar_wait_warp(&sm.p_full[vbuf], vbphase, &sm.failed);
+            for (int it = 0; it < items; ++it) {               // O += P_hi V_lo + P_lo V_hi + P_hi V_hi
+                if (i == 0 || j >= m0) bar_wait_warp(&sm.v_full[stage], phase, &sm.failed);
+                bar_wait_warp(&sm.p_full[buf], bphase, &sm.failed);
                 tc_fence_after();
-                const uint64_t vd = smem_desc(vb + vstage * 2 * PR_HALF);
-                const uint32_t d = TM_O + 128 * vi, w = TM_S + 64 * vbuf;
-                const bool last = vi == 1 || vj >= m1;
+                const uint64_t vd = smem_desc(vb + stage * 2 * PR_HALF);
+                const uint32_t d = TM_O + 128 * i, w = TM_S + 64 * buf;
+                const bool last = i == 1 || j >= m1;
                 if (elect_one()) {
 #pragma unroll
                     for (int part = 0; part < 3; ++part)
 #pragma unroll
                         for (int x = 0; x < 4; ++x)
                             tc_mma(d, w + (part == 1 ? 16 : 0) + 32 * (x >> 1) + 8 * (x & 1), vd + (((part == 0 ? PR_HALF : 0) + x * 32) >> 4), instr_desc(128),
-                                   vj > 0 || part + x > 0);
-                    tc_commit(&sm.o_done[vbuf]);
-                    if (last) tc_commit(&sm.v_empty[vstage]);
-                    if (vj == (vi ? m1 : m0) - 1) tc_commit(&sm.o_last[vi]);
+                                   j > 0 || part + x > 0);
+                    tc_commit(&sm.o_done[buf]);
+                    if (last) tc_commit(&sm.v_empty[stage]);
+                    if (j == (i ? m1 : m0) - 1) tc_commit(&sm.o_last[i]);
                 }
                 __syncwarp();
-                if (last) {
-                    ++vj;
-                    vi = vj < m0 ? 0 : 1;
-                    if (++vstage == PR_VSTAGES) { vstage = 0; vphase ^= 1; }
-                } else {
-                    vi = 1;
-                }
-                if (++vbuf == PR_SBUFS) { vbuf = 0; vbphase ^= 1; }
+                next(last, PR_VSTAGES);
             }
-            if (it < items) {                                  // S = Q K_lo + Q K_hi
-                if (ki == 0 || kj >= m0) {
-                    bar_wait_warp(&sm.k_full[kstage], kphase, &sm.failed);
-                    tc_fence_after();
-                }
-                const uint64_t kd = smem_desc(kb + kstage * 2 * PR_HALF);
-                const uint32_t d = TM_S + 64 * kbuf;
-                const bool last = ki == 1 || kj >= m1;
+        } else {
+            bar_wait_warp(&sm.q_full[0], 0, &sm.failed);
+            if (m1 > 0) bar_wait_warp(&sm.q_full[1], 0, &sm.failed);
+#pragma unroll 1
+            for (int it = 0; it < items; ++it) {               // S = Q K_lo + Q K_hi
+                if (i == 0 || j >= m0) bar_wait_warp(&sm.k_full[stage], phase, &sm.failed);
+                if (it >= PR_SBUFS) bar_wait_warp(&sm.o_done[buf], bphase ^ 1, &sm.failed);
+                tc_fence_after();
+                const uint64_t kd = smem_desc(kb + stage * 2 * PR_HALF);
+                const uint32_t d = TM_S + 64 * buf;
+                const bool last = i == 1 || j >= m1;
                 if (elect_one()) {
-                    if (ki == 0) {
+                    if (i == 0) {
 #pragma unroll
                         for (int x = 0; x < 16; ++x)
                             tc_mma(d, TM_Q + 8 * (x & 7), kd + (((x < 8 ? PR_HALF : 0) + ((x & 7) >> 2) * 8192 + (x & 3) * 32) >> 4), instr_desc(64), x > 0);
@@ -702,27 +710,20 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
                             tc_mma_shared(d, qd + ((((x & 7) >> 2) * PR_HALF + (x & 3) * 32) >> 4),
                                           kd + (((x < 8 ? PR_HALF : 0) + ((x & 7) >> 2) * 8192 + (x & 3) * 32) >> 4), instr_desc(64), x > 0);
                     }
-                    tc_commit(&sm.s_full[kbuf]);
-                    if (last) tc_commit(&sm.k_empty[kstage]);
+                    tc_commit(&sm.s_full[buf]);
+                    if (last) tc_commit(&sm.k_empty[stage]);
                 }
                 __syncwarp();
-                if (last) {
-                    ++kj;
-                    ki = kj < m0 ? 0 : 1;
-                    if (++kstage == PR_KSTAGES) { kstage = 0; kphase ^= 1; }
-                } else {
-                    ki = 1;
-                }
-                if (++kbuf == PR_SBUFS) kbuf = 0;
+                next(last, PR_KSTAGES);
             }
         }
         if (sm.failed) {       // gave up: let what was issued finish before the block goes
             int go = 0;
-            if (elect_one()) tc_commit(&sm.drained);
+            if (elect_one()) tc_commit(&sm.drained[scores]);
             __syncwarp();
-            bar_wait_warp(&sm.drained, 0, &go);
+            bar_wait_warp(&sm.drained[scores], 0, &go);
         }
-    } else if (warp < 19) {
+    } else {
         // ---------------- parameter tables: warp 17 of the keys, warp 18 of the values ----------------
         const bool keys = warp == 17;
         uint64_t *full = keys ? sm.kpar_full : sm.vpar_full, *empty = keys ? sm.kpar_empty : sm.vpar_empty;

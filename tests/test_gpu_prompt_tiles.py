@@ -92,15 +92,26 @@ def _prompt(wl):
     return gcfg, gc, q
 
 
+def _same_every_time(gcfg, gc, q, pos0, times):
+    first = kv.prefill_attention(gcfg, gc, q, pos0)
+    for _ in range(times):
+        out, lse = (torch.full_like(x, float("nan")) for x in first)
+        kv.prefill_attention(gcfg, gc, q, pos0, out=out, lse=lse)
+        assert torch.equal(out, first[0]) and torch.equal(lse, first[1])
+    assert kv.read_status(gc) == 0
+
+
 # one query head per KV head: the second row tile of a block has two steps more than the first, which ends while the other's products go on
 @pytest.mark.parametrize("bits,T", [(2, 700), (3, 333), (4, 512)])
 def test_a_tile_that_ends_before_the_other(bits, T):
     wl = TINY.scaled(bits=bits, head_dim=128, group=64, n_q_heads=16, n_kv_heads=16, batch=2, seq=T, topk=5, pfn_n=1, seed=24000 + bits)
     _check(wl, T, 0)
+    _same_every_time(*_prompt(wl), 0, times=20)
+
+
+# long streams of steps: the weights of a step make room for the scores of a later one many times over
+@pytest.mark.parametrize("bits,hq,hkv,batch", [(2, 32, 8, 2), (3, 8, 8, 4), (4, 64, 8, 1)])
+def test_many_steps_over_the_same_score_buffers(bits, hq, hkv, batch):
+    wl = TINY.scaled(bits=bits, head_dim=128, group=128, n_q_heads=hq, n_kv_heads=hkv, batch=batch, seq=3000, topk=30, pfn_n=1, seed=24100 + bits)
     gcfg, gc, q = _prompt(wl)
-    first = kv.prefill_attention(gcfg, gc, q, 0)
-    for _ in range(20):
-        out, lse = (torch.full_like(x, float("nan")) for x in first)
-        kv.prefill_attention(gcfg, gc, q, 0, out=out, lse=lse)
-        assert torch.equal(out, first[0]) and torch.equal(lse, first[1])
-    assert kv.read_status(gc) == 0
+    _same_every_time(gcfg, gc, q[:, :, -900:], 2100, times=10)
