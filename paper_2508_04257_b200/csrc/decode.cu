@@ -20,7 +20,6 @@ __global__ void decode_merge_kernel(const float *__restrict__ part_ws, int nspli
     // launched with programmatic stream serialization: the blocks may start while the split kernel drains, and wait
     // here until all of it has completed and its records are visible
     pdl_wait();
-    pdl_release();
     float M = M_INIT;
     for (int s = sl; s < nsplit; s += MERGE_SLICES) M = fmaxf(M, base[(size_t)s * PS + D]);
     float acc = 0.f, L = 0.f;

@@ -262,7 +262,6 @@ append_one_kernel(Params p, kvsink_cache c, const __half *__restrict__ k_src, co
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t unit = (int64_t)blockIdx.x * QA_WARPS + warp;
     pdl_wait();
-    pdl_release();
     if (unit >= (int64_t)p.B * p.Hkv) return;
     if (!in_bounds(pos >= 0 && pos < p.max_seq, c.status)) return;
     const int b = (int)(unit / p.Hkv), h = (int)(unit % p.Hkv);
