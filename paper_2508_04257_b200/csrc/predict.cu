@@ -27,7 +27,6 @@ __global__ void sink_score_listed(const uint16_t *__restrict__ H, int S, int64_t
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     int b = blockIdx.y;
     pdl_wait();
-    pdl_release();
     if (i >= S) return;
     const uint16_t *row = H + b * sb + i * ss;
     // the listed channels sit in different sectors of a row: all loads are issued before the first one is used
@@ -50,7 +49,6 @@ __global__ void sink_score_all(const uint16_t *__restrict__ H, int S, int d, int
     int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     int b = blockIdx.y;
     pdl_wait();
-    pdl_release();
     if (warp >= S) return;
     const uint16_t *row = H + b * sb + warp * ss;
     unsigned best = 0;
@@ -145,7 +143,6 @@ sink_select(const uint16_t *__restrict__ score, int score_stride, int S, int k, 
     const uint16_t *sc = score + (size_t)b * score_stride;
     const int kk = k < S ? k : S;
     pdl_wait();
-    pdl_release();
     int vstar = 0x10000, r = 0;   // no score exceeds 0x10000: no top-k selection when kk == 0
     if (kk > 0) {
         if (tid < 256) hist[tid] = 0;
@@ -250,7 +247,6 @@ sink_select_cluster(const uint16_t *__restrict__ score, int score_stride, int S,
     const int kk = k < S ? k : S;
     const int lo = min(S, rk * slice), hi = min(S, lo + slice);
     pdl_wait();
-    pdl_release();
     int vstar = 0x10000, r = 0;   // no score exceeds 0x10000: no top-k selection when kk == 0
     if (tid == 0) { s_neq = 0; s_nsel = 0; }
     // keys of this block's steps (TPT consecutive tokens per thread and step), loaded once (all loads in flight together) and
