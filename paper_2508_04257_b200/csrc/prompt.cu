@@ -61,6 +61,7 @@ struct PromptSmem {
     uint64_t s_full[PR_SBUFS], p_full[PR_SBUFS], o_done[PR_SBUFS], o_last[2], q_full[2], drained[2];
     uint32_t tmem;
     int failed;
+    int odd_values;                             // a sink token of the steps so far has a value that is infinite or NaN
 };
 
 // The block holds all 512 columns of TMEM, so its addresses start at 0.  Columns: accumulators, queries of row tile 0 (with those of
@@ -204,6 +205,7 @@ __device__ __forceinline__ float warp_top(float v)      // largest of the lanes'
 }
 __device__ __forceinline__ __half2 as_half2(uint32_t x) { return *reinterpret_cast<__half2 *>(&x); }
 __device__ __forceinline__ uint32_t as_u32(__half2 x) { return *reinterpret_cast<uint32_t *>(&x); }
+__device__ __forceinline__ bool is_finite(float x) { return fabsf(x) <= 65504.f; }       // of an fp16 value
 
 // Fields of one 16 x 16 matrix of a packed tile, each half ORed into 1024.0: the half is 1024 + code * 2^position.
 // mm: first or second of the warp's two matrices; word(s) as load_words delivers them.
@@ -346,6 +348,7 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
             }
             for (int i = 0; i < PR_HDRS; ++i) bar_init(&sm.v_hdr[i], 1);
             sm.failed = 0;
+            sm.odd_values = 0;
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         }
         __syncwarp();
@@ -503,6 +506,19 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
                 }
             }
             if (a.lse && valid) a.lse[oq] = l > 0.f ? (M + log2f(l)) * 0.6931471805599453f : -INFINITY;
+            // values of sink tokens that are infinite or NaN were left out of the products, where they would reach every row of the
+            // tile; only rows that see the token get them
+            if (valid && *(volatile int *)&sm.odd_values) {
+#pragma unroll 1
+                for (int y = 0; y < min(c.sink_count[b], p.cap); ++y) {
+                    const int tok = c.sink_pos[(size_t)b * p.cap + y];
+                    if (tok < 0 || tok >= lim || !mask_bit(c.sink_bitmask + (size_t)b * p.mask_words, tok)) continue;
+                    const __half *v = (const __half *)c.sink_v + ((size_t)unit * p.cap + y) * D;
+#pragma unroll 1
+                    for (int ch = 0; ch < D; ++ch)
+                        if (!is_finite(__half2float(v[ch]))) a.out[oq * D + ch] += __half2float(v[ch]);
+                }
+            }
         }
     } else if (warp < 16) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
@@ -554,6 +570,7 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
                         left &= left - 1;
                         const int r = ranks[idx++];
                         if (r >= 0) x[k] = __half2float(rows[(size_t)r * D]);
+                        if (!keys && !is_finite(x[k])) x[k] = 0.f;     // a weight of 0 does not hide it: added at the end
                     }
                 }
 #pragma unroll
@@ -777,7 +794,7 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
                 bits[1] = mask_word(j + 1, 1);
             }
             float top = 0.f;
-            bool far = false;
+            bool far = false, odd = false;
             auto look = [&](const Pair &r) {                             // largest |scale * (code - zero)|
                 top = max3(top, r.s0 * fmaxf(fabsf(r.z0), fabsf(QMAX - r.z0)), r.s1 * fmaxf(fabsf(r.z1), fabsf(QMAX - r.z1)));
                 far |= fabsf(r.z0) > PR_NEAR || fabsf(r.z1) > PR_NEAR;
@@ -817,10 +834,17 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
                     if (r >= 0) {
                         const uint2 v = *(const uint2 *)(rows + (size_t)r * D);
                         const float2 v0 = __half22float2(as_half2(v.x)), v1 = __half22float2(as_half2(v.y));
-                        top = fmaxf(fmaxf(fmaxf(fabsf(v0.x), fabsf(v0.y)), fmaxf(fabsf(v1.x), fabsf(v1.y))), top);
+                        const float w[4] = {v0.x, v0.y, v1.x, v1.y};
+#pragma unroll
+                        for (int z = 0; z < 4; ++z) {
+                            const float mag = fabsf(w[z]);
+                            odd |= !is_finite(mag);
+                            top = fmaxf(top, is_finite(mag) ? mag : 0.f);
+                        }
                     }
                 }
                 rank0 += ns;
+                if (!keys && __any_sync(0xffffffffu, odd) && lane == 0) *(volatile int *)&sm.odd_values = 1;
             }
             int e = fit_exponent(warp_top(top));
             if (keys && tok0 + PR_STEP > n_body && seq_len > n_body) e = min(e, 0);    // fp16 rows of the open group, as they are

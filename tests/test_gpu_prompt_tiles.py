@@ -115,3 +115,35 @@ def test_many_steps_over_the_same_score_buffers(bits, hq, hkv, batch):
     wl = TINY.scaled(bits=bits, head_dim=128, group=128, n_q_heads=hq, n_kv_heads=hkv, batch=batch, seq=3000, topk=30, pfn_n=1, seed=24100 + bits)
     gcfg, gc, q = _prompt(wl)
     _same_every_time(gcfg, gc, q[:, :, -900:], 2100, times=10)
+
+
+# a sink token's row may hold infinities and NaN (it is kept as it came): queries before it must not see them
+@pytest.mark.parametrize("bits,topk", [(2, 6), (3, 6), (4, 90)])
+def test_sink_rows_that_are_not_finite_stay_hidden_from_queries_before_them(bits, topk):
+    wl = TINY.scaled(bits=bits, head_dim=128, group=32, n_q_heads=16, n_kv_heads=4, batch=2, seq=300, topk=topk, pfn_n=1, seed=25000 + bits)
+    ocfg, gcfg = configs(wl)
+    H = synth.make_hidden(wl, "cuda")
+    K, V = synth.make_kv(wl, 0, "cuda")
+    bm, pos, cnt = oracle.predict_sinks(ocfg, np16(H))
+    gc, oc = kv.KVCache(gcfg, kv.predict_sinks(gcfg, H, kv.SinkSet(gcfg))), oracle.Cache(ocfg, bm, pos, cnt)
+    kv.quantize_append(gcfg, gc, K, V)
+    oracle.quantize_append(ocfg, oc, np16(K), np16(V))
+    slot = [int(cnt[b]) // 2 for b in range(2)]
+    at = [int(pos[b, s]) for b, s in enumerate(slot)]
+    assert all(0 < t < 290 for t in at)
+    for b, s in enumerate(slot):          # [sequence, KV head, slot, channel]
+        for cache in (gc, oc):
+            k, v = (x.view(2, 4, -1, 128) if cache is gc else x.view(np.float16).reshape(2, 4, -1, 128) for x in (cache.sink_k, cache.sink_v))
+            v[b, 0, s, 5], v[b, 1, s, 7], v[b, 1, s, 127], v[b, 2, s, 0], k[b, 3, s, 64] = np.inf, -np.inf, np.inf, np.nan, np.inf
+    q = torch.randn((2, 16, 300, 128), device="cuda", generator=torch.Generator("cuda").manual_seed(wl.seed)).half()
+    out, lse = (x.cpu().numpy() for x in kv.prefill_attention(gcfg, gc, q, 0))
+    ref, ref_lse = oracle.prefill_attention(ocfg, oc, np16(q), 0)
+    assert kv.read_status(gc) == 0
+    for b, t in enumerate(at):
+        out[b, 12:, t:], lse[b, 12:, t:], ref[b, 12:, t:], ref_lse[b, 12:, t:] = 0, 0, 0, 0      # queries that see the infinite key
+    assert np.array_equal(np.isfinite(out), np.isfinite(ref))
+    for value in (np.inf, -np.inf):
+        assert np.array_equal(out == value, ref == value)
+    fine = np.isfinite(ref)
+    assert_close(out[fine], ref[fine], "prompt attention")
+    assert np.abs(lse - ref_lse).max() <= 2e-3 + 1e-3 * np.abs(ref_lse).max()
