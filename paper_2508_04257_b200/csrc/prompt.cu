@@ -331,6 +331,8 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
         return row0 + 128 * i < n_rows ? (row_limit(row0 + 128 * i + 127) + PR_STEP - 1) / PR_STEP : 0;
     };
     const int n0 = tile_steps(0), n1 = tile_steps(1), n_steps = max(n0, n1);
+    // every thread alike, and before anything is set up; index checks of single accesses are at the accesses
+    if (!in_bounds(b < p.B && row0 < n_rows && a.q_pos0 >= 0 && a.q_pos0 + a.T <= seq_len && seq_len <= p.max_seq && p.cap >= 0, c.status)) return;
 
     if (warp == 16) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&sm.tmem)), "r"(512) : "memory");
@@ -533,6 +535,7 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
         constexpr int TILE = 16 * D * BITS / 8;
         auto fetch = [&](int j) {
             const uint8_t *tile = codes + (size_t)j * 4 * TILE;
+            if (!in_bounds(min((j + 1) * PR_STEP, (coded + KVSINK_TILE - 1) / KVSINK_TILE * KVSINK_TILE) <= p.max_seq, c.status)) return;
             if ((j + 1) * PR_STEP <= coded) {
 #pragma unroll
                 for (int tt = 0; tt < 4; ++tt) load_words<BITS>(tile + tt * TILE, w, lane, next[tt]);
@@ -569,7 +572,7 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
                         tk[k] = __ffsll((long long)left) - 1;
                         left &= left - 1;
                         const int r = ranks[idx++];
-                        if (r >= 0) x[k] = __half2float(rows[(size_t)r * D]);
+                        if (r >= 0 && in_bounds(idx <= 64 && r < p.cap, c.status)) x[k] = __half2float(rows[(size_t)r * D]);
                         if (!keys && !is_finite(x[k])) x[k] = 0.f;     // a weight of 0 does not hide it: added at the end
                     }
                 }
@@ -635,13 +638,13 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
 #pragma unroll
                         for (int y = 0; y < 4; ++y) {
                             const int tk = tok + (lane >> 2) + 8 * (y & 1);
-                            const uint32_t v = tk < seq_len ? *(const uint32_t *)(tail + (size_t)(tk - n_body) * D + 16 * (2 * w + mm) + 8 * (y >> 1) + 2 * t) : 0u;
+                            const uint32_t v = tk < seq_len && in_bounds(tk - n_body < p.G, c.status) ? *(const uint32_t *)(tail + (size_t)(tk - n_body) * D + 16 * (2 * w + mm) + 8 * (y >> 1) + 2 * t) : 0u;
                             hi[y] = as_u32(__hmul2_rn(as_half2(v), up2));
                             lo[y] = 0u;
                         }
                     } else {
                         uint32_t f[4], words[2] = {0u, 0u};
-                        if (tok < coded) load_words<BITS>(codes + (size_t)(tok >> 4) * p.tile_bytes, w, lane, words);
+                        if (tok < coded && in_bounds(tok + KVSINK_TILE <= p.max_seq, c.status)) load_words<BITS>(codes + (size_t)(tok >> 4) * p.tile_bytes, w, lane, words);
                         matrix_fields<BITS>(words, mm, w & 1, f);
                         const int e = entry(tt, mm, second);
                         expand_matrix<BITS, true>(f, tab[e], tab[e + 4], add[e], add[e + 4], hi, lo);
@@ -761,6 +764,7 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
             const int tok = j * PR_STEP + 2 * lane;
             const int64_t at = keys ? (int64_t)(g + (n >> 1)) * D + 2 * lane + 64 * (n & 1) : (int64_t)tok * p.NGv + n;
             Pair r = {0.f, 0.f, 0.f, 0.f};
+            if (n < entries && !in_bounds(keys ? (g + (n >> 1) + 1) * p.G <= n_body : n < p.NGv, c.status)) return r;
             if (n < entries && (keys || tok < seq_len)) { r.s0 = __ldg(ps + at); r.z0 = __ldg(pz + at); }
             if (n < entries && (keys || tok + 1 < seq_len)) { r.s1 = __ldg(ps + at + apart); r.z1 = __ldg(pz + at + apart); }
             return r;
@@ -772,7 +776,7 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
         };
         auto mask_word = [&](int j, int x) {
             const int left = seq_len - (j * PR_STEP + 32 * x);
-            uint32_t w = left > 0 ? __ldg(bm + 2 * j + x) : 0u;
+            uint32_t w = left > 0 && in_bounds(2 * j + x < p.mask_words, c.status) ? __ldg(bm + 2 * j + x) : 0u;
             return left > 0 && left < 32 ? w & ((1u << left) - 1u) : w;
         };
         int g0 = 0, second = p.G, entries = count(0, p.G);
@@ -832,6 +836,7 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
                 for (int y = 0; y < ns; ++y) {
                     const int r = rank[buf][y];
                     if (r >= 0) {
+                        if (!in_bounds(r < p.cap, c.status)) continue;
                         const uint2 v = *(const uint2 *)(rows + (size_t)r * D);
                         const float2 v0 = __half22float2(as_half2(v.x)), v1 = __half22float2(as_half2(v.y));
                         const float w[4] = {v0.x, v0.y, v1.x, v1.y};

@@ -35,3 +35,28 @@ def test_debug_build_runs_the_path_with_a_clean_status_word():
     env = dict(os.environ, KVSINK_LIB=kv_build.DEBUG_LIB)
     r = subprocess.run([sys.executable, "-c", SCRIPT, ROOT], capture_output=True, text=True, env=env, timeout=600)
     assert r.returncode == 0 and "debug build ok" in r.stdout, r.stdout[-1500:] + r.stderr[-3000:]
+
+
+PROMPTS = r"""
+import sys
+sys.path.insert(0, sys.argv[1]); sys.path.insert(0, sys.argv[1] + "/tests")
+from paper_2508_04257_b200 import synth
+from test_gpu_prompt_tiles import _check, _far
+TINY = synth.WORKLOADS["tiny"]
+for bits, group, hq, hkv, batch, T, pos0, topk in ((2, 128, 16, 16, 8, 64, 0, 3), (4, 144, 12, 4, 4, 171, 29, 90), (3, 64, 32, 4, 8, 129, 0, 90),
+                                                   (4, 32, 8, 8, 8, 130, 190, 3)):
+    wl = TINY.scaled(bits=bits, head_dim=128, group=group, n_q_heads=hq, n_kv_heads=hkv, batch=batch, seq=pos0 + T, topk=min(topk, pos0 + T), pfn_n=2,
+                     seed=26000 + bits)
+    _check(wl, T, pos0)                  # asserts parity and a zero status word
+_check(TINY.scaled(bits=2, head_dim=128, group=32, n_q_heads=16, n_kv_heads=4, batch=2, seq=300, topk=6, pfn_n=1, seed=26100), 300, 0, _far, _far)
+print("debug prompts ok")
+"""
+
+
+@pytest.mark.gpu
+def test_prompts_of_many_rows_run_with_index_checks_and_a_clean_status_word():
+    if not os.path.exists(kv_build.DEBUG_LIB):
+        pytest.skip("libkvsink_debug.so has not been built (python -m paper_2508_04257_b200.build --debug)")
+    env = dict(os.environ, KVSINK_LIB=kv_build.DEBUG_LIB)
+    r = subprocess.run([sys.executable, "-c", PROMPTS, ROOT], capture_output=True, text=True, env=env, timeout=600)
+    assert r.returncode == 0 and "debug prompts ok" in r.stdout, r.stdout[-1500:] + r.stderr[-3000:]
