@@ -141,7 +141,9 @@ int kvsink_predict_sinks(const kvsink_config *cfg, const void *hidden, int32_t S
  *                 strides in elements, multiples of 8; both tensors share the strides.
  *   T             any T >= 0 at any time (prefill, chunked prefill, one decode token): a chunk may start and end inside
  *                 a key group; the result is the same as appending its tokens one by one.
- * On success cache->seq_len (host) is advanced by T.
+ * On success cache->seq_len (host) is advanced by T.  An error leaves it and the open group as they were, so the call can be made
+ * again; only where the launch of the whole groups' kernel itself failed behind that of the chunk's ragged ends
+ * (KVSINK_ERR_CUDA with one kernel launched) the rows of the open group in k_tail are undefined.
  */
 int kvsink_quantize_append(const kvsink_config *cfg, kvsink_cache *cache, const void *k_new, const void *v_new, int32_t T,
                            int64_t stride_b, int64_t stride_h, int64_t stride_t, void *cuda_stream);

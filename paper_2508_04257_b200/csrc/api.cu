@@ -4,6 +4,10 @@
 using namespace kvsink;
 
 std::atomic<unsigned long long> kvsink::g_launches{0};
+#ifdef KVSINK_DEBUG
+std::atomic<int> kvsink::g_fail_host_call{0};
+extern "C" void kvsink_debug_fail_host_call(int n) { g_fail_host_call = n; }
+#endif
 
 static int derive(const kvsink_config *cfg, Params *p)
 {
@@ -36,16 +40,16 @@ static int derive(const kvsink_config *cfg, Params *p)
     return KVSINK_OK;
 }
 
-// Whole groups: the streaming kernel where the shape has one, else the generic kernel.
+// Whole groups, behind the chunk's edges if it has any: the streaming kernel where the shape has one, else the generic kernel.
 static int quantize_groups(const Params &p, const kvsink_cache &c, const __half *k, const __half *v, int first_token, int n_groups,
-                           int64_t sb, int64_t sh, int64_t stt, bool do_v_and_sinks, bool after_edges, cudaStream_t st)
+                           int64_t sb, int64_t sh, int64_t stt, bool do_v_and_sinks, const AppendEdges *edges, cudaStream_t st)
 {
     int rc = KVSINK_ERR_UNSUPPORTED;
-    if (do_v_and_sinks) rc = launch_quantize_groups_bulk(p, c, k, v, first_token, n_groups, sb, sh, stt, after_edges, st);
+    if (do_v_and_sinks) rc = launch_quantize_groups_bulk(p, c, k, v, first_token, n_groups, sb, sh, stt, edges, st);
     if (rc != KVSINK_ERR_UNSUPPORTED) return rc;
-    rc = launch_quantize_groups_fast(p, c, k, v, first_token, n_groups, sb, sh, stt, do_v_and_sinks, st);
+    rc = launch_quantize_groups_fast(p, c, k, v, first_token, n_groups, sb, sh, stt, do_v_and_sinks, edges, st);
     if (rc != KVSINK_ERR_UNSUPPORTED) return rc;
-    return launch_quantize_groups(p, c, k, v, first_token, n_groups, sb, sh, stt, do_v_and_sinks, st);
+    return launch_quantize_groups(p, c, k, v, first_token, n_groups, sb, sh, stt, do_v_and_sinks, edges, st);
 }
 
 static bool aligned16(const void *ptr) { return ptr && ((uintptr_t)ptr & 15u) == 0; }
@@ -122,15 +126,12 @@ extern "C" int kvsink_quantize_append(const kvsink_config *cfg, kvsink_cache *ca
     // small enough for it, else token by token.
     if (T > 1 && G <= 128) {
         const int head = S0 % G == 0 ? 0 : (T < G - S0 % G ? T : G - S0 % G), n_groups = (T - head) / G, rem = T - head - n_groups * G;
-        if (head > 0 || rem > 0) {
-            rc = launch_append_edges(p, *cache, k, v, S0, head, T - rem, rem, stride_b, stride_h, stride_t, st);
-            if (rc) return rc;
-        }
-        if (n_groups > 0) {
-            rc = quantize_groups(p, *cache, k + (int64_t)head * stride_t, v + (int64_t)head * stride_t, S0 + head, n_groups, stride_b, stride_h,
-                                 stride_t, true, head > 0 || rem > 0, st);
-            if (rc) return rc;
-        }
+        const AppendEdges edges = {k, v, S0, head, T - rem, rem, stride_b, stride_h, stride_t};
+        const bool ragged = head > 0 || rem > 0;
+        rc = n_groups > 0 ? quantize_groups(p, *cache, k + (int64_t)head * stride_t, v + (int64_t)head * stride_t, S0 + head, n_groups, stride_b,
+                                            stride_h, stride_t, true, ragged ? &edges : nullptr, st)
+                          : launch_append_edges(p, *cache, edges, st);
+        if (rc) return rc;
         cache->seq_len = S0 + T;
         return KVSINK_OK;
     }
@@ -142,7 +143,7 @@ extern "C" int kvsink_quantize_append(const kvsink_config *cfg, kvsink_cache *ca
         if ((S0 + head) % G == 0) {
             // the open group is complete: quantize its keys per channel from the fp16 tail
             rc = quantize_groups(p, *cache, (const __half *)cache->k_tail, (const __half *)cache->k_tail, S0 + head - G, 1,
-                                 (int64_t)p.Hkv * G * p.D, (int64_t)G * p.D, p.D, false, false, st);
+                                 (int64_t)p.Hkv * G * p.D, (int64_t)G * p.D, p.D, false, nullptr, st);
             if (rc) return rc;
         }
         done = head;
@@ -151,7 +152,7 @@ extern "C" int kvsink_quantize_append(const kvsink_config *cfg, kvsink_cache *ca
         const int n_groups = (T - done) / G;
         if (n_groups > 0) {
             rc = quantize_groups(p, *cache, k + (int64_t)done * stride_t, v + (int64_t)done * stride_t, S0 + done, n_groups, stride_b,
-                                 stride_h, stride_t, true, false, st);
+                                 stride_h, stride_t, true, nullptr, st);
             if (rc) return rc;
         }
         rc = launch_quantize_tokens(p, *cache, k, v, done + n_groups * G, S0 + done + n_groups * G, T - done - n_groups * G, stride_b,

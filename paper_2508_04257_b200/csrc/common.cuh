@@ -122,6 +122,20 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
     return cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
 }
 
+// Leave for a kernel to use `bytes` of dynamic shared memory.  In debug builds kvsink_debug_fail_host_call(n) makes the n-th call
+// from then on report a failure, so that tests can look at what an entry point leaves behind that gives up half way.
+#ifdef KVSINK_DEBUG
+extern std::atomic<int> g_fail_host_call;
+#endif
+template <typename Kernel>
+inline bool allow_smem(Kernel kern, size_t bytes)
+{
+#ifdef KVSINK_DEBUG
+    if (g_fail_host_call > 0 && --g_fail_host_call == 0) return false;
+#endif
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
+}
+
 // Decode attention: warps per block, the "no score yet" value of a running maximum, and 2^x.
 constexpr int DEC_WARPS = 4;
 constexpr float M_INIT = -1.0e30f;
@@ -146,19 +160,28 @@ __device__ __forceinline__ bool in_bounds(bool, int32_t *) { return true; }
 
 __device__ __forceinline__ bool mask_bit(const uint32_t *__restrict__ bm, int pos) { return (bm[pos >> 5] >> (pos & 31)) & 1u; }
 
+// The ragged ends of a chunk (append_edges_kernel), whose kernel goes ahead of the whole groups'.  It overwrites rows of the open
+// group, which a call that fails has to leave as they are: a launcher of the whole groups that is given the edges launches
+// them itself, once, behind everything of its own that can fail or be refused on the host.
+struct AppendEdges {
+    const __half *k_src, *v_src;
+    int head_first, head_n;      // position and number of the tokens inside the open group
+    int rem_src, rem_n;          // offset in the source and number of the tokens behind the last whole group
+    int64_t sb, sh, stt;
+};
+
 // Launchers implemented in the kernel translation units; all return a KVSINK_* code.
 int launch_predict_sinks(const Params &p, const __half *hidden, int S, int64_t stride_b, int64_t stride_s, uint32_t *bitmask,
                          int32_t *sink_pos, int32_t *sink_count, void *workspace, cudaStream_t st);
 int launch_quantize_groups(const Params &p, const kvsink_cache &c, const __half *k_src, const __half *v_src, int first_token,
-                           int n_groups, int64_t sb, int64_t sh, int64_t stt, bool do_v_and_sinks, cudaStream_t st);
+                           int n_groups, int64_t sb, int64_t sh, int64_t stt, bool do_v_and_sinks, const AppendEdges *edges, cudaStream_t st);
 int launch_quantize_groups_fast(const Params &p, const kvsink_cache &c, const __half *k_src, const __half *v_src, int first_token,
-                                int n_groups, int64_t sb, int64_t sh, int64_t stt, bool do_v_and_sinks, cudaStream_t st);
+                                int n_groups, int64_t sb, int64_t sh, int64_t stt, bool do_v_and_sinks, const AppendEdges *edges, cudaStream_t st);
 int launch_quantize_groups_bulk(const Params &p, const kvsink_cache &c, const __half *k_src, const __half *v_src, int first_token,
-                                int n_groups, int64_t sb, int64_t sh, int64_t stt, bool after_edges, cudaStream_t st);
+                                int n_groups, int64_t sb, int64_t sh, int64_t stt, const AppendEdges *edges, cudaStream_t st);
 int launch_quantize_tokens(const Params &p, const kvsink_cache &c, const __half *k_src, const __half *v_src, int src_offset,
                            int first_token, int n_tokens, int64_t sb, int64_t sh, int64_t stt, cudaStream_t st);
-int launch_append_edges(const Params &p, const kvsink_cache &c, const __half *k_src, const __half *v_src, int head_first, int head_n, int rem_src,
-                        int rem_n, int64_t sb, int64_t sh, int64_t stt, cudaStream_t st);
+int launch_append_edges(const Params &p, const kvsink_cache &c, const AppendEdges &edges, cudaStream_t st);
 int launch_decode(const Params &p, const kvsink_cache &c, const kvsink_static_params *cal, int mode, const __half *q, float *out, float *lse, void *workspace,
                   size_t workspace_bytes, cudaStream_t st);
 int launch_prefill_b2(const Params &p, const kvsink_cache &c, const __half *q, int T, int q_pos0, int64_t sb, int64_t sh, int64_t stt, float *out,

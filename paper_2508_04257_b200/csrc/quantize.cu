@@ -147,13 +147,14 @@ static size_t groups_smem_bytes(const Params &p)
 }
 
 int launch_quantize_groups(const Params &p, const kvsink_cache &c, const __half *k_src, const __half *v_src, int first_token,
-                           int n_groups, int64_t sb, int64_t sh, int64_t stt, bool do_v_and_sinks, cudaStream_t st)
+                           int n_groups, int64_t sb, int64_t sh, int64_t stt, bool do_v_and_sinks, const AppendEdges *edges, cudaStream_t st)
 {
     if (n_groups <= 0) return KVSINK_OK;
     size_t smem = groups_smem_bytes(p);
     if (smem > 227 * 1024) return KVSINK_ERR_UNSUPPORTED;
-    if (cudaFuncSetAttribute(quantize_groups_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return KVSINK_ERR_CUDA;
+    if (!allow_smem(quantize_groups_kernel, smem)) return KVSINK_ERR_CUDA;
+    if (edges)
+        if (const int rc = launch_append_edges(p, c, *edges, st)) return rc;
     dim3 grid(n_groups, p.Hkv, p.B);
     note_launch();
     quantize_groups_kernel<<<grid, QG_THREADS, smem, st>>>(p, c, k_src, v_src, first_token, sb, sh, stt, do_v_and_sinks ? 1 : 0);
@@ -508,22 +509,21 @@ append_edges_kernel(Params p, kvsink_cache c, const __half *__restrict__ k_src, 
 }
 
 // Groups of more than 128 tokens keep the kernels that go token by token (the group would not fit a block's shared memory).
-int launch_append_edges(const Params &p, const kvsink_cache &c, const __half *k_src, const __half *v_src, int head_first, int head_n, int rem_src,
-                        int rem_n, int64_t sb, int64_t sh, int64_t stt, cudaStream_t st)
+int launch_append_edges(const Params &p, const kvsink_cache &c, const AppendEdges &a, cudaStream_t st)
 {
     if (p.G > 128) return KVSINK_ERR_UNSUPPORTED;
     auto tiles = [](int first, int n) { return n > 0 ? (first + n - 1) / KVSINK_TILE - first / KVSINK_TILE + 1 : 0; };
     EdgeShape e;
-    e.head_first = head_first;
-    e.head_n = head_n;
-    e.flush = head_n > 0 && (head_first + head_n) % p.G == 0;
-    e.rem_first = head_first + rem_src;
-    e.rem_n = rem_n;
-    e.rem_src = rem_src;
-    e.head_tiles = tiles(head_first, head_n);
-    const dim3 grid(p.D / QE_CH + e.head_tiles + tiles(e.rem_first, rem_n), p.Hkv, p.B);
+    e.head_first = a.head_first;
+    e.head_n = a.head_n;
+    e.flush = a.head_n > 0 && (a.head_first + a.head_n) % p.G == 0;
+    e.rem_first = a.head_first + a.rem_src;
+    e.rem_n = a.rem_n;
+    e.rem_src = a.rem_src;
+    e.head_tiles = tiles(a.head_first, a.head_n);
+    const dim3 grid(p.D / QE_CH + e.head_tiles + tiles(e.rem_first, e.rem_n), p.Hkv, p.B);
     const size_t smem = e.flush ? (size_t)p.G * ((QE_CH + 8) * 2 + QE_CH) : 0;
-    return launch_pdl(append_edges_kernel, grid, dim3(QE_THREADS), smem, st, p, c, k_src, v_src, e, sb, sh, stt) == cudaSuccess ? KVSINK_OK : KVSINK_ERR_CUDA;
+    return launch_pdl(append_edges_kernel, grid, dim3(QE_THREADS), smem, st, p, c, a.k_src, a.v_src, e, a.sb, a.sh, a.stt) == cudaSuccess ? KVSINK_OK : KVSINK_ERR_CUDA;
 }
 
 int launch_quantize_tokens(const Params &p, const kvsink_cache &c, const __half *k_src, const __half *v_src, int src_offset,

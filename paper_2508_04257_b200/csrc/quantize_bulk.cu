@@ -875,7 +875,7 @@ bool make_map(CUtensorMap *tm, const __half *base, const Params &p, int T, int64
 
 template <int BITS, int G, int MODE = 0>
 int launch_bulk(const Params &p, const kvsink_cache &c, const kvsink_static_params &sp, const __half *k_src, const __half *v_src, int first_token,
-                int n_groups, int64_t sb, int64_t sh, int64_t stt, cudaStream_t st, bool after_edges = false)
+                int n_groups, int64_t sb, int64_t sh, int64_t stt, cudaStream_t st, const AppendEdges *edges = nullptr)
 {
     using Geo = QbGeo<G, BITS>;
     CUtensorMap tm_k, tm_v;
@@ -889,16 +889,18 @@ int launch_bulk(const Params &p, const kvsink_cache &c, const kvsink_static_para
     constexpr size_t smem = (size_t)NW * (QB_STAGE_BYTES + 8 + Geo::SCRATCH);
     static_assert(smem <= 227 * 1024, "stages too large");
     auto kern = quantize_bulk_kernel<BITS, G, MODE>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return KVSINK_ERR_CUDA;
     QbShape shp;
     shp.first_token = first_token;
     shp.n_groups = n_groups;
-    shp.after_edges = after_edges;
+    shp.after_edges = edges != nullptr;
     const long n_items = (long)p.B * p.Hkv * n_groups * Geo::IPG;
     if (n_items >= (1L << 30)) return KVSINK_ERR_UNSUPPORTED;
     shp.n_items = (unsigned)n_items;
     long blocks = (n_items + NW - 1) / NW;
     if (blocks > 148) blocks = 148;
+    if (!allow_smem(kern, smem)) return KVSINK_ERR_CUDA;
+    if (edges)
+        if (const int rc = launch_append_edges(p, c, *edges, st)) return rc;
     return launch_pdl(kern, dim3((unsigned)blocks), dim3(32 * NW), smem, st, p, c, tm_k, tm_v, shp, sp) == cudaSuccess ? KVSINK_OK : KVSINK_ERR_CUDA;
 }
 
@@ -907,15 +909,15 @@ int launch_bulk(const Params &p, const kvsink_cache &c, const kvsink_static_para
 // Whole groups of a bulk append (keys, values and sink rows).  Returns KVSINK_ERR_UNSUPPORTED when the shape has no
 // kernel of this kind or the inputs cannot be described by a tensor map; the caller then uses another kernel.
 int launch_quantize_groups_bulk(const Params &p, const kvsink_cache &c, const __half *k_src, const __half *v_src, int first_token,
-                                int n_groups, int64_t sb, int64_t sh, int64_t stt, bool after_edges, cudaStream_t st)
+                                int n_groups, int64_t sb, int64_t sh, int64_t stt, const AppendEdges *edges, cudaStream_t st)
 {
     if (p.D != QB_D || n_groups < 1) return KVSINK_ERR_UNSUPPORTED;
     const kvsink_static_params none = {nullptr, nullptr, nullptr, nullptr};
-    if (p.bits == 2 && p.G == 128) return launch_bulk<2, 128>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, after_edges);
-    if (p.bits == 2 && p.G == 64) return launch_bulk<2, 64>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, after_edges);
-    if (p.bits == 3 && p.G == 64) return launch_bulk<3, 64>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, after_edges);
-    if (p.bits == 4 && p.G == 128) return launch_bulk<4, 128>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, after_edges);
-    if (p.bits == 4 && p.G == 64) return launch_bulk<4, 64>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, after_edges);
+    if (p.bits == 2 && p.G == 128) return launch_bulk<2, 128>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, edges);
+    if (p.bits == 2 && p.G == 64) return launch_bulk<2, 64>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, edges);
+    if (p.bits == 3 && p.G == 64) return launch_bulk<3, 64>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, edges);
+    if (p.bits == 4 && p.G == 128) return launch_bulk<4, 128>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, edges);
+    if (p.bits == 4 && p.G == 64) return launch_bulk<4, 64>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, edges);
     return KVSINK_ERR_UNSUPPORTED;
 }
 

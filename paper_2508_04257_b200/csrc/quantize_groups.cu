@@ -574,13 +574,15 @@ quantize_groups_stream(Params p, kvsink_cache c, const __half *__restrict__ k_sr
 
 template <int BITS, int D, int G>
 static int launch_stream(const Params &p, const kvsink_cache &c, const __half *k_src, const __half *v_src, int first_token, int n_groups,
-                         int64_t sb, int64_t sh, int64_t stt, bool do_v, cudaStream_t st)
+                         int64_t sb, int64_t sh, int64_t stt, bool do_v, const AppendEdges *edges, cudaStream_t st)
 {
     constexpr int NT = G / KVSINK_TILE, W = D * BITS / 64, NW = D / 16;
     constexpr size_t smem = 2 * (size_t)G * D * 2 + (size_t)NT * 32 * W * 4 + NW * sizeof(WarpScratch) + 2 * NT * 4 + 16;
     static_assert(smem <= 227 * 1024, "tile too large");
     auto kern = quantize_groups_stream<BITS, D, G>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return KVSINK_ERR_CUDA;
+    if (!allow_smem(kern, smem)) return KVSINK_ERR_CUDA;
+    if (edges)
+        if (const int rc = launch_append_edges(p, c, *edges, st)) return rc;
     const int kinds = do_v ? 2 : 1;
     const long n_items = (long)p.B * p.Hkv * n_groups * kinds;
     int per_sm = (int)((227 * 1024) / (smem + 1024));
@@ -595,27 +597,27 @@ static int launch_stream(const Params &p, const kvsink_cache &c, const __half *k
 
 template <int BITS, int D>
 static int launch_fast(const Params &p, const kvsink_cache &c, const __half *k_src, const __half *v_src, int first_token, int n_groups,
-                       int64_t sb, int64_t sh, int64_t stt, bool do_v, cudaStream_t st)
+                       int64_t sb, int64_t sh, int64_t stt, bool do_v, const AppendEdges *edges, cudaStream_t st)
 {
     switch (p.G) {
-    case 32: return launch_stream<BITS, D, 32>(p, c, k_src, v_src, first_token, n_groups, sb, sh, stt, do_v, st);
-    case 64: return launch_stream<BITS, D, 64>(p, c, k_src, v_src, first_token, n_groups, sb, sh, stt, do_v, st);
-    case 128: return launch_stream<BITS, D, 128>(p, c, k_src, v_src, first_token, n_groups, sb, sh, stt, do_v, st);
+    case 32: return launch_stream<BITS, D, 32>(p, c, k_src, v_src, first_token, n_groups, sb, sh, stt, do_v, edges, st);
+    case 64: return launch_stream<BITS, D, 64>(p, c, k_src, v_src, first_token, n_groups, sb, sh, stt, do_v, edges, st);
+    case 128: return launch_stream<BITS, D, 128>(p, c, k_src, v_src, first_token, n_groups, sb, sh, stt, do_v, edges, st);
     default: return KVSINK_ERR_UNSUPPORTED;
     }
 }
 
 // Returns KVSINK_ERR_UNSUPPORTED when the shape has no streaming kernel (the caller then uses the generic one).
 int launch_quantize_groups_fast(const Params &p, const kvsink_cache &c, const __half *k_src, const __half *v_src, int first_token,
-                                int n_groups, int64_t sb, int64_t sh, int64_t stt, bool do_v_and_sinks, cudaStream_t st)
+                                int n_groups, int64_t sb, int64_t sh, int64_t stt, bool do_v_and_sinks, const AppendEdges *edges, cudaStream_t st)
 {
     if (p.D == 128) {
-        if (p.bits == 2) return launch_fast<2, 128>(p, c, k_src, v_src, first_token, n_groups, sb, sh, stt, do_v_and_sinks, st);
-        if (p.bits == 3) return launch_fast<3, 128>(p, c, k_src, v_src, first_token, n_groups, sb, sh, stt, do_v_and_sinks, st);
-        if (p.bits == 4) return launch_fast<4, 128>(p, c, k_src, v_src, first_token, n_groups, sb, sh, stt, do_v_and_sinks, st);
+        if (p.bits == 2) return launch_fast<2, 128>(p, c, k_src, v_src, first_token, n_groups, sb, sh, stt, do_v_and_sinks, edges, st);
+        if (p.bits == 3) return launch_fast<3, 128>(p, c, k_src, v_src, first_token, n_groups, sb, sh, stt, do_v_and_sinks, edges, st);
+        if (p.bits == 4) return launch_fast<4, 128>(p, c, k_src, v_src, first_token, n_groups, sb, sh, stt, do_v_and_sinks, edges, st);
     } else if (p.D == 64) {
-        if (p.bits == 2) return launch_fast<2, 64>(p, c, k_src, v_src, first_token, n_groups, sb, sh, stt, do_v_and_sinks, st);
-        if (p.bits == 4) return launch_fast<4, 64>(p, c, k_src, v_src, first_token, n_groups, sb, sh, stt, do_v_and_sinks, st);
+        if (p.bits == 2) return launch_fast<2, 64>(p, c, k_src, v_src, first_token, n_groups, sb, sh, stt, do_v_and_sinks, edges, st);
+        if (p.bits == 4) return launch_fast<4, 64>(p, c, k_src, v_src, first_token, n_groups, sb, sh, stt, do_v_and_sinks, edges, st);
     }
     return KVSINK_ERR_UNSUPPORTED;
 }

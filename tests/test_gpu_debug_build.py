@@ -60,3 +60,48 @@ def test_prompts_of_many_rows_run_with_index_checks_and_a_clean_status_word():
     env = dict(os.environ, KVSINK_LIB=kv_build.DEBUG_LIB)
     r = subprocess.run([sys.executable, "-c", PROMPTS, ROOT], capture_output=True, text=True, env=env, timeout=600)
     assert r.returncode == 0 and "debug prompts ok" in r.stdout, r.stdout[-1500:] + r.stderr[-3000:]
+
+
+FAILING_APPEND = r"""
+import sys
+sys.path.insert(0, sys.argv[1]); sys.path.insert(0, sys.argv[1] + "/tests")
+import torch
+import oracle
+import paper_2508_04257_b200 as kv
+from paper_2508_04257_b200 import binding, synth
+from parity_util import compare_cache, configs, np16
+TINY = synth.WORKLOADS["tiny"]
+# bulk, streaming and generic kernels for the whole groups; the chunk ends the open group and leaves a remainder behind its last group
+for bits, d, group in ((3, 128, 64), (2, 128, 128), (2, 128, 32), (4, 64, 80)):
+    wl = TINY.scaled(bits=bits, head_dim=d, group=group, n_q_heads=4, n_kv_heads=2, batch=2, seq=4 * group, topk=9, pfn_n=1, seed=51 + bits)
+    ocfg, gcfg = configs(wl)
+    H, (K, V) = synth.make_hidden(wl, "cuda"), synth.make_kv(wl, 0, "cuda")
+    gc = kv.KVCache(gcfg, kv.predict_sinks(gcfg, H, kv.SinkSet(gcfg)))
+    oc = oracle.Cache(ocfg, *oracle.predict_sinks(ocfg, np16(H)))
+    cut, end = group // 2 + 3, 3 * group + group // 2
+    k, v = K[:, :, cut:end], V[:, :, cut:end]
+    kv.quantize_append(gcfg, gc, K[:, :, :cut], V[:, :, :cut])
+    before = binding.lib().kvsink_launch_count()
+    binding.lib().kvsink_debug_fail_host_call(1)
+    try:
+        kv.quantize_append(gcfg, gc, k, v)
+        raise SystemExit("the append did not report the failed call")
+    except kv.KvsinkError as e:
+        assert e.code == -7, e
+    assert gc.seq_len == cut and binding.lib().kvsink_launch_count() == before
+    kv.quantize_append(gcfg, gc, k, v)             # once more, and this time it works
+    oracle.quantize_append(ocfg, oc, np16(K[:, :, :cut]), np16(V[:, :, :cut]))
+    oracle.quantize_append(ocfg, oc, np16(k), np16(v))
+    compare_cache(gc, oc, wl)
+    assert kv.read_status(gc) == 0
+print("failed append ok")
+"""
+
+
+@pytest.mark.gpu
+def test_an_append_that_fails_on_the_host_leaves_the_open_group():
+    if not os.path.exists(kv_build.DEBUG_LIB):
+        pytest.skip("libkvsink_debug.so has not been built (python -m paper_2508_04257_b200.build --debug)")
+    env = dict(os.environ, KVSINK_LIB=kv_build.DEBUG_LIB)
+    r = subprocess.run([sys.executable, "-c", FAILING_APPEND, ROOT], capture_output=True, text=True, env=env, timeout=600)
+    assert r.returncode == 0 and "failed append ok" in r.stdout, r.stdout[-1500:] + r.stderr[-3000:]
