@@ -91,7 +91,8 @@ __device__ __forceinline__ uint32_t code_exact(float x, float scale, float zero,
 // Programmatic stream serialization (dependent launch).  A kernel launched with launch_pdl may be scheduled while its
 // predecessor in the stream is still draining; it must call pdl_wait() before it reads or writes anything a predecessor
 // may have touched.  pdl_wait() returns once every prerequisite grid has completed and its writes are visible (at once
-// when the kernel was launched the ordinary way).
+// when the kernel was launched the ordinary way).  One kernel reads before it waits: the whole groups' kernel behind the
+// kernel of the same chunk's edges (quantize_bulk.cu says why it may).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // From here on the next kernel in the stream may be scheduled beside this one, up to its own wait.  Only after pdl_wait(), so
 // that a kernel that waits for this one has waited for everything before it too.

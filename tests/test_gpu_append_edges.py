@@ -53,3 +53,46 @@ def test_flat_chunks(scheme, bits, group):
     wl = TINY.scaled(bits=bits, head_dim=128, group=group, n_q_heads=3, n_kv_heads=3, batch=2, seq=sum(chunks), topk=40, pfn_n=1,
                      seed=33000 + bits * 100 + group)
     (test_gpu_calibrated if scheme == "static" else test_gpu_pertoken)._both(wl, chunks=chunks)
+
+
+# the whole groups' kernel of a ragged chunk starts beside the edges' kernel: its inputs, rewritten in place right before it by
+# kernels of the same stream, have to be the new ones every time
+@pytest.mark.parametrize("bits,group", [(3, 64), (2, 128), (4, 64)])
+def test_inputs_rewritten_in_place_right_before_a_ragged_chunk(bits, group):
+    T, cut, rounds = 9 * group + 11, group // 2 + 1, 8
+    wl = TINY.scaled(bits=bits, head_dim=128, group=group, n_q_heads=8, n_kv_heads=8, batch=4, seq=T, topk=40, pfn_n=1, seed=32000 + bits)
+    _, gcfg = configs(wl)
+    sources = []
+    for r in range(rounds):
+        one = wl.scaled(seed=wl.seed + 10 * r)
+        sources.append((synth.make_hidden(one, "cuda"), *synth.make_kv(one, 0, "cuda")))
+    names = [n for n in CACHE_BUFFERS if n != "status"]
+
+    def passes(wait):
+        H, K, V = (torch.empty_like(x) for x in sources[0])
+        gs = kv.SinkSet(gcfg)
+        gc = kv.KVCache(gcfg, gs)
+        seen = []
+        torch.cuda.synchronize()
+        for src in sources:
+            gc.seq_len = 0
+            H.copy_(src[0])
+            K[:, :, :cut].copy_(src[1][:, :, :cut])
+            V[:, :, :cut].copy_(src[2][:, :, :cut])
+            kv.predict_sinks(gcfg, H, gs)
+            wait()
+            kv.quantize_append(gcfg, gc, K[:, :, :cut], V[:, :, :cut])
+            wait()
+            K.copy_(src[1])
+            V.copy_(src[2])
+            kv.predict_sinks(gcfg, H, gs)
+            wait()
+            kv.quantize_append(gcfg, gc, K[:, :, cut:], V[:, :, cut:])
+            wait()
+            seen.append([getattr(gc, n).clone() for n in names])
+        assert kv.read_status(gc) == 0
+        return seen
+
+    for r, (got, ref) in enumerate(zip(passes(lambda: None), passes(torch.cuda.synchronize))):
+        for n, a, b in zip(names, got, ref):
+            assert torch.equal(a.view(torch.uint8), b.view(torch.uint8)), f"{n}, round {r}"
