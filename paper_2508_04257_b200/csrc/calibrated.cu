@@ -469,9 +469,10 @@ static int launch_tokens(const Params &p, const kvsink_cache &c, const kvsink_st
         return launch_pdl(append_one_flat_kernel<PT>, dim3((unsigned)((units + CO_WARPS - 1) / CO_WARPS)), dim3(32 * CO_WARPS), 0, st, p, c, sp, k_src,
                           v_src, first_token, sb, sh) == cudaSuccess ? KVSINK_OK : KVSINK_ERR_CUDA;
     }
-    // tokens before the next tile boundary go by themselves where whole tiles follow (the same chunk at 3 bit, G = 128: 680 -> 322 us)
+    // tokens before the next tile boundary go by themselves where whole tiles that follow have a kernel of their own, at head size 128
+    // (2859 tokens from 1237, 8 x 32 units, 3 bit, G = 128: 680 -> 322 us)
     const int lead = (KVSINK_TILE - first_token % KVSINK_TILE) % KVSINK_TILE;
-    if (lead > 0 && n_tokens >= lead + KVSINK_TILE) {
+    if (p.D == 128 && lead > 0 && n_tokens >= lead + KVSINK_TILE) {
         const int rc = launch_tokens<PT>(p, c, sp, k_src, v_src, first_token, lead, sb, sh, stt, st);
         return rc ? rc : launch_tokens<PT>(p, c, sp, k_src + (int64_t)lead * stt, v_src + (int64_t)lead * stt, first_token + lead, n_tokens - lead, sb, sh,
                                            stt, st);
@@ -498,7 +499,7 @@ int launch_quantize_calibrated(const Params &p, const kvsink_cache &c, const kvs
 {
     // whole G-token spans go to the bulk quantizer where it has a static form (G only shapes its work items); the tokens before the
     // first multiple of G and behind the last go to the others.  A chunk of 2859 tokens from 1237, 8 x 32 units, before only chunks
-    // that began on a multiple were split: static pairs at 2 bit 579 -> 105 us, per-token keys at 4 bit 743 -> 143 us
+    // that began on a multiple were split: 2 bit, 579 -> 105 us
     const int head = (p.G - first_token % p.G) % p.G, n_groups = (n_tokens - head) / p.G;
     if (n_tokens >= head + p.G) {
         const int64_t skip = (int64_t)head * stt;
@@ -518,9 +519,7 @@ int launch_quantize_pertoken(const Params &p, const kvsink_cache &c, const __hal
                              int64_t sb, int64_t sh, int64_t stt, cudaStream_t st)
 {
     const kvsink_static_params none = {nullptr, nullptr, nullptr, nullptr};
-    // whole G-token spans go to the bulk quantizer where it has this form (G only shapes its work items); the tokens before the
-    // first multiple of G and behind the last go to the others.  A chunk of 2859 tokens from 1237, 8 x 32 units, before only chunks
-    // that began on a multiple were split: static pairs at 2 bit 579 -> 105 us, per-token keys at 4 bit 743 -> 143 us
+    // split as with static parameters (per-token keys at 4 bit, the same chunk: 743 -> 143 us)
     const int head = (p.G - first_token % p.G) % p.G, n_groups = (n_tokens - head) / p.G;
     if (n_tokens >= head + p.G) {
         const int64_t skip = (int64_t)head * stt;

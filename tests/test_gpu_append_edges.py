@@ -96,3 +96,20 @@ def test_inputs_rewritten_in_place_right_before_a_ragged_chunk(bits, group):
     for r, (got, ref) in enumerate(zip(passes(lambda: None), passes(torch.cuda.synchronize))):
         for n, a, b in zip(names, got, ref):
             assert torch.equal(a.view(torch.uint8), b.view(torch.uint8)), f"{n}, round {r}"
+
+
+@pytest.mark.parametrize("d,launches", [(64, 1), (128, 3)])
+def test_tokens_before_a_tile_boundary_go_by_themselves_only_where_tiles_have_a_kernel(d, launches):
+    # 100 tokens from position 5 with G = 144 (no whole span): at head size 128 the 11 up to the boundary, five tiles, the last nine
+    cfg = kv.Config(1, 2, 2, d, 64, 2, 144, 144, 2, 1, (1,))
+    g = torch.Generator("cuda").manual_seed(1)
+    K, V = (torch.randn((1, 2, 105, d), device="cuda", generator=g).half() for _ in range(2))
+    sinks = kv.predict_sinks(cfg, torch.randn((1, 105, 64), device="cuda", generator=g).half(), kv.SinkSet(cfg))
+    params = kv.calibrate(cfg, K, V, sinks)
+    cache, whole = kv.KVCache(cfg, sinks), kv.KVCache(cfg, sinks)
+    kv.quantize_append_calibrated(cfg, whole, params, K, V)
+    kv.quantize_append_calibrated(cfg, cache, params, K[:, :, :5], V[:, :, :5])
+    before = kv.launch_count()
+    kv.quantize_append_calibrated(cfg, cache, params, K[:, :, 5:], V[:, :, 5:])
+    assert kv.launch_count() - before == launches
+    assert torch.equal(cache.k_codes, whole.k_codes) and torch.equal(cache.v_codes, whole.v_codes)
