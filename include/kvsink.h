@@ -169,10 +169,14 @@ int kvsink_decode_attention(const kvsink_config *cfg, const kvsink_cache *cache,
  *   q     device, fp16, element (b, hq, t, c) at q + b*stride_b + hq*stride_h + t*stride_t + c (strides in elements,
  *         multiples of 8).
  *   out   device out, float [B][Hq][T][D].      lse  device out, float [B][Hq][T] or NULL.
- * No workspace: every block of eight (query token, query head) rows streams its own prefix of the cache.
+ * No workspace: every block of rows (query token, query head) of one KV head streams its own prefix of the cache, 256 rows a block at
+ * head size 128 where that fills the chip, else eight.
  */
 int kvsink_prefill_attention(const kvsink_config *cfg, const kvsink_cache *cache, const void *q, int32_t T, int32_t q_pos0, int64_t stride_b,
                              int64_t stride_h, int64_t stride_t, float *out, float *lse, void *cuda_stream);
+
+/* Rows a block of kvsink_prefill_attention takes for T query tokens, 256 or 8 (host only, no CUDA call), or a KVSINK_ERR_* code. */
+int kvsink_prefill_rows(const kvsink_config *cfg, int32_t T);
 
 /*
  * kvsink_decode_attention for callers that cannot allocate device memory.  (No counterpart in the paper: this is

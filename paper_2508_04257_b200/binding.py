@@ -17,7 +17,7 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 _LIB_PATH = os.environ.get("KVSINK_LIB") or os.path.join(_HERE, "libkvsink.so")
 
 EXPORTS = ("kvsink_cache_sizes", "kvsink_predict_sinks", "kvsink_quantize_append", "kvsink_decode_attention",
-           "kvsink_decode_attention_static", "kvsink_prefill_attention", "kvsink_calibrate", "kvsink_quantize_append_calibrated",
+           "kvsink_decode_attention_static", "kvsink_prefill_attention", "kvsink_prefill_rows", "kvsink_calibrate", "kvsink_quantize_append_calibrated",
            "kvsink_decode_attention_calibrated", "kvsink_quantize_append_pertoken", "kvsink_decode_attention_pertoken",
            "kvsink_channel_absmax", "kvsink_quant_error", "kvsink_read_status",
            "kvsink_launch_count", "kvsink_strerror")
@@ -61,6 +61,7 @@ _ARGS = {
     "kvsink_decode_attention": (_P, _P, _P, _P, _P, _P, _Z, _P),
     "kvsink_decode_attention_static": (_P, _P, _P, _P, _P, _P),
     "kvsink_prefill_attention": (_P, _P, _P, _I, _I, _L, _L, _L, _P, _P, _P),
+    "kvsink_prefill_rows": (_P, _I),
     "kvsink_calibrate": (_P, _P, _P, _I, _L, _L, _L, _P, _P, _P, _Z, _P),
     "kvsink_quantize_append_calibrated": (_P, _P, _P, _P, _P, _I, _L, _L, _L, _P),
     "kvsink_decode_attention_calibrated": (_P, _P, _P, _P, _P, _P, _P, _Z, _P),
@@ -244,6 +245,14 @@ def prefill_attention(cfg: Config, cache: KVCache, q: torch.Tensor, q_pos0: int,
     if rc:
         raise KvsinkError(rc, "kvsink_prefill_attention")
     return out, lse
+
+
+def prefill_rows(cfg: Config, T: int) -> int:
+    """kvsink_prefill_rows: rows a block of prefill_attention takes for T query tokens, 256 (tensor-core blocks) or 8."""
+    rc = lib().kvsink_prefill_rows(C.byref(cfg.c()), T)
+    if rc < 0:
+        raise KvsinkError(rc, "kvsink_prefill_rows")
+    return rc
 
 
 def decode_attention_static(cfg: Config, cache: KVCache, q: torch.Tensor, out: torch.Tensor, lse: Optional[torch.Tensor] = None):

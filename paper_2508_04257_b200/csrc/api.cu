@@ -196,6 +196,15 @@ extern "C" int kvsink_prefill_attention(const kvsink_config *cfg, const kvsink_c
     return launch_prefill_b4(p, *cache, qq, T, q_pos0, stride_b, stride_h, stride_t, out, lse, st);
 }
 
+extern "C" int kvsink_prefill_rows(const kvsink_config *cfg, int32_t T)
+{
+    Params p;
+    const int rc = derive(cfg, &p);
+    if (rc) return rc;
+    if (T < 1) return KVSINK_ERR_BAD_ARG;
+    return prompt_takes(p, T) ? 256 : 8;
+}
+
 extern "C" int kvsink_decode_attention_static(const kvsink_config *cfg, const kvsink_cache *cache, const void *q, float *out,
                                               float *lse, void *cuda_stream)
 {

@@ -58,3 +58,13 @@ def test_null_and_misaligned_pointers_are_refused_before_any_launch():
     assert lib.kvsink_decode_attention(C.byref(cfg), C.byref(cache), null, null, null, null, C.c_size_t(0), null) == -1
     assert lib.kvsink_cache_sizes(None, None) == -1
     assert b"unknown" in lib.kvsink_strerror(12345)
+
+
+def test_prefill_rows_is_decided_on_the_host():
+    cfg = lambda **k: kv.Config(**{**dict(batch=8, n_q_heads=32, n_kv_heads=32, head_dim=128, hidden=64, bits=2, group=128, max_seq=4096, topk=8, pfn_n=1), **k})
+    assert kv.prefill_rows(cfg(), 4096) == 256 and kv.prefill_rows(cfg(), 1) == 8
+    assert kv.prefill_rows(cfg(head_dim=64), 4096) == 8
+    for bad, code in ((cfg(bits=5), -2), (cfg(), -1)):
+        with pytest.raises(kv.KvsinkError) as e:
+            kv.prefill_rows(bad, 0)
+        assert e.value.code == code

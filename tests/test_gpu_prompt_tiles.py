@@ -32,6 +32,7 @@ def _check(wl, T, pos0, shape_keys=None, shape_values=None, strided=False):
     q = torch.randn((wl.batch, wl.n_q_heads, T, wl.head_dim), device="cuda", generator=g).half()
     if strided:     # [B, T, Hq, D] storage
         q = q.permute(0, 2, 1, 3).contiguous().permute(0, 2, 1, 3)
+    assert kv.prefill_rows(gcfg, T) == 256
     out, lse = kv.prefill_attention(gcfg, gc, q, pos0)
     ref, ref_lse = oracle.prefill_attention(ocfg, oc, np16(q), pos0)
     torch.cuda.synchronize()
@@ -40,6 +41,7 @@ def _check(wl, T, pos0, shape_keys=None, shape_values=None, strided=False):
     top = float(V.abs().max())
     assert_close(out.cpu().numpy(), ref, "prompt attention", atol=2e-3 * max(1.0, top / 6.0))
     assert np.abs(lse.cpu().numpy() - ref_lse).max() <= 2e-3 + 1e-3 * np.abs(ref_lse).max()
+    return [np.linalg.norm(x.cpu().numpy() - r) / np.linalg.norm(r) for x, r in ((out, ref), (lse, ref_lse))]
 
 
 # rows of a unit: 64, 8 x 63, 8 x 129 (five blocks), 4 x 257, 3 x 171 = 513, 513; sequence ends inside a step, a tile, a group
@@ -92,6 +94,50 @@ def _prompt(wl):
     return gcfg, gc, q
 
 
+# Keys, values and weights are carried as fp16 pairs (22 bits).  Without the second half of one of them a factor keeps 11 bits, which
+# moves every weight or value by up to 2^-12 of itself, some 1.5e-4 in the mean, and the outputs, whose terms carry random signs, as much
+# (a numpy model of each of the three gives 1.6e-4 to 2.1e-4).  Sums in 32 bits over a few hundred terms stay below 1e-5
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("hq,hkv,T,pos0", [(16, 4, 400, 0), (16, 16, 300, 77)])
+def test_precision(bits, hq, hkv, T, pos0):
+    wl = TINY.scaled(bits=bits, head_dim=128, group=64, n_q_heads=hq, n_kv_heads=hkv, batch=2, seq=pos0 + T, topk=6, pfn_n=1, seed=27000 + bits)
+    out, lse = _check(wl, T, pos0)
+    assert out <= 3e-5 and lse <= 1e-6, (out, lse)
+
+
+# queries whose last one is not the cache's last token: a step's and a group's tokens behind them are masked, the open group among them
+@pytest.mark.parametrize("bits,group,behind", [(2, 128, 1), (3, 64, 63), (4, 64, 200), (2, 32, 500)])
+def test_chunk_that_ends_before_the_cache(bits, group, behind):
+    wl = TINY.scaled(bits=bits, head_dim=128, group=group, n_q_heads=16, n_kv_heads=8, batch=4, seq=310 + behind, topk=40, pfn_n=1, seed=28000 + bits + behind)
+    _check(wl, 210, 100)
+
+
+def test_without_the_log_sum():
+    wl = TINY.scaled(bits=4, head_dim=128, group=64, n_q_heads=16, n_kv_heads=8, batch=2, seq=257, topk=6, pfn_n=1, seed=28500)
+    gcfg, gc, q = _prompt(wl)
+    assert kv.prefill_rows(gcfg, wl.seq) == 256
+    out, lse = kv.prefill_attention(gcfg, gc, q, 0, want_lse=False)
+    assert lse is None and torch.equal(out, kv.prefill_attention(gcfg, gc, q, 0)[0])
+
+
+# a mask bit without an entry in the position list: the token has no row anywhere, so it takes no part, as on the eight-row blocks
+@pytest.mark.parametrize("bits", [2, 4])
+def test_mask_bit_without_a_list_entry(bits):
+    wl = TINY.scaled(bits=bits, head_dim=128, group=64, n_q_heads=16, n_kv_heads=8, batch=2, seq=300, topk=6, pfn_n=1, seed=29000 + bits)
+    gcfg, gc, q = _prompt(wl)
+    listed = set(gc.sinks.pos.cpu().tolist())
+    extra = [t for t in (2, 64, 100, 130, 131, 255, 290) if t not in listed]
+    words = gc.sinks.bitmask.view(wl.batch, -1)
+    for t in extra:
+        words[:, t // 32] |= (1 << t % 32) - (1 << 32 if t % 32 == 31 else 0)
+    assert kv.prefill_rows(gcfg, 300) == 256 and kv.prefill_rows(gcfg, 12) == 8
+    out, lse = kv.prefill_attention(gcfg, gc, q, 0)
+    for t in range(0, 300, 12):
+        small, small_lse = kv.prefill_attention(gcfg, gc, q[:, :, t:t + 12], t)
+        assert_close(out[:, :, t:t + 12].cpu().numpy(), small.cpu().numpy(), f"queries {t}")
+        assert (lse[:, :, t:t + 12] - small_lse).abs().max() <= 2e-3 + 1e-3 * small_lse.abs().max()
+
+
 def _same_every_time(gcfg, gc, q, pos0, times):
     first = kv.prefill_attention(gcfg, gc, q, pos0)
     for _ in range(times):
@@ -114,6 +160,7 @@ def test_a_tile_that_ends_before_the_other(bits, T):
 def test_many_steps_over_the_same_score_buffers(bits, hq, hkv, batch):
     wl = TINY.scaled(bits=bits, head_dim=128, group=128, n_q_heads=hq, n_kv_heads=hkv, batch=batch, seq=3000, topk=30, pfn_n=1, seed=24100 + bits)
     gcfg, gc, q = _prompt(wl)
+    assert kv.prefill_rows(gcfg, 900) == 256
     _same_every_time(gcfg, gc, q[:, :, -900:], 2100, times=10)
 
 
