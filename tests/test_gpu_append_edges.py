@@ -113,3 +113,35 @@ def test_tokens_before_a_tile_boundary_go_by_themselves_only_where_tiles_have_a_
     kv.quantize_append_calibrated(cfg, cache, params, K[:, :, 5:], V[:, :, 5:])
     assert kv.launch_count() - before == launches
     assert torch.equal(cache.k_codes, whole.k_codes) and torch.equal(cache.v_codes, whole.v_codes)
+
+
+# static appends of shapes that decode has no kernel for (codes and sink rows only): two channels a lane, four channel groups a row,
+# groups longer than a row; single tokens on fresh tiles and on used ones, and chunks around tile and span boundaries
+@pytest.mark.parametrize("d,bits,group", [(64, 2, 32), (64, 4, 32), (64, 2, 64), (64, 4, 64), (128, 2, 32), (128, 3, 32), (128, 4, 144), (128, 3, 144)])
+def test_static_shapes_without_decode(d, bits, group):
+    chunks = (1, 1, 14, 1, 20, 1, 2 * group + 35, 1, 9, 1, 1)
+    wl = TINY.scaled(bits=bits, head_dim=d, group=group, n_q_heads=3, n_kv_heads=3, batch=2, seq=sum(chunks), topk=60, pfn_n=1, seed=34000 + bits + d + group)
+    ocfg, gcfg = configs(wl)
+    H = synth.make_hidden(wl, "cuda")
+    K, V = synth.make_kv(wl, 0, "cuda")
+    gs = guard(kv.SinkSet(gcfg), SINK_BUFFERS)
+    kv.predict_sinks(gcfg, H, gs)
+    bm, pos, cnt = oracle.predict_sinks(ocfg, np16(H))
+    gp, op = kv.calibrate(gcfg, K[:, :, :90], V[:, :, :90], gs), oracle.calibrate(ocfg, np16(K[:, :, :90]), np16(V[:, :, :90]), bm)
+    gc, oc = guard(kv.KVCache(gcfg, gs), CACHE_BUFFERS), oracle.Cache(ocfg, bm, pos, cnt)
+    at = 0
+    for n in chunks:
+        k, v = K[:, :, at:at + n], V[:, :, at:at + n]
+        kv.quantize_append_calibrated(gcfg, gc, gp, k, v)
+        oracle.quantize_append_calibrated(ocfg, oc, op, np16(k), np16(v))
+        at += n
+        used, per = (at + 15) // 16 * 16 * d * bits // 8, wl.max_seq * d * bits // 8
+        for name in ("k_codes", "v_codes"):
+            g, o = (x.reshape(-1, per)[:, :used] for x in (getattr(gc, name).cpu().numpy(), getattr(oc, name)))
+            assert g.tobytes() == o.tobytes(), f"{name} after {at} tokens"
+        for name in ("sink_k", "sink_v"):
+            g = getattr(gc, name).cpu().numpy().reshape(-1)
+            assert g.tobytes() == getattr(oc, name).tobytes(), f"{name} after {at} tokens"
+    assert kv.read_status(gc) == 0
+    check_guards(gs)
+    check_guards(gc)
