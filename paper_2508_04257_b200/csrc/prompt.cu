@@ -57,7 +57,7 @@ struct PromptSmem {
     StepHeader hdr[PR_HDRS];
     int k_rank[2][64], v_rank[2][64];           // side buffer rows of the step's sink tokens, in token order
     uint64_t k_full[PR_KSTAGES], k_empty[PR_KSTAGES], v_full[PR_VSTAGES], v_empty[PR_VSTAGES];
-    uint64_t kpar_full[2], kpar_empty[2], vpar_full[2], vpar_empty[2], v_hdr[PR_HDRS];
+    uint64_t kpar_full[2], kpar_empty[2], vpar_full[2], vpar_empty[2], hdr_full[PR_HDRS];
     uint64_t s_full[PR_SBUFS], p_full[PR_SBUFS], o_done[PR_SBUFS], o_last[2], q_full[2], drained[2];
     uint32_t tmem;
     int failed;
@@ -332,7 +332,10 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
     };
     const int n0 = tile_steps(0), n1 = tile_steps(1), n_steps = max(n0, n1);
     // every thread alike, and before anything is set up; index checks of single accesses are at the accesses
-    if (!in_bounds(b < p.B && row0 < n_rows && a.q_pos0 >= 0 && a.q_pos0 + a.T <= seq_len && seq_len <= p.max_seq && p.cap >= 0, c.status)) return;
+    if (!in_bounds(b < p.B && row0 < n_rows && a.q_pos0 >= 0 && a.q_pos0 + a.T <= seq_len && seq_len <= p.max_seq && p.cap >= 0, c.status)) {
+        pdl_wait();
+        return;
+    }
 
     if (warp == 16) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&sm.tmem)), "r"(512) : "memory");
@@ -348,7 +351,7 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
                 bar_init(&sm.o_last[i], 1);
                 bar_init(&sm.drained[i], 1);
             }
-            for (int i = 0; i < PR_HDRS; ++i) bar_init(&sm.v_hdr[i], 1);
+            for (int i = 0; i < PR_HDRS; ++i) bar_init(&sm.hdr_full[i], 2);
             sm.failed = 0;
             sm.odd_values = 0;
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -358,8 +361,8 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
     }
     __syncthreads();
     tc_fence_after();
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    pdl_wait();
+    pdl_release();
 
     // 96 registers per thread at launch: 2 x 128 threads to 128, 2 x 128 to 80, 128 to 64 add up to the same 61440
     if (warp < 8) {
@@ -413,7 +416,7 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
             const int sb = item % PR_SBUFS;
             const uint32_t t_s = lanes + TM_S + 64 * sb;
             if (!(ok = bar_wait_warp(&sm.s_full[sb], (item / PR_SBUFS) & 1, &sm.failed))) break;
-            if (!(ok = bar_wait_warp(&sm.v_hdr[j & (PR_HDRS - 1)], (j / PR_HDRS) & 1, &sm.failed))) break;
+            if (!(ok = bar_wait_warp(&sm.hdr_full[j & (PR_HDRS - 1)], (j / PR_HDRS) & 1, &sm.failed))) break;
             tc_fence_after();
             const StepHeader &hd = sm.hdr[j & (PR_HDRS - 1)];
             const float c1 = qscale * hd.k_down, ef = hd.e, vup = hd.v_up;
@@ -880,7 +883,7 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
             __syncwarp();
             if (lane == 0) {
                 bar_arrive(&full[buf]);
-                if (!keys) bar_arrive(&sm.v_hdr[j & (PR_HDRS - 1)]);
+                bar_arrive(&sm.hdr_full[j & (PR_HDRS - 1)]);        // for the softmax: both warps' halves of the header
             }
         }
     }
