@@ -1224,13 +1224,15 @@ static int launch_decode_p(const Params &p, const kvsink_cache &c, const kvsink_
     pdl[0].val.programmaticStreamSerializationAllowed = 1;
     // up to eight splits (the portable cluster size): the splits of a unit are launched as one thread-block cluster and
     // merged inside the kernel through distributed shared memory, which saves the merge kernel's 1 to 1.8 us (4 x 32 units of 2048
-    // tokens, 2 bit: 12.3 -> 10.5 us).  A cluster has to be placed as a whole, though, and where the grid fills the chip with
-    // long blocks the slots it leaves empty cost more: 18 x 8 units of 47328 tokens in four splits, 3 bit, 232 us as clusters and
-    // 181 us without, 11 x 8 units of 9068 in six, 4 bit, 29.2 and 26.6 us; pairs are better off alone from some 256 KB a block
-    // (25.1 against 26.6 us at 128 KB, 417 against 412 us at 512 KB)
+    // tokens in fours, 2 bit: 12.2 -> 11.2 us).  A cluster has to be placed as a whole, though, and where the grid fills the chip with
+    // long blocks the slots it leaves empty cost more (clusters, and none; append and decode): fours, 18 x 8 units of 30000 tokens 106
+    // and 86 us at 2 bit, 160 and 133 at 4; sixes, 3 x 32 of 12000, 2 bit, 53 and 38.  Pairs of 2 and 4 bit
+    // win or tie at every length measured (32 x 8 of 9000 with four heads each 71.5 and 74.1, 97.5 and 100.2; 8 x 32 of 16384, 4 bit, 134.3 and
+    // 134.8), at 3 bit up to some 256 KB a block (16 x 32 of 8192, 384 KB a block, 137 and 136)
     const int64_t blocks = (int64_t)nsplit * p.Hkv * qchunks * p.B;
     const int64_t block_bytes = (int64_t)gps * (PM != 0 ? CT * KVSINK_TILE : p.G) * 2 * p.row_bytes;
-    bool cluster_merge = nsplit > 1 && nsplit <= 8 && (blocks <= 2 * 148 || block_bytes < (nsplit == 2 ? 256 : 64) * 1024);
+    const bool pairs = nsplit == 2 && p.bits != 3;
+    bool cluster_merge = nsplit > 1 && nsplit <= 8 && (pairs || blocks <= 2 * 148 || block_bytes < (nsplit == 2 ? 256 : 64) * 1024);
     for (;;) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(nsplit, p.Hkv * qchunks, p.B);
