@@ -6,7 +6,7 @@
 
 namespace kvsink {
 
-// Merge of the sequence splits (more than eight per unit): one block per (sequence, query head); thread (ch, sl) folds the
+// Merge of the sequence splits (where the splits of a unit are not launched as a cluster): one block per (sequence, query head); thread (ch, sl) folds the
 // records sl, sl + MERGE_SLICES, ... of channel ch, and the slices are combined in a fixed order (bit-reproducible).
 constexpr int MERGE_SLICES = 4;
 
@@ -75,10 +75,12 @@ int max_splits(const Params &p)
     return (int)(ns < 1 ? 1 : ns);
 }
 
-// Two and four bit: whole waves of resident blocks times the groups of a warp.  Three bit is bound by issue slots, so an SM's time
-// goes with the number of blocks it gets in all (four resident ones run at full rate, two at three quarters of it), each with the
-// groups of a warp and about one group's time for its prologue and epilogue: 16 x 32 units of 8101 tokens take two splits of
-// 512 blocks' work (7 blocks on the fullest SM instead of 4 of twice the size), 150 -> 129 us.
+// Two and four bit: whole waves of resident blocks times the groups of a warp.  At three bit an SM's time goes with the number of
+// blocks it gets in all (four resident ones run at full rate, two at three quarters of it, by measurement), each with the
+// groups of a warp and about one group's time for its prologue and epilogue.  Measured, microseconds, this rule's choice first and
+// other split counts behind it: 16 x 32 units of 8101 tokens 2: 129 (1: 143, 3: 134; 7 blocks on the fullest SM instead of 4 of
+// twice the size); 8 x 32 of 4096 4: 39 (1: 47, 2: 42); 1 x 8 of 131072 with four heads 74: 54 (37: 59, 64: 57, 96: 64);
+// 4 x 8 of 30000 with four heads 18: 50 (8: 70, 12: 57, 37: 55); 37 x 8 of 9000 2: 85 (1: 98, 3: 87).
 int choose_splits(const Params &p, int n_groups)
 {
     const int qchunks = decode_qchunks(p);

@@ -14,11 +14,12 @@
 // tile's scores are in the softmax the tensor cores run the other tile's products.
 //
 // What bounds it: five matrix products of 128 x 64 x 128 per row tile and step are 2560 clocks for both tiles (2816 with tile 1's
-// queries in shared memory); measured are about 4400: issue slots (the softmax's ~320 instructions for 64 scores of a row, the
-// expansion's ~300 per warp) and instruction fetch, which is why every loop here is kept short and in one copy (with 145 KB of
-// unrolled code a step took 9000 clocks).  4096 queries over 4096 tokens, 8 sequences of 32 heads, 2 bit: 12.8 -> 2.5 ms
-// (434 TFLOP/s of causal pairs, 1085 TFLOP/s of executed products); 1003 queries with four heads per KV head over 7403 tokens,
-// 4 bit: 1.64 -> 0.30 ms.  Relative error against 64 bits 5.3e-5 -> 2.7e-6 and 4.6e-5 -> 8.9e-6.
+// queries in shared memory); measured are about 4700.  Neither the tensor pipe (active 60 % of the cycles) nor the issue slots (52 %)
+// are full: it is the chain of hand-overs (scores, softmax, outputs, the buffers' return) and of the parameter warps.  Every loop is
+// kept short and in one copy (unrolled, the warps waited for instructions: 9000 clocks a step).  4096 queries over 4096 tokens, 8
+// sequences of 32 heads, 2 bit, with the append, back to back: 12.8 ms on the eight-row kernel, 2.75 here; alone 2.41 (457 TFLOP/s of
+// causal pairs, 1140 of executed products).  1003 queries with four heads per KV head over 7403 tokens, 4 bit, with the append: 1.64 and
+// 0.294 ms.  Relative error of the outputs against 64 bits: 5.3e-5 there, 2.6e-6 here, and 4.6e-5, 8.2e-6.
 #include "common.cuh"
 
 namespace kvsink {
@@ -78,8 +79,7 @@ __device__ __forceinline__ void bar_arrive(uint64_t *bar)
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
 // Bounded wait of a whole warp; false after the limit, or soon after another warp of the block ran into its own.  All exits are
-// votes: a loop that lanes could leave one by one makes the code around it divergent for the compiler, and descriptors of
-// matrix instructions then leave the uniform registers (41 instructions instead of 7 for each of them).
+// votes, so that the warp stays converged for the matrix instructions behind it.
 __device__ __forceinline__ bool bar_wait_warp(uint64_t *bar, unsigned parity, int *failed)
 {
     const uint32_t a = smem_addr(bar);
@@ -107,8 +107,8 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr)
 // kind::f16, fp16 operands, fp32 accumulators, M = 128
 __host__ __device__ constexpr uint32_t instr_desc(int n) { return (1u << 4) | ((uint32_t)(n / 8) << 17) | (8u << 24); }
 
-// Issued by one elected lane of a converged warp.  Descriptors and addresses have to stay in uniform registers: under a branch on
-// the lane number instead of elect.sync an instruction took 53 clocks to issue, whatever its size.
+// Issued by one elected lane of a converged warp: under a branch on the lane number instead of elect.sync an instruction took 53
+// clocks to issue, whatever its size.
 __device__ __forceinline__ bool elect_one()
 {
     unsigned yes;
