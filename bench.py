@@ -640,7 +640,7 @@ def run_ours(args):
             "peak_kind": f"{peak_kind} copy bandwidth", "unit": "GB/s", "frac": head["q_gbs"] / peak,
             "frac_of_nominal_8TBs": head["q_gbs"] / NOMINAL_HBM_GBS, "algorithmic_bytes_per_launch": head["qb"],
             "us_per_launch": head["us"]["quantize"], "traffic": ncu_traffic("quantize_bulk_kernel", wl.name) if args.batch == 0 else None}
-    roof_d = {"bound": "hbm", "kernel": "decode_kernel (+ decode_merge_kernel beyond eight splits)", "achieved": head["d_gbs"], "peak": peak,
+    roof_d = {"bound": "hbm", "kernel": "decode_kernel (+ decode_merge_kernel where the splits of a unit are not a cluster)", "achieved": head["d_gbs"], "peak": peak,
               "unit": "GB/s", "frac": head["d_gbs"] / peak, "frac_of_nominal_8TBs": head["d_gbs"] / NOMINAL_HBM_GBS,
               "algorithmic_bytes_per_launch": head["db"], "us_per_launch": head["us"]["decode"],
               "traffic": ncu_traffic("decode_kernel", wl.name) if args.batch == 0 else None}
