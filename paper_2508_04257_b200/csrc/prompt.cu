@@ -14,12 +14,14 @@
 // tile's scores are in the softmax the tensor cores run the other tile's products.
 //
 // What bounds it: five matrix products of 128 x 64 x 128 per row tile and step are 2560 clocks for both tiles (2816 with tile 1's
-// queries in shared memory); measured are about 4700.  Neither the tensor pipe (active 60 % of the cycles) nor the issue slots (52 %)
-// are full: it is the chain of hand-overs (scores, softmax, outputs, the buffers' return) and of the parameter warps.  Every loop is
-// kept short and in one copy (unrolled, the warps waited for instructions: 9000 clocks a step).  4096 queries over 4096 tokens, 8
-// sequences of 32 heads, 2 bit, with the append, back to back: 12.8 ms on the eight-row kernel, 2.75 here; alone 2.41 (457 TFLOP/s of
-// causal pairs, 1140 of executed products).  1003 queries with four heads per KV head over 7403 tokens, 4 bit, with the append: 1.64 and
-// 0.294 ms.  Relative error of the outputs against 64 bits: 5.3e-5 there, 2.6e-6 here, and 4.6e-5, 8.2e-6.
+// queries in shared memory); a step takes about 3700, with the tensor pipe active for 3150 of them (82 %) and 73 to 80 % of the issue
+// slots taken.  What counts is how little code the five roles have between them: at 71 KB, with the loops unrolled, the warps
+// waited for instructions (1.9 of their stalls an issue; a step with a sink token, whose code was seldom there, took 4500 clocks
+// more), at 54 KB hardly (0.3).  So every role is one short loop: tiles two at a time, one pass over a row's scores, parameters
+// and sink rows through shared memory.  4096 queries over 4096 tokens, 8 sequences of 32 heads, 2 bit, with the append, back to
+// back: 2657 us at 71 KB, 2556 now (the power cap holds the clock at some 1.4 GHz).  1003 queries with four heads per KV head over 7403 tokens,
+// 4 bit, with the append: 308 and 270 us; the same at 3 bit with 128-token groups 319 and 275; 2048 queries, 2 x 32 heads, 2 bit with
+// 64-token groups 239 and 212.  Relative error of the outputs against 64 bits: 2.6e-6 and 8.2e-6 for the first two.
 #include "common.cuh"
 
 namespace kvsink {
@@ -35,8 +37,9 @@ constexpr int PR_HALF = 16384;                  // 64 tokens x 128 channels of f
 constexpr int PR_HDRS = 8;
 // A zero point up to this size is subtracted from the code in fp16 exactly; farther ones go through an additive term.
 constexpr float PR_NEAR = 1000.f;
-constexpr long long PR_WAIT_CLOCKS = 1ll << 29;  // about 0.3 s: far beyond any real wait
 constexpr uint32_t PR_WAIT_NS = 20000;          // a poll sleeps up to this long (without the hint it comes back after some 60 clocks)
+constexpr int PR_WAIT_POLLS = 1 << 16;          // 1.3 s of such polls: far beyond any real wait
+constexpr int PR_ROWS_KEPT = 8;                 // sink rows of a step that the parameter warps leave in shared memory
 
 struct StepHeader {
     float k_down, k_up, v_up;                   // 2^-kappa, 2^kappa, 2^e: the step's units of K and V
@@ -56,7 +59,9 @@ struct PromptSmem {
     uint4 vtab[2][4][32];                       // per value channel group and token pair
     uint2 kadd[2][2][64], vadd[2][4][32];       // additive terms hi, lo of far zero points
     StepHeader hdr[PR_HDRS];
+    float k_raw[2][2][2][128], v_raw[2][2][256];   // parameters as they are in memory, by the step's buffer: keys [group][scale, zero][channel], values [scale, zero][token][group]
     int k_rank[2][64], v_rank[2][64];           // side buffer rows of the step's sink tokens, in token order
+    uint4 k_kept[2][PR_ROWS_KEPT][16], v_kept[2][PR_ROWS_KEPT][16];   // the first of those rows
     uint64_t k_full[PR_KSTAGES], k_empty[PR_KSTAGES], v_full[PR_VSTAGES], v_empty[PR_VSTAGES];
     uint64_t kpar_full[2], kpar_empty[2], vpar_full[2], vpar_empty[2], hdr_full[PR_HDRS];
     uint64_t s_full[PR_SBUFS], p_full[PR_SBUFS], o_done[PR_SBUFS], o_last[2], q_full[2], drained[2];
@@ -83,15 +88,13 @@ __device__ __forceinline__ void bar_arrive(uint64_t *bar)
 __device__ __forceinline__ bool bar_wait_warp(uint64_t *bar, unsigned parity, int *failed)
 {
     const uint32_t a = smem_addr(bar);
-    long long start = 0;
 #pragma unroll 1
-    for (unsigned polls = 0;; ++polls) {
+    for (int polls = 0; polls < PR_WAIT_POLLS; ++polls) {
         unsigned ok;
         asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3; selp.u32 %0, 1, 0, p; }"
                      : "=r"(ok) : "r"(a), "r"(parity), "r"(PR_WAIT_NS) : "memory");
         if (__all_sync(0xffffffffu, ok != 0)) return true;
-        if (polls == 0) start = clock64();
-        if (__any_sync(0xffffffffu, *(volatile int *)failed || clock64() - start > PR_WAIT_CLOCKS)) break;
+        if (__any_sync(0xffffffffu, *(volatile int *)failed)) break;
     }
     *(volatile int *)failed = 1;
     return false;
@@ -421,35 +424,34 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
             const StepHeader &hd = sm.hdr[j & (PR_HDRS - 1)];
             const float c1 = qscale * hd.k_down, ef = hd.e, vup = hd.v_up;
             const uint32_t dead0 = hd.dead[0], dead1 = hd.dead[1];
-            // tokens that the row does not see; the two passes over the scores (largest, weights) re-read them from TMEM, half a
-            // step at a time: one copy of the code for both halves
-            const bool masked = (j + 1) * PR_STEP > lim_min || (dead0 | dead1);
+            // tokens that the row does not see: -inf over their scores, in the steps that have any
             const int left = lim - j * PR_STEP;
-            auto load = [&](int half, uint32_t (&v)[32]) {
-                tm_load32(t_s + 32 * half, v);
-                tm_wait_load();
-                if (masked) {
-                    const int n = left - 32 * half;
-                    const uint32_t gone = (half ? dead1 : dead0) | (n <= 0 ? 0xffffffffu : (n >= 32 ? 0u : 0xffffffffu << n));
-#pragma unroll
-                    for (int x = 0; x < 32; ++x)
-                        if (gone >> x & 1u) v[x] = 0xff800000u;
-                }
-            };
-            float top = -INFINITY;
+            if ((j + 1) * PR_STEP > lim_min || (dead0 | dead1)) {
 #pragma unroll 1
-            for (int half = 0; half < 2; ++half) {
-                uint32_t v[32];
-                load(half, v);
-                float tops[4];
+                for (int x = 0; x < 64; x += 16) {
+                    uint32_t v[16];
+                    tm_load16(t_s + x, v);
+                    tm_wait_load();
+                    const int n = left - x;
+                    const uint32_t gone = (x < 32 ? dead0 : dead1) >> (x & 16) | (n <= 0 ? 0xffffu : (n >= 16 ? 0u : 0xffffu << n));
 #pragma unroll
-                for (int x = 0; x < 4; ++x) tops[x] = __uint_as_float(v[x]);
-#pragma unroll
-                for (int x = 4; x < 32; x += 8)
-#pragma unroll
-                    for (int y = 0; y < 4; ++y) tops[y] = x + 4 + y < 32 ? max3(tops[y], __uint_as_float(v[x + y]), __uint_as_float(v[x + 4 + y])) : fmaxf(tops[y], __uint_as_float(v[x + y]));
-                top = max3(max3(tops[0], tops[1], tops[2]), tops[3], top);
+                    for (int y = 0; y < 16; ++y)
+                        if (gone >> y & 1u) v[y] = 0xff800000u;
+                    tm_store16(t_s + x, v);
+                }
+                tm_wait_store();
             }
+            uint32_t v0[32], v1[32];
+            tm_load32(t_s, v0);
+            tm_load32(t_s + 32, v1);
+            tm_wait_load();
+            float top = max3(__uint_as_float(v0[0]), __uint_as_float(v1[0]), -INFINITY), top2 = -INFINITY;
+#pragma unroll
+            for (int x = 1; x < 31; x += 2) {
+                top = max3(top, __uint_as_float(v0[x]), __uint_as_float(v0[x + 1]));
+                top2 = max3(top2, __uint_as_float(v1[x]), __uint_as_float(v1[x + 1]));
+            }
+            top = max3(max3(top, top2, __uint_as_float(v0[31])), __uint_as_float(v1[31]), -INFINITY);
             top = fmaf(top, c1, -ef);
             if (__any_sync(0xffffffffu, top > M + 15.f)) {
                 const float Mn = top > M + 15.f ? top - 8.f : M, f = ex2(M - Mn);
@@ -471,22 +473,21 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
             }
             const float2 c2 = make_float2(c1, c1), sub2 = make_float2(-(M + ef), -(M + ef));
             float2 sum = make_float2(0.f, 0.f);
-#pragma unroll 1
-            for (int half = 0; half < 2; ++half) {       // the half's weights take its scores' place: hi, then lo
-                uint32_t v[32], hi[16], lo[16];
-                load(half, v);
+            auto weights = [&](uint32_t (&v)[32], uint32_t to) {       // the half's weights take its scores' place: hi, then lo
+                uint32_t r[32];
 #pragma unroll
                 for (int x = 0; x < 16; ++x) {
                     float2 w = fma2(make_float2(__uint_as_float(v[2 * x]), __uint_as_float(v[2 * x + 1])), c2, sub2);
                     w.x = ex2(w.x); w.y = ex2(w.y);
                     sum = add2(sum, w);
                     const __half2 wh = __floats2half2_rn(w.x, w.y);
-                    hi[x] = as_u32(wh);
-                    lo[x] = as_u32(__floats2half2_rn(residual(__low2half(wh), w.x), residual(__high2half(wh), w.y)));
+                    r[x] = as_u32(wh);
+                    r[16 + x] = as_u32(__floats2half2_rn(residual(__low2half(wh), w.x), residual(__high2half(wh), w.y)));
                 }
-                tm_store16(t_s + 32 * half, hi);
-                tm_store16(t_s + 32 * half + 16, lo);
-            }
+                tm_store32(to, r);
+            };
+            weights(v0, t_s);
+            weights(v1, t_s + 32);
             l = fmaf(sum.x + sum.y, vup, l);
             tm_wait_store();
             tc_fence_before();
@@ -534,60 +535,38 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
         const int coded = keys ? n_body : seq_len;                       // tokens below it have codes
         // stmatrix: lane l gives the address of row l % 8 of the 8 x 8 matrix l / 8 (row half l/8 % 2, column half l / 16)
         const int sr = (lane & 7) + 8 * ((lane >> 3) & 1), sc = lane >> 4;
-        uint32_t next[4][2], cur[4][2];
         constexpr int TILE = 16 * D * BITS / 8;
-        auto fetch = [&](int j) {
-            const uint8_t *tile = codes + (size_t)j * 4 * TILE;
-            if (!in_bounds(min((j + 1) * PR_STEP, (coded + KVSINK_TILE - 1) / KVSINK_TILE * KVSINK_TILE) <= p.max_seq, c.status)) return;
-            if ((j + 1) * PR_STEP <= coded) {
-#pragma unroll
-                for (int tt = 0; tt < 4; ++tt) load_words<BITS>(tile + tt * TILE, w, lane, next[tt]);
-            } else {
-#pragma unroll
-                for (int tt = 0; tt < 4; ++tt) {
-                    next[tt][0] = next[tt][1] = 0u;
-                    if (j * PR_STEP + 16 * tt < coded) load_words<BITS>(tile + tt * TILE, w, lane, next[tt]);
-                }
-            }
-        };
-        auto take = [&](int j) {       // the words of step j, and the loads of the next
-#pragma unroll
-            for (int tt = 0; tt < 4; ++tt) { cur[tt][0] = next[tt][0]; cur[tt][1] = next[tt][1]; }
-            if (j + 1 < n_steps) fetch(j + 1);
+        // words of the next four tiles, each loaded when the one four before it is taken
+        uint32_t words[4][2];
+        auto fetch = [&](int tile, uint32_t (&to)[2]) {
+            to[0] = to[1] = 0u;
+            if (tile < 4 * n_steps && 16 * tile < coded && in_bounds(16 * (tile + 1) <= p.max_seq, c.status)) load_words<BITS>(codes + (size_t)tile * TILE, w, lane, to);
         };
         // keys: row = token, 16-byte chunk = eight channels, two panels of 64; values: row = channel, chunk = eight tokens
         auto place = [](int r, int ck) { return (uint32_t)((ck >> 3) * 8192 + r * 128 + (((ck & 7) ^ (r & 7)) << 4)); };
         // sink tokens: their exact rows over the expanded ones
-        auto put_sinks = [&](const uint32_t (&sink)[2], const int *ranks, uint32_t base, float up) {
+        auto put_sinks = [&](const uint32_t (&sink)[2], const int *ranks, const uint4 (*kept)[16], uint32_t base, float up) {
             __syncwarp();
             const int ch = 32 * w + lane;
-            const __half *rows = (const __half *)(keys ? c.sink_k : c.sink_v) + (size_t)unit * p.cap * D + ch;
+            const __half *rows = (const __half *)(keys ? c.sink_k : c.sink_v) + (size_t)unit * p.cap * D + ch, *near = (const __half *)kept + ch;
             uint64_t left = (uint64_t)sink[1] << 32 | sink[0];
-            int idx = 0;
-            while (left) {
-                int tk[8];
-                float x[8];
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {      // the loads of eight rows together
-                    tk[k] = -1;
-                    x[k] = 0.f;
-                    if (left) {
-                        tk[k] = __ffsll((long long)left) - 1;
-                        left &= left - 1;
-                        const int r = ranks[idx++];
-                        if (r >= 0 && in_bounds(idx <= 64 && r < p.cap, c.status)) x[k] = __half2float(rows[(size_t)r * D]);
-                        if (!keys && !is_finite(x[k])) x[k] = 0.f;     // a weight of 0 does not hide it: added at the end
-                    }
+#pragma unroll 1
+            for (int idx = 0; left; ++idx) {
+                const int tk = __ffsll((long long)left) - 1;
+                left &= left - 1;
+                float x = 0.f;
+                if (idx < PR_ROWS_KEPT) {
+                    x = __half2float(near[idx * D]);
+                } else {
+                    const int r = ranks[idx];
+                    if (r >= 0 && in_bounds(r < p.cap, c.status)) x = __half2float(rows[(size_t)r * D]);
                 }
-#pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    if (tk[k] >= 0) {
-                        const int r = keys ? tk[k] : ch, col = keys ? ch : tk[k];
-                        const uint32_t at = base + place(r, col >> 3) + 2 * (col & 7);
-                        const unsigned short v = __half_as_ushort(__float2half_rn(x[k] * up));
-                        asm volatile("st.shared.u16 [%0], %1;" ::"r"(at), "h"(v) : "memory");
-                        asm volatile("st.shared.u16 [%0], %1;" ::"r"(at + PR_HALF), "h"((unsigned short)0) : "memory");
-                    }
+                if (!keys && !is_finite(x)) x = 0.f;     // a weight of 0 does not hide it: added at the end
+                const int r = keys ? tk : ch, col = keys ? ch : tk;
+                const uint32_t at = base + place(r, col >> 3) + 2 * (col & 7);
+                const unsigned short v = __half_as_ushort(__float2half_rn(x * up));
+                asm volatile("st.shared.u16 [%0], %1;" ::"r"(at), "h"(v) : "memory");
+                asm volatile("st.shared.u16 [%0], %1;" ::"r"(at + PR_HALF), "h"((unsigned short)0) : "memory");
             }
         };
         const __half *tail = (const __half *)c.k_tail + (size_t)unit * p.G * D;
@@ -596,18 +575,16 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
         // byte offsets of the lane's stmatrix rows for tile tt, matrix mm, and table entries of its columns: by channel pair (keys,
         // the step's second group 64 entries on) or by token pair (values)
         const int jg = 32 * w / p.Gv;                                    // value channel group of the warp's channels
-        auto row_at = [&](int tt, int mm) { return keys ? place(16 * tt + sr, 4 * w + 2 * mm + sc) : place(32 * w + 16 * mm + sr, 2 * tt + sc); };
-        auto entry = [&](int tt, int mm, int second) { return keys ? (tt >= second ? 64 : 0) + 16 * w + 8 * mm + t : 32 * jg + 8 * tt + t; };
-        uint32_t at[4][2];
+        const uint32_t at0 = keys ? place(sr, 4 * w + sc) : place(32 * w + sr, sc), at1 = keys ? place(sr, 4 * w + 2 + sc) : place(32 * w + 16 + sr, sc);
+        const uint32_t add_tile = keys ? 2048 : 0, xor_tile = keys ? 0 : 32;
+        const int entry0 = keys ? 16 * w + t : 32 * jg + t, entry_mm = keys ? 8 : 0;
 #pragma unroll
-        for (int tt = 0; tt < 4; ++tt) { at[tt][0] = row_at(tt, 0); at[tt][1] = row_at(tt, 1); }
-        fetch(0);
+        for (int tt = 0; tt < 4; ++tt) fetch(tt, words[tt]);
         const int stages = keys ? PR_KSTAGES : PR_VSTAGES;
         int stage = 0, phase = 0;
 #pragma unroll 1
         for (int j = 0; j < n_steps; ++j) {
             const int buf = j & 1;
-            take(j);
             if (!bar_wait_warp(&par_full[buf], (j >> 1) & 1, &sm.failed)) break;
             if (j >= stages && !bar_wait_warp(&empty[stage], phase ^ 1, &sm.failed)) break;
             const StepHeader &hd = sm.hdr[j & (PR_HDRS - 1)];
@@ -618,46 +595,50 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
             const bool far = keys ? hd.k_far : hd.v_far;
             const uint4 *tab = keys ? &sm.ktab[buf][0][0] : &sm.vtab[buf][0][0];
             const uint32_t base = smem_addr(keys ? &sm.k[stage][0][0] : &sm.v[stage][0][0]);
-            if (!far && (!keys || (j + 1) * PR_STEP <= n_body)) {
+#pragma unroll 2      // two tiles' chains at a time; all four are slower by a tenth, one by a twentieth
+            for (int tt = 0; tt < 4; ++tt) {
+                const uint32_t cur[2] = {words[0][0], words[0][1]};
 #pragma unroll
-                for (int tt = 0; tt < 4; ++tt)
+                for (int x = 0; x < 3; ++x) { words[x][0] = words[x + 1][0]; words[x][1] = words[x + 1][1]; }
+                fetch(4 * j + tt + 4, words[3]);
+                const int entry = entry0 + (keys ? (tt >= second ? 64 : 0) : 8 * tt), tok = j * PR_STEP + 16 * tt;
+                const uint32_t to0 = base + ((at0 + tt * add_tile) ^ (tt * xor_tile)), to1 = base + ((at1 + tt * add_tile) ^ (tt * xor_tile));
+                if (!far && (!keys || tok < n_body)) {
 #pragma unroll
                     for (int mm = 0; mm < 2; ++mm) {
                         uint32_t f[4], hi[4], lo[4];
-                        matrix_fields<BITS>(cur[tt], mm, w & 1, f);
-                        const uint4 *e = tab + entry(tt, mm, second);
+                        matrix_fields<BITS>(cur, mm, w & 1, f);
+                        const uint4 *e = tab + entry + mm * entry_mm;
                         expand_matrix<BITS, false>(f, e[0], e[4], make_uint2(0u, 0u), make_uint2(0u, 0u), hi, lo);
-                        st_matrix<0>(base + at[tt][mm], hi);
-                        st_matrix<PR_HALF>(base + at[tt][mm], lo);
+                        st_matrix<0>(mm ? to1 : to0, hi);
+                        st_matrix<PR_HALF>(mm ? to1 : to0, lo);
                     }
-            } else {                                      // far zero points, or key tiles of the open group
-                const uint2 *add = keys ? &sm.kadd[buf][0][0] : &sm.vadd[buf][0][0];
+                } else {                                  // far zero points, or a key tile of the open group
+                    const uint2 *add = keys ? &sm.kadd[buf][0][0] : &sm.vadd[buf][0][0];
 #pragma unroll 1
-                for (int x = 0; x < 8; ++x) {
-                    const int tt = x >> 1, mm = x & 1, tok = j * PR_STEP + 16 * tt;
-                    uint32_t hi[4], lo[4];
-                    if (keys && tok >= n_body) {          // exact fp16 rows from the tail
-                        const __half2 up2 = __half2half2(__float2half(up));
+                    for (int mm = 0; mm < 2; ++mm) {
+                        uint32_t hi[4], lo[4];
+                        if (keys && tok >= n_body) {      // exact fp16 rows from the tail
+                            const __half2 up2 = __half2half2(__float2half(up));
 #pragma unroll
-                        for (int y = 0; y < 4; ++y) {
-                            const int tk = tok + (lane >> 2) + 8 * (y & 1);
-                            const uint32_t v = tk < seq_len && in_bounds(tk - n_body < p.G, c.status) ? *(const uint32_t *)(tail + (size_t)(tk - n_body) * D + 16 * (2 * w + mm) + 8 * (y >> 1) + 2 * t) : 0u;
-                            hi[y] = as_u32(__hmul2_rn(as_half2(v), up2));
-                            lo[y] = 0u;
+                            for (int y = 0; y < 4; ++y) {
+                                const int tk = tok + (lane >> 2) + 8 * (y & 1);
+                                const uint32_t v = tk < seq_len && in_bounds(tk - n_body < p.G, c.status) ? *(const uint32_t *)(tail + (size_t)(tk - n_body) * D + 16 * (2 * w + mm) + 8 * (y >> 1) + 2 * t) : 0u;
+                                hi[y] = as_u32(__hmul2_rn(as_half2(v), up2));
+                                lo[y] = 0u;
+                            }
+                        } else {
+                            uint32_t f[4];
+                            matrix_fields<BITS>(cur, mm, w & 1, f);
+                            const int e = entry + mm * entry_mm;
+                            expand_matrix<BITS, true>(f, tab[e], tab[e + 4], add[e], add[e + 4], hi, lo);
                         }
-                    } else {
-                        uint32_t f[4], words[2] = {0u, 0u};
-                        if (tok < coded && in_bounds(tok + KVSINK_TILE <= p.max_seq, c.status)) load_words<BITS>(codes + (size_t)(tok >> 4) * p.tile_bytes, w, lane, words);
-                        matrix_fields<BITS>(words, mm, w & 1, f);
-                        const int e = entry(tt, mm, second);
-                        expand_matrix<BITS, true>(f, tab[e], tab[e + 4], add[e], add[e + 4], hi, lo);
+                        st_matrix<0>(mm ? to1 : to0, hi);
+                        st_matrix<PR_HALF>(mm ? to1 : to0, lo);
                     }
-                    const uint32_t to = base + row_at(tt, mm);
-                    st_matrix<0>(to, hi);
-                    st_matrix<PR_HALF>(to, lo);
                 }
             }
-            if (sink[0] | sink[1]) put_sinks(sink, keys ? sm.k_rank[buf] : sm.v_rank[buf], base, up);
+            if (sink[0] | sink[1]) put_sinks(sink, keys ? sm.k_rank[buf] : sm.v_rank[buf], keys ? sm.k_kept[buf] : sm.v_kept[buf], base, up);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
             if (lane == 0) { bar_arrive(&full[stage]); bar_arrive(&par_empty[buf]); }
@@ -698,7 +679,7 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
                 const uint32_t d = TM_O + 128 * i, w = TM_S + 64 * buf;
                 const bool last = i == 1 || j >= m1;
                 if (elect_one()) {
-#pragma unroll
+#pragma unroll 1
                     for (int part = 0; part < 3; ++part)
 #pragma unroll
                         for (int x = 0; x < 4; ++x)
@@ -723,15 +704,17 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
                 const uint32_t d = TM_S + 64 * buf;
                 const bool last = i == 1 || j >= m1;
                 if (elect_one()) {
-                    if (i == 0) {
+#pragma unroll 1
+                    for (int part = 0; part < 4; ++part) {     // K_lo, K_hi, each by its two panels of 64 channels
+                        const uint64_t kp = kd + (((part < 2 ? PR_HALF : 0) + (part & 1) * 8192) >> 4);
+                        if (i == 0) {
 #pragma unroll
-                        for (int x = 0; x < 16; ++x)
-                            tc_mma(d, TM_Q + 8 * (x & 7), kd + (((x < 8 ? PR_HALF : 0) + ((x & 7) >> 2) * 8192 + (x & 3) * 32) >> 4), instr_desc(64), x > 0);
-                    } else {
+                            for (int x = 0; x < 4; ++x) tc_mma(d, TM_Q + 32 * (part & 1) + 8 * x, kp + 2 * x, instr_desc(64), part + x > 0);
+                        } else {
+                            const uint64_t qp = qd + ((part & 1) * PR_HALF >> 4);
 #pragma unroll
-                        for (int x = 0; x < 16; ++x)
-                            tc_mma_shared(d, qd + ((((x & 7) >> 2) * PR_HALF + (x & 3) * 32) >> 4),
-                                          kd + (((x < 8 ? PR_HALF : 0) + ((x & 7) >> 2) * 8192 + (x & 3) * 32) >> 4), instr_desc(64), x > 0);
+                            for (int x = 0; x < 4; ++x) tc_mma_shared(d, qp + 2 * x, kp + 2 * x, instr_desc(64), part + x > 0);
+                        }
                     }
                     tc_commit(&sm.s_full[buf]);
                     if (last) tc_commit(&sm.k_empty[stage]);
@@ -756,60 +739,78 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
         const uint32_t *bm = c.sink_bitmask + (size_t)b * p.mask_words;
         const int32_t *pos = c.sink_pos + (size_t)b * p.cap;
         const int n_pos = min(c.sink_count[b], p.cap);
-        const __half *rows = (const __half *)(keys ? c.sink_k : c.sink_v) + (size_t)unit * p.cap * D + 4 * lane;
+        const __half *rows = (const __half *)(keys ? c.sink_k : c.sink_v) + (size_t)unit * p.cap * D + 8 * (lane & 15);
+        uint4 (*kept)[PR_ROWS_KEPT][16] = keys ? sm.k_kept : sm.v_kept;
         int rank0 = 0;                                                   // sink tokens before the step
-        // Entries of a step: keys, two channel pairs a lane for each of the (at most two) groups that meet it: G is 32, 64 or at
-        // least 128; values, one token pair a lane for each channel group.  The first two, mostly all, are read one step ahead.
+        // A step's parameters come into shared memory a step ahead, as they are: of the (at most two) key groups that meet the step (G
+        // is 32, 64 or at least 128), of its tokens' values.  Entries: keys, two channel pairs a lane for each group; values, one
+        // token pair a lane for each channel group.
         const float *ps = keys ? ks : vs, *pz = keys ? kz : vz;
-        const int apart = keys ? 1 : p.NGv;                              // from one column's parameter to the other's
-        struct Pair { float s0, z0, s1, z1; };
-        auto fetch = [&](int j, int g, int n, int entries) {
-            const int tok = j * PR_STEP + 2 * lane;
-            const int64_t at = keys ? (int64_t)(g + (n >> 1)) * D + 2 * lane + 64 * (n & 1) : (int64_t)tok * p.NGv + n;
-            Pair r = {0.f, 0.f, 0.f, 0.f};
-            if (n < entries && !in_bounds(keys ? (g + (n >> 1) + 1) * p.G <= n_body : n < p.NGv, c.status)) return r;
-            if (n < entries && (keys || tok < seq_len)) { r.s0 = __ldg(ps + at); r.z0 = __ldg(pz + at); }
-            if (n < entries && (keys || tok + 1 < seq_len)) { r.s1 = __ldg(ps + at + apart); r.z1 = __ldg(pz + at + apart); }
-            return r;
-        };
         // group of the step's first token, tokens of the step before the next group, and the step's entries
+        int g0 = 0, second = p.G;
         auto count = [&](int j, int second) {
             const int body = n_body - j * PR_STEP;
             return keys ? (body > 0 ? (min(body, PR_STEP) > second ? 4 : 2) : 0) : p.NGv;
+        };
+        auto fetch = [&](int j, int g) {
+            const int n = keys ? (count(j, second) >> 1) : 1, chunks = keys ? 32 : 16 * p.NGv;     // 16 bytes each
+            float *to = keys ? &sm.k_raw[j & 1][0][0][0] : &sm.v_raw[j & 1][0][0];
+            const int half = keys ? 128 : 256;
+#pragma unroll 1
+            for (int y = 0; y < n; ++y, to += 256)
+#pragma unroll 1
+                for (int x = lane; x < chunks; x += 32) {
+                    const int64_t at = keys ? (int64_t)(g + y) * D + 4 * x : (int64_t)j * PR_STEP * p.NGv + 4 * x;
+                    if (keys ? !in_bounds((g + y + 1) * p.G <= n_body, c.status) : at >= (int64_t)seq_len * p.NGv) continue;
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(smem_addr(to + 4 * x)), "l"(ps + at) : "memory");
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(smem_addr(to + half + 4 * x)), "l"(pz + at) : "memory");
+                }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        struct Pair { float s0, z0, s1, z1; };
+        auto pair = [&](int j, int n) {
+            Pair r = {0.f, 0.f, 0.f, 0.f};
+            if (keys) {
+                const float *at = &sm.k_raw[j & 1][n >> 1][0][2 * lane + 64 * (n & 1)];
+                const float2 s = *(const float2 *)at, z = *(const float2 *)(at + 128);
+                r.s0 = s.x; r.s1 = s.y; r.z0 = z.x; r.z1 = z.y;
+            } else {
+                const float *at = &sm.v_raw[j & 1][0][2 * lane * p.NGv + n];
+                const int left = seq_len - (j * PR_STEP + 2 * lane);
+                if (left > 0) { r.s0 = at[0]; r.z0 = at[256]; }
+                if (left > 1) { r.s1 = at[p.NGv]; r.z1 = at[256 + p.NGv]; }
+            }
+            return r;
         };
         auto mask_word = [&](int j, int x) {
             const int left = seq_len - (j * PR_STEP + 32 * x);
             uint32_t w = left > 0 && in_bounds(2 * j + x < p.mask_words, c.status) ? __ldg(bm + 2 * j + x) : 0u;
             return left > 0 && left < 32 ? w & ((1u << left) - 1u) : w;
         };
-        int g0 = 0, second = p.G, entries = count(0, p.G);
-        Pair next[2] = {fetch(0, 0, 0, entries), fetch(0, 0, 1, entries)};
+        fetch(0, 0);
         uint32_t bits[2] = {mask_word(0, 0), mask_word(0, 1)};
 #pragma unroll 1
         for (int j = 0; j < n_steps; ++j) {
             const int buf = j & 1, tok0 = j * PR_STEP;
-            const Pair first[2] = {next[0], next[1]};
             const uint32_t sink[2] = {bits[0], bits[1]};
-            const int g = g0, split = second, n_entries = entries;
+            const int split = second, n_entries = count(j, second);
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            __syncwarp();
             if (j + 1 < n_steps) {
                 second -= PR_STEP;
                 while (second <= 0) { second += p.G; ++g0; }
-                entries = count(j + 1, second);
-                next[0] = fetch(j + 1, g0, 0, entries);
-                next[1] = fetch(j + 1, g0, 1, entries);
+                fetch(j + 1, g0);
                 bits[0] = mask_word(j + 1, 0);
                 bits[1] = mask_word(j + 1, 1);
             }
             float top = 0.f;
             bool far = false, odd = false;
-            auto look = [&](const Pair &r) {                             // largest |scale * (code - zero)|
+#pragma unroll 1
+            for (int n = 0; n < n_entries; ++n) {                        // largest |scale * (code - zero)|
+                const Pair r = pair(j, n);
                 top = max3(top, r.s0 * fmaxf(fabsf(r.z0), fabsf(QMAX - r.z0)), r.s1 * fmaxf(fabsf(r.z1), fabsf(QMAX - r.z1)));
                 far |= fabsf(r.z0) > PR_NEAR || fabsf(r.z1) > PR_NEAR;
-            };
-            look(first[0]);
-            look(first[1]);
-#pragma unroll 1
-            for (int n = 2; n < n_entries; ++n) look(fetch(j, g, n, n_entries));
+            }
             if (j >= 2 && !bar_wait_warp(&empty[buf], ((j >> 1) - 1) & 1, &sm.failed)) break;
             // sink tokens of the step and their side buffer rows
             uint32_t dead0 = 0u, dead1 = 0u;
@@ -835,22 +836,22 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
                     else dead0 = m;
                 }
                 __syncwarp();
-#pragma unroll 4
-                for (int y = 0; y < ns; ++y) {
+                __half2 large = __float2half2_rn(0.f);
+#pragma unroll 2
+                for (int y = lane >> 4; y < ns; y += 2) {                // half a warp a row
                     const int r = rank[buf][y];
-                    if (r >= 0) {
-                        if (!in_bounds(r < p.cap, c.status)) continue;
-                        const uint2 v = *(const uint2 *)(rows + (size_t)r * D);
-                        const float2 v0 = __half22float2(as_half2(v.x)), v1 = __half22float2(as_half2(v.y));
-                        const float w[4] = {v0.x, v0.y, v1.x, v1.y};
-#pragma unroll
-                        for (int z = 0; z < 4; ++z) {
-                            const float mag = fabsf(w[z]);
-                            odd |= !is_finite(mag);
-                            top = fmaxf(top, is_finite(mag) ? mag : 0.f);
-                        }
-                    }
+                    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+                    if (r >= 0 && in_bounds(r < p.cap, c.status)) v = *(const uint4 *)(rows + (size_t)r * D);
+                    if (y < PR_ROWS_KEPT) kept[buf][y][lane & 15] = v;
+                    auto look = [&](uint32_t x) {
+                        const __half2 mag = __habs2(as_half2(x));
+                        const uint32_t finite = __hle2_mask(mag, __float2half2_rn(65504.f));
+                        odd |= finite != 0xffffffffu;
+                        large = __hmax2(large, as_half2(as_u32(mag) & finite));
+                    };
+                    look(v.x); look(v.y); look(v.z); look(v.w);
                 }
+                top = max3(top, __low2float(large), __high2float(large));
                 rank0 += ns;
                 if (!keys && __any_sync(0xffffffffu, odd) && lane == 0) *(volatile int *)&sm.odd_values = 1;
             }
@@ -859,13 +860,12 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
             const float up = exp2i(e);
             StepHeader &hd = sm.hdr[j & (PR_HDRS - 1)];
             far = __any_sync(0xffffffffu, far);
-            const bool general = far || tok0 + PR_STEP > n_body;         // the step's keys take the general path, which reads the additive terms
             uint4 *tab = keys ? &sm.ktab[buf][0][0] : &sm.vtab[buf][0][0];
             uint2 *add = keys ? &sm.kadd[buf][0][0] : &sm.vadd[buf][0][0];
 #pragma unroll 1
             for (int n = 0; n < n_entries; ++n) {
-                const Pair r = n == 0 ? first[0] : (n == 1 ? first[1] : fetch(j, g, n, n_entries));
-                table_entry<BITS>(r.s0, r.z0, r.s1, r.z1, up, (lane >> 2) & 1, general, tab + 32 * n + lane, add + 32 * n + lane);
+                const Pair r = pair(j, n);
+                table_entry<BITS>(r.s0, r.z0, r.s1, r.z1, up, (lane >> 2) & 1, far, tab + 32 * n + lane, add + 32 * n + lane);
             }
             if (lane == 0) {
                 if (keys) {

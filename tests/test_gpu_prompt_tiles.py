@@ -83,6 +83,13 @@ def test_every_token_a_sink():
     _check(wl, 270, 0)
 
 
+# one step holds all sinks: up to eight of its rows are left in shared memory by the warps that look at them first, the others are not
+@pytest.mark.parametrize("bits,topk", [(2, 7), (3, 8), (4, 9), (2, 17)])
+def test_sink_rows_of_one_step(bits, topk):
+    wl = TINY.scaled(bits=bits, head_dim=128, group=32, n_q_heads=32, n_kv_heads=16, batch=4, seq=64, topk=topk, pfn_n=0, seed=23100 + topk)
+    _check(wl, 64, 0)
+
+
 def _prompt(wl):
     """A cache that holds a whole prompt, and queries for all of it."""
     _, gcfg = configs(wl)
