@@ -1,4 +1,5 @@
-"""ctypes binding of libkvsink.so: the same entry points as include/kvsink.h, argument marshalling only.
+"""Binding of libkvsink.so: the same entry points as include/kvsink.h, argument marshalling only.  The calls of a layer's step
+(prediction, appends, attention) go through _calls.so (csrc/calls.cpp), the others through ctypes.
 
 Tensors are torch CUDA tensors used for device memory and the current stream; every step of the path runs in
 the library's kernels.  The library must be present: there is no fallback.
@@ -89,6 +90,19 @@ def lib():
             getattr(loaded, name).argtypes = _ARGS[name]
         _lib = loaded
     return _lib
+
+
+_calls = None
+
+
+def _native():
+    """Loads _calls.so and gives it the library's entry points; raises if it has not been built."""
+    global _calls
+    if _calls is None:
+        from . import _calls as module
+        module.bind({n: C.cast(getattr(lib(), n), C.c_void_p).value for n in EXPORTS}, Config, KVCache, StaticParams, KvsinkError)
+        _calls = module
+    return _calls
 
 
 def strerror(code: int) -> str:
@@ -188,63 +202,25 @@ class KVCache:
 
 def predict_sinks(cfg: Config, hidden: torch.Tensor, sinks: SinkSet, workspace: Optional[torch.Tensor] = None) -> SinkSet:
     """kvsink_predict_sinks: hidden fp16 [B, S, d] on the device (last axis contiguous)."""
-    assert hidden.is_cuda and hidden.dtype == torch.float16 and hidden.dim() == 3 and hidden.stride(2) == 1
-    if workspace is None:
-        workspace = hidden.new_empty(_size(cfg, "predict_workspace_bytes"), dtype=torch.uint8)
-    rc = lib().kvsink_predict_sinks(C.byref(cfg.c()), _ptr(hidden), hidden.shape[1], hidden.stride(0),
-                                    hidden.stride(1), _ptr(sinks.bitmask), _ptr(sinks.pos), _ptr(sinks.count),
-                                    _ptr(workspace), workspace.numel(), _stream())
-    if rc:
-        raise KvsinkError(rc, "kvsink_predict_sinks")
-    return sinks
+    return (_calls or _native()).predict_sinks(cfg, hidden, sinks, workspace)
 
 
 def quantize_append(cfg: Config, cache: KVCache, k_new: torch.Tensor, v_new: torch.Tensor) -> None:
     """kvsink_quantize_append: k_new, v_new fp16 [B, Hkv, T, D] on the device with equal strides."""
-    assert k_new.is_cuda and k_new.dtype == torch.float16 and k_new.dim() == 4 and k_new.stride(3) == 1
-    assert v_new.shape == k_new.shape and v_new.stride() == k_new.stride() and v_new.dtype == torch.float16
-    cc = cache.c()
-    rc = lib().kvsink_quantize_append(C.byref(cfg.c()), C.byref(cc), _ptr(k_new), _ptr(v_new), k_new.shape[2],
-                                      k_new.stride(0), k_new.stride(1), k_new.stride(2), _stream())
-    if rc:
-        raise KvsinkError(rc, "kvsink_quantize_append")
-    cache.seq_len = cc.seq_len
+    (_calls or _native()).quantize_append(0, cfg, cache, None, k_new, v_new)
 
 
 def decode_attention(cfg: Config, cache: KVCache, q: torch.Tensor, out: Optional[torch.Tensor] = None,
                      lse: Optional[torch.Tensor] = None, workspace: Optional[torch.Tensor] = None, want_lse: bool = True):
     """kvsink_decode_attention: q fp16 [B, Hq, D] contiguous. Returns (out fp32 [B,Hq,D], lse fp32 [B,Hq] or None)."""
-    assert q.is_cuda and q.dtype == torch.float16 and q.is_contiguous()
-    if out is None:
-        out = q.new_empty((cfg.batch, cfg.n_q_heads, cfg.head_dim), dtype=torch.float32)
-    if lse is None and want_lse:
-        lse = q.new_empty((cfg.batch, cfg.n_q_heads), dtype=torch.float32)
-    if workspace is None:
-        workspace = q.new_empty(cache.sizes["decode_workspace_bytes"], dtype=torch.uint8)
-    cc = cache.c()
-    rc = lib().kvsink_decode_attention(C.byref(cfg.c()), C.byref(cc), _ptr(q), _ptr(out), _ptr(lse), _ptr(workspace),
-                                       workspace.numel(), _stream())
-    if rc:
-        raise KvsinkError(rc, "kvsink_decode_attention")
-    return out, lse
+    return (_calls or _native()).decode_attention(0, cfg, cache, None, q, out, lse, workspace, want_lse)
 
 
 def prefill_attention(cfg: Config, cache: KVCache, q: torch.Tensor, q_pos0: int, out: Optional[torch.Tensor] = None,
                       lse: Optional[torch.Tensor] = None, want_lse: bool = True):
     """kvsink_prefill_attention: q fp16 [B, Hq, T, D] on the device (last axis contiguous); query t sits at position q_pos0 + t.
     Returns (out fp32 [B,Hq,T,D], lse fp32 [B,Hq,T] or None)."""
-    assert q.is_cuda and q.dtype == torch.float16 and q.dim() == 4 and q.stride(3) == 1
-    T = q.shape[2]
-    if out is None:
-        out = q.new_empty((cfg.batch, cfg.n_q_heads, T, cfg.head_dim), dtype=torch.float32)
-    if lse is None and want_lse:
-        lse = q.new_empty((cfg.batch, cfg.n_q_heads, T), dtype=torch.float32)
-    cc = cache.c()
-    rc = lib().kvsink_prefill_attention(C.byref(cfg.c()), C.byref(cc), _ptr(q), T, q_pos0, q.stride(0),
-                                        q.stride(1), q.stride(2), _ptr(out), _ptr(lse), _stream())
-    if rc:
-        raise KvsinkError(rc, "kvsink_prefill_attention")
-    return out, lse
+    return (_calls or _native()).prefill_attention(cfg, cache, q, q_pos0, out, lse, want_lse)
 
 
 def prefill_rows(cfg: Config, T: int) -> int:
@@ -307,64 +283,26 @@ def calibrate(cfg: Config, k_cal: torch.Tensor, v_cal: torch.Tensor, sinks: Sink
 
 def quantize_append_calibrated(cfg: Config, cache: KVCache, params: StaticParams, k_new: torch.Tensor, v_new: torch.Tensor) -> None:
     """kvsink_quantize_append_calibrated: k_new, v_new fp16 [B, Hkv, T, D] on the device with equal strides."""
-    assert k_new.is_cuda and k_new.dtype == torch.float16 and k_new.dim() == 4 and k_new.stride(3) == 1
-    assert v_new.shape == k_new.shape and v_new.stride() == k_new.stride() and v_new.dtype == torch.float16
-    cc, cs = cache.c(), params.c()
-    rc = lib().kvsink_quantize_append_calibrated(C.byref(cfg.c()), C.byref(cc), C.byref(cs), _ptr(k_new), _ptr(v_new), k_new.shape[2],
-                                                 k_new.stride(0), k_new.stride(1), k_new.stride(2), _stream())
-    if rc:
-        raise KvsinkError(rc, "kvsink_quantize_append_calibrated")
-    cache.seq_len = cc.seq_len
+    (_calls or _native()).quantize_append(1, cfg, cache, params, k_new, v_new)
 
 
 def decode_attention_calibrated(cfg: Config, cache: KVCache, params: StaticParams, q: torch.Tensor, out: Optional[torch.Tensor] = None,
                                 lse: Optional[torch.Tensor] = None, workspace: Optional[torch.Tensor] = None, want_lse: bool = True):
     """kvsink_decode_attention_calibrated: q fp16 [B, Hq, D] contiguous. Returns (out fp32 [B,Hq,D], lse fp32 [B,Hq] or None)."""
-    assert q.is_cuda and q.dtype == torch.float16 and q.is_contiguous()
-    if out is None:
-        out = q.new_empty((cfg.batch, cfg.n_q_heads, cfg.head_dim), dtype=torch.float32)
-    if lse is None and want_lse:
-        lse = q.new_empty((cfg.batch, cfg.n_q_heads), dtype=torch.float32)
-    if workspace is None:
-        workspace = q.new_empty(cache.sizes["decode_workspace_bytes"], dtype=torch.uint8)
-    cc, cs = cache.c(), params.c()
-    rc = lib().kvsink_decode_attention_calibrated(C.byref(cfg.c()), C.byref(cc), C.byref(cs), _ptr(q), _ptr(out), _ptr(lse), _ptr(workspace),
-                                                  workspace.numel(), _stream())
-    if rc:
-        raise KvsinkError(rc, "kvsink_decode_attention_calibrated")
-    return out, lse
+    return (_calls or _native()).decode_attention(1, cfg, cache, params, q, out, lse, workspace, want_lse)
 
 
 def quantize_append_pertoken(cfg: Config, cache: KVCache, k_new: torch.Tensor, v_new: torch.Tensor) -> None:
     """kvsink_quantize_append_pertoken: k_new, v_new fp16 [B, Hkv, T, D] on the device with equal strides."""
     assert cache.per_token_keys, "the cache was not sized for per-token key parameters"
-    assert k_new.is_cuda and k_new.dtype == torch.float16 and k_new.dim() == 4 and k_new.stride(3) == 1
-    assert v_new.shape == k_new.shape and v_new.stride() == k_new.stride() and v_new.dtype == torch.float16
-    cc = cache.c()
-    rc = lib().kvsink_quantize_append_pertoken(C.byref(cfg.c()), C.byref(cc), _ptr(k_new), _ptr(v_new), k_new.shape[2],
-                                               k_new.stride(0), k_new.stride(1), k_new.stride(2), _stream())
-    if rc:
-        raise KvsinkError(rc, "kvsink_quantize_append_pertoken")
-    cache.seq_len = cc.seq_len
+    (_calls or _native()).quantize_append(2, cfg, cache, None, k_new, v_new)
 
 
 def decode_attention_pertoken(cfg: Config, cache: KVCache, q: torch.Tensor, out: Optional[torch.Tensor] = None,
                               lse: Optional[torch.Tensor] = None, workspace: Optional[torch.Tensor] = None, want_lse: bool = True):
     """kvsink_decode_attention_pertoken: q fp16 [B, Hq, D] contiguous. Returns (out fp32 [B,Hq,D], lse fp32 [B,Hq] or None)."""
     assert cache.per_token_keys, "the cache was not sized for per-token key parameters"
-    assert q.is_cuda and q.dtype == torch.float16 and q.is_contiguous()
-    if out is None:
-        out = q.new_empty((cfg.batch, cfg.n_q_heads, cfg.head_dim), dtype=torch.float32)
-    if lse is None and want_lse:
-        lse = q.new_empty((cfg.batch, cfg.n_q_heads), dtype=torch.float32)
-    if workspace is None:
-        workspace = q.new_empty(cache.sizes["decode_workspace_bytes"], dtype=torch.uint8)
-    cc = cache.c()
-    rc = lib().kvsink_decode_attention_pertoken(C.byref(cfg.c()), C.byref(cc), _ptr(q), _ptr(out), _ptr(lse), _ptr(workspace),
-                                                workspace.numel(), _stream())
-    if rc:
-        raise KvsinkError(rc, "kvsink_decode_attention_pertoken")
-    return out, lse
+    return (_calls or _native()).decode_attention(2, cfg, cache, None, q, out, lse, workspace, want_lse)
 
 
 def channel_absmax(hidden: torch.Tensor, out: Optional[torch.Tensor] = None) -> torch.Tensor:

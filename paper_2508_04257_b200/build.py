@@ -1,4 +1,4 @@
-"""Builds libkvsink.so (hand-written CUDA for sm_100a) in-tree with nvcc.
+"""Builds libkvsink.so (hand-written CUDA for sm_100a) in-tree with nvcc, and _calls.so, the Python side of its calls, with g++.
 
 Every translation unit is compiled to an object of its own (in parallel, only when it is older than its sources) and
 the objects are linked into the shared library; no kernel calls device code of another unit, so no device link step
@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import os
 import subprocess
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -17,6 +18,10 @@ LIB = os.path.join(HERE, "libkvsink.so")
 HEADER = os.path.join(os.path.dirname(HERE), "include", "kvsink.h")
 SOURCES = ["api.cu", "predict.cu", "quantize.cu", "quantize_groups.cu", "quantize_bulk.cu", "decode.cu", "decode_b2.cu", "decode_b3.cu", "decode_b4.cu", "prompt.cu", "analysis.cu", "calibrated.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC"]
+
+
+CALLS = os.path.join(HERE, "_calls.so")
+CALLS_SOURCE = os.path.join(CSRC, "calls.cpp")
 
 
 def _headers():
@@ -31,6 +36,25 @@ def _older(target: str, deps) -> bool:
 
 
 DEBUG_LIB = os.path.join(HERE, "libkvsink_debug.so")
+
+
+def build_calls(force: bool = False) -> str:
+    """_calls.so: an extension module against the headers of Python and the installed torch."""
+    if force or _older(CALLS, [CALLS_SOURCE, HEADER]):
+        import torch
+        at = os.path.dirname(torch.__file__)
+        cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
+        include = [sysconfig.get_paths()["include"], os.path.join(cuda, "include"), os.path.join(at, "include"),
+                   os.path.join(at, "include", "torch", "csrc", "api", "include")]
+        abi = f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"
+        cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", abi] + [f"-I{d}" for d in include] + \
+              [CALLS_SOURCE, "-o", CALLS, "-L" + os.path.join(at, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
+        r = subprocess.run(cmd, capture_output=True, text=True)
+        if r.returncode != 0:
+            if os.path.exists(CALLS):
+                os.remove(CALLS)
+            raise RuntimeError(f"g++ failed on calls.cpp\n{r.stderr[-4000:]}")
+    return CALLS
 
 
 def build(force: bool = False, verbose: bool = False, debug: bool = False) -> str:
@@ -74,6 +98,7 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False) -> st
             if os.path.exists(LIB):
                 os.remove(LIB)
             raise RuntimeError(f"link failed with status {r.returncode}")
+    build_calls(force and not debug)
     return LIB
 
 

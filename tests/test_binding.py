@@ -69,3 +69,60 @@ def test_work_goes_to_the_current_stream(raw, monkeypatch):
     side = torch.cuda.Stream()
     with torch.cuda.stream(side):
         assert binding._stream() == side.cuda_stream != 0
+
+
+@pytest.mark.parametrize("bad", ["device", "strides", "type"])
+def test_inputs_that_the_calls_refuse(bad):
+    cache = _cache()
+    k = torch.zeros((1, 8, 2, 128), dtype=torch.float32 if bad == "type" else torch.float16)
+    k = k.transpose(2, 3) if bad == "strides" else k
+    with pytest.raises(AssertionError):
+        kv.quantize_append(cache.cfg, cache, k, k)
+    with pytest.raises(AssertionError):
+        kv.decode_attention(cache.cfg, cache, k[:, :, 0])
+    with pytest.raises(AssertionError):
+        kv.prefill_attention(cache.cfg, cache, k, 0)
+    with pytest.raises(AssertionError):
+        kv.predict_sinks(cache.cfg, k[0], cache.sinks)
+    with pytest.raises(AttributeError):
+        kv.decode_attention(cache.cfg, cache, None)
+    assert cache.seq_len == 0
+
+
+@pytest.mark.gpu
+def test_calls_take_records_results_and_errors_as_ctypes_did():
+    class OwnConfig(kv.Config):
+        def c(self):
+            return super().c()
+
+    class OwnCache(kv.KVCache):
+        def c(self):
+            return super().c()
+
+    got, refs = [], []
+    for config, cache_type in ((kv.Config, kv.KVCache), (OwnConfig, OwnCache)):
+        cfg = config(2, 4, 4, 128, 512, 2, 64, 256, 2, 1, (1,))
+        g = torch.Generator("cuda").manual_seed(3)
+        K, V = (torch.randn((2, 4, 101, 128), device="cuda", generator=g).half() for _ in range(2))
+        H, q = torch.randn((2, 101, 512), device="cuda", generator=g).half(), torch.randn((2, 4, 128), device="cuda", generator=g).half()
+        cache = cache_type(cfg, kv.predict_sinks(cfg, H, kv.SinkSet(cfg)))
+        kv.quantize_append(cfg, cache, K, V)
+        assert cache.seq_len == 101
+        out, lse = torch.empty((2, 4, 128), device="cuda"), torch.empty((2, 4), device="cuda")
+        work = torch.empty(cache.sizes["decode_workspace_bytes"], dtype=torch.uint8, device="cuda")
+        given = kv.decode_attention(cfg, cache, q, out, lse, work)
+        assert given[0] is out and given[1] is lse
+        new = kv.decode_attention(cfg, cache, q)
+        assert torch.equal(new[0], out) and torch.equal(new[1], lse) and new[1].shape == lse.shape
+        assert kv.decode_attention(cfg, cache, q, want_lse=False)[1] is None
+        whole = kv.prefill_attention(cfg, cache, q[:, :, None], 100)
+        assert whole[0].shape == (2, 4, 1, 128) and whole[1].shape == (2, 4, 1)
+        got.append([cache.k_codes, out, *whole])
+        with pytest.raises(kv.KvsinkError):
+            kv.decode_attention(config(2, 4, 4, 128, 512, 5, 64, 256, 2, 1, (1,)), cache, q, out, lse, work)      # no such code width
+        refs.append([sys.getrefcount(x) for x in (cfg.batch, out, lse, work, cache.k_codes, cache.sinks)])
+        for _ in range(50):
+            kv.decode_attention(cfg, cache, q, out, lse, work)
+            kv.quantize_append(cfg, cache, K[:, :, :0], V[:, :, :0])
+        assert refs[-1][1:] == [sys.getrefcount(x) for x in (out, lse, work, cache.k_codes, cache.sinks)]
+    assert all(torch.equal(a, b) for a, b in zip(*got))
