@@ -1,5 +1,5 @@
-// Decode attention kernels for 2-bit codes (see decode_kernel.cuh).
-#include "decode_kernel.cuh"
+// Decode attention kernels for 2-bit codes (see decode_kernel.cuh and decode_one.cuh).
+#include "decode_launch.cuh"
 
 namespace kvsink {
 

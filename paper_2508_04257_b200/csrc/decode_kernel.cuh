@@ -204,16 +204,14 @@ struct DecodePlan {
 // column 2h multiplies by the fp16 factor q*scale and column 2h+1 by its fp16 rounding residual, so every score carries
 // the factor to ~22 bits at no extra instruction.  Without PL (five to eight heads) head h owns column h and the
 // residual of channels with large factors goes through a second multiply.
-// I8 (one query head per KV head): the key side runs on the integer tensor path.  The four bytes of a stored
-// word are four channels of one token row.  2 bit: the word masked with 0x03.., 0x0c.., 0x30.., 0xc0.. is the u8 A
-// fragment of one m16n8k32 (fields in place: x1, x4 for the rows g + 8, x16 for the upper contraction slots, x64 for
-// both).  4 bit: a word masked with 0x0f.. and 0xf0.. gives the registers of rows g and g + 8 (x16), two words (two
-// matrices) make one fragment.  The B operand holds the factor q * scale * 2^sh of each channel as three signed 7-bit
-// limbs in four accumulator columns (2, 3 bit: divided by 16 beforehand for the upper slots); sums are exact in int32.
-// 3 bit: the low two bits as for 2 bit, the high bits of the second section (same byte structure) through four more
-// MMAs with the same B operands into accumulators of their own.
-// I8 = 2 (two to four query heads per KV head, 2 and 4 bit): the same with two B operands per word, which hold the upper
-// and the lower byte pair of every head's factors in the pair layout's columns.
+// One query head per KV head at head size 128 has a kernel of its own (decode_one.cuh).
+// I8: the key side runs on the integer tensor path.  The four bytes of a stored word are four channels of one token row.  2 bit: the
+// word masked with 0x03.., 0x0c.., 0x30.., 0xc0.. is the u8 A fragment of one m16n8k32 (fields in place: x1, x4 for the rows
+// g + 8, x16 for the upper contraction slots, x64 for both).  4 bit: a word masked with 0x0f.. and 0xf0.. gives the registers of
+// rows g and g + 8 (x16), two words (two matrices) make one fragment.  The B operand holds the factor q * scale * 2^sh of each
+// channel as four signed bytes (2 bit: divided by 16 beforehand for the upper slots); sums are exact in int32.
+// I8 = 2 (two to four query heads per KV head, 2 and 4 bit): two B operands per word, which hold the upper and the lower byte pair
+// of every head's factors in the pair layout's columns.
 // I8 = 3 (five to eight rows: query heads, or the rows of a block of prompt queries; 2 and 4 bit): two operand tables of the
 // I8 = 2 kind, one for the even rows and one for the odd rows, multiplied with the same masked words, so that lane t finds
 // rows 2t and 2t+1 in its accumulators: the two columns it owns on the (eight-column, fp16) value side.  The key sums are
@@ -243,7 +241,7 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
               float *__restrict__ part_ws, int nsplit, int groups_per_split, int qchunks, int seq_len, int cluster_merge, PrefillShape pre)
 {
     using G_ = Geo<BITS, D>;
-    constexpr int NQMAX = I8 == 1 ? 1 : (PL ? 4 : 8);
+    constexpr int NQMAX = PL ? 4 : 8;
     using Plan = DecodePlan<BITS, D, NGv, CT, NQMAX, PM == 2>;
     constexpr int NM = G_::NM, W = G_::W, BST = Plan::BST, TILE_WORDS = 32 * W;
     constexpr int NSLOT = Plan::NSLOT, SLOT_BYTES = Plan::SLOT_BYTES, KV_BYTES = Plan::KV_BYTES, SZ_BYTES = Plan::SZ_BYTES;
@@ -262,7 +260,7 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
     static_assert(!KT || (I8 != 0 && NGv <= 2 && (BITS != 3 || NGv == 1)), "per-token keys: integer key side, one or two channel groups");
     // decode: grid (splits, KV heads x blocks of eight query heads, sequences); prompt queries: grid (row blocks, KV heads, sequences)
     const int split = PRE ? 0 : blockIdx.x, h = PRE ? blockIdx.y : blockIdx.y / qchunks, qc = PRE ? blockIdx.x : blockIdx.y % qchunks, b = blockIdx.z;
-    const int nq = I8 == 1 ? 1 : (PRE ? min(NQMAX, pre.T * p.rep - 8 * qc) : min(NQMAX, p.rep - NQMAX * qc)), hq0 = h * p.rep + (PRE ? 0 : NQMAX * qc);
+    const int nq = PRE ? min(NQMAX, pre.T * p.rep - 8 * qc) : min(NQMAX, p.rep - NQMAX * qc), hq0 = h * p.rep + (PRE ? 0 : NQMAX * qc);
     // prompt queries: row i of the block is query token (8 qc + i) / rep, query head (8 qc + i) % rep of this KV head
     auto row_token = [&](int i) { return (8 * qc + i) / p.rep; };
     auto row_limit = [&](int i) { return i < nq ? pre.q_pos0 + row_token(i) + 1 : 0; };    // cached tokens the row sees
@@ -514,7 +512,6 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
         for (int e = 0; e < 4; ++e) {
             i8_ch[e] = BITS != 4 ? 16 * (2 * mi + (e & 1)) + 8 * c2 + 2 * tq + (e >> 1)
                                  : 16 * (2 * mi + c2) + 8 * (e & 1) + 2 * tq + (e >> 1);
-            if (I8 == 1) i8_q[e] = qs[i8_ch[e]];
         }
     }
 
@@ -615,47 +612,9 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
                 __syncwarp();   // the parameters are in registers: the slot can take the next group's while this one streams
                 if (gi + 1 < my_groups) issue_params(gi + 1);
             }
-            if constexpr (I8 == 1) {
-                // limbs of the one head's factors: F = rint(q * scale * 2^sh) with the largest |F| in [2^29, 2^30), cut into
-                // four signed bytes (radix 256): every factor is kept to 2^-30 of the group's largest one (2^-26 where the
-                // factor is pre-divided for the upper contraction slots), finer than binary32 keeps the factor itself.
-                // Adding 0x808080 propagates the carries of the signed digits and the exclusive-or removes the offset again.
-                float v[4], amax = 0.f, bsum = 0.f;
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    v[e] = i8_q[e] * scv[e];
-                    amax = fmaxf(amax, fabsf(v[e]));
-                    // the zero-point term takes the unrounded factor: the limbs' rounding then meets the codes (at most
-                    // qmax) only, not code - zero, which is large for a channel far from zero with a narrow range
-                    bsum = fmaf(v[e], zev[e], bsum);
-                }
-                amax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(amax)));   // non-negative floats order as integers
-                int sh = 29 - floor_log2(amax);
-                sh = sh > 60 ? 60 : (sh < -60 ? -60 : sh);
-                const bool upper = BITS != 4 && (lane & 4) != 0;   // 2, 3 bit: this lane's channels sit in the upper contraction slots (x16 in place)
-                const float pre = upper ? pow2i(sh - 4) : pow2i(sh);
-                uint32_t d[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) d[e] = ((uint32_t)__float2int_rn(v[e] * pre) + 0x00808080u) ^ 0x00808080u;
-                // byte transpose: word j = byte j of the four channels, in contraction-slot order
-                const uint32_t t0 = __byte_perm(d[0], d[1], 0x5140), t1 = __byte_perm(d[0], d[1], 0x7362);
-                const uint32_t t2 = __byte_perm(d[2], d[3], 0x5140), t3 = __byte_perm(d[2], d[3], 0x7362);
-                // table [MMA][lower / upper slots][limb, most significant first][t][byte]: this lane owns one 4-byte slot group
-                uint32_t *tab = reinterpret_cast<uint32_t *>(Bs) + (lane >> 2) * 16 + (lane & 3);
-                tab[0] = __byte_perm(t1, t3, 0x7632);
-                tab[4] = __byte_perm(t1, t3, 0x5410);
-                tab[8] = __byte_perm(t0, t2, 0x7632);
-                tab[12] = __byte_perm(t0, t2, 0x5410);
-                if constexpr (KT && NGv == 2) {
-                    // per-token keys, two channel groups: the query's sum over each (lanes 0-15 hold channels 0-63)
-                    const float b0s = warp_sum(lane < 16 ? bsum : 0.f), b1s = warp_sum(lane < 16 ? 0.f : bsum);
-                    if (t == 0) { bias0 = b0s; bias1 = b1s; ks0 = pow2i(-sh); }
-                } else {
-                    bsum = warp_sum(bsum);
-                    if (t == 0) { bias0 = bsum; ks0 = pow2i(-sh); }
-                }
-            } else if constexpr (I8 >= 2) {
-                // up to four heads: the same four signed bytes per factor and head, each head with its own power of two.
+            if constexpr (I8 >= 2) {
+                // up to four heads: the four signed bytes of F = rint(q * scale * 2^sh) (radix 256, as in decode_one.cuh) per factor and
+                // head, each head with its own power of two.
                 // The two most significant bytes of every head fill the eight columns of one B operand (head h in columns
                 // 2h, 2h+1), the two less significant ones those of a second: lane t then finds both halves of head t's sum
                 // in its own accumulators.  Table [MMA][lower / upper slots][operand][column][t] in 32-bit words.
@@ -779,15 +738,6 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
                     bk[i][c2] = e[0];
                     bk[4 + i][c2] = e[32];
                 }
-        } else if constexpr (I8 == 1) {
-            // B fragments of the four words: column g = limb g, contraction slots 4t .. 4t + 3 (lower, upper)
-#pragma unroll
-            for (int m = 0; m < NM; ++m) bk[m][0] = bk[m][1] = 0u;
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int c2 = 0; c2 < 2; ++c2)
-                    bk[i][c2] = g < 4 ? *reinterpret_cast<const uint32_t *>(reinterpret_cast<const signed char *>(Bs) + (i * 2 + c2) * 64 + g * 16 + 4 * t) : 0u;
         } else {
 #pragma unroll
         for (int m = 0; m < NM; ++m) {
@@ -889,73 +839,6 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
                         s[k][0] = fmaf(tg[0], ks0, -bias0); s[k][1] = fmaf(ug, ks1, -bias1);
                         s[k][2] = fmaf(th[0], ks0 * (BITS == 4 ? 0.0625f : 0.25f), -bias0);
                         s[k][3] = fmaf(uh, ks1 * (BITS == 4 ? 0.0625f : 0.25f), -bias1);
-                    } else {
-                        s[k][0] = fmaf(tg[0], ks0, -bias0); s[k][1] = -INFINITY;
-                        s[k][2] = fmaf(th[0], ks0 * (BITS == 4 ? 0.0625f : 0.25f), -bias0); s[k][3] = -INFINITY;
-                    }
-                    continue;
-                }
-                if constexpr (I8 == 1) {
-                    uint32_t kw[W];
-                    load_tile_shared<BITS, D>(kt + k * TILE_WORDS, lane, kw);
-                    int iag[NGK][4];                                    // per-token keys: one set per channel group
-#pragma unroll
-                    for (int j = 0; j < NGK; ++j)
-#pragma unroll
-                        for (int x = 0; x < 4; ++x) iag[j][x] = 0;
-                    int ih0[4] = {0, 0, 0, 0}, ih1[4] = {0, 0, 0, 0};   // 3 bit: the high bits of the even / odd words
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        int (&ia)[4] = iag[NGK == 2 ? (i >> 1) : 0];
-                        uint32_t a0, a1, a2, a3;
-                        if constexpr (BITS == 3) {
-                            // the second section has the byte structure of the first: the high bits of word i sit at bits
-                            // 2, 3, 6, 7 (even i) or 0, 1, 4, 5 (odd i) of the bytes of word 4 + i / 2
-                            const uint32_t hw = kw[4 + (i >> 1)];
-                            if ((i & 1) == 0) {
-                                asm volatile("mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                                             : "+r"(ih0[0]), "+r"(ih0[1]), "+r"(ih0[2]), "+r"(ih0[3])
-                                             : "r"(hw & 0x04040404u), "r"(hw & 0x08080808u), "r"(hw & 0x40404040u), "r"(hw & 0x80808080u), "r"(bk[i][0]), "r"(bk[i][1]));
-                            } else {
-                                asm volatile("mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                                             : "+r"(ih1[0]), "+r"(ih1[1]), "+r"(ih1[2]), "+r"(ih1[3])
-                                             : "r"(hw & 0x01010101u), "r"(hw & 0x02020202u), "r"(hw & 0x10101010u), "r"(hw & 0x20202020u), "r"(bk[i][0]), "r"(bk[i][1]));
-                            }
-                        }
-                        if constexpr (BITS != 4) {
-                            const uint32_t x = kw[i];
-                            a0 = x & 0x03030303u; a1 = x & 0x0c0c0c0cu; a2 = x & 0x30303030u; a3 = x & 0xc0c0c0c0u;
-                        } else {
-                            const uint32_t x = kw[2 * i], y = kw[2 * i + 1];
-                            a0 = x & 0x0f0f0f0fu; a1 = x & 0xf0f0f0f0u; a2 = y & 0x0f0f0f0fu; a3 = y & 0xf0f0f0f0u;
-                        }
-                        asm volatile("mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                                     : "+r"(ia[0]), "+r"(ia[1]), "+r"(ia[2]), "+r"(ia[3])
-                                     : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(bk[i][0]), "r"(bk[i][1]));
-                    }
-                    if constexpr (BITS == 3) {
-                        // code = low + 4 * high; in place the high bits weigh 4, 8 (rows g, g + 8) in even words and 1, 2 in
-                        // odd ones, the low fields 1, 4: rows g in units of 1, rows g + 8 in units of 4
-                        int (&ia)[4] = iag[0];
-                        ia[0] += ih0[0] + 4 * ih1[0]; ia[1] += ih0[1] + 4 * ih1[1];
-                        ia[2] += 2 * ih0[2] + 8 * ih1[2]; ia[3] += 2 * ih0[3] + 8 * ih1[3];
-                    }
-                    // lane t = 0 holds limbs 0, 1 (columns 0, 1), its neighbour limbs 2, 3 (columns 2, 3): each lane combines
-                    // its pair (every column sum is below 2^24, exact in binary32), then the pairs combine
-                    float tg[NGK], th[NGK];
-#pragma unroll
-                    for (int j = 0; j < NGK; ++j) {
-                        const float xg = fmaf((float)iag[j][0], 256.f, (float)iag[j][1]), xh = fmaf((float)iag[j][2], 256.f, (float)iag[j][3]);
-                        const float yg = __shfl_down_sync(0xffffffffu, xg, 1), yh = __shfl_down_sync(0xffffffffu, xh, 1);
-                        tg[j] = fmaf(xg, 65536.f, yg);
-                        th[j] = fmaf(xh, 65536.f, yh);
-                    }
-                    // lanes t != 0 hold no head: their factor and bias are zero, their columns are never read
-                    if constexpr (KT) {
-#pragma unroll
-                        for (int j = 0; j < NGK; ++j) { tg[j] *= ks0; th[j] *= ks0 * (BITS == 4 ? 0.0625f : 0.25f); }
-                        s[k][0] = token_score(tg, k * 16 + g); s[k][1] = -INFINITY;
-                        s[k][2] = token_score(th, k * 16 + g + 8); s[k][3] = -INFINITY;
                     } else {
                         s[k][0] = fmaf(tg[0], ks0, -bias0); s[k][1] = -INFINITY;
                         s[k][2] = fmaf(th[0], ks0 * (BITS == 4 ? 0.0625f : 0.25f), -bias0); s[k][3] = -INFINITY;
@@ -1201,187 +1084,6 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
         }
         cluster.sync();   // nobody's shared memory goes away while the first block reads it
     }
-}
-
-// ---- launch: one instantiation per (bits, head size, value groups per row, chunk size, key-side variant) ----
-template <int BITS, int D, int NGV, int CT, bool PL, int I8 = 0, int PM = 0>
-static int launch_decode_p(const Params &p, const kvsink_cache &c, const kvsink_static_params *cal, const __half *q, float *out, float *lse, float *ws,
-                           cudaStream_t st)
-{
-    // the units the sequence is split in: key groups, or ring chunks when the parameters are static
-    const int n_groups = PM != 0 ? (c.seq_len + CT * KVSINK_TILE - 1) / (CT * KVSINK_TILE) : c.seq_len / p.G;
-    const kvsink_static_params sp = PM == 1 ? *cal : kvsink_static_params{nullptr, nullptr, nullptr, nullptr};
-    const int nsplit = choose_splits(p, n_groups);
-    const int gps = n_groups > 0 ? (n_groups + nsplit - 1) / nsplit : 0;
-    const int qchunks = decode_qchunks(p);      // blocks per KV head; each serves up to NQMAX query heads
-    if (qchunks * (I8 == 1 ? 1 : (PL ? 4 : 8)) < p.rep) return KVSINK_ERR_UNSUPPORTED;
-    const size_t smem = DecodePlan<BITS, D, NGV, CT, I8 == 1 ? 1 : (PL ? 4 : 8), PM == 2>::BYTES;
-    auto kern = decode_kernel<BITS, D, NGV, CT, PL, I8, PM>;
-    // up to 48 KB need no leave, which costs a call
-    if (smem > 48 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return KVSINK_ERR_CUDA;
-    cudaLaunchAttribute pdl[2];
-    pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    pdl[0].val.programmaticStreamSerializationAllowed = 1;
-    // up to eight splits (the portable cluster size): the splits of a unit are launched as one thread-block cluster and
-    // merged inside the kernel through distributed shared memory, which saves the merge kernel's 1 to 1.8 us (4 x 32 units of 2048
-    // tokens in fours, 2 bit: 12.2 -> 11.2 us).  A cluster has to be placed as a whole, though, and where the grid fills the chip with
-    // long blocks the slots it leaves empty cost more (clusters, and none; append and decode): fours, 18 x 8 units of 30000 tokens 106
-    // and 86 us at 2 bit, 160 and 133 at 4; sixes, 3 x 32 of 12000, 2 bit, 53 and 38.  Pairs of 2 and 4 bit
-    // win or tie at every length measured (32 x 8 of 9000 with four heads each 71.5 and 74.1, 97.5 and 100.2; 8 x 32 of 16384, 4 bit, 134.3 and
-    // 134.8), at 3 bit up to some 256 KB a block (16 x 32 of 8192, 384 KB a block, 137 and 136)
-    const int64_t blocks = (int64_t)nsplit * p.Hkv * qchunks * p.B;
-    const int64_t block_bytes = (int64_t)gps * (PM != 0 ? CT * KVSINK_TILE : p.G) * 2 * p.row_bytes;
-    const bool pairs = nsplit == 2 && p.bits != 3;
-    bool cluster_merge = nsplit > 1 && nsplit <= 8 && (pairs || blocks <= 2 * 148 || block_bytes < (nsplit == 2 ? 256 : 64) * 1024);
-    for (;;) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(nsplit, p.Hkv * qchunks, p.B);
-        cfg.blockDim = dim3(DEC_THREADS);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = st;
-        cfg.attrs = pdl;
-        cfg.numAttrs = 1;
-        if (cluster_merge) {
-            pdl[1].id = cudaLaunchAttributeClusterDimension;
-            pdl[1].val.clusterDim.x = nsplit;
-            pdl[1].val.clusterDim.y = 1;
-            pdl[1].val.clusterDim.z = 1;
-            cfg.numAttrs = 2;
-        }
-        if (cudaLaunchKernelEx(&cfg, kern, p, c, sp, q, out, lse, ws, nsplit, gps, qchunks, (int)c.seq_len, (int)cluster_merge, PrefillShape{0, 0, 0, 0, 0}) == cudaSuccess) {
-            note_launch();
-            break;
-        }
-        (void)cudaGetLastError();
-        if (!cluster_merge) return KVSINK_ERR_CUDA;
-        cluster_merge = false;   // a cluster that cannot be placed: the same launch without one, merged by the second kernel
-    }
-    if (nsplit > 1 && !cluster_merge) return launch_decode_merge(ws, nsplit, D, p.B * p.Hq, out, lse, st);
-    return KVSINK_OK;
-}
-
-// Prompt queries (the eight-column fp16 path): one block per eight (query token, query head) rows of a KV head.
-template <int BITS, int D, int NGV, int CT>
-static int launch_prefill_p(const Params &p, const kvsink_cache &c, const __half *q, const PrefillShape &pre, float *out, float *lse, cudaStream_t st)
-{
-    const size_t smem = DecodePlan<BITS, D, NGV, CT, 8>::BYTES;
-    auto kern = decode_kernel<BITS, D, NGV, CT, false, (D == 128 && BITS != 3) ? 3 : 0, 0, true>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return KVSINK_ERR_CUDA;
-    const long long blocks = ((long long)pre.T * p.rep + 7) / 8;
-    if (blocks > 0x7fffffffLL) return KVSINK_ERR_UNSUPPORTED;
-    cudaLaunchAttribute pdl[1];
-    pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    pdl[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)blocks, p.Hkv, p.B);
-    cfg.blockDim = dim3(DEC_THREADS);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cfg.attrs = pdl;
-    cfg.numAttrs = 1;
-    const kvsink_static_params none = {nullptr, nullptr, nullptr, nullptr};
-    if (cudaLaunchKernelEx(&cfg, kern, p, c, none, q, out, lse, (float *)nullptr, 1, 0, (int)blocks, (int)c.seq_len, 0, pre) != cudaSuccess)
-        return KVSINK_ERR_CUDA;
-    note_launch();
-    return KVSINK_OK;
-}
-
-template <int BITS, int D, int NGV>
-static int launch_prefill_n(const Params &p, const kvsink_cache &c, const __half *q, const PrefillShape &pre, float *out, float *lse, cudaStream_t st)
-{
-    // several channel groups per row mean G = D / NGV tokens per group: only chunk sizes that divide such a group are built;
-    // four groups per row take one tile per chunk (their parameter registers would spill otherwise)
-    constexpr int TPG_MAX = NGV == 1 ? 4 : D / NGV / KVSINK_TILE;
-    if constexpr (TPG_MAX % 4 == 0 && 4 * (2 * 128 * (D * BITS / 64) + 2 * 16 * NGV * 4) <= 4800)
-        if ((p.G / KVSINK_TILE) % 4 == 0) return launch_prefill_p<BITS, D, NGV, 4>(p, c, q, pre, out, lse, st);
-    if constexpr (TPG_MAX % 2 == 0 && NGV < 4)
-        if ((p.G / KVSINK_TILE) % 2 == 0) return launch_prefill_p<BITS, D, NGV, 2>(p, c, q, pre, out, lse, st);
-    return launch_prefill_p<BITS, D, NGV, 1>(p, c, q, pre, out, lse, st);
-}
-
-template <int BITS, int D>
-static int launch_prefill_t(const Params &p, const kvsink_cache &c, const __half *q, const PrefillShape &pre, float *out, float *lse, cudaStream_t st)
-{
-    if (p.NGv == 1) return launch_prefill_n<BITS, D, 1>(p, c, q, pre, out, lse, st);
-    if (p.NGv == 2) return launch_prefill_n<BITS, D, 2>(p, c, q, pre, out, lse, st);
-    if (p.NGv == 4) return launch_prefill_n<BITS, D, 4>(p, c, q, pre, out, lse, st);
-    return KVSINK_ERR_UNSUPPORTED;
-}
-
-template <int BITS>
-static int launch_prefill_bits(const Params &p, const kvsink_cache &c, const __half *q, int T, int q_pos0, int64_t sb, int64_t sh, int64_t stt,
-                               float *out, float *lse, cudaStream_t st)
-{
-    const PrefillShape pre = {T, q_pos0, sb, sh, stt};
-    if (p.D == 128) return launch_prefill_t<BITS, 128>(p, c, q, pre, out, lse, st);
-    if constexpr (BITS != 3)
-        if (p.D == 64) return launch_prefill_t<BITS, 64>(p, c, q, pre, out, lse, st);
-    return KVSINK_ERR_UNSUPPORTED;
-}
-
-template <int BITS, int D, int NGV, int CT, int PM>
-static int launch_decode_c(const Params &p, const kvsink_cache &c, const kvsink_static_params *cal, const __half *q, float *out, float *lse, float *ws,
-                           cudaStream_t st)
-{
-    // key side by head size, code width and query heads per KV head; only the reachable kernels are built
-    if constexpr (D == 128)
-        if (p.rep == 1) return launch_decode_p<BITS, D, NGV, CT, true, 1, PM>(p, c, cal, q, out, lse, ws, st);
-    if constexpr (D == 128 && BITS != 3) {
-        if (p.rep <= 4) return launch_decode_p<BITS, D, NGV, CT, true, 2, PM>(p, c, cal, q, out, lse, ws, st);
-        if constexpr (PM != 2) return launch_decode_p<BITS, D, NGV, CT, false, 3, PM>(p, c, cal, q, out, lse, ws, st);
-        else return KVSINK_ERR_UNSUPPORTED;      // per-token keys: at most four query heads per KV head
-    } else if constexpr (PM == 2) {
-        return KVSINK_ERR_UNSUPPORTED;           // per-token keys run on the integer key side only
-    } else if constexpr (D == 128) {
-        return launch_decode_p<BITS, D, NGV, CT, true, 0, PM>(p, c, cal, q, out, lse, ws, st);   // 3 bit: pair layout, four heads at a time
-    } else {
-        if (p.rep <= 4) return launch_decode_p<BITS, D, NGV, CT, true, 0, PM>(p, c, cal, q, out, lse, ws, st);
-        return launch_decode_p<BITS, D, NGV, CT, false, 0, PM>(p, c, cal, q, out, lse, ws, st);
-    }
-}
-
-template <int BITS, int D, int NGV, int PM>
-static int launch_decode_n(const Params &p, const kvsink_cache &c, const kvsink_static_params *cal, const __half *q, float *out, float *lse, float *ws,
-                           cudaStream_t st)
-{
-    // ring chunks of four tiles where a key group divides into them and two slots of that size stay below ~9 KB per
-    // warp, else of two tiles (G a multiple of 32), else of one
-    // several channel groups per row mean G = D / NGV tokens per group: only chunk sizes that divide such a group are built;
-    // four groups per row take one tile per chunk (their parameter registers would spill otherwise)
-    constexpr int TPG_MAX = NGV == 1 ? 4 : D / NGV / KVSINK_TILE;
-    if constexpr (TPG_MAX % 4 == 0 && 4 * (2 * 128 * (D * BITS / 64) + (PM == 2 ? 4 : 2) * 16 * NGV * 4) <= (PM == 2 ? 5200 : 4800))
-        if ((p.G / KVSINK_TILE) % 4 == 0) return launch_decode_c<BITS, D, NGV, 4, PM>(p, c, cal, q, out, lse, ws, st);
-    if constexpr (TPG_MAX % 2 == 0 && NGV < 4)
-        if ((p.G / KVSINK_TILE) % 2 == 0) return launch_decode_c<BITS, D, NGV, 2, PM>(p, c, cal, q, out, lse, ws, st);
-    return launch_decode_c<BITS, D, NGV, 1, PM>(p, c, cal, q, out, lse, ws, st);
-}
-
-template <int BITS, int D, int PM>
-static int launch_decode_t(const Params &p, const kvsink_cache &c, const kvsink_static_params *cal, const __half *q, float *out, float *lse, float *ws,
-                           cudaStream_t st)
-{
-    if (p.NGv == 1) return launch_decode_n<BITS, D, 1, PM>(p, c, cal, q, out, lse, ws, st);
-    if constexpr (PM != 2 || BITS != 3)
-        if (p.NGv == 2) return launch_decode_n<BITS, D, 2, PM>(p, c, cal, q, out, lse, ws, st);
-    if constexpr (PM == 0)
-        if (p.NGv == 4) return launch_decode_n<BITS, D, 4, PM>(p, c, cal, q, out, lse, ws, st);
-    return KVSINK_ERR_UNSUPPORTED;
-}
-
-// Dispatch over head size for one code width; each width is compiled in a translation unit of its own.  mode 0: dynamic
-// per-channel key parameters (`cal` null); 1: static parameters `cal`; 2: per-token key parameters.  Modes 1 and 2 are
-// built for head size 128 with one or two channel groups per row; mode 2 for at most four query heads per KV head
-// (3 bit: one, with one channel group).
-template <int BITS>
-static int launch_decode_bits(const Params &p, const kvsink_cache &c, const kvsink_static_params *cal, int mode, const __half *q, float *out,
-                              float *lse, float *ws, cudaStream_t st)
-{
-    if (mode == 2) return p.D == 128 ? launch_decode_t<BITS, 128, 2>(p, c, cal, q, out, lse, ws, st) : KVSINK_ERR_UNSUPPORTED;
-    if (mode == 1) return p.D == 128 && cal ? launch_decode_t<BITS, 128, 1>(p, c, cal, q, out, lse, ws, st) : KVSINK_ERR_UNSUPPORTED;
-    if (p.D == 128) return launch_decode_t<BITS, 128, 0>(p, c, cal, q, out, lse, ws, st);
-    if constexpr (BITS != 3)
-        if (p.D == 64) return launch_decode_t<BITS, 64, 0>(p, c, cal, q, out, lse, ws, st);
-    return KVSINK_ERR_UNSUPPORTED;
 }
 
 }  // namespace kvsink

@@ -1,0 +1,87 @@
+"""Decode with one query head per KV head (decode_one.cuh): tile pairs, lane-owned tokens, weights in fixed point."""
+import copy
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2508_04257_b200 as kv
+from paper_2508_04257_b200 import synth
+from parity_util import assert_close, configs, np16
+
+pytestmark = pytest.mark.gpu
+
+
+def _workload(bits, group, seq, batch=2, heads=3):
+    return synth.WORKLOADS["tiny"].scaled(bits=bits, head_dim=128, group=group, n_q_heads=heads, n_kv_heads=heads, batch=batch, seq=seq, topk=3, pfn_n=1)
+
+
+def _both(wl, H, K, V, q):
+    ocfg, gcfg = configs(wl)
+    sinks = kv.predict_sinks(gcfg, H, kv.SinkSet(gcfg))
+    cache = kv.KVCache(gcfg, sinks)
+    kv.quantize_append(gcfg, cache, K, V)
+    oc = oracle.Cache(ocfg, *oracle.predict_sinks(ocfg, np16(H)))
+    oracle.quantize_append(ocfg, oc, np16(K), np16(V))
+    out, lse = kv.decode_attention(gcfg, cache, q)
+    assert kv.read_status(cache) == 0
+    return out.cpu().numpy(), lse.cpu().numpy(), oracle.decode_attention(ocfg, oc, np16(q))
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("group,seq", [(32, 31), (32, 33), (32, 160), (32, 352), (64, 64), (64, 79), (64, 1000), (128, 128), (128, 145), (128, 1300),
+                                       (144, 577), (144, 432)])
+def test_odd_lengths_and_groups(bits, group, seq):
+    wl = _workload(bits, group, seq)
+    H = synth.make_hidden(wl, "cuda")
+    K, V = synth.make_kv(wl, 0, "cuda")
+    out, lse, (ref, ref_lse) = _both(wl, H, K, V, synth.make_query(wl, K))
+    assert_close(out, ref, "attention output")
+    assert np.abs(lse - ref_lse).max() <= 2e-3 + 1e-3 * np.abs(ref_lse).max()
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("rising", [True, False])
+def test_weights_that_move_the_unit(bits, rising):
+    """Scores that climb (or fall) by 30 along the sequence and value rows between 2^-8 and 2^8: the reference and the unit of the weights
+    move in most steps, or the first step's stays too large for the rest."""
+    wl = _workload(bits, 64, 1000)
+    H = synth.make_hidden(wl, "cuda")
+    g = torch.Generator("cuda").manual_seed(bits)
+    q = torch.randn((2, 3, 128), device="cuda", generator=g).half()
+    K = 0.1 * torch.randn((2, 3, 1000, 128), device="cuda", generator=g)
+    along = torch.linspace(0, 30, 1000, device="cuda") * 128 ** 0.5
+    K += (along if rising else along.flip(0))[:, None] * (q.float() / q.float().pow(2).sum(-1, keepdim=True))[:, :, None]
+    V = torch.randn((2, 3, 1000, 128), device="cuda", generator=g) * 2.0 ** (16 * torch.rand((2, 3, 1000, 1), device="cuda", generator=g) - 8)
+    out, lse, (ref, ref_lse) = _both(wl, H, K.half(), V.half(), q)
+    # the outputs are as large as the loudest rows near the top score: the tolerance goes with them
+    assert np.abs(out - ref).max() <= (2e-3 + 1e-2) * np.abs(ref).max()
+    assert np.abs(lse - ref_lse).max() <= 2e-3 + 1e-3 * np.abs(ref_lse).max()
+
+
+@pytest.mark.parametrize("bits", [2, 4])
+def test_sums_beyond_32_bits(bits):
+    """A query of zeros gives every token the weight 1: a warp's byte sums pass int32 unless they are set aside on the way (every 2048
+    tiles; 592 units leave one split, whose four warps take 2112 tiles each).  All units hold one unit's cache."""
+    units, seq = 592, 4 * 2112 * 16
+    one = kv.Config(1, 1, 1, 128, 512, bits, 128, seq, 2, 1, (1,))
+    many = kv.Config(1, units, units, 128, 512, bits, 128, seq, 2, 1, (1,))
+    g = torch.Generator("cuda").manual_seed(7)
+    K, V = (torch.randn((1, 1, seq, 128), device="cuda", generator=g).half() for _ in range(2))
+    V += 3                                                     # most values of a row near its middle, all far from zero
+    H = torch.randn((1, seq, 512), device="cuda", generator=g).half()
+    sinks = kv.predict_sinks(one, H, kv.SinkSet(one))
+    small = kv.KVCache(one, sinks)
+    kv.quantize_append(one, small, K, V)
+    big = copy.copy(small)
+    big.cfg, big.sizes = many, kv.cache_sizes(many)
+    for name in ("k_codes", "v_codes", "k_scale", "k_zero", "v_scale", "v_zero", "k_tail", "sink_k", "sink_v"):
+        setattr(big, name, getattr(small, name).repeat(units))
+    out, lse = kv.decode_attention(many, big, torch.zeros((1, units, 128), device="cuda", dtype=torch.float16))
+    ref, ref_lse = kv.decode_attention(one, small, torch.zeros((1, 1, 128), device="cuda", dtype=torch.float16))     # short ranges: many splits
+    assert kv.read_status(small) == 0
+    assert torch.equal(out, out[:, :1].expand_as(out)) and abs(lse[0, 0].item() - np.log(seq)) < 1e-4
+    # the same 32-bit arithmetic in another order: 135168 terms, each side within n * 2^-24 of the sum at worst, some 2^-20 of it in earnest
+    assert (out[0, 0] - ref[0, 0]).abs().max() <= 2.0 ** -18 * ref.abs().max()
+    assert (ref[0, 0] - V.float().mean((0, 1, 2))).abs().max() < 0.05
