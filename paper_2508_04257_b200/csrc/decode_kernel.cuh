@@ -177,6 +177,9 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, unsigned
                  ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
 
+template <int N>
+struct Count { static constexpr int value = N; };
+
 constexpr int DEC_WAIT_LIMIT = 1 << 22;   // polls of a full-barrier before a warp gives up (far beyond any real latency)
 
 // Shared-memory plan of a decode block, shared by the kernel and the launcher.  CT = tiles per ring chunk, NQMAX = the
@@ -297,25 +300,33 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
     // the next kernel in the stream may be scheduled from now on: its blocks take whatever room this grid leaves, set
     // themselves up, and wait at the same point until this grid has completed
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    // Sink rows of the side buffer are shared out over all warps of all splits and handled after the stream; the
-    // first row of this warp is fetched now, so that its latency hides behind the stream.
+    // Sink rows of the side buffer are shared out over all warps of all splits and handled after the stream, SB at a time: all of
+    // their loads together, a batch ahead (one row at a time cost 1311 rows of eight units in 64 splits 3.6 us: five trips to memory a warp).
+    // The first row is asked for here; there are no registers for more of them to wait in.
+    constexpr int SB = PL ? 4 : 2;
     const int sink_n = min(c.sink_count[b], p.cap);
     const int sink_worker = split * DEC_WARPS + warp, sink_workers = nsplit * DEC_WARPS;
-    int sink_pos_next = -1;
-    uint32_t sink_k_next[CPL / 2], sink_v_next[CPL / 2];
-    auto fetch_sink = [&](int j) {
-        sink_pos_next = -1;
+    int sink_pos[SB];
+    uint32_t sink_k[SB][CPL / 2], sink_v[SB][CPL / 2];
+    auto fetch_sinks = [&](int first, int from, int to) {
 #pragma unroll
-        for (int e = 0; e < CPL / 2; ++e) sink_k_next[e] = sink_v_next[e] = 0u;
-        if (j < sink_n) {
-            sink_pos_next = c.sink_pos[(size_t)b * p.cap + j];
-            const uint32_t *kr = (const uint32_t *)((const __half *)c.sink_k + ((size_t)unit * p.cap + j) * D + lane * CPL);
-            const uint32_t *vr = (const uint32_t *)((const __half *)c.sink_v + ((size_t)unit * p.cap + j) * D + lane * CPL);
+        for (int i = 0; i < SB; ++i) {
+            if (i < from || i >= to) continue;
+            const int j = first + i * sink_workers;
+            sink_pos[i] = -1;
 #pragma unroll
-            for (int e = 0; e < CPL / 2; ++e) { sink_k_next[e] = kr[e]; sink_v_next[e] = vr[e]; }
+            for (int e = 0; e < CPL / 2; ++e) sink_k[i][e] = sink_v[i][e] = 0u;
+            if (j < sink_n) {
+                sink_pos[i] = c.sink_pos[(size_t)b * p.cap + j];
+                const uint32_t *kr = (const uint32_t *)((const __half *)c.sink_k + ((size_t)unit * p.cap + j) * D + lane * CPL);
+                const uint32_t *vr = (const uint32_t *)((const __half *)c.sink_v + ((size_t)unit * p.cap + j) * D + lane * CPL);
+#pragma unroll
+                for (int e = 0; e < CPL / 2; ++e) { sink_k[i][e] = kr[e]; sink_v[i][e] = vr[e]; }
+            }
         }
     };
-    fetch_sink(sink_worker);
+
+    fetch_sinks(sink_worker, 0, 1);
 
     // ---------------- packed stream ----------------
     float m0 = M_INIT, m1 = M_INIT, l0 = 0.f, l1 = 0.f;             // running max / sum of query heads 2t and 2t+1
@@ -944,6 +955,8 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
     }
     if (!stream_ok && lane == 0) atomicOr(c.status, KVSINK_STATUS_TIMEOUT);
 
+    fetch_sinks(sink_worker, 1, SB);      // used when the packed partial is done
+
     // ---- this warp's packed partial: finish the reductions over the token lanes, convert units ----
 #pragma unroll
     for (int o = 4; o < 32; o <<= 1) {
@@ -996,32 +1009,58 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
 #pragma unroll
             for (int e = 0; e < CPL; ++e) os[i][e] = 0.f;
         }
-        for (int j = sink_worker; j < sink_n; j += sink_workers) {
-            const int pos = sink_pos_next;
-            float kf[CPL], vf[CPL];
+        for (int first = sink_worker; first < sink_n; first += SB * sink_workers) {
+            // most warps have one row, if any: the work of a whole batch only where there are more
+            auto rows = [&](auto batch) {
+            constexpr int N = decltype(batch)::value;
+            float kf[N][CPL], vf[N][CPL];
+            int pos[N];
 #pragma unroll
-            for (int e = 0; e < CPL / 2; ++e) {
-                const float2 k2 = __half22float2(*reinterpret_cast<const __half2 *>(&sink_k_next[e]));
-                const float2 v2 = __half22float2(*reinterpret_cast<const __half2 *>(&sink_v_next[e]));
-                kf[2 * e] = k2.x; kf[2 * e + 1] = k2.y; vf[2 * e] = v2.x; vf[2 * e + 1] = v2.y;
+            for (int i = 0; i < N; ++i) {
+                pos[i] = sink_pos[i] >= 0 && sink_pos[i] < n ? sink_pos[i] : -1;
+#pragma unroll
+                for (int e = 0; e < CPL / 2; ++e) {
+                    const float2 k2 = __half22float2(*reinterpret_cast<const __half2 *>(&sink_k[i][e]));
+                    const float2 v2 = __half22float2(*reinterpret_cast<const __half2 *>(&sink_v[i][e]));
+                    kf[i][2 * e] = k2.x; kf[i][2 * e + 1] = k2.y;
+                    vf[i][2 * e] = v2.x; vf[i][2 * e + 1] = v2.y;
+                }
             }
-            fetch_sink(j + sink_workers);   // the next row streams in while this one is used
-            if (pos < 0 || pos >= n) continue;
+            if (N == SB && first + SB * sink_workers < sink_n) fetch_sinks(first + SB * sink_workers, 0, SB);   // they stream in while these are used
 #pragma unroll
             for (int i = 0; i < NQMAX; ++i) {
-                if (i < nq && (!PRE || pos < row_limit(i))) {
-                    float d = 0.f;
+                if (i < nq) {
+                    float sc[N], mnew = ms[i];
 #pragma unroll
-                    for (int e = 0; e < CPL; ++e) d += qs[i * D + lane * CPL + e] * kf[e];
-                    const float sc = warp_sum(d);
-                    const float mnew = fmaxf(ms[i], sc);
-                    const float corr = ex2(ms[i] - mnew), pp = ex2(sc - mnew);
-                    ls[i] = ls[i] * corr + pp;
+                    for (int k = 0; k < N; ++k) {
+                        float d = 0.f;
 #pragma unroll
-                    for (int e = 0; e < CPL; ++e) os[i][e] = os[i][e] * corr + pp * vf[e];
+                        for (int e = 0; e < CPL; ++e) d += qs[i * D + lane * CPL + e] * kf[k][e];
+                        sc[k] = warp_sum(d);
+                    }
+#pragma unroll
+                    for (int k = 0; k < N; ++k) {
+                        if (pos[k] < 0 || (PRE && pos[k] >= row_limit(i))) sc[k] = -INFINITY;
+                        mnew = fmaxf(mnew, sc[k]);
+                    }
+                    const float corr = ex2(ms[i] - mnew);
+                    ls[i] *= corr;
+#pragma unroll
+                    for (int e = 0; e < CPL; ++e) os[i][e] *= corr;
+#pragma unroll
+                    for (int k = 0; k < N; ++k) {
+                        if (sc[k] == -INFINITY) continue;      // warp-uniform; a row that is not seen may hold anything
+                        const float pp = ex2(sc[k] - mnew);
+                        ls[i] += pp;
+#pragma unroll
+                        for (int e = 0; e < CPL; ++e) os[i][e] = fmaf(pp, vf[k][e], os[i][e]);
+                    }
                     ms[i] = mnew;
                 }
             }
+            };
+            if (first + sink_workers < sink_n) rows(Count<SB>());
+            else rows(Count<1>());
         }
         float *sp = my_part + (size_t)nq * PS;
 #pragma unroll
@@ -1053,20 +1092,21 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
             if (lse && ch == 0) lse[oq] = L > 0.f ? (M + log2f(L)) * 0.6931471805599453f : -INFINITY;
         } else {
             // the split's record: to the workspace for the merge kernel, or, when the splits of a unit form a thread-block
-            // cluster, to this block's shared memory (the query tables are no longer needed) for the cluster's first block
+            // cluster, to this block's shared memory (the query tables are no longer needed) for the cluster
             float *wsr = cluster_merge ? qs + (size_t)qh * PS : part_ws + (oq * nsplit + split) * PS;
             wsr[ch] = acc;
             if (ch == 0) { wsr[D] = M; wsr[D + 1] = L; }
         }
     }
     if (cluster_merge) {
-        // the splits of a unit are the blocks of one cluster: its first block reads the records of the others through
-        // distributed shared memory and merges them in split order (the same arithmetic as the merge kernel)
+        // the splits of a unit are the blocks of one cluster: they read one another's records through
+        // distributed shared memory and merge them in split order (the same arithmetic as the merge kernel)
         namespace cg = cooperative_groups;
         cg::cluster_group cluster = cg::this_cluster();
         cluster.sync();
-        if (split == 0) {
-            for (int idx = tid; idx < nq * D; idx += DEC_THREADS) {
+        {
+            // the outputs are shared out over the blocks
+            for (int idx = split * DEC_THREADS + tid; idx < nq * D; idx += nsplit * DEC_THREADS) {
                 const int qh = idx / D, ch = idx % D;
                 float M = M_INIT;
                 for (int sp = 0; sp < nsplit; ++sp) M = fmaxf(M, cluster.map_shared_rank(qs, sp)[(size_t)qh * PS + D]);
@@ -1082,7 +1122,7 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
                 if (lse && ch == 0) lse[oq] = L > 0.f ? (M + log2f(L)) * 0.6931471805599453f : -INFINITY;
             }
         }
-        cluster.sync();   // nobody's shared memory goes away while the first block reads it
+        cluster.sync();   // nobody's shared memory goes away while another block reads it
     }
 }
 

@@ -22,22 +22,21 @@ static int launch_decode_p(const Params &p, const kvsink_cache &c, const kvsink_
         if constexpr (I8 == 1) return decode_one_kernel<BITS, NGV, CT, PM>;
         else return decode_kernel<BITS, D, NGV, CT, PL, I8, PM>;
     }();
-    // up to 48 KB need no leave, which costs a call
-    if (smem > 48 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return KVSINK_ERR_CUDA;
     cudaLaunchAttribute pdl[2];
     pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     pdl[0].val.programmaticStreamSerializationAllowed = 1;
     // up to eight splits (the portable cluster size): the splits of a unit are launched as one thread-block cluster and
-    // merged inside the kernel through distributed shared memory, which saves the merge kernel's 1 to 1.8 us (4 x 32 units of 2048
-    // tokens in fours, 2 bit: 12.2 -> 11.2 us).  A cluster has to be placed as a whole, though, and where the grid fills the chip with
-    // long blocks the slots it leaves empty cost more (clusters, and none; append and decode): fours, 18 x 8 units of 30000 tokens 106
-    // and 86 us at 2 bit, 160 and 133 at 4; sixes, 3 x 32 of 12000, 2 bit, 53 and 38.  Pairs of 2 and 4 bit
-    // win or tie at every length measured (32 x 8 of 9000 with four heads each 71.5 and 74.1, 97.5 and 100.2; 8 x 32 of 16384, 4 bit, 134.3 and
-    // 134.8), at 3 bit up to some 256 KB a block (16 x 32 of 8192, 384 KB a block, 137 and 136)
+    // merged inside the kernel through distributed shared memory, which saves the merge kernel's 2 to 3 us.  A cluster has to be placed
+    // as a whole, though, and a grid that nearly fills the chip's 592 slots does not fit in one round any more (decode alone,
+    // clusters and none: sixes, 576 blocks, 3 x 32 units of 4000 tokens 20.3 and 14.4 us, of 12000 40.7 and 28.1; fours, 576 blocks, 18 x 8 of 9000
+    // 54 and 40; fours and eights, 512 blocks, 4 x 32 of 2048 9.8 and 10.7, 8 x 8 of 4096 with four heads 14.9 and 16.2, 4 bit 17.6 and 19.0,
+    // 16 x 8 of 30000 99.2 and 100.4).  Pairs, whose second block finds room anywhere, lose beyond a round only (20 x 32 of 3000 44.9 and 39.8;
+    // 592 blocks, 37 x 8 of 9000, 66.5 and 67.6); at 3 bit up to some 256 KB a block (16 x 32 of 8192, 384 KB a block, 137 and 136).
     const int64_t blocks = (int64_t)nsplit * p.Hkv * qchunks * p.B;
     const int64_t block_bytes = (int64_t)gps * (PM != 0 ? CT * KVSINK_TILE : p.G) * 2 * p.row_bytes;
-    const bool pairs = nsplit == 2 && p.bits != 3;
-    bool cluster_merge = nsplit > 1 && nsplit <= 8 && (pairs || blocks <= 2 * 148 || block_bytes < (nsplit == 2 ? 256 : 64) * 1024);
+    bool cluster_merge = nsplit > 1 && nsplit <= 8 && (nsplit == 2 ? blocks <= 4 * 148 && (p.bits != 3 || block_bytes < 256 * 1024) : blocks <= 512);
+    // up to 48 KB need no leave, which costs a call
+    if (smem > 48 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return KVSINK_ERR_CUDA;
     for (;;) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(nsplit, p.Hkv * qchunks, p.B);
