@@ -1,4 +1,4 @@
-// Decode attention kernels for 2-bit codes (see decode_kernel.cuh and decode_one.cuh).
+// Decode attention kernels for 2-bit codes (see decode_kernel.cuh and decode_few.cuh).
 #include "decode_launch.cuh"
 
 namespace kvsink {

@@ -207,7 +207,8 @@ struct DecodePlan {
 // column 2h multiplies by the fp16 factor q*scale and column 2h+1 by its fp16 rounding residual, so every score carries
 // the factor to ~22 bits at no extra instruction.  Without PL (five to eight heads) head h owns column h and the
 // residual of channels with large factors goes through a second multiply.
-// One query head per KV head at head size 128 has a kernel of its own (decode_one.cuh).
+// At head size 128 one query head per KV head has a kernel of its own (decode_one.cuh), and so have two to four (decode_few.cuh) but for
+// three and four at 2 bit with one channel group a row.
 // I8: the key side runs on the integer tensor path.  The four bytes of a stored word are four channels of one token row.  2 bit: the
 // word masked with 0x03.., 0x0c.., 0x30.., 0xc0.. is the u8 A fragment of one m16n8k32 (fields in place: x1, x4 for the rows
 // g + 8, x16 for the upper contraction slots, x64 for both).  4 bit: a word masked with 0x0f.. and 0xf0.. gives the registers of

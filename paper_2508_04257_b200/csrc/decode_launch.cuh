@@ -1,12 +1,13 @@
 // Launches of the decode kernels, included once per code width.
 #pragma once
 #include "decode_kernel.cuh"
+#include "decode_few.cuh"
 #include "decode_one.cuh"
 
 namespace kvsink {
 
 // ---- launch: one instantiation per (bits, head size, value groups per row, chunk size, key-side variant) ----
-template <int BITS, int D, int NGV, int CT, bool PL, int I8 = 0, int PM = 0>
+template <int BITS, int D, int NGV, int CT, bool PL, int I8 = 0, int PM = 0, int R = 0>
 static int launch_decode_p(const Params &p, const kvsink_cache &c, const kvsink_static_params *cal, const __half *q, float *out, float *lse, float *ws,
                            cudaStream_t st)
 {
@@ -16,10 +17,12 @@ static int launch_decode_p(const Params &p, const kvsink_cache &c, const kvsink_
     const int nsplit = choose_splits(p, n_groups);
     const int gps = n_groups > 0 ? (n_groups + nsplit - 1) / nsplit : 0;
     const int qchunks = decode_qchunks(p);      // blocks per KV head; each serves up to NQMAX query heads
-    if (qchunks * (I8 == 1 ? 1 : (PL ? 4 : 8)) < p.rep) return KVSINK_ERR_UNSUPPORTED;
-    const size_t smem = DecodePlan<BITS, D, NGV, CT, I8 == 1 ? 1 : (PL ? 4 : 8), PM == 2>::BYTES;
+    constexpr int NQ = R ? R : (PL ? 4 : 8);
+    if (qchunks * NQ < p.rep) return KVSINK_ERR_UNSUPPORTED;
+    const size_t smem = DecodePlan<BITS, D, NGV, CT, NQ, PM == 2>::BYTES;
     const auto kern = [] {
-        if constexpr (I8 == 1) return decode_one_kernel<BITS, NGV, CT, PM>;
+        if constexpr (R == 1) return decode_one_kernel<BITS, NGV, CT, PM>;
+        else if constexpr (R != 0) return decode_few_kernel<BITS, NGV, CT, PM, R>;
         else return decode_kernel<BITS, D, NGV, CT, PL, I8, PM>;
     }();
     cudaLaunchAttribute pdl[2];
@@ -53,7 +56,8 @@ static int launch_decode_p(const Params &p, const kvsink_cache &c, const kvsink_
             cfg.numAttrs = 2;
         }
         cudaError_t launched;
-        if constexpr (I8 == 1) launched = cudaLaunchKernelEx(&cfg, kern, p, c, sp, q, out, lse, ws, nsplit, gps, (int)c.seq_len, (int)cluster_merge);
+        if constexpr (R == 1) launched = cudaLaunchKernelEx(&cfg, kern, p, c, sp, q, out, lse, ws, nsplit, gps, (int)c.seq_len, (int)cluster_merge);
+        else if constexpr (R != 0) launched = cudaLaunchKernelEx(&cfg, kern, p, c, sp, q, out, lse, ws, nsplit, gps, qchunks, (int)c.seq_len, (int)cluster_merge);
         else launched = cudaLaunchKernelEx(&cfg, kern, p, c, sp, q, out, lse, ws, nsplit, gps, qchunks, (int)c.seq_len, (int)cluster_merge, PrefillShape{0, 0, 0, 0, 0});
         if (launched == cudaSuccess) {
             note_launch();
@@ -130,17 +134,23 @@ template <int BITS, int D, int NGV, int CT, int PM>
 static int launch_decode_c(const Params &p, const kvsink_cache &c, const kvsink_static_params *cal, const __half *q, float *out, float *lse, float *ws,
                            cudaStream_t st)
 {
-    // key side by head size, code width and query heads per KV head; only the reachable kernels are built
-    if constexpr (D == 128 && NGV < 4)
-        if (p.rep == 1) return launch_decode_p<BITS, D, NGV, CT, true, 1, PM>(p, c, cal, q, out, lse, ws, st);
-    if constexpr (D == 128 && BITS != 3) {
-        if (p.rep <= 4) return launch_decode_p<BITS, D, NGV, CT, true, 2, PM>(p, c, cal, q, out, lse, ws, st);
-        if constexpr (PM != 2) return launch_decode_p<BITS, D, NGV, CT, false, 3, PM>(p, c, cal, q, out, lse, ws, st);
-        else return KVSINK_ERR_UNSUPPORTED;      // per-token keys: at most four query heads per KV head
-    } else if constexpr (PM == 2) {
-        return KVSINK_ERR_UNSUPPORTED;           // per-token keys run on the integer key side only
-    } else if constexpr (D == 128) {
-        return launch_decode_p<BITS, D, NGV, CT, true, 0, PM>(p, c, cal, q, out, lse, ws, st);   // 3 bit: pair layout, four heads at a time
+    // kernel by head size, code width and query heads per KV head; only the reachable ones are built
+    if constexpr (D == 128) {
+        if constexpr (PM == 2 && BITS == 3)
+            if (p.rep > 1) return KVSINK_ERR_UNSUPPORTED;
+        if constexpr (NGV < 4 || CT == 2) {
+            if (p.rep == 1) return launch_decode_p<BITS, D, NGV, CT, true, 0, PM, 1>(p, c, cal, q, out, lse, ws, st);
+            if (p.rep == 2) return launch_decode_p<BITS, D, NGV, CT, true, 0, PM, 2>(p, c, cal, q, out, lse, ws, st);
+            // 2 bit with one channel group a row: as many instructions as with fp16 values, and more registers (8 x 8 units of 16000 tokens,
+            // static parameters, 34.0 and 32.1 us; of 8000 tokens, per-token keys, 30.1 and 27.8)
+            if constexpr (BITS == 2 && NGV == 1) {
+                if (p.rep <= 4) return launch_decode_p<BITS, D, NGV, CT, true, 2, PM>(p, c, cal, q, out, lse, ws, st);
+            } else {
+                if (p.rep <= 4 || BITS == 3) return launch_decode_p<BITS, D, NGV, CT, true, 0, PM, 4>(p, c, cal, q, out, lse, ws, st);
+            }
+        }
+        if constexpr (PM != 2 && BITS != 3 && (NGV < 4 || CT == 1)) return launch_decode_p<BITS, D, NGV, CT, false, 3, PM>(p, c, cal, q, out, lse, ws, st);
+        return KVSINK_ERR_UNSUPPORTED;           // per-token keys: at most four query heads per KV head
     } else {
         if (p.rep <= 4) return launch_decode_p<BITS, D, NGV, CT, true, 0, PM>(p, c, cal, q, out, lse, ws, st);
         return launch_decode_p<BITS, D, NGV, CT, false, 0, PM>(p, c, cal, q, out, lse, ws, st);
@@ -160,8 +170,8 @@ static int launch_decode_n(const Params &p, const kvsink_cache &c, const kvsink_
         if ((p.G / KVSINK_TILE) % 4 == 0) return launch_decode_c<BITS, D, NGV, 4, PM>(p, c, cal, q, out, lse, ws, st);
     if constexpr (TPG_MAX % 2 == 0 && NGV < 4)
         if ((p.G / KVSINK_TILE) % 2 == 0) return launch_decode_c<BITS, D, NGV, 2, PM>(p, c, cal, q, out, lse, ws, st);
-    if constexpr (NGV == 4 && D == 128)      // one query head: a lane keeps the parameters of one token of a pair only
-        if (p.rep == 1) return launch_decode_p<BITS, D, NGV, 2, true, 1, PM>(p, c, cal, q, out, lse, ws, st);
+    if constexpr (NGV == 4 && D == 128)      // up to four heads (3 bit: always) a lane keeps the parameters of few tokens
+        if (p.rep <= 4 || BITS == 3) return launch_decode_c<BITS, D, NGV, 2, PM>(p, c, cal, q, out, lse, ws, st);
     return launch_decode_c<BITS, D, NGV, 1, PM>(p, c, cal, q, out, lse, ws, st);
 }
 

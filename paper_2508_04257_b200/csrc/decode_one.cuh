@@ -31,6 +31,14 @@ __device__ __forceinline__ void imma16832(int (&c)[4], const uint32_t (&a)[4], u
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+// The two nibble words of a 3-bit word: rows g (me) and rows g + 8 (mo), three bits at 4 j.
+__device__ __forceinline__ void nibbles3(const uint32_t *w, int i, uint32_t *me, uint32_t *mo)
+{
+    const uint32_t x = w[i], hh = (i & 1) ? (w[4 + i / 2] << 2) : w[4 + i / 2];
+    *me = (x & 0x33333333u) | (hh & 0xccccccccu);
+    *mo = ((x >> 2) & 0x33333333u) | ((hh >> 1) & 0xccccccccu);
+}
+
 // A fragment i (channels 32 i ... 32 i + 31) of a tile's words.
 template <int BITS>
 __device__ __forceinline__ void byte_frag(const uint32_t (&w)[2 * BITS], int i, uint32_t (&a)[4])
@@ -41,8 +49,8 @@ __device__ __forceinline__ void byte_frag(const uint32_t (&w)[2 * BITS], int i, 
         const uint32_t x = w[2 * i], y = w[2 * i + 1];
         a[0] = x & 0x0f0f0f0fu; a[1] = x & 0xf0f0f0f0u; a[2] = y & 0x0f0f0f0fu; a[3] = y & 0xf0f0f0f0u;
     } else {
-        const uint32_t x = w[i], hh = (i & 1) ? (w[4 + i / 2] << 2) : w[4 + i / 2];
-        const uint32_t me = (x & 0x33333333u) | (hh & 0xccccccccu), mo = ((x >> 2) & 0x33333333u) | ((hh >> 1) & 0xccccccccu);
+        uint32_t me, mo;
+        nibbles3(w, i, &me, &mo);
         a[0] = me & 0x07070707u; a[1] = mo & 0x07070707u; a[2] = me & 0x70707070u; a[3] = mo & 0x70707070u;
     }
 }

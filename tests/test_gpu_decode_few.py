@@ -1,4 +1,4 @@
-"""Decode with one query head per KV head (decode_one.cuh): tile pairs, lane-owned tokens, weights in fixed point."""
+"""Decode with few query heads per KV head (decode_few.cuh): tile pairs, lane-owned tokens, weights in fixed point."""
 import copy
 
 import numpy as np
@@ -13,8 +13,8 @@ from parity_util import assert_close, configs, np16
 pytestmark = pytest.mark.gpu
 
 
-def _workload(bits, group, seq, batch=2, heads=3):
-    return synth.WORKLOADS["tiny"].scaled(bits=bits, head_dim=128, group=group, n_q_heads=heads, n_kv_heads=heads, batch=batch, seq=seq, topk=3, pfn_n=1)
+def _workload(bits, group, seq, rows=1, batch=2, heads=3):
+    return synth.WORKLOADS["tiny"].scaled(bits=bits, head_dim=128, group=group, n_q_heads=rows * heads, n_kv_heads=heads, batch=batch, seq=seq, topk=3, pfn_n=1)
 
 
 def _both(wl, H, K, V, q):
@@ -30,10 +30,10 @@ def _both(wl, H, K, V, q):
 
 
 @pytest.mark.parametrize("bits", [2, 3, 4])
-@pytest.mark.parametrize("group,seq", [(32, 31), (32, 33), (32, 160), (32, 352), (64, 64), (64, 79), (64, 1000), (128, 128), (128, 145), (128, 1300),
-                                       (144, 577), (144, 432)])
-def test_odd_lengths_and_groups(bits, group, seq):
-    wl = _workload(bits, group, seq)
+@pytest.mark.parametrize("rows", [1, 2, 3, 4])
+@pytest.mark.parametrize("group,seq", [(32, 31), (32, 352), (64, 79), (64, 1000), (128, 128), (128, 1300), (144, 577), (144, 432)])
+def test_odd_lengths_and_groups(bits, rows, group, seq):
+    wl = _workload(bits, group, seq, rows)
     H = synth.make_hidden(wl, "cuda")
     K, V = synth.make_kv(wl, 0, "cuda")
     out, lse, (ref, ref_lse) = _both(wl, H, K, V, synth.make_query(wl, K))
@@ -42,17 +42,20 @@ def test_odd_lengths_and_groups(bits, group, seq):
 
 
 @pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("rows", [1, 2, 4])
 @pytest.mark.parametrize("rising", [True, False])
-def test_weights_that_move_the_unit(bits, rising):
+def test_weights_that_move_the_unit(bits, rows, rising):
     """Scores that climb (or fall) by 30 along the sequence and value rows between 2^-8 and 2^8: the reference and the unit of the weights
     move in most steps, or the first step's stays too large for the rest."""
-    wl = _workload(bits, 64, 1000)
+    wl = _workload(bits, 64, 1000, rows)
     H = synth.make_hidden(wl, "cuda")
     g = torch.Generator("cuda").manual_seed(bits)
     q = torch.randn((2, 3, 128), device="cuda", generator=g).half()
     K = 0.1 * torch.randn((2, 3, 1000, 128), device="cuda", generator=g)
     along = torch.linspace(0, 30, 1000, device="cuda") * 128 ** 0.5
     K += (along if rising else along.flip(0))[:, None] * (q.float() / q.float().pow(2).sum(-1, keepdim=True))[:, :, None]
+    # the other rows of a KV head climb at other rates, or fall
+    q = torch.stack([q * (1 - 0.7 * r) for r in range(rows)], 2).reshape(2, 3 * rows, 128).contiguous()
     V = torch.randn((2, 3, 1000, 128), device="cuda", generator=g) * 2.0 ** (16 * torch.rand((2, 3, 1000, 1), device="cuda", generator=g) - 8)
     out, lse, (ref, ref_lse) = _both(wl, H, K.half(), V.half(), q)
     # the outputs are as large as the loudest rows near the top score: the tolerance goes with them
@@ -60,13 +63,13 @@ def test_weights_that_move_the_unit(bits, rising):
     assert np.abs(lse - ref_lse).max() <= 2e-3 + 1e-3 * np.abs(ref_lse).max()
 
 
-@pytest.mark.parametrize("bits", [2, 4])
-def test_sums_beyond_32_bits(bits):
-    """A query of zeros gives every token the weight 1: a warp's byte sums pass int32 unless they are set aside on the way (every 2048
+@pytest.mark.parametrize("bits,rows", [(2, 1), (4, 1), (2, 2), (4, 4), (3, 4)])
+def test_sums_beyond_32_bits(bits, rows):
+    """A query of zeros gives every token the weight 1: a warp's byte sums pass int32 unless they are carried on the way (every 2048
     tiles; 592 units leave one split, whose four warps take 2112 tiles each).  All units hold one unit's cache."""
     units, seq = 592, 4 * 2112 * 16
-    one = kv.Config(1, 1, 1, 128, 512, bits, 128, seq, 2, 1, (1,))
-    many = kv.Config(1, units, units, 128, 512, bits, 128, seq, 2, 1, (1,))
+    one = kv.Config(1, rows, 1, 128, 512, bits, 128, seq, 2, 1, (1,))
+    many = kv.Config(1, rows * units, units, 128, 512, bits, 128, seq, 2, 1, (1,))
     g = torch.Generator("cuda").manual_seed(7)
     K, V = (torch.randn((1, 1, seq, 128), device="cuda", generator=g).half() for _ in range(2))
     V += 3                                                     # most values of a row near its middle, all far from zero
@@ -78,10 +81,10 @@ def test_sums_beyond_32_bits(bits):
     big.cfg, big.sizes = many, kv.cache_sizes(many)
     for name in ("k_codes", "v_codes", "k_scale", "k_zero", "v_scale", "v_zero", "k_tail", "sink_k", "sink_v"):
         setattr(big, name, getattr(small, name).repeat(units))
-    out, lse = kv.decode_attention(many, big, torch.zeros((1, units, 128), device="cuda", dtype=torch.float16))
-    ref, ref_lse = kv.decode_attention(one, small, torch.zeros((1, 1, 128), device="cuda", dtype=torch.float16))     # short ranges: many splits
+    out, lse = kv.decode_attention(many, big, torch.zeros((1, rows * units, 128), device="cuda", dtype=torch.float16))
+    ref, ref_lse = kv.decode_attention(one, small, torch.zeros((1, rows, 128), device="cuda", dtype=torch.float16))     # short ranges: many splits
     assert kv.read_status(small) == 0
-    assert torch.equal(out, out[:, :1].expand_as(out)) and abs(lse[0, 0].item() - np.log(seq)) < 1e-4
+    assert torch.equal(out, out[:, :rows].repeat(1, units, 1)) and abs(lse[0, 0].item() - np.log(seq)) < 1e-4
     # the same 32-bit arithmetic in another order: 135168 terms, each side within n * 2^-24 of the sum at worst, some 2^-20 of it in earnest
     assert (out[0, 0] - ref[0, 0]).abs().max() <= 2.0 ** -18 * ref.abs().max()
     assert (ref[0, 0] - V.float().mean((0, 1, 2))).abs().max() < 0.05
