@@ -7,7 +7,7 @@
 // Values: a pair of tiles is multiplied together: the bytes of both tiles' words that belong to one 16-channel matrix are put in one word
 // (4 bit: they are already), so that all 32 contraction slots are tokens and no column is spent on telling matrices apart.
 //   weight = rint(2^(s - ref) * scale * 2^ev), below 2^31, per row; sums of a byte are exact in int32.  When a weight does not fit (one vote a
-//   step) a row's reference moves by whole bytes, so that the sums only change places: with four rows there are 64 of them a lane, and
+//   step) the references and units of the rows move by whole bits and the sums with them, in place: with four rows there are 64 of them a lane, and
 //   rescaling them in binary32 (another 64 values, which only fit local memory) took 1.5 times as long as everything else.
 // Append and decode, us a pass, fp16 values before and this kernel (start of both: the same merge and splits): 16 x 8 units of 30000 tokens, four
 // heads each, 4 bit, 140 -> 123; 4 x 8 of 30000, 3 bit, 53 -> 49; 8 x 8 of 16000, groups of 32, 2 bit, 67 -> 58, groups of 64 46 -> 44; two heads,
@@ -58,6 +58,7 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
     constexpr float ROWF = BITS == 2 ? 0.25f : (BITS == 4 ? 0.0625f : 1.f);      // rows g + 8 of a fragment: place of their field
     constexpr float UPF = BITS == 4 ? 1.f : 0.0625f;                             // upper contraction slots: place of their field
     constexpr float WEIGHT_LIMIT = 2130706432.f;                                 // 0x7f000000: its carries still fit a signed byte
+    constexpr int PLACE = BITS == 4 ? 24 : 26;                                   // a new unit puts the largest weight into [2^PLACE, 2^(PLACE + 1))
 
     const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), g = lane >> 2, t = lane & 3;
     const bool odd = t & 1;
@@ -140,21 +141,24 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
 #pragma unroll
     for (int j = 0; j < NGv; ++j) bv[j] = 0.f;
 
-    // The sums of the lanes with `on` in a unit 256 times as large: every byte's sum becomes the next lower byte's.
-    auto shift_bytes = [&](bool on) {
+    // The sums in a unit 2^k times as large (k <= 8, the same for a row's lanes): what a byte's sum loses at its lower end goes to the next
+    // lower byte, and only the lowest one's is rounded.
+    auto shift_sums = [&](int k) {
+        const int lost = (1 << k) - 1, half = (1 << k) >> 1, up = 1 << (8 - k);
 #pragma unroll
         for (int i = 0; i < 8; ++i)
 #pragma unroll
             for (int x = 0; x < 4; x += 2) {
                 if constexpr (R == 2) {      // bytes 3, 2 are the even lane's, 1, 0 the odd one's
-                    const int hi = O[i][x], lo = O[i][x + 1], other = __shfl_xor_sync(0xffffffffu, lo, 1);
-                    if (on) { O[i][x] = odd ? other : 0; O[i][x + 1] = odd ? hi + ((lo + 128) >> 8) : hi; }
-                } else if (on) {
+                    const int hi = O[i][x], lo = O[i][x + 1], above = __shfl_xor_sync(0xffffffffu, lo, 1);
+                    O[i][x] = (hi >> k) + (odd ? (above & lost) * up : 0);
+                    O[i][x + 1] = ((lo + (odd ? half : 0)) >> k) + (hi & lost) * up;
+                } else {
                     int (&u)[4] = O[i], (&v)[4] = O[(8 + i) % (8 * NT)];
-                    v[x + 1] = v[x] + ((v[x + 1] + 128) >> 8);
-                    v[x] = u[x + 1];
-                    u[x + 1] = u[x];
-                    u[x] = 0;
+                    v[x + 1] = ((v[x + 1] + half) >> k) + (v[x] & lost) * up;
+                    v[x] = (v[x] >> k) + (u[x + 1] & lost) * up;
+                    u[x + 1] = (u[x + 1] >> k) + (u[x] & lost) * up;
+                    u[x] >>= k;
                 }
             }
     };
@@ -195,9 +199,12 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
         for (int o = 4; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         return v;
     };
-    // Weights of a step's tokens of this lane: pw = 2^(s - ref) and x = pw * scale in units of 2^-ev, after moving the rows' references if
-    // one weight of the warp does not fit.  The first move puts a row's largest weight into [2^28, 2^29); later ones are by whole bytes
-    // (ref by 8, 16, ...), so that the sums so far only change places and the largest weight stays above 2^22.
+    // Weights of a step's tokens of this lane: pw = 2^(s - ref) and x = pw * scale in units of 2^-ev, after moving the rows' references and
+    // units if one weight of the warp does not fit.  References are whole numbers, so that the sums so far move by whole bits; a new unit
+    // puts the row's largest weight of the step into [2^PLACE, 2^(PLACE + 1)), where it is not finer than the old one: 22 bits of it also in the upper
+    // slots, which take a sixteenth, and room for weights 16 (4 bit: 64) times as large.  A move costs a few hundred instructions, most of them
+    // for the sums, and more room means fewer moves: 2 bits more of it and 2 (4 bit: 4) bits less, append and decode of 4 x 8 units of 30000 tokens,
+    // four heads, 3 bit, 52.4 and 54.3 us; 16 x 8, 4 bit, 131.7 with four bits less.
     auto weights = [&](const auto &s, const auto &sv, auto &pw, auto &x) {
         constexpr int N = sizeof(pw) / sizeof(pw[0]);
         bool moves = false;
@@ -216,7 +223,7 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
         float top = ref;
 #pragma unroll
         for (int k = 0; k < N; ++k) top = fmaxf(top, s[k]);
-        top = row_max(top);
+        top = ceilf(row_max(top));
         float wm = 0.f;
 #pragma unroll
         for (int k = 0; k < N; ++k) {
@@ -225,33 +232,21 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
             for (int j = 0; j < NGv; ++j) wm = fmaxf(wm, pw[k] * fabsf(sv[k][j]));
         }
         wm = row_max(wm);
-        const float rise = top - ref;
-        if (__all_sync(0xffffffffu, ref == M_INIT)) {
-            // nothing has been added yet (the rows see the same tokens: they all start here)
-            ref = top;
-            ev = 28 - floor_log2(wm);
-            ev = ev > 60 ? 60 : (ev < -60 ? -60 : ev);
-        } else {
-            // bytes by which the largest weight is too large, and by which 2^(s - ref) is although the scales are small
-            const float over = (float)(floor_log2(wm) + ev) + rise - 29.9f;
-            int k = over > 0.f ? (int)fminf(ceilf(over * 0.125f), 1.0e8f) : 0;
-            int j = rise - 8.f * k > 64.f ? (int)fminf(ceilf((rise - 8.f * k - 64.f) * 0.125f), 1.0e8f) : 0;
-            if (j > 0 && ev + 8 * (long long)j > 100) { k += j; j = 0; }
-            for (int i = 0; i < 4 && __any_sync(0xffffffffu, k > i); ++i) shift_bytes(k > i);
-            ev += 8 * j;
-            const float f = k + j > 15 ? 0.f : pow2i(-8 * (k + j));
-            l *= f;
+        const int rise = (int)fminf(top - ref, 200.f);      // of a row that has no sums yet: 200
+        const int to = min(max(min(PLACE - floor_log2(wm), 60), -60), ev + rise);
+        // the sums are below 2^56
+        for (int left = ref == M_INIT ? 0 : min(ev + rise - to, 56); __any_sync(0xffffffffu, left > 0); left -= 8) shift_sums(min(max(left, 0), 8));
+        const float f = rise > 126 ? 0.f : pow2i(-rise);
+        l *= f;
 #pragma unroll
-            for (int i = 0; i < NGv; ++i) bv[i] *= f;
-            ref = k + j > 15 ? top : ref + 8.f * (float)(k + j);
-        }
+        for (int i = 0; i < NGv; ++i) bv[i] *= f;
+        ref = top;
+        ev = to;
         evf = pow2i(ev);
 #pragma unroll
-        for (int k = 0; k < N; ++k) {
-            pw[k] = ex2(s[k] - ref);
+        for (int k = 0; k < N; ++k)
 #pragma unroll
             for (int j = 0; j < NGv; ++j) x[k][j] = pw[k] * (sv[k][j] * (evf * up_of(k)));
-        }
     };
     // The value products of a pair: this lane's tokens' weights and parameters, and the two tiles' words.
     const uint32_t pair_sel = R == 2 && odd ? 0x4051u : 0x6273u;     // bytes of two tokens for this lane's two columns
@@ -654,9 +649,9 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
             }
             // a tile adds less than 2^19 to a sum of bytes
             if ((ci & (2048 / CT - 1)) == 2048 / CT - 1 && __any_sync(0xffffffffu, carry_bytes())) {
-                shift_bytes(true);
+                shift_sums(1);
                 carry_bytes();
-                ev -= 8;
+                ev -= 1;
                 evf = pow2i(ev);
             }
         }

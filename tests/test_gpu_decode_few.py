@@ -63,6 +63,53 @@ def test_weights_that_move_the_unit(bits, rows, rising):
     assert np.abs(lse - ref_lse).max() <= 2e-3 + 1e-3 * np.abs(ref_lse).max()
 
 
+UNITS = 592      # as many units as the chip has slots: one split, whose four warps take a quarter of the sequence each
+
+
+def _long_ranges(bits, group, K, V, q):
+    """Decode of one unit's cache (K, V [seq, 128], q [rows, 128]) that all of UNITS units hold, and the oracle's result for one of them."""
+    rows, seq = q.shape[0], K.shape[0]
+    args = lambda units: (1, rows * units, units, 128, 512, bits, group, seq, 2, 1, (1,))
+    one, many, ocfg = kv.Config(*args(1)), kv.Config(*args(UNITS)), oracle.Config(*args(1))
+    K, V = K[None, None].half(), V[None, None].half()
+    H = torch.randn((1, seq, 512), device="cuda", generator=torch.Generator("cuda").manual_seed(7)).half()
+    small = kv.KVCache(one, kv.predict_sinks(one, H, kv.SinkSet(one)))
+    kv.quantize_append(one, small, K, V)
+    big = copy.copy(small)
+    big.cfg, big.sizes = many, kv.cache_sizes(many)
+    for name in ("k_codes", "v_codes", "k_scale", "k_zero", "v_scale", "v_zero", "k_tail", "sink_k", "sink_v"):
+        setattr(big, name, getattr(small, name).repeat(UNITS))
+    out, lse = kv.decode_attention(many, big, q.half().repeat(UNITS, 1)[None].contiguous())
+    assert kv.read_status(small) == 0
+    assert torch.equal(out, out[:, :rows].repeat(1, UNITS, 1)) and torch.equal(lse, lse[:, :rows].repeat(1, UNITS))
+    oc = oracle.Cache(ocfg, *oracle.predict_sinks(ocfg, np16(H)))
+    oracle.quantize_append(ocfg, oc, np16(K), np16(V))
+    ref, ref_lse = oracle.decode_attention(ocfg, oc, np16(q.half())[None])
+    return out[0, :rows].cpu().numpy(), lse[0, :rows].cpu().numpy(), ref[0], ref_lse[0]
+
+
+def _queries(rows, g):
+    """Queries of one direction, each a fifth shorter than the one before, and what a key is made of so that the first one's score is 1."""
+    q = torch.randn(128, device="cuda", generator=g).half().float()
+    return torch.stack([q * (1 - 0.2 * r) for r in range(rows)]).half(), q * (128 ** 0.5 / q.pow(2).sum())
+
+
+# jump in nats, length of the row: the reference moves by 48 to 173 bits at once, the largest weight by up to 8 more
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("rows", [1, 2, 3, 4])
+def test_one_token_far_above_the_rest(bits, rows):
+    g = torch.Generator("cuda").manual_seed(11 * bits + rows)
+    q, key = _queries(rows, g)
+    flat = torch.randn((32768, 128), device="cuda", generator=g) + 1
+    for jump, loud in ((33, 1), (45, 1), (60, 16), (60, 256), (85, 1), (85, 16), (85, 256), (120, 256)):
+        K, V = torch.zeros_like(flat), flat.clone()      # equal tokens, 8192 a warp, before it
+        K[-100], V[-100] = jump * key, loud * V[-100]
+        out, lse, ref, ref_lse = _long_ranges(bits, 64 if bits == 2 and rows > 2 else 128, K, V, q)      # the shapes that decode_few.cuh takes
+        err = np.abs(out - ref).max(1) / np.abs(ref).max(1)
+        assert err.max() <= 5e-5, (jump, loud, err)
+        assert np.abs(lse - ref_lse).max() <= 1e-5 * np.abs(ref_lse).max(), (jump, loud)
+
+
 @pytest.mark.parametrize("bits,rows", [(2, 1), (4, 1), (2, 2), (4, 4), (3, 4)])
 def test_sums_beyond_32_bits(bits, rows):
     """A query of zeros gives every token the weight 1: a warp's byte sums pass int32 unless they are carried on the way (every 2048
