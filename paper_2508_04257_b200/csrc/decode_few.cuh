@@ -6,9 +6,10 @@
 // Keys: a row's four signed bytes in four of the eight columns of an operand (R = 4: two operands, the upper bytes and the lower).
 // Values: a pair of tiles is multiplied together: the bytes of both tiles' words that belong to one 16-channel matrix are put in one word
 // (4 bit: they are already), so that all 32 contraction slots are tokens and no column is spent on telling matrices apart.
-//   weight = rint(2^(s - ref) * scale * 2^ev), below 2^31, per row; sums of a byte are exact in int32.  When a weight does not fit (one vote a
-//   step) the references and units of the rows move by whole bits and the sums with them, in place: with four rows there are 64 of them a lane, and
-//   rescaling them in binary32 (another 64 values, which only fit local memory) took 1.5 times as long as everything else.
+//   weight = rint(2^(s - ref) * scale * 2^ev), below 2^31, ref per row and ev per row and value channel group; sums of a byte are exact in
+//   int32.  When a weight does not fit (one vote a step) the references and units of the rows move by whole bits and the sums with them, in place:
+//   with four rows there are 64 of them a lane, and rescaling them in binary32 (another 64 values, which only fit local memory) took 1.5 times as
+//   long as everything else.
 // Append and decode, us a pass, fp16 values before and this kernel (start of both: the same merge and splits): 16 x 8 units of 30000 tokens, four
 // heads each, 4 bit, 140 -> 123; 4 x 8 of 30000, 3 bit, 53 -> 49; 8 x 8 of 16000, groups of 32, 2 bit, 67 -> 58, groups of 64 46 -> 44; two heads,
 // 2 bit 34.8 -> 30.3, 4 bit 44.2 -> 38.6.  Error against 64 bits 5e-5 -> 1e-6.  Four heads at 2 bit with one channel group a row stay in
@@ -132,8 +133,9 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
     int O[8 * NT][4];
     const float up = (BITS != 4 && odd) ? 0.0625f : 1.f;             // R = 2: this lane's tokens stand in the upper contraction slots
     auto up_of = [&](int k) { return R == 4 ? ((BITS != 4 && (k & 1)) ? 0.0625f : 1.f) : up; };
-    int ev = 60;
-    float evf = pow2i(60);
+    float evf[NGv];                       // 2^ev, a value channel group's own: groups may lie far apart in size
+#pragma unroll
+    for (int j = 0; j < NGv; ++j) evf[j] = pow2i(60);
 #pragma unroll
     for (int i = 0; i < 8 * NT; ++i)
 #pragma unroll
@@ -141,12 +143,12 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
 #pragma unroll
     for (int j = 0; j < NGv; ++j) bv[j] = 0.f;
 
-    // The sums in a unit 2^k times as large (k <= 8, the same for a row's lanes): what a byte's sum loses at its lower end goes to the next
-    // lower byte, and only the lowest one's is rounded.
-    auto shift_sums = [&](int k) {
+    // The sums of value channel group j in a unit 2^k times as large (k <= 8, the same for a row's lanes): what a byte's sum loses at its lower
+    // end goes to the next lower byte, and only the lowest one's is rounded.
+    auto shift_sums = [&](int j, int k) {
         const int lost = (1 << k) - 1, half = (1 << k) >> 1, up = 1 << (8 - k);
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
+        for (int i = 8 / NGv * j; i < 8 / NGv * (j + 1); ++i)
 #pragma unroll
             for (int x = 0; x < 4; x += 2) {
                 if constexpr (R == 2) {      // bytes 3, 2 are the even lane's, 1, 0 the odd one's
@@ -200,8 +202,8 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
         return v;
     };
     // Weights of a step's tokens of this lane: pw = 2^(s - ref) and x = pw * scale in units of 2^-ev, after moving the rows' references and
-    // units if one weight of the warp does not fit.  References are whole numbers, so that the sums so far move by whole bits; a new unit
-    // puts the row's largest weight of the step into [2^PLACE, 2^(PLACE + 1)), where it is not finer than the old one: 22 bits of it also in the upper
+    // (each channel group's) units if one weight of the warp does not fit.  References are whole numbers, so that the sums so far move by
+    // whole bits; a new unit puts the row's largest weight of the step into [2^PLACE, 2^(PLACE + 1)), where it is not finer than the old one: 22 bits of it also in the upper
     // slots, which take a sixteenth, and room for weights 16 (4 bit: 64) times as large.  A move costs a few hundred instructions, most of them
     // for the sums, and more room means fewer moves: 2 bits more of it and 2 (4 bit: 4) bits less, append and decode of 4 x 8 units of 30000 tokens,
     // four heads, 3 bit, 52.4 and 54.3 us; 16 x 8, 4 bit, 131.7 with four bits less.
@@ -215,7 +217,7 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
             moves |= d > 64.f;
 #pragma unroll
             for (int j = 0; j < NGv; ++j) {
-                x[k][j] = pw[k] * (sv[k][j] * (evf * up_of(k)));
+                x[k][j] = pw[k] * (sv[k][j] * (evf[j] * up_of(k)));
                 moves |= fabsf(x[k][j]) >= WEIGHT_LIMIT * up_of(k);
             }
         }
@@ -224,29 +226,26 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
 #pragma unroll
         for (int k = 0; k < N; ++k) top = fmaxf(top, s[k]);
         top = ceilf(row_max(top));
-        float wm = 0.f;
-#pragma unroll
-        for (int k = 0; k < N; ++k) {
-            pw[k] = ex2(s[k] - top);
-#pragma unroll
-            for (int j = 0; j < NGv; ++j) wm = fmaxf(wm, pw[k] * fabsf(sv[k][j]));
-        }
-        wm = row_max(wm);
+        const bool first = ref == M_INIT;
         const int rise = (int)fminf(top - ref, 200.f);      // of a row that has no sums yet: 200
-        const int to = min(max(min(PLACE - floor_log2(wm), 60), -60), ev + rise);
-        // the sums are below 2^56
-        for (int left = ref == M_INIT ? 0 : min(ev + rise - to, 56); __any_sync(0xffffffffu, left > 0); left -= 8) shift_sums(min(max(left, 0), 8));
         const float f = rise > 126 ? 0.f : pow2i(-rise);
+        ref = top;
         l *= f;
 #pragma unroll
-        for (int i = 0; i < NGv; ++i) bv[i] *= f;
-        ref = top;
-        ev = to;
-        evf = pow2i(ev);
+        for (int k = 0; k < N; ++k) pw[k] = ex2(s[k] - ref);
 #pragma unroll
-        for (int k = 0; k < N; ++k)
+        for (int j = 0; j < NGv; ++j) {
+            float wm = 0.f;
 #pragma unroll
-            for (int j = 0; j < NGv; ++j) x[k][j] = pw[k] * (sv[k][j] * (evf * up_of(k)));
+            for (int k = 0; k < N; ++k) wm = fmaxf(wm, pw[k] * fabsf(sv[k][j]));
+            const int ev = floor_log2(evf[j]), to = min(max(min(PLACE - floor_log2(row_max(wm)), 60), -60), ev + rise);
+            // the sums are below 2^56
+            for (int left = first ? 0 : min(ev + rise - to, 56); __any_sync(0xffffffffu, left > 0); left -= 8) shift_sums(j, min(max(left, 0), 8));
+            evf[j] = pow2i(to);
+            bv[j] *= f;
+#pragma unroll
+            for (int k = 0; k < N; ++k) x[k][j] = pw[k] * (sv[k][j] * (evf[j] * up_of(k)));
+        }
     };
     // The value products of a pair: this lane's tokens' weights and parameters, and the two tiles' words.
     const uint32_t pair_sel = R == 2 && odd ? 0x4051u : 0x6273u;     // bytes of two tokens for this lane's two columns
@@ -649,10 +648,12 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
             }
             // a tile adds less than 2^19 to a sum of bytes
             if ((ci & (2048 / CT - 1)) == 2048 / CT - 1 && __any_sync(0xffffffffu, carry_bytes())) {
-                shift_sums(1);
+#pragma unroll
+                for (int j = 0; j < NGv; ++j) {
+                    shift_sums(j, 1);
+                    evf[j] *= 0.5f;
+                }
                 carry_bytes();
-                ev -= 1;
-                evf = pow2i(ev);
             }
         }
     }
@@ -678,7 +679,7 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
                 o += __shfl_xor_sync(0xffffffffu, o, 1);
             }
             if (row < nq && (R == 4 || odd == (half == 1)))
-                my_part[row * PS + 16 * m + 8 * half + g] = o * (pow2i(-ev) * (half ? ROWF : 1.f)) - bv[m * NGv / 8];
+                my_part[row * PS + 16 * m + 8 * half + g] = o * (pow2i(-floor_log2(evf[m * NGv / 8])) * (half ? ROWF : 1.f)) - bv[m * NGv / 8];
         }
     if (row < nq && g == 0 && (R == 4 || !odd)) { my_part[row * PS + D] = ref; my_part[row * PS + D + 1] = l; }
 

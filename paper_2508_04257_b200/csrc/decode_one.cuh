@@ -16,7 +16,7 @@
 // Values: a stored byte pair belongs to one channel and two tokens, and the two byte pairs of a 2- or 3-bit word (the two words of a
 // 4-bit fragment) to two 16-channel matrices.  The weights' four signed bytes therefore stand in eight columns, 2 l + matrix, with
 // zeros where the other matrix' codes are: lane t finds byte t of both matrices' sums in its accumulators.
-//   weight = rint(2^(s - R) * scale * 2^ev), below 2^31; R and ev move only when a weight would not fit (one vote a step).  The sums
+//   weight = rint(2^(s - R) * scale * 2^ev), below 2^31, ev per value channel group; R and ev move only when a weight would not fit (one vote a step).  The sums
 //   of a byte are exact in int32; when R or ev moves they are added to binary32 ones and start from zero.  The upper contraction
 //   slots' tokens of 2 and 3 bit carry a weight divided by 16, kept to 2^-25 of the largest or better.
 #pragma once
@@ -135,18 +135,17 @@ decode_one_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
     float Of[4][4];                       // the part of them from before the last move of R or ev
     const float up = (BITS != 4 && odd) ? 0.0625f : 1.f;             // this lane's token stands in the upper contraction slots
     const float w_limit = WEIGHT_LIMIT * up;
-    int ev = 60;
-    float evl = pow2i(60) * up;
+    float evl[NGv];                       // 2^ev, a value channel group's own (groups may lie far apart in size), of this lane's slots
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int x = 0; x < 4; ++x) { O[i][x] = 0; Of[i][x] = 0.f; }
 #pragma unroll
-    for (int j = 0; j < NGv; ++j) bv[j] = 0.f;
+    for (int j = 0; j < NGv; ++j) { bv[j] = 0.f; evl[j] = pow2i(60) * up; }
 
-    auto settle = [&](float f) {
+    auto settle = [&](int j, float f) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 4 / NGv * j; i < 4 / NGv * (j + 1); ++i)
 #pragma unroll
             for (int x = 0; x < 4; ++x) { Of[i][x] = (Of[i][x] + (float)O[i][x]) * f; O[i][x] = 0; }
     };
@@ -161,38 +160,33 @@ decode_one_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
             pw[k] = ex2(d);
             moves |= d > 20.f;
 #pragma unroll
-            for (int j = 0; j < NGv; ++j) { x[k][j] = pw[k] * (sv[k][j] * evl); moves |= fabsf(x[k][j]) >= w_limit; }
+            for (int j = 0; j < NGv; ++j) { x[k][j] = pw[k] * (sv[k][j] * evl[j]); moves |= fabsf(x[k][j]) >= w_limit; }
         }
         if (!__any_sync(0xffffffffu, moves)) return;
         float top = R;
 #pragma unroll
         for (int k = 0; k < N; ++k) top = fmaxf(top, s[k]);
         top = warp_max(top);
-        float wm = 0.f;
-#pragma unroll
-        for (int k = 0; k < N; ++k) {
-            pw[k] = ex2(s[k] - top);
-#pragma unroll
-            for (int j = 0; j < NGv; ++j) wm = fmaxf(wm, pw[k] * fabsf(sv[k][j]));
-        }
-        wm = warp_max(wm);
         const float corr = ex2(R - top);
-        int to = 28 - floor_log2(wm);
-        // not finer than the weights so far allow: they shrink by corr
-        const int most = ev + max(0, -floor_log2(corr) - 1);
-        to = min(to, R == M_INIT ? 60 : most);
-        to = to > 60 ? 60 : (to < -60 ? -60 : to);
-        settle(corr * pow2i(to - ev));
-        ev = to;
-        evl = pow2i(ev) * up;
+        const int rise = max(0, -floor_log2(corr) - 1);
+        const bool first = R == M_INIT;
+        R = top;
         l *= corr;
 #pragma unroll
-        for (int j = 0; j < NGv; ++j) bv[j] *= corr;
-        R = top;
+        for (int k = 0; k < N; ++k) pw[k] = ex2(s[k] - R);
 #pragma unroll
-        for (int k = 0; k < N; ++k)
+        for (int j = 0; j < NGv; ++j) {
+            float wm = 0.f;
 #pragma unroll
-            for (int j = 0; j < NGv; ++j) x[k][j] = pw[k] * (sv[k][j] * evl);
+            for (int k = 0; k < N; ++k) wm = fmaxf(wm, pw[k] * fabsf(sv[k][j]));
+            // not finer than the weights so far allow: they shrink by corr
+            const int ev = floor_log2(evl[j]) - floor_log2(up), to = max(min(28 - floor_log2(warp_max(wm)), first ? 60 : min(60, ev + rise)), -60);
+            settle(j, corr * pow2i(to - ev));
+            evl[j] = pow2i(to) * up;
+            bv[j] *= corr;
+#pragma unroll
+            for (int k = 0; k < N; ++k) x[k][j] = pw[k] * (sv[k][j] * evl[j]);
+        }
     };
     // The value products of a pair: this lane's token's weight and parameters, the two tiles' words.
     const int col_src = (g >> 2) * 4 + t;                            // lane that holds the byte pair of column g's byte, of token quarter 0
@@ -518,7 +512,10 @@ decode_one_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
                 pair_values(pw[pr], x[pr], sv[pr], zv[pr],
                             [&](int k, uint32_t (&w)[W]) { load_tile_shared<BITS, D>(vt + (pr * TP + k) * TILE_WORDS, lane, w); });
             // a tile adds less than 2^19 to a sum of bytes
-            if ((ci & (2048 / CT - 1)) == 2048 / CT - 1) settle(1.f);
+            if ((ci & (2048 / CT - 1)) == 2048 / CT - 1) {
+#pragma unroll
+                for (int j = 0; j < NGv; ++j) settle(j, 1.f);
+            }
         }
     }
     if (!stream_ok && lane == 0) atomicOr(c.status, KVSINK_STATUS_TIMEOUT);
@@ -538,7 +535,7 @@ decode_one_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
                 float o = ((float)O[i][x] + Of[i][x]) * unit_t;      // this lane's byte; the quad's four make the sum
                 o += __shfl_xor_sync(0xffffffffu, o, 1);
                 o += __shfl_xor_sync(0xffffffffu, o, 2);
-                if (t == x) my_part[16 * (2 * i + (x & 1)) + 8 * (x >> 1) + g] = o * (pow2i(-ev) * (x >= 2 ? ROWF : 1.f)) - bv[i * NGv / 4];
+                if (t == x) my_part[16 * (2 * i + (x & 1)) + 8 * (x >> 1) + g] = o * (pow2i(floor_log2(up) - floor_log2(evl[i * NGv / 4])) * (x >= 2 ? ROWF : 1.f)) - bv[i * NGv / 4];
             }
         if (lane == 0) { my_part[D] = R; my_part[D + 1] = l; }
     }

@@ -110,6 +110,20 @@ def test_one_token_far_above_the_rest(bits, rows):
         assert np.abs(lse - ref_lse).max() <= 1e-5 * np.abs(ref_lse).max(), (jump, loud)
 
 
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("rows", [1, 2, 4])
+@pytest.mark.parametrize("group", [32, 64])
+def test_value_channel_groups_of_different_size(bits, rows, group):
+    """The channel groups of a value row lie 2^15 apart in size: the quiet ones keep their digits."""
+    g = torch.Generator("cuda").manual_seed(13 * bits + rows)
+    size = torch.tensor([300.0, 0.01, 0.3, 300.0], device="cuda").repeat_interleave(32) if group == 32 else torch.tensor([300.0, 0.01], device="cuda").repeat_interleave(64)
+    K, V = torch.randn((8192, 128), device="cuda", generator=g), (torch.randn((8192, 128), device="cuda", generator=g) + 1) * size
+    out, lse, ref, ref_lse = _long_ranges(bits, group, K, V, 2 * torch.randn((rows, 128), device="cuda", generator=g))
+    err = np.abs(out - ref).reshape(rows, -1, group).max(2) / np.abs(ref).reshape(rows, -1, group).max(2)
+    # weights of 22 bits at least and scores of binary32 (below 2^5: 2^-20 each), 2048 tokens a warp; one unit for all groups: 7e-3 to 0.2
+    assert err.max() <= 2e-5, err
+
+
 @pytest.mark.parametrize("bits,rows", [(2, 1), (4, 1), (2, 2), (4, 4), (3, 4)])
 def test_sums_beyond_32_bits(bits, rows):
     """A query of zeros gives every token the weight 1: a warp's byte sums pass int32 unless they are carried on the way (every 2048
