@@ -133,6 +133,7 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
     int O[8 * NT][4];
     const float up = (BITS != 4 && odd) ? 0.0625f : 1.f;             // R = 2: this lane's tokens stand in the upper contraction slots
     auto up_of = [&](int k) { return R == 4 ? ((BITS != 4 && (k & 1)) ? 0.0625f : 1.f) : up; };
+    float dither = (lane + 0.5f) * (1.f / 32) - 0.5f;
     float evf[NGv];                       // 2^ev, a value channel group's own: groups may lie far apart in size
 #pragma unroll
     for (int j = 0; j < NGv; ++j) evf[j] = pow2i(60);
@@ -201,7 +202,7 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
         for (int o = 4; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         return v;
     };
-    // Weights of a step's tokens of this lane: pw = 2^(s - ref) and x = pw * scale in units of 2^-ev, after moving the rows' references and
+    // Weights of a step's tokens of this lane: pw = 2^(s - ref) and x = pw * scale in units of 2^-ev (plus the dither), after moving the rows' references and
     // (each channel group's) units if one weight of the warp does not fit.  References are whole numbers, so that the sums so far move by
     // whole bits; a new unit puts the row's largest weight of the step into [2^PLACE, 2^(PLACE + 1)), where it is not finer than the old one: 22 bits of it also in the upper
     // slots, which take a sixteenth, and room for weights 16 (4 bit: 64) times as large.  A move costs a few hundred instructions, most of them
@@ -209,6 +210,7 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
     // four heads, 3 bit, 52.4 and 54.3 us; 16 x 8, 4 bit, 131.7 with four bits less.
     auto weights = [&](const auto &s, const auto &sv, auto &pw, auto &x) {
         constexpr int N = sizeof(pw) / sizeof(pw[0]);
+        dither = next_dither(dither);
         bool moves = false;
 #pragma unroll
         for (int k = 0; k < N; ++k) {
@@ -217,7 +219,7 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
             moves |= d > 64.f;
 #pragma unroll
             for (int j = 0; j < NGv; ++j) {
-                x[k][j] = pw[k] * (sv[k][j] * (evf[j] * up_of(k)));
+                x[k][j] = fmaf(pw[k], sv[k][j] * (evf[j] * up_of(k)), dither);
                 moves |= fabsf(x[k][j]) >= WEIGHT_LIMIT * up_of(k);
             }
         }
@@ -244,7 +246,7 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
             evf[j] = pow2i(to);
             bv[j] *= f;
 #pragma unroll
-            for (int k = 0; k < N; ++k) x[k][j] = pw[k] * (sv[k][j] * (evf[j] * up_of(k)));
+            for (int k = 0; k < N; ++k) x[k][j] = fmaf(pw[k], sv[k][j] * (evf[j] * up_of(k)), dither);
         }
     };
     // The value products of a pair: this lane's tokens' weights and parameters, and the two tiles' words.

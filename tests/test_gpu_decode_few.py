@@ -124,6 +124,26 @@ def test_value_channel_groups_of_different_size(bits, rows, group):
     assert err.max() <= 2e-5, err
 
 
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("rows", [1, 2, 4])
+def test_a_long_tail_of_small_weights(bits, rows):
+    """Each warp has one token far above 32767 others: a 2^-25th of its weight apiece (2^-20th and 2^-15th for the third and fourth row), a
+    thousandth of the output together."""
+    g = torch.Generator("cuda").manual_seed(17 * bits + rows)
+    q, key = _queries(rows, g)
+    V = torch.randn((131072, 128), device="cuda", generator=g) + 1
+    for depth in (24.5, 25.2, 26, 30):
+        K = torch.zeros_like(V)
+        K[::32768] = depth * np.log(2) * key
+        out, lse, ref, ref_lse = _long_ranges(bits, 64 if bits == 2 and rows > 2 else 128, K, V, q)
+        err = np.abs(out - ref).max(1) / np.abs(ref).max(1)
+        # scores of binary32 near 26 (2^-19 each), and binary32 sums of the weights: the lane that holds the large one (a 32nd, 16th or 8th of
+        # a row's) loses half a digit of its sum, or a whole weight, at every small one, and so do its sums of weight * scale * zero.  Weights rounded to
+        # nearest lose half of the tail, or all
+        lost = np.minimum(2.0 ** (-depth * (1 - 0.2 * np.arange(rows))), 2.0 ** -24) * 32768 * {1: 1 / 32, 2: 1 / 16, 4: 1 / 8}[rows]
+        assert (err <= 2e-5 + 2 * lost).all(), (depth, err, lost)
+
+
 @pytest.mark.parametrize("bits,rows", [(2, 1), (4, 1), (2, 2), (4, 4), (3, 4)])
 def test_sums_beyond_32_bits(bits, rows):
     """A query of zeros gives every token the weight 1: a warp's byte sums pass int32 unless they are carried on the way (every 2048
