@@ -40,7 +40,7 @@ PyObject *name[NAMES];
 
 struct Ref {      // an owned reference
     PyObject *o;
-    explicit Ref(PyObject *x) : o(x) {}
+    explicit Ref(PyObject *x = nullptr) : o(x) {}
     ~Ref() { Py_XDECREF(o); }
     Ref(const Ref &) = delete;
     Ref &operator=(const Ref &) = delete;
@@ -272,16 +272,16 @@ PyObject *quantize_append(PyObject *, PyObject *const *a, Py_ssize_t n)      // 
     END_HANDLE_TH_ERRORS
 }
 
-// out and lse (None where it is not wanted), as given or new
-bool results(PyObject *out, PyObject *lse, PyObject *want_lse, const at::Tensor &q, const kvsink_config &c, int64_t T, PyObject **o, PyObject **l)
+// out and lse (None where it is not wanted), as given or new; an allocation that throws leaves what was made before it to its owner
+bool results(PyObject *out, PyObject *lse, PyObject *want_lse, const at::Tensor &q, const kvsink_config &c, int64_t T, Ref *o, Ref *l)
 {
     const int want = lse == Py_None ? PyObject_IsTrue(want_lse) : 0;
     if (want < 0) return false;
     const int64_t shape[4] = {c.batch, c.n_q_heads, T < 0 ? (int64_t)c.head_dim : T, c.head_dim};
-    *o = result(out, q, at::IntArrayRef(shape, T < 0 ? 3 : 4), at::kFloat);
-    if (!*o) return false;
-    *l = want ? result(lse, q, at::IntArrayRef(shape, T < 0 ? 2 : 3), at::kFloat) : Py_NewRef(lse);
-    return *l != nullptr;
+    o->o = result(out, q, at::IntArrayRef(shape, T < 0 ? 3 : 4), at::kFloat);
+    if (!o->o) return false;
+    l->o = want ? result(lse, q, at::IntArrayRef(shape, T < 0 ? 2 : 3), at::kFloat) : Py_NewRef(lse);
+    return l->o != nullptr;
 }
 
 PyObject *decode_attention(PyObject *, PyObject *const *a, Py_ssize_t n)      // mode, cfg, cache, params, q, out, lse, workspace, want_lse
@@ -295,10 +295,8 @@ PyObject *decode_attention(PyObject *, PyObject *const *a, Py_ssize_t n)      //
     kvsink_cache cache;
     kvsink_static_params sp;
     if (!read_config(a[1], &c)) return nullptr;
-    PyObject *out_ = nullptr, *lse_ = nullptr;
-    const bool made = results(a[5], a[6], a[8], *q, c, -1, &out_, &lse_);
-    Ref out(out_), lse(lse_);
-    if (!made) return nullptr;
+    Ref out, lse;
+    if (!results(a[5], a[6], a[8], *q, c, -1, &out, &lse)) return nullptr;
     int64_t need = 0;
     if (a[7] == Py_None) {
         Ref sizes(PyObject_GetAttr(a[2], name[SIZES]));
@@ -337,11 +335,9 @@ PyObject *prefill_attention(PyObject *, PyObject *const *a, Py_ssize_t n)      /
     kvsink_cache cache;
     if (!read_config(a[0], &c)) return nullptr;
     const int64_t T = q->size(2), sb = q->stride(0), sh = q->stride(1), stt = q->stride(2);
-    PyObject *out_ = nullptr, *lse_ = nullptr;
-    const bool made = results(a[4], a[5], a[6], *q, c, T, &out_, &lse_);
-    Ref out(out_), lse(lse_);
+    Ref out, lse;
     void *o, *l;
-    if (!made || !address(out.o, &o) || !address(lse.o, &l) || !read_cache(a[1], &cache)) return nullptr;
+    if (!results(a[4], a[5], a[6], *q, c, T, &out, &lse) || !address(out.o, &o) || !address(lse.o, &l) || !read_cache(a[1], &cache)) return nullptr;
     const void *qp = q->data_ptr();
     void *st = stream();
     if (!done(released([&] { return f_prefill_attention(&c, &cache, qp, (int32_t)T, pos0, sb, sh, stt, (float *)o, (float *)l, st); }), "kvsink_prefill_attention")) return nullptr;

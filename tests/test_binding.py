@@ -126,3 +126,17 @@ def test_calls_take_records_results_and_errors_as_ctypes_did():
             kv.quantize_append(cfg, cache, K[:, :, :0], V[:, :, :0])
         assert refs[-1][1:] == [sys.getrefcount(x) for x in (out, lse, work, cache.k_codes, cache.sinks)]
     assert all(torch.equal(a, b) for a, b in zip(*got))
+
+
+@pytest.mark.gpu
+def test_a_result_that_cannot_be_allocated_leaves_the_other_to_its_owner():
+    cache = _cache()
+    q, out = torch.zeros((1, 8, 1, 128), device="cuda").half(), torch.zeros((1, 8, 128), device="cuda")
+    cfg = kv.Config(1 << 20, 1 << 20, 8, 128, 512, 2, 64, 256, 2, 1, (1,))      # an lse of four terabytes
+    before = sys.getrefcount(out)
+    for _ in range(5):
+        with pytest.raises(torch.OutOfMemoryError):
+            kv.decode_attention(cfg, cache, q, out)
+        with pytest.raises(torch.OutOfMemoryError):
+            kv.prefill_attention(cfg, cache, q, 0, out)
+    assert sys.getrefcount(out) == before
