@@ -10,6 +10,7 @@ import os
 import subprocess
 import sysconfig
 from concurrent.futures import ThreadPoolExecutor
+from typing import Optional
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
@@ -38,10 +39,14 @@ def _older(target: str, deps) -> bool:
 DEBUG_LIB = os.path.join(HERE, "libkvsink_debug.so")
 
 
-def build_calls(force: bool = False) -> str:
-    """_calls.so: an extension module against the headers of Python and the installed torch."""
+def build_calls(force: bool = False) -> Optional[str]:
+    """_calls.so: an extension module against the headers of Python and the installed torch.  None, with a message, where torch has no CUDA: the
+    library needs no torch, and there is no device for the calls."""
+    import torch
+    if torch.version.cuda is None:
+        print("torch was built without CUDA: _calls.so is left out", flush=True)
+        return None
     if force or _older(CALLS, [CALLS_SOURCE, HEADER]):
-        import torch
         at = os.path.dirname(torch.__file__)
         cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
         include = [sysconfig.get_paths()["include"], os.path.join(cuda, "include"), os.path.join(at, "include"),

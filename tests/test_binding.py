@@ -8,7 +8,7 @@ import pytest
 import torch
 
 import paper_2508_04257_b200 as kv
-from paper_2508_04257_b200 import binding
+from paper_2508_04257_b200 import binding, build
 
 
 def _cache():
@@ -140,3 +140,9 @@ def test_a_result_that_cannot_be_allocated_leaves_the_other_to_its_owner():
         with pytest.raises(torch.OutOfMemoryError):
             kv.prefill_attention(cfg, cache, q, 0, out)
     assert sys.getrefcount(out) == before
+
+
+def test_a_torch_without_cuda_builds_the_library_alone(monkeypatch, capsys):
+    monkeypatch.setattr(torch.version, "cuda", None)
+    monkeypatch.setattr(build.subprocess, "run", lambda *a, **k: pytest.fail("nothing to compile"))
+    assert build.build_calls(force=True) is None and "without CUDA" in capsys.readouterr().out
