@@ -96,10 +96,13 @@ _calls = None
 
 
 def _native():
-    """Loads _calls.so and gives it the library's entry points; raises if it has not been built."""
+    """Loads _calls.so and gives it the library's entry points; raises if it has not been built, or for another torch or Python."""
     global _calls
     if _calls is None:
         from . import _calls as module
+        from .build import calls_abi
+        if module.abi != calls_abi():
+            raise ImportError(f"_calls.so was built for {module.abi}, this is {calls_abi()}: build it with `python -m paper_2508_04257_b200.build`")
         module.bind({n: C.cast(getattr(lib(), n), C.c_void_p).value for n in EXPORTS}, Config, KVCache, StaticParams, KvsinkError)
         _calls = module
     return _calls

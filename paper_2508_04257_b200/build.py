@@ -39,26 +39,37 @@ def _older(target: str, deps) -> bool:
 DEBUG_LIB = os.path.join(HERE, "libkvsink_debug.so")
 
 
+def calls_abi() -> str:
+    """What _calls.so is tied to: the torch and the Python that it is built for."""
+    import torch
+    return f"torch {torch.__version__}, {sysconfig.get_config_var('SOABI')}"
+
+
 def build_calls(force: bool = False) -> Optional[str]:
-    """_calls.so: an extension module against the headers of Python and the installed torch.  None, with a message, where torch has no CUDA: the
-    library needs no torch, and there is no device for the calls."""
+    """_calls.so: an extension module against the headers of Python and the installed torch, built anew when either is another one.  None, with
+    a message, where torch has no CUDA: the library needs no torch, and there is no device for the calls."""
     import torch
     if torch.version.cuda is None:
         print("torch was built without CUDA: _calls.so is left out", flush=True)
         return None
-    if force or _older(CALLS, [CALLS_SOURCE, HEADER]):
+    built_for = os.path.join(OBJ, "calls_abi.txt")
+    stale = force or _older(CALLS, [CALLS_SOURCE, HEADER]) or not os.path.exists(built_for) or open(built_for).read() != calls_abi()
+    if stale:
         at = os.path.dirname(torch.__file__)
         cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
         include = [sysconfig.get_paths()["include"], os.path.join(cuda, "include"), os.path.join(at, "include"),
                    os.path.join(at, "include", "torch", "csrc", "api", "include")]
-        abi = f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"
-        cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", abi] + [f"-I{d}" for d in include] + \
+        defines = [f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", f'-DKVSINK_CALLS_ABI="{calls_abi()}"']
+        cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden"] + defines + [f"-I{d}" for d in include] + \
               [CALLS_SOURCE, "-o", CALLS, "-L" + os.path.join(at, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             if os.path.exists(CALLS):
                 os.remove(CALLS)
             raise RuntimeError(f"g++ failed on calls.cpp\n{r.stderr[-4000:]}")
+        os.makedirs(OBJ, exist_ok=True)
+        with open(built_for, "w") as out:
+            out.write(calls_abi())
     return CALLS
 
 

@@ -383,5 +383,10 @@ PyMODINIT_FUNC PyInit__calls(void)
 {
     for (int i = 0; i < NAMES; ++i)
         if (!(name[i] = PyUnicode_InternFromString(NAME[i]))) return nullptr;
-    return PyModule_Create(&module);
+    PyObject *m = PyModule_Create(&module);
+    if (m && PyModule_AddStringConstant(m, "abi", KVSINK_CALLS_ABI)) {      // what it was built for, compared by binding.py
+        Py_DECREF(m);
+        return nullptr;
+    }
+    return m;
 }

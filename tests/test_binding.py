@@ -146,3 +146,28 @@ def test_a_torch_without_cuda_builds_the_library_alone(monkeypatch, capsys):
     monkeypatch.setattr(torch.version, "cuda", None)
     monkeypatch.setattr(build.subprocess, "run", lambda *a, **k: pytest.fail("nothing to compile"))
     assert build.build_calls(force=True) is None and "without CUDA" in capsys.readouterr().out
+
+
+def test_the_calls_are_built_anew_for_another_torch_or_python(monkeypatch, tmp_path):
+    compiled = []
+
+    def run(cmd, **kw):
+        compiled.append([a for a in cmd if a.startswith("-DKVSINK_CALLS_ABI=")])
+        (tmp_path / "_calls.so").write_bytes(b"")
+        return subprocess.CompletedProcess(cmd, 0, "", "")
+
+    monkeypatch.setattr(build, "CALLS", str(tmp_path / "_calls.so"))
+    monkeypatch.setattr(build, "OBJ", str(tmp_path / "objects"))
+    monkeypatch.setattr(build.subprocess, "run", run)
+    for abi, builds in (("one", 1), ("one", 1), ("two", 2), ("two", 2)):
+        monkeypatch.setattr(build, "calls_abi", lambda: abi)
+        build.build_calls()
+        assert len(compiled) == builds and compiled[-1] == [f'-DKVSINK_CALLS_ABI="{abi}"']
+
+
+def test_calls_of_another_torch_are_refused(monkeypatch):
+    assert binding._native().abi == build.calls_abi()
+    monkeypatch.setattr(binding, "_calls", None)
+    monkeypatch.setattr(build, "calls_abi", lambda: "another")
+    with pytest.raises(ImportError, match="another"):
+        kv.predict_sinks(None, None, None)
