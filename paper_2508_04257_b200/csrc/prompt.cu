@@ -38,7 +38,8 @@ constexpr int PR_HDRS = 8;
 // A zero point up to this size is subtracted from the code in fp16 exactly; farther ones go through an additive term.
 constexpr float PR_NEAR = 1000.f;
 constexpr uint32_t PR_WAIT_NS = 20000;          // a poll sleeps up to this long (without the hint it comes back after some 60 clocks)
-constexpr int PR_WAIT_POLLS = 1 << 16;          // 1.3 s of such polls: far beyond any real wait
+constexpr long long PR_WAIT_CLOCKS = 1ll << 29; // 0.27 s at the highest clock, at least: far beyond any real wait
+constexpr unsigned PR_WAIT_LOOK = 256;               // polls between two looks at the clock, at most 5 ms
 constexpr int PR_ROWS_KEPT = 8;                 // sink rows of a step that the parameter warps leave in shared memory
 
 struct StepHeader {
@@ -88,13 +89,19 @@ __device__ __forceinline__ void bar_arrive(uint64_t *bar)
 __device__ __forceinline__ bool bar_wait_warp(uint64_t *bar, unsigned parity, int *failed)
 {
     const uint32_t a = smem_addr(bar);
+    long long start = 0;
 #pragma unroll 1
-    for (int polls = 0; polls < PR_WAIT_POLLS; ++polls) {
+    for (unsigned polls = 1;; ++polls) {
         unsigned ok;
         asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3; selp.u32 %0, 1, 0, p; }"
                      : "=r"(ok) : "r"(a), "r"(parity), "r"(PR_WAIT_NS) : "memory");
         if (__all_sync(0xffffffffu, ok != 0)) return true;
         if (__any_sync(0xffffffffu, *(volatile int *)failed)) break;
+        if (polls % PR_WAIT_LOOK == 0) {
+            const long long now = clock64();
+            if (polls == PR_WAIT_LOOK) start = now;
+            else if (__any_sync(0xffffffffu, now - start > PR_WAIT_CLOCKS)) break;
+        }
     }
     *(volatile int *)failed = 1;
     return false;
