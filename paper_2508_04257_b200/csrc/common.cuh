@@ -215,8 +215,8 @@ int launch_decode_b4(const Params &p, const kvsink_cache &c, const kvsink_static
 int launch_decode_merge(const float *ws, int nsplit, int D, int n_rows, float *out, float *lse, cudaStream_t st);
 // Query heads of one KV head that one decode block serves, and the blocks per KV head that makes.  Up to four heads share a
 // block.  Five to eight share one where a path with eight columns exists: the integer key side with two operand tables (2 and
-// 4 bit, head size 128) or the eight-column fp16 path (head size 64); at 3 bit with head size 128 they go four at a time to
-// the fp16 pair layout, whose residual columns the eight-column fp16 path lacks.
+// 4 bit, head size 128) or the eight-column fp16 path (head size 64); at 3 bit with head size 128 they go four at a time
+// (decode_few.cuh).
 inline int decode_heads_per_block(const Params &p) { return p.rep <= 4 ? 4 : (p.D == 128 && p.bits == 3 ? 4 : 8); }
 inline int decode_qchunks(const Params &p) { return (p.rep + decode_heads_per_block(p) - 1) / decode_heads_per_block(p); }
 int max_splits(const Params &p);

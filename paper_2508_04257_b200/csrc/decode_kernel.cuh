@@ -183,7 +183,7 @@ struct Count { static constexpr int value = N; };
 constexpr int DEC_WAIT_LIMIT = 1 << 22;   // polls of a full-barrier before a warp gives up (far beyond any real latency)
 
 // Shared-memory plan of a decode block, shared by the kernel and the launcher.  CT = tiles per ring chunk, NQMAX = the
-// most query heads a block of this instantiation serves (1 on the integer key side, 4 with the pair layout, else 8).
+// most query heads a block of this instantiation serves (1 in decode_one.cuh, 2 or 4 in decode_few.cuh, here 4 with the pair layout, else 8).
 template <int BITS, int D, int NGv, int CT, int NQMAX, bool KTOK = false>
 struct DecodePlan {
     static constexpr int W = D * BITS / 64, TILE_BYTES = 128 * W;
@@ -203,7 +203,7 @@ struct DecodePlan {
     static constexpr int BYTES = FIXED + (RING > PART ? RING : PART);
 };
 
-// PL ("pair layout", for at most four query heads per KV head): query head h owns accumulator columns 2h and 2h+1;
+// PL ("pair layout", for at most four query heads per KV head; head size 64, and I8 = 2): query head h owns accumulator columns 2h and 2h+1;
 // column 2h multiplies by the fp16 factor q*scale and column 2h+1 by its fp16 rounding residual, so every score carries
 // the factor to ~22 bits at no extra instruction.  Without PL (five to eight heads) head h owns column h and the
 // residual of channels with large factors goes through a second multiply.
@@ -214,7 +214,7 @@ struct DecodePlan {
 // g + 8, x16 for the upper contraction slots, x64 for both).  4 bit: a word masked with 0x0f.. and 0xf0.. gives the registers of
 // rows g and g + 8 (x16), two words (two matrices) make one fragment.  The B operand holds the factor q * scale * 2^sh of each
 // channel as four signed bytes (2 bit: divided by 16 beforehand for the upper slots); sums are exact in int32.
-// I8 = 2 (two to four query heads per KV head, 2 and 4 bit): two B operands per word, which hold the upper and the lower byte pair
+// I8 = 2 (three and four query heads per KV head, 2 bit, one channel group a row): two B operands per word, which hold the upper and the lower byte pair
 // of every head's factors in the pair layout's columns.
 // I8 = 3 (five to eight rows: query heads, or the rows of a block of prompt queries; 2 and 4 bit): two operand tables of the
 // I8 = 2 kind, one for the even rows and one for the odd rows, multiplied with the same masked words, so that lane t finds
@@ -225,10 +225,10 @@ struct DecodePlan {
 // token.  There are no token groups: the key B operand is prepared once per block, a ring chunk holds code words only, the
 // stream covers every tile up to the sequence length (tokens beyond it are masked) and there is no fp16 tail.
 //
-// KT (per-token keys, PM = 2): keys carry one (scale, zero) per token and channel group like the values, so the key B operand
-// holds the query alone (prepared once per block) and a token's parameters are applied to its dot products afterwards:
-// score = sum over channel groups j of scale[t][j] * (dot_j - zero[t][j] * sum of the query over group j).  The parameters
-// of a chunk's tokens arrive with the chunk.  Like CAL there are no token groups and no tail.  Integer key side only.
+// KT (per-token keys, PM = 2): keys carry one (scale, zero) per token like the values, so the key B operand holds the query alone
+// (prepared once per block) and a token's parameters are applied to its dot product afterwards: score = scale[t] * (dot - zero[t] *
+// sum of the query).  The parameters of a chunk's tokens arrive with the chunk.  Like CAL there are no token groups and no tail.
+// Integer key side only.
 //
 // PRE (attention of a chunk of prompt queries over the cache, Algorithm 1's attention statement): the eight accumulator
 // columns of a block are eight (query token, query head) rows of one KV head, token-major; query token t sits at position
@@ -258,10 +258,11 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
 
     const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), g = lane >> 2, t = lane & 3;
     constexpr bool CAL = PM == 1, KT = PM == 2, FLAT = PM != 0;    // static parameters / per-token keys / either: no token groups
-    constexpr int NGK = KT ? NGv : 1;                              // separate dot products per tile on the key side
     static_assert(!PRE || (!PL && (I8 == 0 || I8 == 3) && !FLAT), "prompt queries take an eight-column path");
     static_assert(I8 != 3 || (!PL && !KT && D == 128 && BITS != 3), "eight rows on the integer key side: 2 and 4 bit, head size 128");
-    static_assert(!KT || (I8 != 0 && NGv <= 2 && (BITS != 3 || NGv == 1)), "per-token keys: integer key side, one or two channel groups");
+    static_assert(I8 != 2 || (PL && BITS == 2 && D == 128 && NGv == 1), "up to four heads on the integer key side: 2 bit, one channel group");
+    static_assert(!KT || I8 == 2, "per-token keys: the integer key side of up to four heads");
+    static_assert(!PL || I8 == 2 || D == 64, "pair layout of the fp16 key side: head size 64");
     // decode: grid (splits, KV heads x blocks of eight query heads, sequences); prompt queries: grid (row blocks, KV heads, sequences)
     const int split = PRE ? 0 : blockIdx.x, h = PRE ? blockIdx.y : blockIdx.y / qchunks, qc = PRE ? blockIdx.x : blockIdx.y % qchunks, b = blockIdx.z;
     const int nq = PRE ? min(NQMAX, pre.T * p.rep - 8 * qc) : min(NQMAX, p.rep - NQMAX * qc), hq0 = h * p.rep + (PRE ? 0 : NQMAX * qc);
@@ -515,9 +516,8 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
     constexpr int PS = D + 2;                                        // partial record: o[D], m, l
 
     // Integer key side: lane l prepares the B operand bytes of one group of four contraction slots, (MMA l/8, lower or
-    // upper slots (l/4)%2, slots 4(l%4) ... +3); these are its four channels and their query values.
+    // upper slots (l/4)%2, slots 4(l%4) ... +3); these are its four channels.
     int i8_ch[4] = {0, 0, 0, 0};
-    float i8_q[4] = {0.f, 0.f, 0.f, 0.f};
     if constexpr (I8) {
         const int mi = lane >> 3, c2 = (lane >> 2) & 1, tq = lane & 3;
 #pragma unroll
@@ -658,14 +658,9 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
                         const uint32_t t2 = __byte_perm(d[2], d[3], 0x5140), t3 = __byte_perm(d[2], d[3], 0x7362);
                         w3 = __byte_perm(t1, t3, 0x7632); w2 = __byte_perm(t1, t3, 0x5410);
                         w1 = __byte_perm(t0, t2, 0x7632); w0 = __byte_perm(t0, t2, 0x5410);
-                        if constexpr (KT && NGv == 2) {
-                            const float b0s = warp_sum(lane < 16 ? bsum : 0.f), b1s = warp_sum(lane < 16 ? 0.f : bsum);
-                            if (t == hh) { bias0 = b0s; bias1 = b1s; ks0 = pow2i(-sh); }
-                        } else {
-                            bsum = warp_sum(bsum);
-                            if (t == hh) {
-                                if (set == 0) { bias0 = bsum; ks0 = pow2i(-sh); } else { bias1 = bsum; ks1 = pow2i(-sh); }
-                            }
+                        bsum = warp_sum(bsum);
+                        if (t == hh) {
+                            if (set == 0) { bias0 = bsum; ks0 = pow2i(-sh); } else { bias1 = bsum; ks1 = pow2i(-sh); }
                         }
                     }
                     tab[(2 * hh) * 4] = w3;
@@ -783,13 +778,8 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
 
             // per-token keys: (scale, zero) of the chunk's tokens, token-major, delivered with the chunk
             const float *kts = ssv0 + 2 * (SZ_BYTES / 4) + sub * ST * 16 * NGv, *ktz = kts + SZ_BYTES / 4;
-            // score of a token from its group dot products d[j] (already in query units): sum_j scale_j * (d_j - zero_j * qsum_j)
-            auto token_score = [&](const float (&d)[NGK], int tok) {
-                float r = 0.f;
-#pragma unroll
-                for (int j = 0; j < NGK; ++j) r = fmaf(kts[tok * NGv + j], fmaf(-ktz[tok * NGv + j], j == 0 ? bias0 : bias1, d[j]), r);
-                return r;
-            };
+            // score of a token from its dot product d (already in query units): scale * (d - zero * sum of the query)
+            auto token_score = [&](float d, int tok) { return kts[tok] * fmaf(-ktz[tok], bias0, d); };
             // scores of the chunk's tiles
             float s[ST][4];
 #pragma unroll
@@ -797,17 +787,11 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
                 if constexpr (I8 >= 2) {
                     uint32_t kw[W];
                     load_tile_shared<BITS, D>(kt + k * TILE_WORDS, lane, kw);
-                    // upper / lower byte pair of the heads' sums; per-token keys: one set per channel group (MMA i covers
-                    // channels 32 i ... 32 i + 31)
-                    int ia[NGK][4], ib[NGK][4];
+                    // upper / lower byte pair of the heads' sums
+                    int ia[4] = {0, 0, 0, 0}, ib[4] = {0, 0, 0, 0};
                     int ic[4] = {0, 0, 0, 0}, id[4] = {0, 0, 0, 0};   // I8 = 3: the same for the odd rows
 #pragma unroll
-                    for (int j = 0; j < NGK; ++j)
-#pragma unroll
-                        for (int x = 0; x < 4; ++x) ia[j][x] = ib[j][x] = 0;
-#pragma unroll
                     for (int i = 0; i < 4; ++i) {
-                        const int jg = NGK == 2 ? (i >> 1) : 0;
                         uint32_t a0, a1, a2, a3;
                         if constexpr (BITS != 4) {
                             const uint32_t x = kw[i];
@@ -817,10 +801,10 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
                             a0 = x & 0x0f0f0f0fu; a1 = x & 0xf0f0f0f0u; a2 = y & 0x0f0f0f0fu; a3 = y & 0xf0f0f0f0u;
                         }
                         asm volatile("mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                                     : "+r"(ia[jg][0]), "+r"(ia[jg][1]), "+r"(ia[jg][2]), "+r"(ia[jg][3])
+                                     : "+r"(ia[0]), "+r"(ia[1]), "+r"(ia[2]), "+r"(ia[3])
                                      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(bk[i][0]), "r"(bk[i][1]));
                         asm volatile("mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                                     : "+r"(ib[jg][0]), "+r"(ib[jg][1]), "+r"(ib[jg][2]), "+r"(ib[jg][3])
+                                     : "+r"(ib[0]), "+r"(ib[1]), "+r"(ib[2]), "+r"(ib[3])
                                      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(bk[4 + i][0]), "r"(bk[4 + i][1]));
                         if constexpr (I8 == 3) {   // the odd rows' operands from the second table, the same masked words
                             const uint32_t *e0 = reinterpret_cast<const uint32_t *>(Bs) + 512 + (i * 2) * 64 + g * 4 + t;
@@ -834,26 +818,20 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
                         }
                     }
                     // lane t holds head t: bytes 3, 2 of its sum in the first accumulators, bytes 1, 0 in the second
-                    float tg[NGK], th[NGK];
-#pragma unroll
-                    for (int j = 0; j < NGK; ++j) {
-                        tg[j] = fmaf(fmaf((float)ia[j][0], 256.f, (float)ia[j][1]), 65536.f, fmaf((float)ib[j][0], 256.f, (float)ib[j][1]));
-                        th[j] = fmaf(fmaf((float)ia[j][2], 256.f, (float)ia[j][3]), 65536.f, fmaf((float)ib[j][2], 256.f, (float)ib[j][3]));
-                    }
+                    const float tg = fmaf(fmaf((float)ia[0], 256.f, (float)ia[1]), 65536.f, fmaf((float)ib[0], 256.f, (float)ib[1]));
+                    const float th = fmaf(fmaf((float)ia[2], 256.f, (float)ia[3]), 65536.f, fmaf((float)ib[2], 256.f, (float)ib[3]));
                     if constexpr (KT) {
-#pragma unroll
-                        for (int j = 0; j < NGK; ++j) { tg[j] *= ks0; th[j] *= ks0 * (BITS == 4 ? 0.0625f : 0.25f); }
-                        s[k][0] = token_score(tg, k * 16 + g); s[k][1] = -INFINITY;
-                        s[k][2] = token_score(th, k * 16 + g + 8); s[k][3] = -INFINITY;
+                        s[k][0] = token_score(tg * ks0, k * 16 + g); s[k][1] = -INFINITY;
+                        s[k][2] = token_score(th * (ks0 * 0.25f), k * 16 + g + 8); s[k][3] = -INFINITY;
                     } else if constexpr (I8 == 3) {   // rows 2t (even table) and 2t + 1 (odd table): this lane's two columns
                         const float ug = fmaf(fmaf((float)ic[0], 256.f, (float)ic[1]), 65536.f, fmaf((float)id[0], 256.f, (float)id[1]));
                         const float uh = fmaf(fmaf((float)ic[2], 256.f, (float)ic[3]), 65536.f, fmaf((float)id[2], 256.f, (float)id[3]));
-                        s[k][0] = fmaf(tg[0], ks0, -bias0); s[k][1] = fmaf(ug, ks1, -bias1);
-                        s[k][2] = fmaf(th[0], ks0 * (BITS == 4 ? 0.0625f : 0.25f), -bias0);
+                        s[k][0] = fmaf(tg, ks0, -bias0); s[k][1] = fmaf(ug, ks1, -bias1);
+                        s[k][2] = fmaf(th, ks0 * (BITS == 4 ? 0.0625f : 0.25f), -bias0);
                         s[k][3] = fmaf(uh, ks1 * (BITS == 4 ? 0.0625f : 0.25f), -bias1);
                     } else {
-                        s[k][0] = fmaf(tg[0], ks0, -bias0); s[k][1] = -INFINITY;
-                        s[k][2] = fmaf(th[0], ks0 * (BITS == 4 ? 0.0625f : 0.25f), -bias0); s[k][3] = -INFINITY;
+                        s[k][0] = fmaf(tg, ks0, -bias0); s[k][1] = -INFINITY;
+                        s[k][2] = fmaf(th, ks0 * (BITS == 4 ? 0.0625f : 0.25f), -bias0); s[k][3] = -INFINITY;
                     }
                     continue;
                 }
