@@ -30,14 +30,18 @@ static int launch_decode_p(const Params &p, const kvsink_cache &c, const kvsink_
     pdl[0].val.programmaticStreamSerializationAllowed = 1;
     // up to eight splits (the portable cluster size): the splits of a unit are launched as one thread-block cluster and
     // merged inside the kernel through distributed shared memory, which saves the merge kernel's 2 to 3 us.  A cluster has to be placed
-    // as a whole, though, and a grid that nearly fills the chip's 592 slots does not fit in one round any more (decode alone,
-    // clusters and none: sixes, 576 blocks, 3 x 32 units of 4000 tokens 20.3 and 14.4 us, of 12000 40.7 and 28.1; fours, 576 blocks, 18 x 8 of 9000
-    // 54 and 40; fours and eights, 512 blocks, 4 x 32 of 2048 9.8 and 10.7, 8 x 8 of 4096 with four heads 14.9 and 16.2, 4 bit 17.6 and 19.0,
-    // 16 x 8 of 30000 99.2 and 100.4).  Pairs, whose second block finds room anywhere, lose beyond a round only (20 x 32 of 3000 44.9 and 39.8;
+    // as a whole, though: where blocks by themselves would be three an SM some SMs get four, and what nearly fills the chip's 592 slots does
+    // not fit in one round any more.  Decode alone, clusters and none, us: eights, 320 blocks, 40 units of 8000 tokens, 2 bit, 13.6 and 12.4;
+    // sixes, 432, 72 of 6000, 15.7 and 13.9; fours, 384, 96 of 4000, 3 bit, 17.8 and 16.2, 96 of 8000, 4 bit, 35.9 and 26.1; 448, 112 of 16000, 2 bit,
+    // 31.9 and 31.0; sixes, 576, 3 x 32 units of 4000, 20.3 and 14.4, 96 of 3000, 3 bit, 19.7 and 14.8; threes, 576, 192 of 1500, 3 bit,
+    // 19.0 and 14.4.  512 blocks leave no SM more than it would have: eights, 64 units of 8000, four heads, 2 bit, 21.1 and 23.2, fours, 128 of 4000,
+    // 3 bit, 19.6 and 20.2, 128 of 8000, four heads, 4 bit, 45.0 and 46.3; 480 are even (threes, 160 of 3000, 3 bit, 19.1 and 19.3; sixes, 80 of
+    // 6000, 2 bit, 15.8 and 15.1, with four heads 23.1 and 24.5).  Up to 296 blocks clusters stay.
+    // Pairs, whose second block finds room anywhere, lose beyond a round only (20 x 32 of 3000 44.9 and 39.8;
     // 592 blocks, 37 x 8 of 9000, 66.5 and 67.6); at 3 bit up to some 256 KB a block (16 x 32 of 8192, 384 KB a block, 137 and 136).
     const int64_t blocks = (int64_t)nsplit * p.Hkv * qchunks * p.B;
     const int64_t block_bytes = (int64_t)gps * (PM != 0 ? CT * KVSINK_TILE : p.G) * 2 * p.row_bytes;
-    bool cluster_merge = nsplit > 1 && nsplit <= 8 && (nsplit == 2 ? blocks <= 4 * 148 && (p.bits != 3 || block_bytes < 256 * 1024) : blocks <= 512);
+    bool cluster_merge = nsplit > 1 && nsplit <= 8 && (nsplit == 2 ? blocks <= 4 * 148 && (p.bits != 3 || block_bytes < 256 * 1024) : blocks <= 2 * 148 || (blocks > 480 && blocks <= 512));
     // up to 48 KB need no leave, which costs a call
     if (smem > 48 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return KVSINK_ERR_CUDA;
     for (;;) {
