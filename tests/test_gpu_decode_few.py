@@ -41,28 +41,6 @@ def test_odd_lengths_and_groups(bits, rows, group, seq):
     assert np.abs(lse - ref_lse).max() <= 2e-3 + 1e-3 * np.abs(ref_lse).max()
 
 
-@pytest.mark.parametrize("bits", [2, 3, 4])
-@pytest.mark.parametrize("rows", [1, 2, 4])
-@pytest.mark.parametrize("rising", [True, False])
-def test_weights_that_move_the_unit(bits, rows, rising):
-    """Scores that climb (or fall) by 30 along the sequence and value rows between 2^-8 and 2^8: the reference and the unit of the weights
-    move in most steps, or the first step's stays too large for the rest."""
-    wl = _workload(bits, 64, 1000, rows)
-    H = synth.make_hidden(wl, "cuda")
-    g = torch.Generator("cuda").manual_seed(bits)
-    q = torch.randn((2, 3, 128), device="cuda", generator=g).half()
-    K = 0.1 * torch.randn((2, 3, 1000, 128), device="cuda", generator=g)
-    along = torch.linspace(0, 30, 1000, device="cuda") * 128 ** 0.5
-    K += (along if rising else along.flip(0))[:, None] * (q.float() / q.float().pow(2).sum(-1, keepdim=True))[:, :, None]
-    # the other rows of a KV head climb at other rates, or fall
-    q = torch.stack([q * (1 - 0.7 * r) for r in range(rows)], 2).reshape(2, 3 * rows, 128).contiguous()
-    V = torch.randn((2, 3, 1000, 128), device="cuda", generator=g) * 2.0 ** (16 * torch.rand((2, 3, 1000, 1), device="cuda", generator=g) - 8)
-    out, lse, (ref, ref_lse) = _both(wl, H, K.half(), V.half(), q)
-    # the outputs are as large as the loudest rows near the top score: the tolerance goes with them
-    assert np.abs(out - ref).max() <= (2e-3 + 1e-2) * np.abs(ref).max()
-    assert np.abs(lse - ref_lse).max() <= 2e-3 + 1e-3 * np.abs(ref_lse).max()
-
-
 UNITS = 592      # as many units as the chip has slots: one split, whose four warps take a quarter of the sequence each
 
 
@@ -92,6 +70,40 @@ def _queries(rows, g):
     """Queries of one direction, each a fifth shorter than the one before, and what a key is made of so that the first one's score is 1."""
     q = torch.randn(128, device="cuda", generator=g).half().float()
     return torch.stack([q * (1 - 0.2 * r) for r in range(rows)]).half(), q * (128 ** 0.5 / q.pow(2).sum())
+
+
+def _moves(score, size, room):
+    """Steps of 32 tokens in which a warp's largest weight (score in bits, value row of `size`) has outgrown its unit: the fewest of the four warps."""
+    logs = (score + torch.log2(size)).reshape(4, -1, 32).amax(2).tolist()
+    count = []
+    for steps in logs:
+        placed, n = steps[0], 0
+        for w in steps:
+            if w > placed + room:
+                placed, n = w, n + 1
+        count.append(n)
+    return min(count)
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("rows", [1, 2, 4])
+@pytest.mark.parametrize("scores,values", [("rise", "any"), ("rise", "fall"), ("fall", "any")])
+def test_weights_that_move_the_unit(bits, rows, scores, values):
+    """Scores that climb (or fall) by 300 along the sequence, over 100 bits in a warp's range of 64 steps, value rows between 2^-8 and 2^8: the
+    reference and the units of the weights move in most steps, or those of the first step stay too large for the rest."""
+    seq, g = 8192, torch.Generator("cuda").manual_seed(bits)
+    q, key = _queries(rows, g)
+    along = torch.linspace(0, 1, seq, device="cuda")
+    score = 300 * (along if scores == "rise" else along.flip(0))
+    size = 2.0 ** (8 - 16 * along if values == "fall" else 16 * torch.rand(seq, device="cuda", generator=g) - 8)
+    room = 7 if bits == 4 and rows > 1 else 5      # bits that a weight may grow by before a move is certain
+    moves = _moves(score / np.log(2), size, room)
+    assert moves >= 10 if scores == "rise" else moves <= 5
+    K = 0.1 * torch.randn((seq, 128), device="cuda", generator=g) + score[:, None] * key
+    out, lse, ref, ref_lse = _long_ranges(bits, 64, K, torch.randn((seq, 128), device="cuda", generator=g) * size[:, None], q)
+    # scores of binary32 near 433, and of sums of 128 such products: 2^-14 at worst
+    assert (np.abs(out - ref).max(1) <= 2e-4 * np.abs(ref).max(1)).all()
+    assert np.abs(lse - ref_lse).max() <= 1e-5 * np.abs(ref_lse).max()
 
 
 # jump in nats, length of the row: the reference moves by 48 to 173 bits at once, the largest weight by up to 8 more
@@ -144,28 +156,20 @@ def test_a_long_tail_of_small_weights(bits, rows):
         assert (err <= 2e-5 + 2 * lost).all(), (depth, err, lost)
 
 
-@pytest.mark.parametrize("bits,rows", [(2, 1), (4, 1), (2, 2), (4, 4), (3, 4)])
-def test_sums_beyond_32_bits(bits, rows):
-    """A query of zeros gives every token the weight 1: a warp's byte sums pass int32 unless they are carried on the way (every 2048
-    tiles; 592 units leave one split, whose four warps take 2112 tiles each).  All units hold one unit's cache."""
-    units, seq = 592, 4 * 2112 * 16
-    one = kv.Config(1, rows, 1, 128, 512, bits, 128, seq, 2, 1, (1,))
-    many = kv.Config(1, rows * units, units, 128, 512, bits, 128, seq, 2, 1, (1,))
-    g = torch.Generator("cuda").manual_seed(7)
-    K, V = (torch.randn((1, 1, seq, 128), device="cuda", generator=g).half() for _ in range(2))
-    V += 3                                                     # most values of a row near its middle, all far from zero
-    H = torch.randn((1, seq, 512), device="cuda", generator=g).half()
-    sinks = kv.predict_sinks(one, H, kv.SinkSet(one))
-    small = kv.KVCache(one, sinks)
-    kv.quantize_append(one, small, K, V)
-    big = copy.copy(small)
-    big.cfg, big.sizes = many, kv.cache_sizes(many)
-    for name in ("k_codes", "v_codes", "k_scale", "k_zero", "v_scale", "v_zero", "k_tail", "sink_k", "sink_v"):
-        setattr(big, name, getattr(small, name).repeat(units))
-    out, lse = kv.decode_attention(many, big, torch.zeros((1, rows * units, 128), device="cuda", dtype=torch.float16))
-    ref, ref_lse = kv.decode_attention(one, small, torch.zeros((1, rows, 128), device="cuda", dtype=torch.float16))     # short ranges: many splits
-    assert kv.read_status(small) == 0
-    assert torch.equal(out, out[:, :rows].repeat(1, units, 1)) and abs(lse[0, 0].item() - np.log(seq)) < 1e-4
-    # the same 32-bit arithmetic in another order: 135168 terms, each side within n * 2^-24 of the sum at worst, some 2^-20 of it in earnest
-    assert (out[0, 0] - ref[0, 0]).abs().max() <= 2.0 ** -18 * ref.abs().max()
-    assert (ref[0, 0] - V.float().mean((0, 1, 2))).abs().max() < 0.05
+@pytest.mark.parametrize("rows,place", [(1, 28), (2, 24), (4, 24)])
+def test_sums_beyond_32_bits(rows, place):
+    """4 bit, all tokens weigh the same, just below the largest weight that fits, and some channels have the largest code in every token: their
+    sums of bytes pass int32 unless they are carried, or added up in binary32, on the way (every 2048 tiles), and those of the top byte are
+    beyond 2^29 by then.  The unit comes from a warp's first tokens, whose value rows are smaller (it puts the largest weight to 2^place).
+    Codes of 2 and 3 bit add a twentieth as much: no cache is long enough."""
+    tiles, weight = 4800, 1.98
+    seq, g = 4 * tiles * 16, torch.Generator("cuda").manual_seed(7)
+    a_tile = 16 * 15 * 16 * (int(weight * 2 ** 30) >> 24)      # tokens, code, place of the field in a byte of channels 8 to 15, top byte of the weight
+    assert a_tile * (tiles - 4) > 2 ** 31 and 2 ** 31 > a_tile * 2048 > 2 ** 29
+    codes = torch.randint(0, 16, (seq, 128), device="cuda", generator=g).float()
+    codes[:, ::16], codes[:, 9::16] = 0, 15
+    size = torch.full((4, seq // 4, 1), weight, device="cuda")
+    size[:, :64] = 2.0 ** (place - 30)
+    out, lse, ref, ref_lse = _long_ranges(4, 128, torch.zeros_like(codes), codes * size.reshape(seq, 1), torch.zeros((rows, 128), device="cuda"))
+    # equal weights: what is left is the rounding of binary32 sums over 2400 tokens a lane
+    assert np.abs(out - ref).max() <= 1e-5 * np.abs(ref).max() and np.abs(lse - np.log(seq)).max() < 1e-4
