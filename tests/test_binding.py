@@ -71,10 +71,10 @@ def test_work_goes_to_the_current_stream(raw, monkeypatch):
         assert binding._stream() == side.cuda_stream != 0
 
 
-@pytest.mark.parametrize("bad", ["device", "strides", "type"])
+@pytest.mark.parametrize("bad", ["device", pytest.param("strides", marks=pytest.mark.gpu), pytest.param("type", marks=pytest.mark.gpu)])
 def test_inputs_that_the_calls_refuse(bad):
     cache = _cache()
-    k = torch.zeros((1, 8, 2, 128), dtype=torch.float32 if bad == "type" else torch.float16)
+    k = torch.zeros((1, 8, 2, 128), dtype=torch.float32 if bad == "type" else torch.float16, device="cpu" if bad == "device" else "cuda")
     k = k.transpose(2, 3) if bad == "strides" else k
     with pytest.raises(AssertionError):
         kv.quantize_append(cache.cfg, cache, k, k)
@@ -87,6 +87,45 @@ def test_inputs_that_the_calls_refuse(bad):
     with pytest.raises(AttributeError):
         kv.decode_attention(cache.cfg, cache, None)
     assert cache.seq_len == 0
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("bad", ["shape", "strides", "type"])
+def test_values_unlike_the_keys_are_refused(bad):
+    cache = _cache()
+    k = torch.zeros((1, 8, 4, 128), dtype=torch.float16, device="cuda")
+    v = {"shape": k[:, :, :2], "strides": torch.zeros((1, 4, 8, 128), dtype=torch.float16, device="cuda").transpose(1, 2), "type": k.bfloat16()}[bad]
+    with pytest.raises(AssertionError):
+        kv.quantize_append(cache.cfg, cache, k, v)
+    with pytest.raises(AssertionError):
+        kv.quantize_append_calibrated(cache.cfg, cache, kv.StaticParams(cache.cfg), k, v)
+    assert cache.seq_len == 0
+
+
+@pytest.mark.gpu
+def test_the_calls_run_on_the_current_stream():
+    """Inputs that a side stream only writes after some 20 ms: work on any other stream would read what was there before."""
+    cfg = kv.Config(2, 4, 4, 128, 512, 2, 64, 256, 2, 1, (1,))
+    g = torch.Generator("cuda").manual_seed(3)
+    K, V = (torch.randn((2, 4, 101, 128), device="cuda", generator=g).half() for _ in range(2))
+    H, q = torch.randn((2, 101, 512), device="cuda", generator=g).half(), torch.randn((2, 4, 128), device="cuda", generator=g).half()
+
+    def run(cache, H, K, V, q):
+        kv.predict_sinks(cfg, H, cache.sinks)
+        kv.quantize_append(cfg, cache, K, V)
+        return (*kv.decode_attention(cfg, cache, q), *kv.prefill_attention(cfg, cache, q[:, :, None], 100), cache.k_codes, cache.sinks.pos)
+
+    want = run(kv.KVCache(cfg), H, K, V, q)
+    late, cache = [torch.zeros_like(x) for x in (H, K, V, q)], kv.KVCache(cfg)
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(40_000_000)
+        for x, y in zip(late, (H, K, V, q)):
+            x.copy_(y)
+        got = run(cache, *late)
+    side.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(want, got))
 
 
 @pytest.mark.gpu
