@@ -38,8 +38,10 @@ constexpr int PR_HDRS = 8;
 // A zero point up to this size is subtracted from the code in fp16 exactly; farther ones go through an additive term.
 constexpr float PR_NEAR = 1000.f;
 constexpr uint32_t PR_WAIT_NS = 20000;          // a poll sleeps up to this long (without the hint it comes back after some 60 clocks)
-constexpr long long PR_WAIT_CLOCKS = 1ll << 29; // 0.27 s at the highest clock, at least: far beyond any real wait
-constexpr unsigned PR_WAIT_LOOK = 256;               // polls between two looks at the clock, at most 5 ms
+// Between 8 ms (polls of 60 clocks) and 5.2 s (polls that all sleep as long as they may): a real wait is for work of the same block, some 10 us.
+// Counted in polls and not in clocks: a look at the clock every 256 polls made the kernel 6 % slower (2661 and 2825 us), since every wait
+// of every role holds a copy of the loop and code is what it has least room for.
+constexpr int PR_WAIT_POLLS = 1 << 18;
 constexpr int PR_ROWS_KEPT = 8;                 // sink rows of a step that the parameter warps leave in shared memory
 
 struct StepHeader {
@@ -89,19 +91,13 @@ __device__ __forceinline__ void bar_arrive(uint64_t *bar)
 __device__ __forceinline__ bool bar_wait_warp(uint64_t *bar, unsigned parity, int *failed)
 {
     const uint32_t a = smem_addr(bar);
-    long long start = 0;
 #pragma unroll 1
-    for (unsigned polls = 1;; ++polls) {
+    for (int polls = 0; polls < PR_WAIT_POLLS; ++polls) {
         unsigned ok;
         asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3; selp.u32 %0, 1, 0, p; }"
                      : "=r"(ok) : "r"(a), "r"(parity), "r"(PR_WAIT_NS) : "memory");
         if (__all_sync(0xffffffffu, ok != 0)) return true;
         if (__any_sync(0xffffffffu, *(volatile int *)failed)) break;
-        if (polls % PR_WAIT_LOOK == 0) {
-            const long long now = clock64();
-            if (polls == PR_WAIT_LOOK) start = now;
-            else if (__any_sync(0xffffffffu, now - start > PR_WAIT_CLOCKS)) break;
-        }
     }
     *(volatile int *)failed = 1;
     return false;
