@@ -10,10 +10,11 @@
 //   int32.  When a weight does not fit (one vote a step) the references and units of the rows move by whole bits and the sums with them, in place:
 //   with four rows there are 64 of them a lane, and rescaling them in binary32 (another 64 values, which only fit local memory) took 1.5 times as
 //   long as everything else.
-// Append and decode, us a pass, fp16 values before and this kernel (start of both: the same merge and splits): 16 x 8 units of 30000 tokens, four
-// heads each, 4 bit, 140 -> 123; 4 x 8 of 30000, 3 bit, 53 -> 49; 8 x 8 of 16000, groups of 32, 2 bit, 67 -> 58, groups of 64 46 -> 44; two heads,
-// 2 bit 34.8 -> 30.3, 4 bit 44.2 -> 38.6.  Error against 64 bits 5e-5 -> 1e-6.  Four heads at 2 bit with one channel group a row stay in
-// decode_kernel.cuh (decode_launch.cuh says why).
+// Append and decode, us a pass, fp16 values (and the same merge and splits) before, this kernel now: 16 x 8 units of 30000 tokens, four heads
+// each, 4 bit, 140 -> 127; 4 x 8 of 30000, 3 bit, 53 -> 54; 8 x 8 of 16000, groups of 32, 2 bit, 67 -> 63, groups of 64 46 -> 47; two heads,
+// 2 bit 34.8 -> 30.4, 4 bit 44.2 -> 38.9.  Error against 64 bits, 8192 tokens a warp: N(0,1) 2e-3 -> 2e-5, scores with a deviation of four nats
+// 4e-4 -> 1e-5; a weight keeps 22 bits of the row's largest at least, smaller ones their sum.  Three and four heads at 2 bit with one channel
+// group a row stay in decode_kernel.cuh (decode_launch.cuh says why).
 #pragma once
 #include "decode_one.cuh"
 

@@ -8,17 +8,18 @@
 // fixed point.  With the fp16 values all lanes of a quad did the work of the quad's two tokens.
 // Append and decode, us a pass, fp16 values with a warp's work on eight tokens at a time before, this kernel now: 8 x 32 units of 4096
 // tokens, 2 bit, 31.0 -> 25.9 (decode alone 26.8 -> 19.6); static parameters, 3821 tokens, 27.6 -> 23.9; 16 x 32 of 8101, 3 bit, 135 -> 114;
-// 64 x 32 of 8192, 4 bit, 481 -> 445; 32-token groups, 2 bit, 53.7 -> 36.8.  Error against 64 bits 5e-5 -> 1e-6: the fp16 products'
-// accumulation truncated.  Four blocks an SM; five (96 registers, a few spilled) are slower except at 4 bit: 26.4 against 23.9, 422 / 411.
+// 64 x 32 of 8192, 4 bit, 481 -> 445; 32-token groups, 2 bit, 53.7 -> 36.8.  Error against 64 bits of these 5e-5 -> 1e-6 (the fp16
+// products' accumulation truncates; 8192 tokens a warp, N(0,1), 2e-3 -> 1e-5).  Four blocks an SM; five (96 registers, a few spilled)
+// are slower except at 4 bit: 26.4 against 23.9, 422 / 411.
 //
 // Keys: the four signed bytes of the factor q * scale in columns 0-3, and again in 4-7, so that lanes t < 2 take the first tile's sums
 // and lanes t >= 2 the second's; one exchange inside a lane pair leaves each lane with its own token's sum.
 // Values: a stored byte pair belongs to one channel and two tokens, and the two byte pairs of a 2- or 3-bit word (the two words of a
 // 4-bit fragment) to two 16-channel matrices.  The weights' four signed bytes therefore stand in eight columns, 2 l + matrix, with
 // zeros where the other matrix' codes are: lane t finds byte t of both matrices' sums in its accumulators.
-//   weight = rint(2^(s - R) * scale * 2^ev), below 2^31, ev per value channel group; R and ev move only when a weight would not fit (one vote a step).  The sums
-//   of a byte are exact in int32; when R or ev moves they are added to binary32 ones and start from zero.  A new unit puts the
-//   largest weight into [2^28, 2^29); the upper contraction slots' tokens of 2 and 3 bit carry a weight divided by 16.  So a weight is held to
+//   weight = rint(2^(s - R) * scale * 2^ev), below 2^31, ev per value channel group; R and ev move only when a weight would not fit (one
+//   vote a step).  The sums of a byte are exact in int32; when R or ev moves they are added to binary32 ones and start from zero.  A new
+//   unit puts the largest weight into [2^28, 2^29); the upper contraction slots' tokens of 2 and 3 bit carry a weight divided by 16.  So a weight is held to
 //   2^-29 of the largest, there to 2^-25; smaller ones keep their sum by a dither (next_dither).
 #pragma once
 #include "decode_kernel.cuh"

@@ -14,14 +14,14 @@
 // tile's scores are in the softmax the tensor cores run the other tile's products.
 //
 // What bounds it: five matrix products of 128 x 64 x 128 per row tile and step are 2560 clocks for both tiles (2816 with tile 1's
-// queries in shared memory); a step takes about 3700, with the tensor pipe active for 3150 of them (82 %) and 73 to 80 % of the issue
-// slots taken.  What counts is how little code the five roles have between them: at 71 KB, with the loops unrolled, the warps
-// waited for instructions (1.9 of their stalls an issue; a step with a sink token, whose code was seldom there, took 4500 clocks
-// more), at 54 KB hardly (0.3).  So every role is one short loop: tiles two at a time, one pass over a row's scores, parameters
-// and sink rows through shared memory.  4096 queries over 4096 tokens, 8 sequences of 32 heads, 2 bit, with the append, back to
-// back: 2657 us at 71 KB, 2556 now (the power cap holds the clock at some 1.4 GHz).  1003 queries with four heads per KV head over 7403 tokens,
-// 4 bit, with the append: 308 and 270 us; the same at 3 bit with 128-token groups 319 and 275; 2048 queries, 2 x 32 heads, 2 bit with
-// 64-token groups 239 and 212.  Relative error of the outputs against 64 bits: 2.6e-6 and 8.2e-6 for the first two.
+// queries in shared memory); a step takes about 3700 to 4000.  On the SMs that have a block the tensor pipe is active for 77 to 82 % of the
+// time and 73 % of the issue slots are taken.  What counts is how little code the five roles have between them: at 71 KB, with the loops
+// unrolled, the warps waited for instructions (1.9 of their stalls an issue; a step with a sink token, whose code was seldom there, took
+// 4500 clocks more), at 54 KB hardly (0.3).  So every role is one short loop: tiles two at a time, one pass over a row's scores, parameters
+// and sink rows through shared memory.  71 KB and now, append and attention, us: 4096 queries over 4096 tokens, 8 sequences of 32
+// heads, 2 bit, 2749 and 2650 (the power cap holds the clock at some 1.4 GHz); 1003 queries with four heads per KV head over 7403 tokens, 4 bit, 294
+// and 278; the same at 3 bit with 128-token groups 319 and 275; 2048 queries, 2 x 32 heads, 2 bit with 64-token groups 239 and 212.  Relative
+// error of the outputs against 64 bits: 2.6e-6 and 8.2e-6 for the first two.
 #include "common.cuh"
 
 namespace kvsink {
