@@ -201,3 +201,29 @@ def test_sink_rows_that_are_not_finite_stay_hidden_from_queries_before_them(bits
     fine = np.isfinite(ref)
     assert_close(out[fine], ref[fine], "prompt attention")
     assert np.abs(lse - ref_lse).max() <= 2e-3 + 1e-3 * np.abs(ref_lse).max()
+
+
+# several row blocks to a block of the grid, which takes them one after the other: the last ones are their units' first rows, 44 with one row tile, 4, 256
+@pytest.mark.parametrize("bits,group,hq,hkv,batch,T,pos0", [(2, 128, 16, 16, 12, 300, 0), (4, 64, 8, 4, 40, 130, 50), (3, 32, 4, 4, 60, 512, 0)])
+def test_several_row_blocks_to_a_block(bits, group, hq, hkv, batch, T, pos0):
+    wl = TINY.scaled(bits=bits, head_dim=128, group=group, n_q_heads=hq, n_kv_heads=hkv, batch=batch, seq=pos0 + T, topk=5, pfn_n=1, seed=30000 + bits)
+    _check(wl, T, pos0)
+    _same_every_time(*_prompt(wl)[:2], _queries(wl, T), pos0, times=3)
+
+
+def _queries(wl, T):
+    return torch.randn((wl.batch, wl.n_q_heads, T, wl.head_dim), device="cuda", generator=torch.Generator("cuda").manual_seed(wl.seed)).half()
+
+
+# more row blocks than the lists of 148 blocks hold (95 each): a second wave of blocks takes the rest.  Against the eight-row blocks, which
+# eight queries a unit go to
+def test_more_row_blocks_than_the_grid_takes():
+    wl = TINY.scaled(bits=2, head_dim=128, group=64, n_q_heads=32, n_kv_heads=32, batch=450, seq=72, topk=2, pfn_n=1, seed=31000)
+    gcfg, gc, q = _prompt(wl)
+    assert wl.batch * 32 > 148 * 95 and kv.prefill_rows(gcfg, 72) == 256 and kv.prefill_rows(gcfg, 8) == 8
+    out, lse = kv.prefill_attention(gcfg, gc, q, 0)
+    for t in range(0, 72, 8):
+        small, small_lse = kv.prefill_attention(gcfg, gc, q[:, :, t:t + 8], t)
+        assert (out[:, :, t:t + 8] - small).abs().max() <= 2e-3 + 1e-2 * small.abs().max()
+        assert (lse[:, :, t:t + 8] - small_lse).abs().max() <= 2e-3 + 1e-3 * small_lse.abs().max()
+    assert kv.read_status(gc) == 0
