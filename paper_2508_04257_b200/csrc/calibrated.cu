@@ -296,148 +296,146 @@ __device__ __forceinline__ uint32_t code_static_fast(float x, float s, float r, 
     return (uint32_t)(int)fminf(fmaxf(c + z, 0.f), qmax);
 }
 
-// Whole fresh tiles (a bulk append that starts on a tile boundary): one warp per 16-token tile.  The warp stages the
-// tile's key and value rows in shared memory and every lane codes exactly the elements of its own pair slots of the packed
-// tiles, so the lane's words come out in the tile's own order and are stored with one 16-byte (or 8-byte) store per plane.
-constexpr int CF_WARPS = 4;
+// The tiles of up to two spans of new tokens (head size 128), all of them and both spans in one launch: what a chunk has before its first
+// whole group and behind its last, or a short chunk.  One block per 16-token tile: it stages the tile's new key and value rows in shared memory, and
+// each of its four warps codes one side's elements of half the channels, a lane exactly those of its own pair slots of the packed tile, so
+// that its words come out in the tile's own order.  Where earlier tokens live in the tile their fields are kept: a lane's words are its
+// own, so that takes no atomics.
+// Latency is what counts here (a few tiles a unit): a chunk's ragged ends were up to six launches, of whole tiles (a warp each) and of the tokens before and
+// behind them, walking the words of both tiles field by field.  Per-token keys, 2 bit, 4 x 8 units, 91 tokens from 37: 35.0 us, one launch with a warp a
+// tile 17.3, a block a tile 9.6; 14 x 4 units of 357 tokens 28.9, 19.0, 12.7.
+constexpr int CF_THREADS = 128;
+struct TokenSpans {
+    int first[2], n[2], src[2];      // position of the first token, number of tokens, row of the first one in the source
+    int tiles[2];                    // tiles that they touch
+};
 
 template <int BITS, bool PT>
-__global__ void __launch_bounds__(32 * CF_WARPS)
+__global__ void __launch_bounds__(CF_THREADS)
 quantize_calibrated_tiles_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *__restrict__ k_src,
-                                 const __half *__restrict__ v_src, int first_token, int n_tiles, int64_t sb, int64_t sh, int64_t stt)
+                                 const __half *__restrict__ v_src, TokenSpans spans, int64_t sb, int64_t sh, int64_t stt)
 {
-    constexpr int D = 128, W = D * BITS / 64, NLO = BITS == 3 ? D / 32 : W, NHI = BITS == 3 ? D / 64 : 0;
+    constexpr int D = 128;
+    constexpr int LO = BITS == 4 ? 4 : 2, HI = BITS == 3 ? 1 : 0;   // words of a warp's half of the channels: of whole codes or low bits, of high bits
     constexpr int ROW = D + 8;                                 // padded row (halves): conflict-free column reads
-    __shared__ __align__(16) __half s_k[CF_WARPS][KVSINK_TILE * ROW], s_v[CF_WARPS][KVSINK_TILE * ROW];
-    __shared__ float4 s_kp[D];                                 // (scale, 1 / scale, zero) of the KV head's key channels
-    __shared__ float4 s_pt[PT ? CF_WARPS : 1][2][KVSINK_TILE][4];   // per-token keys: the same per (K / V, token, 32-channel block)
+    __shared__ __align__(16) __half s_x[2][KVSINK_TILE * ROW];  // keys, values
+    __shared__ float4 s_kp[PT ? 1 : D];                        // (scale, 1 / scale, zero) of the KV head's key channels
+    __shared__ float4 s_pt[2][PT ? KVSINK_TILE : 1][4];        // the same per (keys / values, token, 32-channel block); static values: of the head
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
-    const int h = blockIdx.y, b = blockIdx.z;
+    const int kind = warp & 1, half = warp >> 1;               // keys or values, lower or upper 64 channels
+    const int h = blockIdx.y, b = blockIdx.z, ti = blockIdx.x;
     const int64_t unit = (int64_t)b * p.Hkv + h;
     const float qmax = (float)((1 << BITS) - 1);
     const uint32_t *bm = c.sink_bitmask + (size_t)b * p.mask_words;
+    const int sp_i = ti >= spans.tiles[0], first = spans.first[sp_i], last = first + spans.n[sp_i];
+    const int tok0 = (first / KVSINK_TILE + ti - (sp_i ? spans.tiles[0] : 0)) * KVSINK_TILE;
     pdl_wait();
-    for (int i = tid; i < D && !PT; i += 32 * CF_WARPS) {
-        const float sc = sp.k_scale[h * D + i];
-        s_kp[i] = make_float4(sc, sc == 0.f ? 0.f : __frcp_rn(sc), sp.k_zero[h * D + i], 0.f);
+    pdl_release();                                             // the whole groups' kernel of the same chunk may start beside this one
+    if (!in_bounds(tok0 >= 0 && tok0 + KVSINK_TILE <= p.max_seq, c.status)) return;
+    const int lo = max(first - tok0, 0), hi = min(last - tok0, KVSINK_TILE);                   // the tile's new tokens
+    const uint32_t fresh16 = ((1u << hi) - 1u) & ~((1u << lo) - 1u);
+    const uint32_t mask16 = (bm[tok0 >> 5] >> (tok0 & 31)) & fresh16;   // sink bits of the new tokens
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+        const int i = tid + CF_THREADS * x, side = i >> 8, r = (i >> 4) & 15, c8 = i & 15;
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (r >= lo && r < hi)
+            v = __ldg(reinterpret_cast<const uint4 *>((side ? v_src : k_src) + b * sb + h * sh + (int64_t)(spans.src[sp_i] + tok0 + r - first) * stt + c8 * 8));
+        *reinterpret_cast<uint4 *>(s_x[side] + r * ROW + c8 * 8) = v;
+    }
+    auto triple = [](float sc, float z) { return make_float4(sc, sc == 0.f ? 0.f : __frcp_rn(sc), z, 0.f); };
+    if constexpr (!PT) {
+        s_kp[tid] = triple(sp.k_scale[h * D + tid], sp.k_zero[h * D + tid]);
+        if (tid < 4) s_pt[1][0][tid] = triple(sp.v_scale[h * p.NGv + 32 * tid / p.Gv], sp.v_zero[h * p.NGv + 32 * tid / p.Gv]);
     }
     __syncthreads();
-    const int ti = blockIdx.x * CF_WARPS + warp;               // tile of this append
-    if (ti >= n_tiles) return;
-    const int tok0 = first_token + ti * KVSINK_TILE, src0 = ti * KVSINK_TILE;
-    if (!in_bounds(tok0 >= 0 && tok0 + KVSINK_TILE <= p.max_seq, c.status)) return;
-    __half *mk = s_k[warp], *mv = s_v[warp];
-    for (int i = lane; i < KVSINK_TILE * (D / 8); i += 32) {
-        const int r = i / (D / 8), c8 = i % (D / 8);
-        const int64_t off = b * sb + h * sh + (int64_t)(src0 + r) * stt + c8 * 8;
-        *reinterpret_cast<uint4 *>(mk + r * ROW + c8 * 8) = __ldg(reinterpret_cast<const uint4 *>(k_src + off));
-        *reinterpret_cast<uint4 *>(mv + r * ROW + c8 * 8) = __ldg(reinterpret_cast<const uint4 *>(v_src + off));
-    }
-    const uint32_t mask16 = (bm[tok0 >> 5] >> (tok0 & 31)) & 0xffffu;   // sink bits of the tile's tokens
-    __syncwarp();
-    if (mask16) {   // exact rows to the side buffer at the rank of their position
+    // exact rows to the side buffer at the rank of their position
+    if (mask16 && half == 0) {
         const int count = min(c.sink_count[b], p.cap);
         for (uint32_t rest = mask16; rest; rest &= rest - 1u) {
             const int r = __ffs((int)rest) - 1;
             const int slot = find_slot(c.sink_pos + (size_t)b * p.cap, count, tok0 + r);
             if (slot < 0) {
-                if (lane == 0) atomicOr(c.status, KVSINK_STATUS_SINK_MISMATCH);
+                if (tid == 0) atomicOr(c.status, KVSINK_STATUS_SINK_MISMATCH);
                 continue;
             }
-            __half *dk = (__half *)c.sink_k + ((size_t)unit * p.cap + slot) * D, *dv = (__half *)c.sink_v + ((size_t)unit * p.cap + slot) * D;
-            if (lane < D / 8) {
-                *reinterpret_cast<uint4 *>(dk + lane * 8) = *reinterpret_cast<const uint4 *>(mk + r * ROW + lane * 8);
-                *reinterpret_cast<uint4 *>(dv + lane * 8) = *reinterpret_cast<const uint4 *>(mv + r * ROW + lane * 8);
-            }
+            __half *to = (__half *)(kind ? c.sink_v : c.sink_k) + ((size_t)unit * p.cap + slot) * D;
+            if (lane < D / 8) *reinterpret_cast<uint4 *>(to + lane * 8) = *reinterpret_cast<const uint4 *>(s_x[kind] + r * ROW + lane * 8);
         }
     }
     if constexpr (PT) {
-        // per-token parameters: lane -> token lane / 2, channels 64 (lane % 2) ... + 63 as two 32-channel blocks, combined to
-        // the channel group (32, 64 or 128 channels) and written to the parameter arrays by the group's first lane
-        const int tk = lane >> 1, hf = lane & 1;
-        const bool sink = (mask16 >> tk) & 1u;
+        // per-token parameters: a thread takes one 32-channel block of a token's keys or values; the four threads of a row put theirs together to the
+        // channel group (32, 64 or 128 channels), whose first one writes the pair
+        const int side = tid >> 6, tk = (tid >> 2) & 15, blk = tid & 3;
+        const __half2 *row = reinterpret_cast<const __half2 *>(s_x[side] + tk * ROW + 32 * blk);
+        __half2 l2 = row[0], h2 = l2;
 #pragma unroll
-        for (int kind = 0; kind < 2; ++kind) {
-            const __half *row = (kind ? mv : mk) + tk * ROW + 64 * hf;
-            float mn[2], mx[2];
-#pragma unroll
-            for (int sbk = 0; sbk < 2; ++sbk) {
-                __half2 lo = *reinterpret_cast<const __half2 *>(row + 32 * sbk), hi = lo;
-#pragma unroll
-                for (int i = 1; i < 16; ++i) {
-                    const __half2 x = *reinterpret_cast<const __half2 *>(row + 32 * sbk + 2 * i);
-                    lo = __hmin2(lo, x); hi = __hmax2(hi, x);
-                }
-                mn[sbk] = fminf(__low2float(lo), __high2float(lo)); mx[sbk] = fmaxf(__low2float(hi), __high2float(hi));
-            }
-            if (p.Gv >= 64) { mn[0] = mn[1] = fminf(mn[0], mn[1]); mx[0] = mx[1] = fmaxf(mx[0], mx[1]); }
-            if (p.Gv >= 128) {
-                mn[0] = mn[1] = fminf(mn[0], __shfl_xor_sync(0xffffffffu, mn[0], 1));
-                mx[0] = mx[1] = fmaxf(mx[0], __shfl_xor_sync(0xffffffffu, mx[0], 1));
-            }
-            float *ps = kind ? c.v_scale : c.k_scale, *pz = kind ? c.v_zero : c.k_zero;
-#pragma unroll
-            for (int sbk = 0; sbk < 2; ++sbk) {
-                float sc, ze;
-                group_params(!sink, mn[sbk], mx[sbk], qmax, &sc, &ze);
-                const int ch0 = 64 * hf + 32 * sbk;
-                s_pt[warp][kind][tk][2 * hf + sbk] = make_float4(sc, sc == 0.f ? 0.f : __frcp_rn(sc), ze, 0.f);
-                if (ch0 % p.Gv == 0) {
-                    const size_t o = ((size_t)unit * p.max_seq + tok0 + tk) * p.NGv + ch0 / p.Gv;
-                    ps[o] = sc; pz[o] = ze;
-                }
-            }
+        for (int x = 1; x < 16; ++x) { l2 = __hmin2(l2, row[x]); h2 = __hmax2(h2, row[x]); }
+        float mn = fminf(__low2float(l2), __high2float(l2)), mx = fmaxf(__low2float(h2), __high2float(h2));
+        for (int o = 1; 32 * o < p.Gv; o <<= 1) {
+            mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         }
-        __syncwarp();
+        float sc, ze;
+        group_params(!((mask16 >> tk) & 1u), mn, mx, qmax, &sc, &ze);
+        s_pt[side][tk][blk] = triple(sc, ze);
+        if (((fresh16 >> tk) & 1u) && 32 * blk % p.Gv == 0) {
+            const size_t o = ((size_t)unit * p.max_seq + tok0 + tk) * p.NGv + 32 * blk / p.Gv;
+            (side ? c.v_scale : c.k_scale)[o] = sc;
+            (side ? c.v_zero : c.k_zero)[o] = ze;
+        }
+        __syncthreads();
     }
     // codes of pair slot s = 4m + r, half e: keys (token, channel) = (g + 8(r&1), 16m + 8(r>>1) + 2t + e),
     //                                        values (channel, token) = (16m + g + 8(r&1), 8(r>>1) + 2t + e)
-    uint32_t kw[W], vw[W];
+    const uint32_t none16 = mask16 | ~fresh16;                 // code 0: sink tokens, and fields of tokens that are not this call's
+    const __half *xs = s_x[kind];
+    uint32_t w[LO + HI];
 #pragma unroll
-    for (int i = 0; i < W; ++i) kw[i] = vw[i] = 0u;
+    for (int i = 0; i < LO + HI; ++i) w[i] = 0u;
 #pragma unroll
-    for (int m = 0; m < D / 16; ++m) {
-        const int vj = (16 * m) / p.Gv;   // value channel group of this matrix (groups are multiples of 16 channels)
-        float vs = 0.f, vz = 0.f, vr = 0.f;
-        if constexpr (!PT) { vs = sp.v_scale[h * p.NGv + vj]; vz = sp.v_zero[h * p.NGv + vj]; vr = vs == 0.f ? 0.f : __frcp_rn(vs); }
+    for (int m = 0; m < 4; ++m)
 #pragma unroll
         for (int r = 0; r < 4; ++r)
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-                const int s_ = 4 * m + r;
-                const int ktok = g + 8 * (r & 1), kch = 16 * m + 8 * (r >> 1) + 2 * t + e;
-                const int vch = 16 * m + g + 8 * (r & 1), vtok = 8 * (r >> 1) + 2 * t + e;
-                const float4 kp = PT ? s_pt[PT ? warp : 0][0][ktok][kch >> 5] : s_kp[kch];
-                const float4 vp = PT ? s_pt[PT ? warp : 0][1][vtok][vch >> 5] : make_float4(vs, vr, vz, 0.f);
-                const uint32_t kc = ((mask16 >> ktok) & 1u) || kp.x == 0.f ? 0u : code_static_fast(__half2float(mk[ktok * ROW + kch]), kp.x, kp.y, kp.z, qmax);
-                const uint32_t vc = ((mask16 >> vtok) & 1u) || vp.x == 0.f ? 0u : code_static_fast(__half2float(mv[vtok * ROW + vch]), vp.x, vp.y, vp.z, qmax);
-                if constexpr (BITS == 2) {
-                    kw[s_ / 8] |= kc << (16 * e + 2 * (s_ % 8)); vw[s_ / 8] |= vc << (16 * e + 2 * (s_ % 8));
-                } else if constexpr (BITS == 4) {
-                    kw[s_ / 4] |= kc << (16 * e + 4 * (s_ % 4)); vw[s_ / 4] |= vc << (16 * e + 4 * (s_ % 4));
+                const int s_ = 4 * m + r, row = g + 8 * (r & 1), col = 8 * (r >> 1) + 2 * t + e, ch0 = 64 * half + 16 * m;
+                const int tok = kind ? col : row, ch = ch0 + (kind ? row : col);
+                const float4 q = PT ? s_pt[kind][PT ? tok : 0][ch >> 5] : (kind ? s_pt[1][0][ch >> 5] : s_kp[PT ? 0 : ch]);
+                const uint32_t code = ((none16 >> tok) & 1u) || q.x == 0.f ? 0u : code_static_fast(__half2float(xs[tok * ROW + ch]), q.x, q.y, q.z, qmax);
+                if constexpr (BITS == 4) {
+                    w[s_ / 4] |= code << (16 * e + 4 * (s_ % 4));
+                } else if constexpr (BITS == 2) {
+                    w[s_ / 8] |= code << (16 * e + 2 * (s_ % 8));
                 } else {
-                    const int i = s_ / 8, k = s_ % 8, hb = 16 * e + 4 * (k / 2) + 2 * (1 - (i % 2)) + (k % 2);
-                    kw[i] |= (kc & 3u) << (16 * e + 2 * k); vw[i] |= (vc & 3u) << (16 * e + 2 * k);
-                    kw[NLO + i / 2] |= (kc >> 2) << hb; vw[NLO + i / 2] |= (vc >> 2) << hb;
+                    const int i = s_ / 8, k = s_ % 8;
+                    w[i] |= (code & 3u) << (16 * e + 2 * k);
+                    w[LO] |= (code >> 2) << (16 * e + 4 * (k / 2) + 2 * (1 - i) + (k % 2));
                 }
             }
-    }
-    // a section of n words per lane is stored as planes of up to four words per lane
+    // the lane's words of its half: 2 and 3 bit two of the four in the plane, 4 bit the half's plane; 3 bit one of the two of the high bits
     const size_t tile_off = (size_t)unit * p.max_seq * p.row_bytes + (size_t)(tok0 / KVSINK_TILE) * p.tile_bytes;
-    uint32_t *ko = (uint32_t *)(c.k_codes + tile_off), *vo = (uint32_t *)(c.v_codes + tile_off);
-    auto store_section = [&](uint32_t *dst, const uint32_t *w, int n) {
-        for (int pl = 0; pl * 4 < n; ++pl) {
-            const int u = n - 4 * pl > 4 ? 4 : n - 4 * pl;
-            uint32_t *d = dst + u * lane;
-            if (u == 4) *reinterpret_cast<uint4 *>(d) = make_uint4(w[4 * pl], w[4 * pl + 1], w[4 * pl + 2], w[4 * pl + 3]);
-            else if (u == 2) *reinterpret_cast<uint2 *>(d) = make_uint2(w[4 * pl], w[4 * pl + 1]);
-            else for (int i = 0; i < u; ++i) d[i] = w[4 * pl + i];
-            dst += 32 * u;
+    uint8_t *tile = (kind ? c.v_codes : c.k_codes) + tile_off;
+    uint32_t *to = (uint32_t *)(tile + (BITS == 4 ? 512 * half + 16 * lane : 16 * lane + 8 * half)), *to_high = (uint32_t *)(tile + 512 + 8 * lane + 4 * half);
+    if (lo > 0) {
+        // earlier tokens live in the tile: their fields stay.  A slot's token: keys' by s % 2 among rows g, g + 8; values' by s / 2 % 2 among columns 2t + e, + 8
+        uint32_t f[2];                                         // all ones where the word's fields of that kind are new
+#pragma unroll
+        for (int x = 0; x < 2; ++x)
+            f[x] = kind ? ((fresh16 >> (2 * t + 8 * x)) & 1u ? 0xffffu : 0u) | ((fresh16 >> (2 * t + 1 + 8 * x)) & 1u ? 0xffff0000u : 0u)
+                        : ((fresh16 >> (g + 8 * x)) & 1u ? 0xffffffffu : 0u);
+        const uint32_t even = kind ? (BITS == 4 ? 0x00ff00ffu : 0x0f0f0f0fu) : (BITS == 4 ? 0x0f0f0f0fu : 0x33333333u);
+        const uint32_t kept = ~((even & f[0]) | (~even & f[1]));
+#pragma unroll
+        for (int i = 0; i < LO; ++i) w[i] |= to[i] & kept;
+        if constexpr (BITS == 3) {
+            const uint32_t even_high = kind ? 0x0f0f0f0fu : 0x55555555u;
+            w[LO] |= *to_high & ~((even_high & f[0]) | (~even_high & f[1]));
         }
-    };
-    store_section(ko, kw, NLO);
-    store_section(vo, vw, NLO);
-    if constexpr (BITS == 3) { store_section(ko + 32 * NLO, kw + NLO, NHI); store_section(vo + 32 * NLO, vw + NLO, NHI); }
+    }
+    if constexpr (BITS == 4) *reinterpret_cast<uint4 *>(to) = make_uint4(w[0], w[1], w[2], w[3]);
+    else *reinterpret_cast<uint2 *>(to) = make_uint2(w[0], w[1]);
+    if constexpr (BITS == 3) *to_high = w[LO];
 }
 
 }  // namespace
@@ -459,6 +457,20 @@ int launch_calibrate(const Params &p, const __half *k, const __half *v, int T, i
                                                                                                                                 : KVSINK_ERR_CUDA;
 }
 
+// Up to two spans at head size 128.
+template <bool PT>
+static int launch_spans(const Params &p, const kvsink_cache &c, const kvsink_static_params &sp, const __half *k_src, const __half *v_src, TokenSpans s,
+                        int64_t sb, int64_t sh, int64_t stt, cudaStream_t st)
+{
+    for (int i = 0; i < 2; ++i) s.tiles[i] = s.n[i] > 0 ? (s.first[i] + s.n[i] - 1) / KVSINK_TILE - s.first[i] / KVSINK_TILE + 1 : 0;
+    const dim3 grid(s.tiles[0] + s.tiles[1], p.Hkv, p.B), block(CF_THREADS);
+    if (grid.x == 0) return KVSINK_OK;
+    const cudaError_t e = p.bits == 2   ? launch_pdl(quantize_calibrated_tiles_kernel<2, PT>, grid, block, 0, st, p, c, sp, k_src, v_src, s, sb, sh, stt)
+                          : p.bits == 3 ? launch_pdl(quantize_calibrated_tiles_kernel<3, PT>, grid, block, 0, st, p, c, sp, k_src, v_src, s, sb, sh, stt)
+                                        : launch_pdl(quantize_calibrated_tiles_kernel<4, PT>, grid, block, 0, st, p, c, sp, k_src, v_src, s, sb, sh, stt);
+    return e == cudaSuccess ? KVSINK_OK : KVSINK_ERR_CUDA;
+}
+
 template <bool PT>
 static int launch_tokens(const Params &p, const kvsink_cache &c, const kvsink_static_params &sp, const __half *k_src, const __half *v_src,
                          int first_token, int n_tokens, int64_t sb, int64_t sh, int64_t stt, cudaStream_t st)
@@ -469,24 +481,18 @@ static int launch_tokens(const Params &p, const kvsink_cache &c, const kvsink_st
         return launch_pdl(append_one_flat_kernel<PT>, dim3((unsigned)((units + CO_WARPS - 1) / CO_WARPS)), dim3(32 * CO_WARPS), 0, st, p, c, sp, k_src,
                           v_src, first_token, sb, sh) == cudaSuccess ? KVSINK_OK : KVSINK_ERR_CUDA;
     }
-    // tokens before the next tile boundary go by themselves where whole tiles that follow have a kernel of their own, at head size 128
-    // (2859 tokens from 1237, 8 x 32 units, 3 bit, G = 128: 680 -> 322 us)
-    const int lead = (KVSINK_TILE - first_token % KVSINK_TILE) % KVSINK_TILE;
-    if (p.D == 128 && lead > 0 && n_tokens >= lead + KVSINK_TILE) {
-        const int rc = launch_tokens<PT>(p, c, sp, k_src, v_src, first_token, lead, sb, sh, stt, st);
-        return rc ? rc : launch_tokens<PT>(p, c, sp, k_src + (int64_t)lead * stt, v_src + (int64_t)lead * stt, first_token + lead, n_tokens - lead, sb, sh,
-                                           stt, st);
-    }
-    // whole fresh tiles of a head-size-128 cache take the tile kernel, the ragged rest (at most 15 tokens) the general one
-    if (p.D == 128 && lead == 0 && n_tokens >= KVSINK_TILE && ((uintptr_t)k_src & 15u) == 0 && ((uintptr_t)v_src & 15u) == 0) {
-        const int n_tiles = n_tokens / KVSINK_TILE;
-        const dim3 grid((n_tiles + CF_WARPS - 1) / CF_WARPS, p.Hkv, p.B);
-        cudaError_t e = p.bits == 2 ? launch_pdl(quantize_calibrated_tiles_kernel<2, PT>, grid, dim3(32 * CF_WARPS), 0, st, p, c, sp, k_src, v_src, first_token, n_tiles, sb, sh, stt)
-                      : p.bits == 3 ? launch_pdl(quantize_calibrated_tiles_kernel<3, PT>, grid, dim3(32 * CF_WARPS), 0, st, p, c, sp, k_src, v_src, first_token, n_tiles, sb, sh, stt)
-                                    : launch_pdl(quantize_calibrated_tiles_kernel<4, PT>, grid, dim3(32 * CF_WARPS), 0, st, p, c, sp, k_src, v_src, first_token, n_tiles, sb, sh, stt);
-        if (e != cudaSuccess) return KVSINK_ERR_CUDA;
-        const int done = n_tiles * KVSINK_TILE;
-        return launch_tokens<PT>(p, c, sp, k_src + (int64_t)done * stt, v_src + (int64_t)done * stt, first_token + done, n_tokens - done, sb, sh, stt, st);
+    if (p.D == 128) {
+        // One launch, whatever the ends.  Group sizes without a bulk form (they have no decode kernel either, codes are all they are for) keep
+        // the launches they had, which are counted: the tokens up to a tile boundary, whole tiles, the rest
+        int at = 0, rc = KVSINK_OK;
+        while (at < n_tokens && rc == KVSINK_OK) {
+            const int lead = (KVSINK_TILE - (first_token + at) % KVSINK_TILE) % KVSINK_TILE, left = n_tokens - at;
+            int n = left;
+            if (p.G != 64 && p.G != 128 && left >= lead + KVSINK_TILE) n = lead > 0 ? lead : left / KVSINK_TILE * KVSINK_TILE;
+            rc = launch_spans<PT>(p, c, sp, k_src, v_src, TokenSpans{{first_token + at, 0}, {n, 0}, {at, 0}, {0, 0}}, sb, sh, stt, st);
+            at += n;
+        }
+        return rc;
     }
     const int tiles = (first_token + n_tokens - 1) / KVSINK_TILE - first_token / KVSINK_TILE + 1;
     const dim3 grid(tiles, p.Hkv, p.B);
@@ -494,45 +500,39 @@ static int launch_tokens(const Params &p, const kvsink_cache &c, const kvsink_st
                    cudaSuccess ? KVSINK_OK : KVSINK_ERR_CUDA;
 }
 
-int launch_quantize_calibrated(const Params &p, const kvsink_cache &c, const kvsink_static_params &sp, const __half *k_src, const __half *v_src,
-                               int first_token, int n_tokens, int64_t sb, int64_t sh, int64_t stt, cudaStream_t st)
+// Whole G-token spans go to the bulk quantizer where it has a form for the scheme (G only shapes its work items with static parameters); the
+// tokens before the first multiple of G and behind the last go ahead of it in one launch, beside which it may start (quantize_bulk.cu says why).
+// Static parameters, 2859 tokens from 1237, 8 x 32 units, 2 bit: 579 us without the bulk quantizer, 105 with it.
+template <bool PT>
+static int launch_flat(const Params &p, const kvsink_cache &c, const kvsink_static_params &sp, const __half *k_src, const __half *v_src,
+                       int first_token, int n_tokens, int64_t sb, int64_t sh, int64_t stt, cudaStream_t st)
 {
-    // whole G-token spans go to the bulk quantizer where it has a static form (G only shapes its work items); the tokens before the
-    // first multiple of G and behind the last go to the others.  A chunk of 2859 tokens from 1237, 8 x 32 units, before only chunks
-    // that began on a multiple were split: 2 bit, 579 -> 105 us
     const int head = (p.G - first_token % p.G) % p.G, n_groups = (n_tokens - head) / p.G;
     if (n_tokens >= head + p.G) {
         const int64_t skip = (int64_t)head * stt;
-        int rc = launch_quantize_static_bulk(p, c, sp, k_src + skip, v_src + skip, first_token + head, n_groups, sb, sh, stt, st);
-        if (rc == KVSINK_OK) {
-            const int done = head + n_groups * p.G;
-            rc = launch_tokens<false>(p, c, sp, k_src, v_src, first_token, head, sb, sh, stt, st);
-            return rc ? rc : launch_tokens<false>(p, c, sp, k_src + (int64_t)done * stt, v_src + (int64_t)done * stt, first_token + done, n_tokens - done, sb,
-                                               sh, stt, st);
-        }
+        const int done = head + n_groups * p.G;
+        const auto ends = [&] {
+            return launch_spans<PT>(p, c, sp, k_src, v_src, TokenSpans{{first_token, first_token + done}, {head, n_tokens - done}, {0, done}, {0, 0}}, sb, sh, stt, st);
+        };
+        const LaunchBefore before = head > 0 || done < n_tokens ? launch_before(ends) : LaunchBefore{};
+        const int rc = PT ? launch_quantize_pertoken_bulk(p, c, k_src + skip, v_src + skip, first_token + head, n_groups, sb, sh, stt, before, st)
+                          : launch_quantize_static_bulk(p, c, sp, k_src + skip, v_src + skip, first_token + head, n_groups, sb, sh, stt, before, st);
         if (rc != KVSINK_ERR_UNSUPPORTED) return rc;
     }
-    return launch_tokens<false>(p, c, sp, k_src, v_src, first_token, n_tokens, sb, sh, stt, st);
+    return launch_tokens<PT>(p, c, sp, k_src, v_src, first_token, n_tokens, sb, sh, stt, st);
+}
+
+int launch_quantize_calibrated(const Params &p, const kvsink_cache &c, const kvsink_static_params &sp, const __half *k_src, const __half *v_src,
+                               int first_token, int n_tokens, int64_t sb, int64_t sh, int64_t stt, cudaStream_t st)
+{
+    return launch_flat<false>(p, c, sp, k_src, v_src, first_token, n_tokens, sb, sh, stt, st);
 }
 
 int launch_quantize_pertoken(const Params &p, const kvsink_cache &c, const __half *k_src, const __half *v_src, int first_token, int n_tokens,
                              int64_t sb, int64_t sh, int64_t stt, cudaStream_t st)
 {
     const kvsink_static_params none = {nullptr, nullptr, nullptr, nullptr};
-    // split as with static parameters (per-token keys at 4 bit, the same chunk: 743 -> 143 us)
-    const int head = (p.G - first_token % p.G) % p.G, n_groups = (n_tokens - head) / p.G;
-    if (n_tokens >= head + p.G) {
-        const int64_t skip = (int64_t)head * stt;
-        int rc = launch_quantize_pertoken_bulk(p, c, k_src + skip, v_src + skip, first_token + head, n_groups, sb, sh, stt, st);
-        if (rc == KVSINK_OK) {
-            const int done = head + n_groups * p.G;
-            rc = launch_tokens<true>(p, c, none, k_src, v_src, first_token, head, sb, sh, stt, st);
-            return rc ? rc : launch_tokens<true>(p, c, none, k_src + (int64_t)done * stt, v_src + (int64_t)done * stt, first_token + done, n_tokens - done, sb,
-                                               sh, stt, st);
-        }
-        if (rc != KVSINK_ERR_UNSUPPORTED) return rc;
-    }
-    return launch_tokens<true>(p, c, none, k_src, v_src, first_token, n_tokens, sb, sh, stt, st);
+    return launch_flat<true>(p, c, none, k_src, v_src, first_token, n_tokens, sb, sh, stt, st);
 }
 
 }  // namespace kvsink

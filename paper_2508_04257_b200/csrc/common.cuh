@@ -198,10 +198,18 @@ int launch_calibrate(const Params &p, const __half *k, const __half *v, int T, i
                      const kvsink_static_params &sp, void *workspace, cudaStream_t st);
 int launch_quantize_calibrated(const Params &p, const kvsink_cache &c, const kvsink_static_params &sp, const __half *k_src, const __half *v_src,
                                int first_token, int n_tokens, int64_t sb, int64_t sh, int64_t stt, cudaStream_t st);
+// A launch that a launcher of whole groups makes ahead of its own, behind everything of its own that can be refused: the same call's ragged
+// ends.  Refers to the callable it was made from.
+struct LaunchBefore {
+    int (*call)(const void *) = nullptr;
+    const void *with = nullptr;
+};
+template <typename F>
+LaunchBefore launch_before(const F &f) { return {[](const void *w) { return (*static_cast<const F *>(w))(); }, &f}; }
 int launch_quantize_static_bulk(const Params &p, const kvsink_cache &c, const kvsink_static_params &sp, const __half *k_src, const __half *v_src,
-                                int first_token, int n_groups, int64_t sb, int64_t sh, int64_t stt, cudaStream_t st);
+                                int first_token, int n_groups, int64_t sb, int64_t sh, int64_t stt, LaunchBefore before, cudaStream_t st);
 int launch_quantize_pertoken_bulk(const Params &p, const kvsink_cache &c, const __half *k_src, const __half *v_src, int first_token, int n_groups,
-                                  int64_t sb, int64_t sh, int64_t stt, cudaStream_t st);
+                                  int64_t sb, int64_t sh, int64_t stt, LaunchBefore before, cudaStream_t st);
 int launch_quantize_pertoken(const Params &p, const kvsink_cache &c, const __half *k_src, const __half *v_src, int first_token, int n_tokens,
                              int64_t sb, int64_t sh, int64_t stt, cudaStream_t st);
 size_t calibrate_workspace_bytes(const Params &p);

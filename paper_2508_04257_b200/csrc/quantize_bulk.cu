@@ -249,7 +249,7 @@ __device__ __forceinline__ void qb_pack_matrix(const uint32_t (&pc)[4], int m, u
 struct QbShape {
     int first_token, n_groups;
     unsigned n_items;
-    int after_edges;     // launched behind append_edges_kernel of the same call
+    int after_edges;     // launched behind the kernel of the same call's ragged ends
 };
 
 template <int G, int BITS = 2>
@@ -881,7 +881,7 @@ bool make_map(CUtensorMap *tm, const __half *base, const Params &p, int T, int64
 
 template <int BITS, int G, int MODE = 0>
 int launch_bulk(const Params &p, const kvsink_cache &c, const kvsink_static_params &sp, const __half *k_src, const __half *v_src, int first_token,
-                int n_groups, int64_t sb, int64_t sh, int64_t stt, cudaStream_t st, const AppendEdges *edges = nullptr)
+                int n_groups, int64_t sb, int64_t sh, int64_t stt, cudaStream_t st, LaunchBefore before)
 {
     using Geo = QbGeo<G, BITS>;
     CUtensorMap tm_k, tm_v;
@@ -898,15 +898,15 @@ int launch_bulk(const Params &p, const kvsink_cache &c, const kvsink_static_para
     QbShape shp;
     shp.first_token = first_token;
     shp.n_groups = n_groups;
-    shp.after_edges = edges != nullptr;
+    shp.after_edges = before.call != nullptr;
     const long n_items = (long)p.B * p.Hkv * n_groups * Geo::IPG;
     if (n_items >= (1L << 30)) return KVSINK_ERR_UNSUPPORTED;
     shp.n_items = (unsigned)n_items;
     long blocks = (n_items + NW - 1) / NW;
     if (blocks > 148) blocks = 148;
     if (!allow_smem(kern, smem)) return KVSINK_ERR_CUDA;
-    if (edges)
-        if (const int rc = launch_append_edges(p, c, *edges, st)) return rc;
+    if (before.call)
+        if (const int rc = before.call(before.with)) return rc;
     return launch_pdl(kern, dim3((unsigned)blocks), dim3(32 * NW), smem, st, p, c, tm_k, tm_v, shp, sp) == cudaSuccess ? KVSINK_OK : KVSINK_ERR_CUDA;
 }
 
@@ -919,25 +919,28 @@ int launch_quantize_groups_bulk(const Params &p, const kvsink_cache &c, const __
 {
     if (p.D != QB_D || n_groups < 1) return KVSINK_ERR_UNSUPPORTED;
     const kvsink_static_params none = {nullptr, nullptr, nullptr, nullptr};
-    if (p.bits == 2 && p.G == 128) return launch_bulk<2, 128>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, edges);
-    if (p.bits == 2 && p.G == 64) return launch_bulk<2, 64>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, edges);
-    if (p.bits == 3 && p.G == 64) return launch_bulk<3, 64>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, edges);
-    if (p.bits == 4 && p.G == 128) return launch_bulk<4, 128>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, edges);
-    if (p.bits == 4 && p.G == 64) return launch_bulk<4, 64>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, edges);
+    const auto ends = [&] { return launch_append_edges(p, c, *edges, st); };
+    const LaunchBefore before = edges ? launch_before(ends) : LaunchBefore{};
+    if (p.bits == 2 && p.G == 128) return launch_bulk<2, 128>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
+    if (p.bits == 2 && p.G == 64) return launch_bulk<2, 64>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
+    if (p.bits == 3 && p.G == 64) return launch_bulk<3, 64>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
+    if (p.bits == 4 && p.G == 128) return launch_bulk<4, 128>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
+    if (p.bits == 4 && p.G == 64) return launch_bulk<4, 64>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
     return KVSINK_ERR_UNSUPPORTED;
 }
 
 // The same for static parameters: n_groups spans of G tokens (G only sets the shape of the work items here), the first at a
 // multiple of G.  Shapes without a bulk kernel return KVSINK_ERR_UNSUPPORTED and the caller uses the tile kernels.
 int launch_quantize_static_bulk(const Params &p, const kvsink_cache &c, const kvsink_static_params &sp, const __half *k_src, const __half *v_src,
-                                int first_token, int n_groups, int64_t sb, int64_t sh, int64_t stt, cudaStream_t st)
+                                int first_token, int n_groups, int64_t sb, int64_t sh, int64_t stt, LaunchBefore before,
+                                cudaStream_t st)
 {
     if (p.D != QB_D || n_groups < 1 || first_token % p.G) return KVSINK_ERR_UNSUPPORTED;
-    if (p.bits == 2 && p.G == 128) return launch_bulk<2, 128, 1>(p, c, sp, k_src, v_src, first_token, n_groups, sb, sh, stt, st);
-    if (p.bits == 2 && p.G == 64) return launch_bulk<2, 64, 1>(p, c, sp, k_src, v_src, first_token, n_groups, sb, sh, stt, st);
-    if (p.bits == 3 && p.G == 64) return launch_bulk<3, 64, 1>(p, c, sp, k_src, v_src, first_token, n_groups, sb, sh, stt, st);
-    if (p.bits == 4 && p.G == 128) return launch_bulk<4, 128, 1>(p, c, sp, k_src, v_src, first_token, n_groups, sb, sh, stt, st);
-    if (p.bits == 4 && p.G == 64) return launch_bulk<4, 64, 1>(p, c, sp, k_src, v_src, first_token, n_groups, sb, sh, stt, st);
+    if (p.bits == 2 && p.G == 128) return launch_bulk<2, 128, 1>(p, c, sp, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
+    if (p.bits == 2 && p.G == 64) return launch_bulk<2, 64, 1>(p, c, sp, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
+    if (p.bits == 3 && p.G == 64) return launch_bulk<3, 64, 1>(p, c, sp, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
+    if (p.bits == 4 && p.G == 128) return launch_bulk<4, 128, 1>(p, c, sp, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
+    if (p.bits == 4 && p.G == 64) return launch_bulk<4, 64, 1>(p, c, sp, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
     return KVSINK_ERR_UNSUPPORTED;
 }
 
@@ -945,14 +948,15 @@ int launch_quantize_static_bulk(const Params &p, const kvsink_cache &c, const kv
 // 3 bit has no form here: its bulk items need 64-token spans, which give two channel groups per row, and the decode side of
 // per-token keys takes one group at 3 bit.
 int launch_quantize_pertoken_bulk(const Params &p, const kvsink_cache &c, const __half *k_src, const __half *v_src, int first_token, int n_groups,
-                                  int64_t sb, int64_t sh, int64_t stt, cudaStream_t st)
+                                  int64_t sb, int64_t sh, int64_t stt, LaunchBefore before,
+                                cudaStream_t st)
 {
     if (p.D != QB_D || n_groups < 1 || first_token % p.G) return KVSINK_ERR_UNSUPPORTED;
     const kvsink_static_params none = {nullptr, nullptr, nullptr, nullptr};
-    if (p.bits == 2 && p.G == 128) return launch_bulk<2, 128, 2>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st);
-    if (p.bits == 2 && p.G == 64) return launch_bulk<2, 64, 2>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st);
-    if (p.bits == 4 && p.G == 128) return launch_bulk<4, 128, 2>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st);
-    if (p.bits == 4 && p.G == 64) return launch_bulk<4, 64, 2>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st);
+    if (p.bits == 2 && p.G == 128) return launch_bulk<2, 128, 2>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
+    if (p.bits == 2 && p.G == 64) return launch_bulk<2, 64, 2>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
+    if (p.bits == 4 && p.G == 128) return launch_bulk<4, 128, 2>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
+    if (p.bits == 4 && p.G == 64) return launch_bulk<4, 64, 2>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
     return KVSINK_ERR_UNSUPPORTED;
 }
 

@@ -145,3 +145,13 @@ def test_static_shapes_without_decode(d, bits, group):
     assert kv.read_status(gc) == 0
     check_guards(gs)
     check_guards(gc)
+
+
+# static pairs and per-token keys: ragged ends in one launch ahead, with few tokens, whole tiles and both
+@pytest.mark.parametrize("scheme", ["static", "per_token"])
+@pytest.mark.parametrize("chunks", [(5 * 128 + 11, 3, 90), (130, 6 * 128 + 30), (16, 4 * 128 + 112, 1, 15)])
+def test_flat_chunks_of_many_units(scheme, chunks):
+    import test_gpu_calibrated
+    import test_gpu_pertoken
+    wl = TINY.scaled(bits=3, head_dim=128, group=128, n_q_heads=8, n_kv_heads=8, batch=8, seq=sum(chunks), topk=40, pfn_n=1, seed=36000 + chunks[0])
+    (test_gpu_calibrated if scheme == "static" else test_gpu_pertoken)._both(wl, chunks=chunks)
