@@ -264,17 +264,22 @@ struct QbGeo {
     static constexpr int Gv = G < D ? G : D, NGv = D / Gv;
     static constexpr int NS = 2 * D / G;          // statistic sets per item: MT for keys, 2 * NGv for values
     static constexpr int KPL = NS / 2;            // keys per lane
-    static constexpr int KROWB = 2 * KC;          // bytes per row of a key item in shared memory
+    static constexpr bool KWIDE = KC > 64;        // a key item has all channels: two boxes of 64, as a value item
+    static constexpr int KROWB = KWIDE ? 128 : 2 * KC;   // bytes per row of a key item's box in shared memory
+    // A word of the 3-bit codes' high bits covers 64 channels, twice a key item's of 128-token groups: a warp takes the two items of
+    // such a pair one after the other and keeps the first one's part of the words
+    static constexpr bool PAIRED = BITS == 3 && KC < 64;
     // per warp and for each of the item's 16 * NS keys: three fp16 thresholds (2 bit), or a coder (stored by key pair)
     // and (scale, zero)
-    // (static pairs: also the two fp16 clamp bounds of every key)
-    static constexpr int SCRATCH = BITS == 2 ? 3 * 16 * NS * 2 : 8 * NS * (int)sizeof(QbCoder2) + 16 * NS * (int)sizeof(float2) + 2 * 16 * NS * 2;
+    // (static pairs: also the two fp16 clamp bounds of every key); then those parts of words, one a tile and lane
+    static constexpr int CODER = BITS == 2 ? 3 * 16 * NS * 2 : 8 * NS * (int)sizeof(QbCoder2) + 16 * NS * (int)sizeof(float2) + 2 * 16 * NS * 2;
+    static constexpr int SCRATCH = CODER + (PAIRED ? NT * 128 : 0);
     static constexpr int TILE_BYTES = 256 * BITS, ROW_BYTES = 16 * BITS;   // packed tile of 16 tokens x 128 channels
     // warps per block, each with one stage, one mbarrier and its scratch: 20 (96 registers per thread) for the 2-bit
-    // coder; 16 (128 registers) for the 3- and 4-bit coder, which spills at 96 and measures 9 % faster this way
-    static constexpr int WARPS = BITS == 2 ? 20 : 16;
-    static_assert(G == 64 || G == 128, "group size");
-    static_assert(BITS != 3 || G == 64, "a 3-bit key item must cover whole words of the high-bit section (64 channels)");
+    // coder; 16 (128 registers) for the 3- and 4-bit coder, which spills at 96 and measures 9 % faster this way, and for the
+    // twice as many statistics of 32-token groups
+    static constexpr int WARPS = BITS == 2 && G > 32 ? 20 : 16;
+    static_assert(G == 32 || G == 64 || G == 128, "group size");
     static_assert(MT == NS && 2 * NGv == NS, "statistic sets");
 };
 
@@ -318,7 +323,7 @@ __device__ __forceinline__ void qb_load_mask(const Params &p, const kvsink_cache
         mw.w0 = __ldg(bm + ((p0 + 32 * q_sub) >> 5));
     } else if (q_sub < QbGeo<G>::NK) {
         mw.w0 = __ldg(bm + (p0 >> 5));
-        mw.w1 = __ldg(bm + (p0 >> 5) + 1);
+        if (G >= 64) mw.w1 = __ldg(bm + (p0 >> 5) + 1);
         if (G == 128) { mw.w2 = __ldg(bm + (p0 >> 5) + 2); mw.w3 = __ldg(bm + (p0 >> 5) + 3); }
     } else {
         mw.w0 = __ldg(bm + ((p0 + 32 * (q_sub - QbGeo<G>::NK)) >> 5));
@@ -331,7 +336,7 @@ __device__ __forceinline__ void qb_issue(const CUtensorMap *tm_k, const CUtensor
 {
     using Geo = QbGeo<G>;
     qb_mbar_expect_tx(bar, QB_STAGE_BYTES);
-    if (KSLAB && q.sub < Geo::NK) {               // per-token keys: the key map has the value map's box
+    if ((KSLAB || Geo::KWIDE) && q.sub < Geo::NK) {   // per-token keys, or all channels in an item: the key map has the value map's box
         const int tok = q.grp * G + 32 * q.sub;
         qb_tma_load(dst, tm_k, 0, tok, q.h, q.b, bar);
         qb_tma_load(dst + 4096, tm_k, 64, tok, q.h, q.b, bar);
@@ -396,7 +401,7 @@ quantize_bulk_kernel(Params p, kvsink_cache c, const __grid_constant__ CUtensorM
     //           matrix 8T + m = tile T x channels [16m, 16m+16): row 16T + rr + 8 (mj >> 1), chunk 2 (m & 3) + (mj & 1)
     //   keys:   KROWB-byte rows of KC channels; matrix NT*mi + T: row 16T + rr + 8 (mj & 1), chunk 2 mi + (mj >> 1)
     const uint32_t lane_v = (uint32_t)((rr + 8 * (mj >> 1)) * 128 + ((((mj & 1) ^ (rr & 1)) | (rr & 6)) << 4));
-    const uint32_t lane_ks = (uint32_t)((rr + 8 * (mj & 1)) * 128 + ((((mj >> 1) ^ (rr & 1)) | (rr & 6)) << 4));   // key slabs (MODE 2): value layout, plain load
+    const uint32_t lane_ks = (uint32_t)((rr + 8 * (mj & 1)) * 128 + ((((mj >> 1) ^ (rr & 1)) | (rr & 6)) << 4));   // key items laid out like values (MODE 2, 32-token groups): plain load
     const uint32_t lane_k = Geo::KROWB == 64 ? (uint32_t)((rr + 8 * (mj & 1)) * 64 + ((((mj >> 1) ^ ((rr >> 1) & 1)) | ((rr >> 1) & 2)) << 4))
                                              : (uint32_t)((rr + 8 * (mj & 1)) * 128 + ((((mj >> 1) ^ (rr & 1)) | (rr & 6)) << 4));
 
@@ -407,12 +412,15 @@ quantize_bulk_kernel(Params p, kvsink_cache c, const __grid_constant__ CUtensorM
     unsigned char *my_stage = stages + (size_t)warp * QB_STAGE_BYTES;
     uint64_t *my_full = full + warp;
 
-    // the block's items: in round r the block takes NW consecutive items, one per warp
-    const unsigned id_step = gridDim.x * NW;
-    const QbPos step = qb_decode<G>(id_step, sh.n_groups, p.Hkv);
-    unsigned id = blockIdx.x * NW + warp;
+    // the block's items: in round r the block takes NW consecutive items, one per warp, or NW pairs of items
+    constexpr unsigned PAIR = Geo::PAIRED ? 2u : 1u;
+    const unsigned id_step = PAIR * gridDim.x * NW - (PAIR - 1u);               // to the next item; from a pair's first one: 1
+    const QbPos step = qb_decode<G>(id_step, sh.n_groups, p.Hkv), one = {1, 0, 0, 0};
+    unsigned id = PAIR * (blockIdx.x * NW + warp);
+    auto after = [&](unsigned i) { return Geo::PAIRED && !(i & 1u) ? i + 1u : i + id_step; };
     QbPos cur = qb_decode<G>(id, sh.n_groups, p.Hkv);
-    QbPos nxt = qb_advance<G>(cur, step, sh.n_groups, p.Hkv);
+    QbPos nxt = qb_advance<G>(cur, Geo::PAIRED ? one : step, sh.n_groups, p.Hkv);
+    uint32_t *high_part = (uint32_t *)(scratch + (size_t)warp * Geo::SCRATCH + Geo::CODER) + lane;
     QbMask mw;
     mw.w0 = mw.w1 = mw.w2 = mw.w3 = 0u;
     if (id < sh.n_items) {
@@ -420,11 +428,12 @@ quantize_bulk_kernel(Params p, kvsink_cache c, const __grid_constant__ CUtensorM
         if (lane == 0) qb_issue<G, MODE == 2>(&tm_k, &tm_v, cur, my_stage, my_full);
     }
     unsigned phase = 0;                           // parity of the stage's current use
-    for (; id < sh.n_items; id += id_step, phase ^= 1u) {
+    for (unsigned next_id; id < sh.n_items; id = next_id, phase ^= 1u) {
+        next_id = after(id);
         // sink bits of the warp's next item, fetched while this one is processed
         QbMask mw_next;
         mw_next.w0 = mw_next.w1 = mw_next.w2 = mw_next.w3 = 0u;
-        if (id + id_step < sh.n_items) qb_load_mask<G, MODE == 2>(p, c, nxt.sub, nxt.grp, nxt.b, sh.first_token, mw_next);
+        if (next_id < sh.n_items) qb_load_mask<G, MODE == 2>(p, c, nxt.sub, nxt.grp, nxt.b, sh.first_token, mw_next);
         if (!__all_sync(0xffffffffu, qb_wait(my_full, phase))) {
             if (lane == 0) atomicOr(c.status, KVSINK_STATUS_TIMEOUT);
             break;
@@ -456,7 +465,8 @@ quantize_bulk_kernel(Params p, kvsink_cache c, const __grid_constant__ CUtensorM
 #pragma unroll
             for (int u = 0; u < 16; ++u) {
                 const int mi = u / NT, T = u % NT;
-                qb_ldmatrix_x4(a[u], ((stage + lane_k) ^ (mi << 5)) + T * 16 * Geo::KROWB);
+                if constexpr (Geo::KWIDE) qb_ldmatrix_x4(a[u], ((stage + lane_ks) ^ ((mi & 3) << 5)) + T * 2048 + (mi >> 2) * 4096);
+                else qb_ldmatrix_x4(a[u], ((stage + lane_k) ^ (mi << 5)) + T * 16 * Geo::KROWB);
             }
         }
         const bool has_sink = (mw.w0 | mw.w1 | mw.w2 | mw.w3) != 0u;   // the same in every lane; false for almost every item
@@ -491,7 +501,7 @@ quantize_bulk_kernel(Params p, kvsink_cache c, const __grid_constant__ CUtensorM
                 __half *dst = side + ((size_t)unit * p.cap + my) * D;
                 uint32_t src;
                 int n16, off;                     // 16-byte chunks of the row held by this item, first channel
-                if (slab) {
+                if (slab || Geo::KWIDE) {
                     src = stage + (lane >> 3) * 4096 + r * 128 + (((lane & 7) ^ (r & 7)) << 4);
                     n16 = 16; off = 0;
                 } else {
@@ -547,9 +557,9 @@ quantize_bulk_kernel(Params p, kvsink_cache c, const __grid_constant__ CUtensorM
         }
         // every lane has consumed its ldmatrix results: the stage can take the warp's next item, which streams in
         // while this one is coded from registers
-        const QbPos nn = qb_advance<G>(nxt, step, sh.n_groups, p.Hkv);
+        const QbPos nn = qb_advance<G>(nxt, Geo::PAIRED && !(next_id & 1u) ? one : step, sh.n_groups, p.Hkv);
         __syncwarp();
-        if (lane == 0 && id + id_step < sh.n_items) qb_issue<G, MODE == 2>(&tm_k, &tm_v, nxt, my_stage, my_full);
+        if (lane == 0 && next_id < sh.n_items) qb_issue<G, MODE == 2>(&tm_k, &tm_v, nxt, my_stage, my_full);
 
         if (kslab) {
             // the other channels of a token row live in the other half of the register and in the other lanes of the quad
@@ -565,25 +575,27 @@ quantize_bulk_kernel(Params p, kvsink_cache c, const __grid_constant__ CUtensorM
                     }
                     mn[s][ab] = lo2; mx[s][ab] = hi2;
                 }
-        } else if (NS == 4 && MODE != 1) {
-            // The other rows of a column live in the lanes that differ in bits 2..4.  Eight (set, side) pairs for the eight
+        } else if (NS >= 4 && MODE != 1) {
+            // The other rows of a column live in the lanes that differ in bits 2..4.  2 NS (set, side) pairs for the eight
             // lanes of a column group: each exchange halves what a lane carries (it keeps the half its own bit names and sends
-            // the other), so that lane g ends with the extremes of pair g alone -- both of its keys, one per half
-            uint32_t vn[8], vx[8];
+            // the other), so that lane g ends with the extremes of its NS / 4 pairs alone -- both keys of each, one per half
+            uint32_t vn[2 * NS], vx[2 * NS];
 #pragma unroll
-            for (int c8 = 0; c8 < 8; ++c8) { vn[c8] = mn[(c8 >> 1) % NS][c8 & 1]; vx[c8] = mx[(c8 >> 1) % NS][c8 & 1]; }
+            for (int c = 0; c < 2 * NS; ++c) { vn[c] = mn[c >> 1][c & 1]; vx[c] = mx[c >> 1][c & 1]; }
 #pragma unroll
-            for (int w = 4; w >= 1; w >>= 1) {
-                const bool up = (lane & (4 * w)) != 0;     // bit 4, 3, 2 of the lane = bit 2, 1, 0 of g
+            for (int w = NS; w >= NS / 4; w >>= 1) {
+                const int o = 16 * w / NS;                 // 16, 8, 4: bit 2, 1, 0 of g
+                const bool up = (lane & o) != 0;
 #pragma unroll
                 for (int i = 0; i < w; ++i) {
                     const uint32_t sn = up ? vn[i] : vn[w + i], kn = up ? vn[w + i] : vn[i];
                     const uint32_t sx = up ? vx[i] : vx[w + i], kx = up ? vx[w + i] : vx[i];
-                    vn[i] = qb_hmin2(kn, __shfl_xor_sync(0xffffffffu, sn, 4 * w));
-                    vx[i] = qb_hmax2(kx, __shfl_xor_sync(0xffffffffu, sx, 4 * w));
+                    vn[i] = qb_hmin2(kn, __shfl_xor_sync(0xffffffffu, sn, o));
+                    vx[i] = qb_hmax2(kx, __shfl_xor_sync(0xffffffffu, sx, o));
                 }
             }
-            mn[0][0] = vn[0]; mx[0][0] = vx[0];
+#pragma unroll
+            for (int j = 0; j < NS / 4; ++j) { mn[j][0] = vn[j]; mx[j][0] = vx[j]; }
         } else {
         // the other rows of a column live in the lanes that differ in bits 2..4
 #pragma unroll
@@ -601,13 +613,13 @@ quantize_bulk_kernel(Params p, kvsink_cache c, const __grid_constant__ CUtensorM
 #pragma unroll
         for (int j = 0; j < KPL; ++j) {
             // the lane's j-th key.  Per-token keys: lane (g, t) takes the token of tile t >> 1, rows g + 8 (t & 1), channel group j
-            // With eight (set, side) pairs (NS = 4) the exchange above left lane g with pair g: its keys are the two halves.
-            const bool scat = NS == 4 && MODE != 1 && !kslab;
-            const int kk = scat ? 2 * g + j : g + 8 * j;
+            // After the exchange above (NS >= 4) lane g has KPL consecutive keys, the halves of its pairs.
+            const bool scat = NS >= 4 && MODE != 1 && !kslab;
+            const int kk = scat ? KPL * g + j : g + 8 * j;
             const int s_ = kslab ? (t4 >> 1) * NGv + j : kk >> 2, ab_ = kslab ? (t4 & 1) : (kk >> 1) & 1, e_ = kslab ? 0 : kk & 1;
             uint32_t smn = 0, smx = 0;
             if (scat) {
-                smn = mn[0][0]; smx = mx[0][0];
+                smn = mn[j >> 1][0]; smx = mx[j >> 1][0];
             } else {
 #pragma unroll
                 for (int s = 0; s < NS; ++s)
@@ -705,14 +717,19 @@ quantize_bulk_kernel(Params p, kvsink_cache c, const __grid_constant__ CUtensorM
                 }
             }
             // ---- packed words: bytes (even matrix lo, odd matrix lo, even matrix hi, odd matrix hi) ----
-            if (slab) {
+            auto whole_tiles = [&](auto at) {          // at(T, m): register of matrix m of tile T
 #pragma unroll
                 for (int T = 0; T < 2; ++T) {
                     uint4 w;
-                    w.x = __byte_perm(bits[8 * T + 0], bits[8 * T + 1], 0x6240); w.y = __byte_perm(bits[8 * T + 2], bits[8 * T + 3], 0x6240);
-                    w.z = __byte_perm(bits[8 * T + 4], bits[8 * T + 5], 0x6240); w.w = __byte_perm(bits[8 * T + 6], bits[8 * T + 7], 0x6240);
+                    w.x = __byte_perm(bits[at(T, 0)], bits[at(T, 1)], 0x6240); w.y = __byte_perm(bits[at(T, 2)], bits[at(T, 3)], 0x6240);
+                    w.z = __byte_perm(bits[at(T, 4)], bits[at(T, 5)], 0x6240); w.w = __byte_perm(bits[at(T, 6)], bits[at(T, 7)], 0x6240);
                     *(uint4 *)(codes + T * Geo::TILE_BYTES + lane * 16) = w;
                 }
+            };
+            if (slab) {
+                whole_tiles([](int T, int m) { return 8 * T + m; });
+            } else if constexpr (Geo::KWIDE) {
+                whole_tiles([](int T, int m) { return NT * m + T; });
             } else {
 #pragma unroll
                 for (int T = 0; T < NT; ++T) {
@@ -801,24 +818,29 @@ quantize_bulk_kernel(Params p, kvsink_cache c, const __grid_constant__ CUtensorM
             __syncwarp();   // the scratch is rewritten by the next item
             // ---- packed words.  4 bit: word m of a lane is matrix m, planes of four words.  3 bit: low section as for
             //      2 bit (word m >> 1, byte m & 1 of each half), high section at 512 bytes (word m >> 2, two per lane) ----
-            if (slab) {
+            auto whole_tiles = [&](auto at) {          // at(T, m): register of matrix m of tile T
 #pragma unroll
                 for (int T = 0; T < 2; ++T) {
                     uint8_t *dst = codes + T * Geo::TILE_BYTES;
                     if constexpr (BITS == 4) {
-                        *(uint4 *)(dst + lane * 16) = make_uint4(lo[8 * T], lo[8 * T + 1], lo[8 * T + 2], lo[8 * T + 3]);
-                        *(uint4 *)(dst + 512 + lane * 16) = make_uint4(lo[8 * T + 4], lo[8 * T + 5], lo[8 * T + 6], lo[8 * T + 7]);
+                        *(uint4 *)(dst + lane * 16) = make_uint4(lo[at(T, 0)], lo[at(T, 1)], lo[at(T, 2)], lo[at(T, 3)]);
+                        *(uint4 *)(dst + 512 + lane * 16) = make_uint4(lo[at(T, 4)], lo[at(T, 5)], lo[at(T, 6)], lo[at(T, 7)]);
                     } else {
                         uint4 w;
-                        w.x = lo[8 * T + 0] | (lo[8 * T + 1] << 8); w.y = lo[8 * T + 2] | (lo[8 * T + 3] << 8);
-                        w.z = lo[8 * T + 4] | (lo[8 * T + 5] << 8); w.w = lo[8 * T + 6] | (lo[8 * T + 7] << 8);
+                        w.x = lo[at(T, 0)] | (lo[at(T, 1)] << 8); w.y = lo[at(T, 2)] | (lo[at(T, 3)] << 8);
+                        w.z = lo[at(T, 4)] | (lo[at(T, 5)] << 8); w.w = lo[at(T, 6)] | (lo[at(T, 7)] << 8);
                         *(uint4 *)(dst + lane * 16) = w;
                         uint2 h;
-                        h.x = hi[8 * T + 0] | hi[8 * T + 1] | hi[8 * T + 2] | hi[8 * T + 3];
-                        h.y = hi[8 * T + 4] | hi[8 * T + 5] | hi[8 * T + 6] | hi[8 * T + 7];
+                        h.x = hi[at(T, 0)] | hi[at(T, 1)] | hi[at(T, 2)] | hi[at(T, 3)];
+                        h.y = hi[at(T, 4)] | hi[at(T, 5)] | hi[at(T, 6)] | hi[at(T, 7)];
                         *(uint2 *)(dst + 512 + lane * 8) = h;
                     }
                 }
+            };
+            if (slab) {
+                whole_tiles([](int T, int m) { return 8 * T + m; });
+            } else if constexpr (Geo::KWIDE) {
+                whole_tiles([](int T, int m) { return NT * m + T; });
             } else {
 #pragma unroll
                 for (int T = 0; T < NT; ++T) {
@@ -827,6 +849,11 @@ quantize_bulk_kernel(Params p, kvsink_cache c, const __grid_constant__ CUtensorM
                         *(uint4 *)(dst + sub * 512 + lane * 16) = make_uint4(lo[T], lo[NT + T], lo[2 * NT + T], lo[3 * NT + T]);
                     } else if constexpr (BITS == 4) {              // matrices 2 sub, 2 sub + 1: half of a lane's plane entry
                         *(uint2 *)(dst + (sub >> 1) * 512 + lane * 16 + (sub & 1) * 8) = make_uint2(lo[T], lo[NT + T]);
+                    } else if constexpr (Geo::PAIRED) {            // 3 bit, 32 channels: one low word and half of a high word
+                        *(uint32_t *)(dst + lane * 16 + sub * 4) = lo[T] | (lo[NT + T] << 8);
+                        const uint32_t h = hi[T] | hi[NT + T];
+                        if (sub & 1) *(uint32_t *)(dst + 512 + lane * 8 + (sub >> 1) * 4) = high_part[32 * T] | h;
+                        else high_part[32 * T] = h;
                     } else {                                       // 3 bit, 64 channels: two low words and one whole high word
                         uint2 w;
                         w.x = lo[T] | (lo[NT + T] << 8);
@@ -886,7 +913,7 @@ int launch_bulk(const Params &p, const kvsink_cache &c, const kvsink_static_para
     using Geo = QbGeo<G, BITS>;
     CUtensorMap tm_k, tm_v;
     const int T = n_groups * G;
-    if (MODE == 2) {
+    if (MODE == 2 || Geo::KWIDE) {
         if (!make_map(&tm_k, k_src, p, T, sb, sh, stt, 64, 32, CU_TENSOR_MAP_SWIZZLE_128B)) return KVSINK_ERR_UNSUPPORTED;
     } else if (!make_map(&tm_k, k_src, p, T, sb, sh, stt, Geo::KC, G, Geo::KROWB == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B))
         return KVSINK_ERR_UNSUPPORTED;
@@ -901,8 +928,15 @@ int launch_bulk(const Params &p, const kvsink_cache &c, const kvsink_static_para
     shp.after_edges = before.call != nullptr;
     const long n_items = (long)p.B * p.Hkv * n_groups * Geo::IPG;
     if (n_items >= (1L << 30)) return KVSINK_ERR_UNSUPPORTED;
+    // Few items: a warp's time for one (of a pair: for two, one after the other) is longer than the other kernels take, which put more warps on
+    // a group.  Items and us, this kernel and the other: 32-token groups, 2 bit 320 7.8 and 6.6, 512 7.2 and 8.3; 3 bit 320 9.7 and 10.3;
+    // 4 bit 320 8.9 and 8.3, 512 8.3 and 8.8; 3 bit, 128-token groups 1024 15.2 and 14.4, 1280 16.0 and 16.5, 2048 15.6 and 22.5, static pairs
+    // 1280 13.1 and 10.9, 2048 12.3 and 15.5, per-token keys 1280 15.6 and 12.0, 2048 15.7 and 18.6.  Elsewhere this one is as fast from the first
+    constexpr long least = Geo::PAIRED ? (MODE == 0 ? 1200 : 1500) : (Geo::KWIDE ? 400 : 0);
+    if (n_items < least) return KVSINK_ERR_UNSUPPORTED;
     shp.n_items = (unsigned)n_items;
-    long blocks = (n_items + NW - 1) / NW;
+    constexpr int per_round = Geo::PAIRED ? 2 * NW : NW;
+    long blocks = (n_items + per_round - 1) / per_round;
     if (blocks > 148) blocks = 148;
     if (!allow_smem(kern, smem)) return KVSINK_ERR_CUDA;
     if (before.call)
@@ -923,7 +957,11 @@ int launch_quantize_groups_bulk(const Params &p, const kvsink_cache &c, const __
     const LaunchBefore before = edges ? launch_before(ends) : LaunchBefore{};
     if (p.bits == 2 && p.G == 128) return launch_bulk<2, 128>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
     if (p.bits == 2 && p.G == 64) return launch_bulk<2, 64>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
+    if (p.bits == 2 && p.G == 32) return launch_bulk<2, 32>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
+    if (p.bits == 3 && p.G == 32) return launch_bulk<3, 32>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
+    if (p.bits == 4 && p.G == 32) return launch_bulk<4, 32>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
     if (p.bits == 3 && p.G == 64) return launch_bulk<3, 64>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
+    if (p.bits == 3 && p.G == 128) return launch_bulk<3, 128>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
     if (p.bits == 4 && p.G == 128) return launch_bulk<4, 128>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
     if (p.bits == 4 && p.G == 64) return launch_bulk<4, 64>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
     return KVSINK_ERR_UNSUPPORTED;
@@ -939,14 +977,14 @@ int launch_quantize_static_bulk(const Params &p, const kvsink_cache &c, const kv
     if (p.bits == 2 && p.G == 128) return launch_bulk<2, 128, 1>(p, c, sp, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
     if (p.bits == 2 && p.G == 64) return launch_bulk<2, 64, 1>(p, c, sp, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
     if (p.bits == 3 && p.G == 64) return launch_bulk<3, 64, 1>(p, c, sp, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
+    if (p.bits == 3 && p.G == 128) return launch_bulk<3, 128, 1>(p, c, sp, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
     if (p.bits == 4 && p.G == 128) return launch_bulk<4, 128, 1>(p, c, sp, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
     if (p.bits == 4 && p.G == 64) return launch_bulk<4, 64, 1>(p, c, sp, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
     return KVSINK_ERR_UNSUPPORTED;
 }
 
 // The same for per-token keys (keys quantized like values; the pairs go to the key parameter arrays in the value parameters' shape).
-// 3 bit has no form here: its bulk items need 64-token spans, which give two channel groups per row, and the decode side of
-// per-token keys takes one group at 3 bit.
+// 3 bit: one channel group a row, since the decode side of per-token keys takes no more.
 int launch_quantize_pertoken_bulk(const Params &p, const kvsink_cache &c, const __half *k_src, const __half *v_src, int first_token, int n_groups,
                                   int64_t sb, int64_t sh, int64_t stt, LaunchBefore before,
                                 cudaStream_t st)
@@ -955,6 +993,7 @@ int launch_quantize_pertoken_bulk(const Params &p, const kvsink_cache &c, const 
     const kvsink_static_params none = {nullptr, nullptr, nullptr, nullptr};
     if (p.bits == 2 && p.G == 128) return launch_bulk<2, 128, 2>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
     if (p.bits == 2 && p.G == 64) return launch_bulk<2, 64, 2>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
+    if (p.bits == 3 && p.G == 128) return launch_bulk<3, 128, 2>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
     if (p.bits == 4 && p.G == 128) return launch_bulk<4, 128, 2>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
     if (p.bits == 4 && p.G == 64) return launch_bulk<4, 64, 2>(p, c, none, k_src, v_src, first_token, n_groups, sb, sh, stt, st, before);
     return KVSINK_ERR_UNSUPPORTED;

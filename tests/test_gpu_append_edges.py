@@ -147,7 +147,38 @@ def test_static_shapes_without_decode(d, bits, group):
     check_guards(gc)
 
 
-# static pairs and per-token keys: ragged ends in one launch ahead, with few tokens, whole tiles and both
+# whole groups of 32 tokens, and of 128 at 3 bit, go to the bulk quantizer from 400 and 1200 work items (4096 elements) on; two rounds of items a warp.
+# 3 bit: two items of 32 channels share the words of the high bits
+def _extremes(x):
+    x[:, :, :, 1] = 0.0
+    x[:, :, :, 2] = -2.5
+    x[:, :, :, 65] *= 300.0
+    x[:, :, :, 66] = 40.0 + x[:, :, :, 66] * 0.01
+    x[:, :, 5:9] = 7.0
+    x[:, :, 40] *= 1e-3
+    return x.clamp_(-60000, 60000)
+
+
+@pytest.mark.parametrize("bits,group,batch,heads,T", [(2, 32, 8, 8, 700), (3, 32, 8, 8, 650), (4, 32, 4, 16, 671), (2, 32, 7, 3, 330), (3, 128, 4, 8, 5 * 128 + 70),
+                                                      (3, 128, 8, 8, 12 * 128)])
+def test_group_sizes_of_the_bulk_quantizer(bits, group, batch, heads, T):
+    wl = TINY.scaled(bits=bits, head_dim=128, group=group, n_q_heads=heads, n_kv_heads=heads, batch=batch, seq=T, topk=40, pfn_n=3, seed=35000 + bits + group + T)
+    ocfg, gcfg = configs(wl)
+    H = synth.make_hidden(wl, "cuda")
+    K, V = (_extremes(x) for x in synth.make_kv(wl, 0, "cuda"))
+    gs = guard(kv.SinkSet(gcfg), SINK_BUFFERS)
+    kv.predict_sinks(gcfg, H, gs)
+    gc, oc = guard(kv.KVCache(gcfg, gs), CACHE_BUFFERS), oracle.Cache(ocfg, *oracle.predict_sinks(ocfg, np16(H)))
+    for at, end in ((0, group + 5), (group + 5, T)):
+        kv.quantize_append(gcfg, gc, K[:, :, at:end], V[:, :, at:end])
+        oracle.quantize_append(ocfg, oc, np16(K[:, :, at:end]), np16(V[:, :, at:end]))
+        compare_cache(gc, oc, wl, f"after {end} tokens: ")
+    assert kv.read_status(gc) == 0
+    check_guards(gs)
+    check_guards(gc)
+
+
+# the same with static pairs and per-token keys (1500 items): ragged ends in one launch ahead, with few tokens, whole tiles and both
 @pytest.mark.parametrize("scheme", ["static", "per_token"])
 @pytest.mark.parametrize("chunks", [(5 * 128 + 11, 3, 90), (130, 6 * 128 + 30), (16, 4 * 128 + 112, 1, 15)])
 def test_flat_chunks_of_many_units(scheme, chunks):
