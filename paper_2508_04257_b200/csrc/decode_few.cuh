@@ -79,13 +79,13 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
     extern __shared__ __align__(128) unsigned char smem_raw[];
     float *qs = (float *)smem_raw;                                   // [R][D] q * log2e/sqrt(D)
     __half *q16 = (__half *)(qs + R * D);                            // [R][D] q as given
-    uint64_t *bars = (uint64_t *)(smem_raw + Plan::Q_BYTES + DEC_WARPS * Plan::B_BYTES);   // [warps][8]: chunk slots, then the parameter slot
+    uint64_t *bars = (uint64_t *)(smem_raw + Plan::Q_BYTES + DEC_WARPS * Plan::B_BYTES);   // [warps]: of the parameter slot
     unsigned char *ring_all = smem_raw + Plan::FIXED;                // [warps][WARP_RING]; later reused for the partials
     float *part = (float *)ring_all;                                 // [2*warps][nq][D+2]
 
-    const uint32_t cbar = smem_addr(bars + warp * 8), pbar = cbar + 4 * 8;
+    const uint32_t pbar = smem_addr(bars + warp);
     if (lane == 0) {
-        for (int i = 0; i < 5; ++i) mbar_init(cbar + 8 * i, 1);
+        mbar_init(pbar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     // everything above overlaps the tail of the kernel before this one; nothing it may have written is read before this point
@@ -299,7 +299,7 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
     };
 
     // ---- the warps take contiguous, nearly equal ranges of the split's groups; a warp's chunks (CT tiles each) are consecutive in
-    //      memory and arrive through a ring of NSLOT bulk-copy slots filled NSLOT - 1 chunks ahead by lane 0; the key parameters
+    //      memory and arrive through a ring of NSLOT slots filled NSLOT - 1 chunks ahead; the key parameters
     //      of a group arrive one group ahead through one more slot ----
     const int g_begin = split * groups_per_split, g_end = min(n_groups, g_begin + groups_per_split);
     const int g_cnt = max(g_end - g_begin, 0);
@@ -314,21 +314,13 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
     const uint32_t ring_s = smem_addr(ring), kp_s = smem_addr(kp_ring);
     auto issue_chunk = [&]() {
         const int slot = iss & (NSLOT - 1);
-        // debug builds: the chunk must lie inside the unit's code arrays (a skipped copy ends in the wait's time-out)
+        // debug builds: the chunk must lie inside the unit's code arrays
         const bool inside = in_bounds((size_t)iss_kv + KV_BYTES <= (size_t)p.max_seq * p.row_bytes, c.status);
-        const uint32_t dst = ring_s + slot * SLOT_BYTES, bar = cbar + 8 * slot;
-        if (lane == 0 && inside) {
-            mbar_expect_tx(bar, CAL ? 2 * KV_BYTES : SLOT_BYTES);
-            bulk_g2s(dst, kc_base + iss_kv, KV_BYTES, bar);
-            bulk_g2s(dst + KV_BYTES, vc_base + iss_kv, KV_BYTES, bar);
-            if constexpr (!CAL) {
-                bulk_g2s(dst + 2 * KV_BYTES, (const unsigned char *)vs_base + iss_sz, SZ_BYTES, bar);
-                bulk_g2s(dst + 2 * KV_BYTES + SZ_BYTES, (const unsigned char *)vz_base + iss_sz, SZ_BYTES, bar);
-            }
-            if constexpr (KT) {
-                bulk_g2s(dst + 2 * KV_BYTES + 2 * SZ_BYTES, (const unsigned char *)ktok_s_base + iss_sz, SZ_BYTES, bar);
-                bulk_g2s(dst + 2 * KV_BYTES + 3 * SZ_BYTES, (const unsigned char *)ktok_z_base + iss_sz, SZ_BYTES, bar);
-            }
+        const uint32_t dst = ring_s + slot * SLOT_BYTES;
+        if (inside) {
+            copy_words<KV_BYTES>(dst, kc_base + iss_kv, lane);
+            copy_words<KV_BYTES>(dst + KV_BYTES, vc_base + iss_kv, lane);
+            if constexpr (!CAL) copy_params<SZ_BYTES, KT ? 4 : 2>(dst + 2 * KV_BYTES, vs_base, vz_base, ktok_s_base, ktok_z_base, iss_sz, lane);
         }
         ++iss;
         iss_kv += KV_BYTES;
@@ -351,7 +343,10 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
     };
     if (my_groups > 0) {
         if (!FLAT) issue_params(0);
-        for (int i = 0; i < NSLOT - 1 && iss < n_chunks; ++i) issue_chunk();
+        for (int i = 0; i < NSLOT - 1; ++i) {      // a group of copies a chunk, empty ones behind the last
+            if (iss < n_chunks) issue_chunk();
+            copies_commit();
+        }
     }
     float cal_sv[NGv], cal_zv[NGv];       // static value parameters of the KV head
 #pragma unroll
@@ -456,8 +451,6 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
                 if (!wait_bar(pbar, (unsigned)gi & 1u)) { stream_ok = false; break; }
 #pragma unroll
                 for (int e = 0; e < CPL; ++e) { scv[e] = kp_ring[i8_ch[e]]; zev[e] = kp_ring[D + i8_ch[e]]; }
-                __syncwarp();   // the parameters are in registers: the slot can take the next group's while this one streams
-                if (gi + 1 < my_groups) issue_params(gi + 1);
             }
             // F = rint(q * scale * 2^sh) with the largest |F| of the row in [2^29, 2^30), cut into four signed bytes (radix 256): every
             // factor is kept to 2^-30 of the group's largest one (2^-26 where it is pre-divided for the upper contraction slots).  Adding
@@ -518,6 +511,8 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
                 ck *= 65536.f;
             }
             __syncwarp();
+            // every lane's parameters have gone into sums over the warp: the slot can take the next group's while this one streams
+            if (!FLAT && gi + 1 < my_groups) issue_params(gi + 1);
             if (R == 2) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
@@ -532,7 +527,8 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
             // refill the slot freed by the previous chunk, then wait for this chunk's bytes
             __syncwarp();
             if (iss < n_chunks) issue_chunk();
-            if (!wait_bar(cbar + 8 * slot, (unsigned)(ci / NSLOT) & 1u)) { stream_ok = false; break; }
+            copies_commit();
+            copies_wait<NSLOT - 1>();
             const uint2 mwords = mword_next;
             if (ci + 1 < n_chunks) mword_next = load_mask_words(grp * TPG + (cj + 1) * CT);   // the warp's chunks are consecutive
             const uint32_t *kt = (const uint32_t *)(ring + slot * SLOT_BYTES), *vt = kt + KV_BYTES / 4;
@@ -660,6 +656,7 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
             }
         }
     }
+    copies_wait<0>();      // the ring's space is used again
     if (!stream_ok && lane == 0) atomicOr(c.status, KVSINK_STATUS_TIMEOUT);
 
     fetch_sinks(sink_worker, 1, SB);

@@ -153,7 +153,7 @@ __device__ __forceinline__ void tile_frags(const uint32_t (&w)[Geo<BITS, D>::W],
     }
 }
 
-// ---- per-warp bulk-copy ring (TMA, cp.async.bulk) ----
+// ---- bulk copies (TMA, cp.async.bulk) ----
 // Barriers and copy destinations are passed as 32-bit shared-window addresses, converted once per warp.
 __device__ __forceinline__ void mbar_init(uint32_t bar, unsigned count)
 {
@@ -177,6 +177,45 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, unsigned
                  ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
 
+// ---- ring chunks: copies of 16 bytes a lane (cp.async), a group of them a chunk ----
+// By bulk copies (four to six a chunk, issued by one lane) a chunk took some 110 instructions, a sixth of the 148 a tile of decode_one_kernel at
+// 2 bit; so some 20.  Decode alone, us, in turn on one GPU: 8 x 32 units of 4096 tokens, 2 bit, 19.6 and 18.8; static, 3821 tokens, 16.7 and 16.2;
+// 16 x 32 of 8101, 3 bit, 103.1 and 97.8; 64 x 32 of 8192, 4 bit, 410 and 404; four heads, 9 x 8 of 9000, 2 bit, 64-token groups, 33.0 and 31.6;
+// two heads, 4 x 8 of 14512, 3 bit, 23.3 and 22.4; head size 64, 12 x 4 of 37403 with four heads 40.9 and 39.5; 1 x 8 of 256 5.35 and 5.11.
+// The parameters of a key group stay with a bulk copy, which is issued only when every lane's loads of the slot's last ones have been used: loads
+// wait in a queue behind the copies of the chunks, a bulk copy does not and has overtaken them (4 bit, 2048 units of 8192 tokens: a few outputs
+// of each call were wrong).
+__device__ __forceinline__ void copy16(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int LEFT>      // all groups but the last LEFT have arrived, for every lane of the warp
+__device__ __forceinline__ void copies_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(LEFT) : "memory");
+    __syncwarp();
+}
+template <int BYTES>
+__device__ __forceinline__ void copy_words(uint32_t dst, const uint8_t *src, int lane)
+{
+#pragma unroll
+    for (int x = 0; x < BYTES / 512; ++x) copy16(dst + 512 * x + 16 * lane, src + 512 * x + 16 * lane);
+    if (BYTES % 512 && lane < BYTES % 512 / 16) copy16(dst + BYTES / 512 * 512 + 16 * lane, src + BYTES / 512 * 512 + 16 * lane);
+}
+// BYTES from `offset` on of each of N parameter arrays, one behind the other
+template <int BYTES, int N>
+__device__ __forceinline__ void copy_params(uint32_t dst, const float *a0, const float *a1, const float *a2, const float *a3, uint32_t offset, int lane)
+{
+    constexpr int PIECES = BYTES / 16;
+#pragma unroll
+    for (int x = 0; x < N * PIECES; x += 32) {
+        const int at = x + lane, i = at / PIECES;
+        const float *base = i == 0 ? a0 : (i == 1 ? a1 : (i == 2 ? a2 : a3));
+        if (N * PIECES - x >= 32 || at < N * PIECES) copy16(dst + 16 * at, (const unsigned char *)base + offset + 16 * (at % PIECES));
+    }
+}
+
 template <int N>
 struct Count { static constexpr int value = N; };
 
@@ -198,7 +237,7 @@ struct DecodePlan {
     // query tables (fp32 scaled, fp16 as given); the same space later holds the block's record for a cluster merge
     static constexpr int Q_BYTES = (NQMAX * D * 6 > NQMAX * PS * 4 ? NQMAX * D * 6 : NQMAX * PS * 4);
     static constexpr int B_BYTES = 2 * NQMAX * BST * 2;                 // per warp: key B operand rows (>= 512 for the limb tables)
-    static constexpr int FIXED = (Q_BYTES + DEC_WARPS * B_BYTES + DEC_WARPS * 8 * 8 + 127) / 128 * 128;
+    static constexpr int FIXED = (Q_BYTES + DEC_WARPS * B_BYTES + DEC_WARPS * 8 + 127) / 128 * 128;
     static constexpr int RING = DEC_WARPS * WARP_RING, PART = 2 * DEC_WARPS * NQMAX * PS * 4;
     static constexpr int BYTES = FIXED + (RING > PART ? RING : PART);
 };
@@ -286,14 +325,14 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
     float *qs = (float *)smem_raw;                                   // [NQMAX][D] q * log2e/sqrt(D)
     __half *q16 = (__half *)(qs + NQMAX * D);                        // [NQMAX][D] q as given
     __half *Bs_all = (__half *)(smem_raw + Plan::Q_BYTES);           // [warps][2][NQMAX][BST] key B operand (hi, lo) of the group
-    uint64_t *bars = (uint64_t *)(smem_raw + Plan::Q_BYTES + DEC_WARPS * Plan::B_BYTES);   // [warps][8]: 4 chunk slots, 2 parameter slots
+    uint64_t *bars = (uint64_t *)(smem_raw + Plan::Q_BYTES + DEC_WARPS * Plan::B_BYTES);   // [warps]: of the parameter slot
     unsigned char *ring_all = smem_raw + Plan::FIXED;                // [warps][WARP_RING]; later reused for the partials
     float *part = (float *)ring_all;                                 // [2*warps][nq][D+2]
 
-    // chunk full-barriers (one per ring slot) and the parameter full-barrier of this warp, as shared-window addresses
-    const uint32_t cbar = smem_addr(bars + warp * 8), pbar = cbar + 4 * 8;
+    // the barrier of this warp's key parameters, as a shared-window address
+    const uint32_t pbar = smem_addr(bars + warp);
     if (lane == 0) {
-        for (int i = 0; i < 5; ++i) mbar_init(cbar + 8 * i, 1);
+        mbar_init(pbar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     // launched with programmatic stream serialization: everything above overlaps the tail of the kernel before this
@@ -432,7 +471,7 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
     };
 
     // ---- complete key groups of this split: the warps take contiguous, nearly equal ranges of its groups.  A warp's
-    //      chunks (CT tiles each) are consecutive in memory and arrive through a ring of NSLOT bulk-copy slots filled
+    //      chunks (CT tiles each) are consecutive in memory and arrive through a ring of NSLOT slots filled
     //      NSLOT - 1 chunks ahead by lane 0; the key parameters of a group arrive one group ahead through one more slot. ----
     const int g_begin = split * groups_per_split, g_end = min(n_groups, g_begin + groups_per_split);
     const int g_cnt = max(g_end - g_begin, 0);
@@ -449,21 +488,13 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
     const uint32_t ring_s = smem_addr(ring), kp_s = smem_addr(kp_ring);
     auto issue_chunk = [&]() {
         const int slot = iss & (NSLOT - 1);
-        // debug builds: the chunk must lie inside the unit's code arrays (a skipped copy ends in the wait's time-out)
+        // debug builds: the chunk must lie inside the unit's code arrays
         const bool inside = in_bounds((size_t)iss_kv + KV_BYTES <= (size_t)p.max_seq * p.row_bytes, c.status);
-        const uint32_t dst = ring_s + slot * SLOT_BYTES, bar = cbar + 8 * slot;
-        if (lane == 0 && inside) {
-            mbar_expect_tx(bar, CAL ? 2 * KV_BYTES : SLOT_BYTES);
-            bulk_g2s(dst, kc_base + iss_kv, KV_BYTES, bar);
-            bulk_g2s(dst + KV_BYTES, vc_base + iss_kv, KV_BYTES, bar);
-            if constexpr (!CAL) {
-                bulk_g2s(dst + 2 * KV_BYTES, (const unsigned char *)vs_base + iss_sz, SZ_BYTES, bar);
-                bulk_g2s(dst + 2 * KV_BYTES + SZ_BYTES, (const unsigned char *)vz_base + iss_sz, SZ_BYTES, bar);
-            }
-            if constexpr (KT) {   // the tokens' key parameters (same shape as the value parameters) follow them in the slot
-                bulk_g2s(dst + 2 * KV_BYTES + 2 * SZ_BYTES, (const unsigned char *)ktok_s_base + iss_sz, SZ_BYTES, bar);
-                bulk_g2s(dst + 2 * KV_BYTES + 3 * SZ_BYTES, (const unsigned char *)ktok_z_base + iss_sz, SZ_BYTES, bar);
-            }
+        const uint32_t dst = ring_s + slot * SLOT_BYTES;
+        if (inside) {
+            copy_words<KV_BYTES>(dst, kc_base + iss_kv, lane);
+            copy_words<KV_BYTES>(dst + KV_BYTES, vc_base + iss_kv, lane);
+            if constexpr (!CAL) copy_params<SZ_BYTES, KT ? 4 : 2>(dst + 2 * KV_BYTES, vs_base, vz_base, ktok_s_base, ktok_z_base, iss_sz, lane);
         }
         ++iss;
         iss_kv += KV_BYTES;
@@ -486,7 +517,10 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
     };
     if (my_groups > 0) {
         if (!FLAT) issue_params(0);
-        for (int i = 0; i < NSLOT - 1 && iss < n_chunks; ++i) issue_chunk();
+        for (int i = 0; i < NSLOT - 1; ++i) {      // a group of copies a chunk, empty ones behind the last
+            if (iss < n_chunks) issue_chunk();
+            copies_commit();
+        }
     }
     // static value parameters of the KV head: the same for every token
     float cal_sv[NGv], cal_zv[NGv];
@@ -621,8 +655,6 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
                     const int ch = I8 ? i8_ch[e] : lane * CPL + e;
                     scv[e] = kp[ch]; zev[e] = kp[D + ch];
                 }
-                __syncwarp();   // the parameters are in registers: the slot can take the next group's while this one streams
-                if (gi + 1 < my_groups) issue_params(gi + 1);
             }
             if constexpr (I8 >= 2) {
                 // up to four heads: the four signed bytes of F = rint(q * scale * 2^sh) (radix 256, as in decode_one.cuh) per factor and
@@ -733,6 +765,8 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
             }
             }
             __syncwarp();
+            // every lane's parameters have gone into sums over the warp: the slot can take the next group's while this one streams
+            if (!FLAT && gi + 1 < my_groups) issue_params(gi + 1);
         }
         if constexpr (I8 >= 2) {
             // (I8 = 3: those of the even rows; the odd rows' are read from the table tile by tile)
@@ -762,7 +796,8 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
             // refill the slot freed by the previous chunk, then wait for this chunk's bytes
             __syncwarp();
             if (iss < n_chunks) issue_chunk();
-            if (!wait_bar(cbar + 8 * slot, (unsigned)(ci / NSLOT) & 1u)) { stream_ok = false; break; }
+            copies_commit();
+            copies_wait<NSLOT - 1>();
             const uint2 mwords = mword_next;
             {   // sink bits of the warp's next chunk, fetched one chunk ahead
                 if (ci + 1 < n_chunks) mword_next = load_mask_words(grp * TPG + (cj + 1) * CT);   // the warp's chunks are consecutive
@@ -932,6 +967,7 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
             }
         }
     }
+    copies_wait<0>();      // the ring's space is used again
     if (!stream_ok && lane == 0) atomicOr(c.status, KVSINK_STATUS_TIMEOUT);
 
     fetch_sinks(sink_worker, 1, SB);      // used when the packed partial is done
