@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 TINY = synth.WORKLOADS["tiny"]
 
 
-def _check(wl, T, pos0, shape_keys=None, shape_values=None, strided=False):
+def _check(wl, T, pos0, shape_keys=None, shape_values=None, strided=False, rows=256):
     ocfg, gcfg = configs(wl)
     H = synth.make_hidden(wl, "cuda")
     K, V = synth.make_kv(wl, 0, "cuda")
@@ -32,7 +32,7 @@ def _check(wl, T, pos0, shape_keys=None, shape_values=None, strided=False):
     q = torch.randn((wl.batch, wl.n_q_heads, T, wl.head_dim), device="cuda", generator=g).half()
     if strided:     # [B, T, Hq, D] storage
         q = q.permute(0, 2, 1, 3).contiguous().permute(0, 2, 1, 3)
-    assert kv.prefill_rows(gcfg, T) == 256
+    assert kv.prefill_rows(gcfg, T) == rows
     out, lse = kv.prefill_attention(gcfg, gc, q, pos0)
     ref, ref_lse = oracle.prefill_attention(ocfg, oc, np16(q), pos0)
     torch.cuda.synchronize()
@@ -201,6 +201,15 @@ def test_sink_rows_that_are_not_finite_stay_hidden_from_queries_before_them(bits
     fine = np.isfinite(ref)
     assert_close(out[fine], ref[fine], "prompt attention")
     assert np.abs(lse - ref_lse).max() <= 2e-3 + 1e-3 * np.abs(ref_lse).max()
+
+
+# few rows a unit, on the side of the line that the tensor-core blocks take: one row tile, not full; and just on the other side of it
+@pytest.mark.parametrize("bits,group,hq,hkv,batch,T,pos0,rows", [
+    (2, 128, 8, 8, 5, 96, 0, 256), (2, 64, 32, 8, 5, 23, 200, 256), (4, 64, 8, 8, 5, 60, 30, 256), (4, 32, 16, 8, 4, 37, 64, 256), (3, 64, 8, 8, 5, 57, 5, 256), (3, 128, 32, 8, 5, 15, 120, 256),
+    (2, 128, 8, 8, 1, 593, 0, 256), (2, 128, 8, 8, 5, 88, 0, 8), (4, 64, 8, 8, 5, 56, 0, 8), (3, 64, 8, 8, 5, 56, 5, 8)])
+def test_few_rows_on_both_sides_of_the_line(bits, group, hq, hkv, batch, T, pos0, rows):
+    wl = TINY.scaled(bits=bits, head_dim=128, group=group, n_q_heads=hq, n_kv_heads=hkv, batch=batch, seq=pos0 + T, topk=4, pfn_n=1, seed=32000 + bits * 100 + T)
+    _check(wl, T, pos0, strided=T % 2 == 1, rows=rows)
 
 
 # several row blocks to a block of the grid, which takes them one after the other: the last ones are their units' first rows, 44 with one row tile, 4, 256
