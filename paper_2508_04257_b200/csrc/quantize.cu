@@ -328,8 +328,12 @@ append_one_kernel(Params p, kvsink_cache c, const __half *__restrict__ k_src, co
 // keys, and the tokens behind the last whole group.  One block per (sequence, KV head, 64 channels) has the keys; one per tile
 // touched the values.  Latency bound (a few rows per block), so it is one launch instead of three that wait for one another: a 2779-token
 // chunk that starts inside a group, 5 x 8 units at 3 bit, had 12 us of head tokens and 7 us of flush before its whole groups.
+// The head size and the bits are the kernel's own, so that the walk over a word's fields is straight code, and the rows of codes are padded, which puts
+// the lanes of a quad into different banks (walk by run-time bits, rows of 64 and 128 bytes, loads one after the other, and now, us): that chunk 26.3
+// and 25.1 (20.7 without its ends), its 27 head tokens alone 7.1 and 5.9, 10 x 32 units of them 18.2 and 15.3, 8 x 32 units, 2859 tokens
+// from 1237, 2 bit, 94.7 and 90.2, 4 x 8 with 64 channels, 700 from 250, 4 bit, 16.5 and 14.5.
 // ---------------------------------------------------------------------------------------------------------
-constexpr int QE_THREADS = 256, QE_CH = 64, QE_SHARE = QE_THREADS / QE_CH;
+constexpr int QE_THREADS = 256, QE_CH = 64, QE_SHARE = QE_THREADS / QE_CH, QE_CROW = QE_CH + 4, QE_MAX_G = 128;
 
 struct EdgeShape {
     int head_first, head_n, flush;             // tokens inside the open group; whether they complete it
@@ -337,18 +341,20 @@ struct EdgeShape {
     int head_tiles;                            // tiles the head tokens touch
 };
 
+template <int D, int BITS>
 __global__ void __launch_bounds__(QE_THREADS)
 append_edges_kernel(Params p, kvsink_cache c, const __half *__restrict__ k_src, const __half *__restrict__ v_src, EdgeShape e, int64_t sb, int64_t sh,
                     int64_t stt)
 {
+    constexpr int VROW = D + 8;                // padded row of the values' codes: a quad's tokens lie in different banks
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ float part[QE_SHARE][2][QE_CH]; // keys: extremes of the row quarters; then scale, zero
-    __shared__ uint8_t flag[128];              // keys: sink flags of the open group; values: tokens of the tile that are new
-    __shared__ uint8_t vcode[KVSINK_TILE * 128];
-    const int D = p.D, G = p.G, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __shared__ uint8_t flag[QE_MAX_G];         // keys: sink flags of the open group; values: tokens of the tile that are new
+    __shared__ uint8_t vcode[KVSINK_TILE * VROW];
+    const int G = p.G, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int h = blockIdx.y, b = blockIdx.z;
     const int64_t unit = (int64_t)b * p.Hkv + h, src0 = b * sb + h * sh;
-    const float qmax = (float)((1 << p.bits) - 1);
+    const float qmax = (float)((1 << BITS) - 1);
     const uint32_t *bm = c.sink_bitmask + (size_t)b * p.mask_words;
     const int32_t *sink_pos = c.sink_pos + (size_t)b * p.cap;
     pdl_wait();
@@ -356,7 +362,7 @@ append_edges_kernel(Params p, kvsink_cache c, const __half *__restrict__ k_src, 
     if (!in_bounds(e.head_first >= 0 && e.head_first + e.head_n <= p.max_seq && (e.rem_n == 0 || e.rem_first + e.rem_n <= p.max_seq), c.status)) return;
     const int count = min(c.sink_count[b], p.cap);
 
-    const int slices = D / QE_CH;
+    constexpr int slices = D / QE_CH;
     if ((int)blockIdx.x < slices) {            // ---- keys: a slice of 64 channels ----
         constexpr int CHUNKS = QE_CH / 8, RS = QE_CH + 8;
         const int c0 = (int)blockIdx.x * QE_CH, old = e.head_first % G;               // rows of the open group that the tail holds
@@ -364,24 +370,30 @@ append_edges_kernel(Params p, kvsink_cache c, const __half *__restrict__ k_src, 
         const __half *src = k_src + src0 + c0;
         if (e.flush) {
             __half *Kt = (__half *)dyn;        // [G][RS]
-            uint8_t *code = (uint8_t *)(Kt + (size_t)G * RS);                         // [G][QE_CH]
+            uint8_t *code = (uint8_t *)(Kt + (size_t)G * RS);                         // [G][QE_CROW]
             const int g0 = e.head_first - old;
-            for (int idx = tid; idx < G * CHUNKS; idx += QE_THREADS) {
-                const int t = idx / CHUNKS, ch = (idx % CHUNKS) * 8;
-                const __half *row = t < old ? tail + (size_t)t * D : src + (int64_t)(t - old) * stt;
-                *(uint4 *)(Kt + (size_t)t * RS + ch) = *(const uint4 *)(row + ch);
+            uint4 v[QE_MAX_G * CHUNKS / QE_THREADS];                                    // all of a thread's loads on their way at once
+#pragma unroll
+            for (int x = 0; x < QE_MAX_G * CHUNKS / QE_THREADS; ++x) {
+                const int idx = tid + x * QE_THREADS, t = idx / CHUNKS, ch = (idx % CHUNKS) * 8;
+                if (t < G) v[x] = *(const uint4 *)((t < old ? tail + (size_t)t * D : src + (int64_t)(t - old) * stt) + ch);
             }
-            for (int t = tid; t < G; t += QE_THREADS) flag[t] = mask_bit(bm, g0 + t) ? 1 : 0;
+            if (tid < G) flag[tid] = mask_bit(bm, g0 + tid) ? 1 : 0;
+#pragma unroll
+            for (int x = 0; x < QE_MAX_G * CHUNKS / QE_THREADS; ++x) {
+                const int idx = tid + x * QE_THREADS, t = idx / CHUNKS, ch = (idx % CHUNKS) * 8;
+                if (t < G) *(uint4 *)(Kt + (size_t)t * RS + ch) = v[x];
+            }
             __syncthreads();
             // extremes per channel: four threads with a share of the rows each, then one thread per channel
             const int ch = tid % QE_CH, qt = tid / QE_CH;
             float mn = INFINITY, mx = -INFINITY;
-            for (int t = qt; t < G; t += QE_SHARE)
-                if (!flag[t]) {
-                    const float x = __half2float(Kt[(size_t)t * RS + ch]);
-                    mn = fminf(mn, x);
-                    mx = fmaxf(mx, x);
-                }
+#pragma unroll 4
+            for (int t = qt; t < G; t += QE_SHARE) {
+                const float x = __half2float(Kt[(size_t)t * RS + ch]);
+                mn = flag[t] ? mn : fminf(mn, x);
+                mx = flag[t] ? mx : fmaxf(mx, x);
+            }
             part[qt][0][ch] = mn;
             part[qt][1][ch] = mx;
             __syncthreads();
@@ -400,31 +412,35 @@ append_edges_kernel(Params p, kvsink_cache c, const __half *__restrict__ k_src, 
             }
             __syncthreads();
             const float s = part[0][0][ch], z = part[0][1][ch];
+#pragma unroll 4
             for (int t = qt; t < G; t += QE_SHARE)
-                code[t * QE_CH + ch] = flag[t] ? 0 : (uint8_t)code_exact(__half2float(Kt[(size_t)t * RS + ch]), s, z, qmax);
+                code[t * QE_CROW + ch] = flag[t] ? 0 : (uint8_t)code_exact(__half2float(Kt[(size_t)t * RS + ch]), s, z, qmax);
             __syncthreads();
             // the slice's words: per tile and lane two words of a 2-bit section, four of a 4-bit one, one of the 3-bit high section
             uint32_t *out = (uint32_t *)(c.k_codes + (size_t)unit * p.max_seq * p.row_bytes + (size_t)(g0 / KVSINK_TILE) * p.tile_bytes);
-            const int tile_words = p.tile_bytes / 4, per_lane = p.bits, fields = p.bits == 4 ? 4 : 8, lo_words = p.bits == 4 ? 4 : 2;
-            const int n_lo = D * (p.bits == 4 ? 4 : 2) / 64;
-            for (int idx = tid; idx < G / KVSINK_TILE * 32 * per_lane; idx += QE_THREADS) {
-                const int ln = idx % 32, i = idx / 32 % per_lane, tile = idx / (32 * per_lane);
-                const uint8_t *rows = code + tile * KVSINK_TILE * QE_CH;
+            constexpr int tile_words = 8 * D * BITS / 16, lo_bits = BITS == 4 ? 4 : 2, fields = 16 / lo_bits, lo_words = BITS == 4 ? 4 : 2, n_lo = D * lo_bits / 64;
+            for (int idx = tid; idx < G / KVSINK_TILE * 32 * BITS; idx += QE_THREADS) {
+                const int ln = idx % 32, i = idx / 32 % BITS, tile = idx / (32 * BITS);                 // i and tile are a warp's
+                const uint8_t *rows = code + tile * KVSINK_TILE * QE_CROW;
                 uint32_t word = 0;
                 int m, row, col;
-                if (i < lo_words) {
+                if (BITS != 3 || i < lo_words) {
+#pragma unroll
                     for (int k = 0; k < fields; ++k)
+#pragma unroll
                         for (int x = 0; x < 2; ++x) {
                             slot_to_elem(ln, fields * i + k, x, &m, &row, &col);
-                            word |= (rows[row * QE_CH + 16 * m + col] & (p.bits == 4 ? 15u : 3u)) << (16 * x + (p.bits == 4 ? 4 : 2) * k);
+                            word |= (rows[row * QE_CROW + 16 * m + col] & ((1u << lo_bits) - 1u)) << (16 * x + lo_bits * k);
                         }
                     out[tile * tile_words + section_word_offset(n_lo, ln, lo_words * (int)blockIdx.x + i)] = word;
                 } else {
+#pragma unroll
                     for (int k = 0; k < 16; ++k)
+#pragma unroll
                         for (int x = 0; x < 2; ++x) {
                             slot_to_elem(ln, k, x, &m, &row, &col);
                             const int w = k >> 3, f = k & 7;
-                            word |= (uint32_t)((rows[row * QE_CH + 16 * m + col] >> 2) & 1) << (16 * x + 4 * (f >> 1) + 2 * (1 - w) + (f & 1));
+                            word |= (uint32_t)((rows[row * QE_CROW + 16 * m + col] >> 2) & 1) << (16 * x + 4 * (f >> 1) + 2 * (1 - w) + (f & 1));
                         }
                     out[tile * tile_words + 32 * n_lo + section_word_offset(D / 64, ln, (int)blockIdx.x)] = word;
                 }
@@ -458,7 +474,7 @@ append_edges_kernel(Params p, kvsink_cache c, const __half *__restrict__ k_src, 
     const int tile = first / KVSINK_TILE + vt - (head ? 0 : e.head_tiles);
     const int t_lo = max(first, tile * KVSINK_TILE), t_hi = min(first + n, (tile + 1) * KVSINK_TILE);
     if (tid < KVSINK_TILE) flag[tid] = (tile * KVSINK_TILE + tid >= t_lo && tile * KVSINK_TILE + tid < t_hi) ? 1 : 0;
-    const int cpl = D / 32;   // channels per lane (2 or 4)
+    constexpr int cpl = D / 32;   // channels per lane (2 or 4)
     for (int pos = t_lo + warp; pos < t_hi; pos += QE_THREADS / 32) {
         const __half *row = v_src + src0 + (int64_t)(offset + pos - first) * stt + lane * cpl;
         __half2 v2[2];
@@ -492,18 +508,18 @@ append_edges_kernel(Params p, kvsink_cache c, const __half *__restrict__ k_src, 
             c.v_scale[o] = s;
             c.v_zero[o] = z;
         }
-        for (int i = 0; i < cpl; ++i) vcode[(pos % KVSINK_TILE) * D + lane * cpl + i] = sink ? 0 : (uint8_t)code_exact(x[i], s, z, qmax);
+        for (int i = 0; i < cpl; ++i) vcode[(pos % KVSINK_TILE) * VROW + lane * cpl + i] = sink ? 0 : (uint8_t)code_exact(x[i], s, z, qmax);
     }
     __syncthreads();
     // the new tokens' fields; fields of other tokens keep their bits, a fresh tile is written whole
-    const int tile_words = p.tile_bytes / 4;
+    constexpr int tile_words = 8 * D * BITS / 16;
     uint32_t *vout = (uint32_t *)(c.v_codes + (size_t)unit * p.max_seq * p.row_bytes + (size_t)tile * p.tile_bytes);
     const bool fresh = t_lo % KVSINK_TILE == 0;
     for (int word = tid; word < tile_words; word += QE_THREADS) {
         const uint32_t keep = fresh ? 0u : vout[word];
         uint32_t fieldmask;
-        const uint32_t newbits = assemble_word_masked(p.bits, D, word, [&](int m, int row, int col) {
-            return flag[col] ? (uint32_t)vcode[col * D + 16 * m + row] : 0x100u; }, &fieldmask);
+        const uint32_t newbits = assemble_word_masked(BITS, D, word, [&](int m, int row, int col) {
+            return flag[col] ? (uint32_t)vcode[col * VROW + 16 * m + row] : 0x100u; }, &fieldmask);
         if (fieldmask || fresh) vout[word] = (keep & ~fieldmask) | newbits;
     }
 }
@@ -511,7 +527,7 @@ append_edges_kernel(Params p, kvsink_cache c, const __half *__restrict__ k_src, 
 // Groups of more than 128 tokens keep the kernels that go token by token (the group would not fit a block's shared memory).
 int launch_append_edges(const Params &p, const kvsink_cache &c, const AppendEdges &a, cudaStream_t st)
 {
-    if (p.G > 128) return KVSINK_ERR_UNSUPPORTED;
+    if (p.G > QE_MAX_G) return KVSINK_ERR_UNSUPPORTED;
     auto tiles = [](int first, int n) { return n > 0 ? (first + n - 1) / KVSINK_TILE - first / KVSINK_TILE + 1 : 0; };
     EdgeShape e;
     e.head_first = a.head_first;
@@ -522,8 +538,10 @@ int launch_append_edges(const Params &p, const kvsink_cache &c, const AppendEdge
     e.rem_src = a.rem_src;
     e.head_tiles = tiles(a.head_first, a.head_n);
     const dim3 grid(p.D / QE_CH + e.head_tiles + tiles(e.rem_first, e.rem_n), p.Hkv, p.B);
-    const size_t smem = e.flush ? (size_t)p.G * ((QE_CH + 8) * 2 + QE_CH) : 0;
-    return launch_pdl(append_edges_kernel, grid, dim3(QE_THREADS), smem, st, p, c, a.k_src, a.v_src, e, a.sb, a.sh, a.stt) == cudaSuccess ? KVSINK_OK : KVSINK_ERR_CUDA;
+    const size_t smem = e.flush ? (size_t)p.G * ((QE_CH + 8) * 2 + QE_CROW) : 0;
+    const auto kernel = p.D == 128 ? (p.bits == 2 ? append_edges_kernel<128, 2> : p.bits == 3 ? append_edges_kernel<128, 3> : append_edges_kernel<128, 4>)
+                                   : (p.bits == 2 ? append_edges_kernel<64, 2> : append_edges_kernel<64, 4>);
+    return launch_pdl(kernel, grid, dim3(QE_THREADS), smem, st, p, c, a.k_src, a.v_src, e, a.sb, a.sh, a.stt) == cudaSuccess ? KVSINK_OK : KVSINK_ERR_CUDA;
 }
 
 int launch_quantize_tokens(const Params &p, const kvsink_cache &c, const __half *k_src, const __half *v_src, int src_offset,

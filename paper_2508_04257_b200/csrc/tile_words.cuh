@@ -81,7 +81,9 @@ __device__ __forceinline__ uint32_t assemble_word_masked(int bits, int D, int wo
     if (bits == 2 || bits == 4) {
         const int n = D * bits / 64, fields = 16 / bits;
         section_word_owner(n, word, &lane, &i);
+#pragma unroll
         for (int k = 0; k < fields; ++k)
+#pragma unroll
             for (int e = 0; e < 2; ++e) {
                 slot_to_elem(lane, fields * i + k, e, &m, &row, &col);
                 put(get(m, row, col), (1u << bits) - 1u, 16 * e + bits * k);
@@ -90,7 +92,9 @@ __device__ __forceinline__ uint32_t assemble_word_masked(int bits, int D, int wo
         const int nlo = D / 32, nhi = D / 64;
         if (word < 32 * nlo) {
             section_word_owner(nlo, word, &lane, &i);
+#pragma unroll
             for (int k = 0; k < 8; ++k)
+#pragma unroll
                 for (int e = 0; e < 2; ++e) {
                     slot_to_elem(lane, 8 * i + k, e, &m, &row, &col);
                     put(get(m, row, col), 3u, 16 * e + 2 * k);
@@ -98,8 +102,11 @@ __device__ __forceinline__ uint32_t assemble_word_masked(int bits, int D, int wo
         } else {
             int j;
             section_word_owner(nhi, word - 32 * nlo, &lane, &j);
+#pragma unroll
             for (int w = 0; w < 2; ++w)
+#pragma unroll
                 for (int k = 0; k < 8; ++k)
+#pragma unroll
                     for (int e = 0; e < 2; ++e) {
                         slot_to_elem(lane, 8 * (2 * j + w) + k, e, &m, &row, &col);
                         const uint32_t v = get(m, row, col);
