@@ -341,6 +341,23 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
         }
         return __all_sync(0xffffffffu, ok);
     };
+    // sink bits of the chunk that starts at tile T: one 32-bit word covers two tiles
+    auto load_mask_words = [&](int T) {
+        uint2 w;
+        w.x = __ldg(bm + (T >> 1));
+        w.y = NP == 2 ? __ldg(bm + (T >> 1) + 1) : 0u;
+        return w;
+    };
+    uint2 mword_next = my_groups > 0 ? load_mask_words(w_begin * TPG) : make_uint2(0u, 0u);
+    // The loads that come next are issued ahead of the first copies of the ring and used behind them: the copies of 16 warps keep the load unit busy,
+    // and what is queued behind them waits (with the queries loaded behind them, us, before and now: 8 x 8 units of 8000 tokens, 2 bit,
+    // 64-token groups, four heads each 27.0 and 26.3, two heads each, 3000 tokens 14.2 and 13.8, static 11.9 and 11.2)
+    float cal_sv[NGv], cal_zv[NGv];       // static value parameters of the KV head
+#pragma unroll
+    for (int j = 0; j < NGv; ++j) { cal_sv[j] = CAL ? sp.v_scale[h * NGv + j] : 0.f; cal_zv[j] = CAL ? sp.v_zero[h * NGv + j] : 0.f; }
+    __half q_v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) q_v[r] = r < nq ? q[((size_t)b * p.Hq + hq0 + r) * D + tid] : __float2half(0.f);
     if (my_groups > 0) {
         if (!FLAT) issue_params(0);
         for (int i = 0; i < NSLOT - 1; ++i) {      // a group of copies a chunk, empty ones behind the last
@@ -348,14 +365,11 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
             copies_commit();
         }
     }
-    float cal_sv[NGv], cal_zv[NGv];       // static value parameters of the KV head
-#pragma unroll
-    for (int j = 0; j < NGv; ++j) { cal_sv[j] = CAL ? sp.v_scale[h * NGv + j] : 0.f; cal_zv[j] = CAL ? sp.v_zero[h * NGv + j] : 0.f; }
     // the first copies are in flight: now the query tables
-    for (int i = tid; i < R * D; i += DEC_THREADS) {
-        const __half v = i / D < nq ? q[((size_t)b * p.Hq + hq0) * D + i] : __float2half(0.f);
-        q16[i] = v;
-        qs[i] = __half2float(v) * qscale;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        q16[r * D + tid] = q_v[r];
+        qs[r * D + tid] = __half2float(q_v[r]) * qscale;
     }
     __syncthreads();
 
@@ -368,14 +382,6 @@ decode_few_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
         i8_ch[e] = BITS != 4 ? 16 * (2 * mi + (e & 1)) + 8 * c2 + 2 * tq + (e >> 1) : 16 * (2 * mi + c2) + 8 * (e & 1) + 2 * tq + (e >> 1);
     }
 
-    // sink bits of the chunk that starts at tile T: one 32-bit word covers two tiles
-    auto load_mask_words = [&](int T) {
-        uint2 w;
-        w.x = __ldg(bm + (T >> 1));
-        w.y = NP == 2 ? __ldg(bm + (T >> 1) + 1) : 0u;
-        return w;
-    };
-    uint2 mword_next = my_groups > 0 ? load_mask_words(w_begin * TPG) : make_uint2(0u, 0u);
     bool stream_ok = true;
     int ci = 0;                                                      // running chunk index of this warp
 

@@ -515,6 +515,18 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
         }
         return __all_sync(0xffffffffu, ok);
     };
+    // the queries' loads go ahead of the ring's first copies, behind which they would wait for the load unit (8 x 8 units of 8000 tokens, four heads each,
+    // 2 bit, 128-token groups 20.8 and 20.0 us)
+    constexpr int QV = NQMAX * D / DEC_THREADS;
+    __half q_v[QV];
+#pragma unroll
+    for (int x = 0; x < QV; ++x) {
+        const int qh = (tid + x * DEC_THREADS) / D, ch = (tid + x * DEC_THREADS) % D;
+        q_v[x] = __float2half(0.f);
+        if (qh < nq)
+            q_v[x] = PRE ? q[b * pre.q_sb + (int64_t)(hq0 + (8 * qc + qh) % p.rep) * pre.q_sh + (int64_t)row_token(qh) * pre.q_st + ch]
+                         : q[((size_t)b * p.Hq + hq0 + qh) * D + ch];
+    }
     if (my_groups > 0) {
         if (!FLAT) issue_params(0);
         for (int i = 0; i < NSLOT - 1; ++i) {      // a group of copies a chunk, empty ones behind the last
@@ -536,14 +548,10 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
         fit_value_scale(mx);
     }
     // the first copies are in flight: now the query tables (the copies do not depend on them)
-    for (int i = tid; i < NQMAX * D; i += DEC_THREADS) {
-        const int qh = i / D, ch = i % D;
-        __half v = __float2half(0.f);
-        if (qh < nq)
-            v = PRE ? q[b * pre.q_sb + (int64_t)(hq0 + (8 * qc + qh) % p.rep) * pre.q_sh + (int64_t)row_token(qh) * pre.q_st + ch]
-                    : q[((size_t)b * p.Hq + hq0 + qh) * D + ch];
-        q16[i] = v;
-        qs[i] = __half2float(v) * qscale;
+#pragma unroll
+    for (int x = 0; x < QV; ++x) {
+        q16[tid + x * DEC_THREADS] = q_v[x];
+        qs[tid + x * DEC_THREADS] = __half2float(q_v[x]) * qscale;
     }
     __syncthreads();
 

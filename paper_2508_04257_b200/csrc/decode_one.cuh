@@ -288,6 +288,22 @@ decode_one_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
         }
         return __all_sync(0xffffffffu, ok);
     };
+    // sink bits of the chunk that starts at tile T: one 32-bit word covers two tiles
+    auto load_mask_words = [&](int T) {
+        uint2 w;
+        w.x = __ldg(bm + (T >> 1));
+        w.y = NP == 2 ? __ldg(bm + (T >> 1) + 1) : 0u;
+        return w;
+    };
+    static_assert(DEC_THREADS == D, "a query value a thread");
+    // The loads that come next are issued ahead of the first copies of the ring and used behind them: the copies of 16 warps keep the load unit busy,
+    // and what is queued behind them waits (with the query loaded behind them, us, before and now: 8 x 32 units of 4096 tokens, 2 bit
+    // 18.6 and 18.1, 3 bit, 64-token groups 32.5 and 31.6, 4 bit, 128-token groups 28.5 and 27.6)
+    float cal_sv[NGv], cal_zv[NGv];       // static value parameters of the KV head
+#pragma unroll
+    for (int j = 0; j < NGv; ++j) { cal_sv[j] = CAL ? sp.v_scale[h * NGv + j] : 0.f; cal_zv[j] = CAL ? sp.v_zero[h * NGv + j] : 0.f; }
+    const __half q_v = q[((size_t)b * p.Hq + h) * D + tid];
+    uint2 mword_next = my_groups > 0 ? load_mask_words(w_begin * TPG) : make_uint2(0u, 0u);
     if (my_groups > 0) {
         if (!FLAT) issue_params(0);
         for (int i = 0; i < NSLOT - 1; ++i) {      // a group of copies a chunk, empty ones behind the last
@@ -295,15 +311,9 @@ decode_one_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
             copies_commit();
         }
     }
-    float cal_sv[NGv], cal_zv[NGv];       // static value parameters of the KV head
-#pragma unroll
-    for (int j = 0; j < NGv; ++j) { cal_sv[j] = CAL ? sp.v_scale[h * NGv + j] : 0.f; cal_zv[j] = CAL ? sp.v_zero[h * NGv + j] : 0.f; }
     // the first copies are in flight: now the query tables
-    for (int i = tid; i < D; i += DEC_THREADS) {
-        const __half v = q[((size_t)b * p.Hq + h) * D + i];
-        q16[i] = v;
-        qs[i] = __half2float(v) * qscale;
-    }
+    q16[tid] = q_v;
+    qs[tid] = __half2float(q_v) * qscale;
     __syncthreads();
 
     // Key operand: lane l prepares the bytes of one group of four contraction slots, (fragment l/8, lower or upper slots (l/4)%2, slots
@@ -317,14 +327,6 @@ decode_one_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
         i8_q[e] = qs[i8_ch[e]];
     }
 
-    // sink bits of the chunk that starts at tile T: one 32-bit word covers two tiles
-    auto load_mask_words = [&](int T) {
-        uint2 w;
-        w.x = __ldg(bm + (T >> 1));
-        w.y = NP == 2 ? __ldg(bm + (T >> 1) + 1) : 0u;
-        return w;
-    };
-    uint2 mword_next = my_groups > 0 ? load_mask_words(w_begin * TPG) : make_uint2(0u, 0u);
     bool stream_ok = true;
     int ci = 0;                                                      // running chunk index of this warp
 
