@@ -12,7 +12,7 @@
 //   long as everything else.
 // Append and decode, us a pass, fp16 values (and the same merge and splits) before, this kernel now: 16 x 8 units of 30000 tokens, four heads
 // each, 4 bit, 140 -> 127; 4 x 8 of 30000, 3 bit, 53 -> 54; 8 x 8 of 16000, groups of 32, 2 bit, 67 -> 63, groups of 64 46 -> 47; two heads,
-// 2 bit 34.8 -> 30.4, 4 bit 44.2 -> 38.9.  Error against 64 bits, 8192 tokens a warp: N(0,1) 2e-3 -> 2e-5, scores with a deviation of four nats
+// 2 bit 34.8 -> 30.4, 4 bit 44.2 -> 38.9 (all of these some 5 % less since the ring is filled by all lanes, behind the queries' loads).  Error against 64 bits, 8192 tokens a warp: N(0,1) 2e-3 -> 2e-5, scores with a deviation of four nats
 // 4e-4 -> 1e-5; a weight keeps 22 bits of the row's largest at least, smaller ones their sum.  Three and four heads at 2 bit with one channel
 // group a row stay in decode_kernel.cuh (decode_launch.cuh says why).
 #pragma once

@@ -7,8 +7,8 @@
 // 32 tokens every lane owns one, 8 t + g, for everything between the two products: the softmax, the parameters, the weight in
 // fixed point.  With the fp16 values all lanes of a quad did the work of the quad's two tokens.
 // Append and decode, us a pass, fp16 values with a warp's work on eight tokens at a time before, this kernel now: 8 x 32 units of 4096
-// tokens, 2 bit, 31.0 -> 25.9 (decode alone 26.8 -> 19.6); static parameters, 3821 tokens, 27.6 -> 23.9; 16 x 32 of 8101, 3 bit, 135 -> 114;
-// 64 x 32 of 8192, 4 bit, 481 -> 445; 32-token groups, 2 bit, 53.7 -> 36.8.  Error against 64 bits of these 5e-5 -> 1e-6 (the fp16
+// tokens, 2 bit, 31.0 -> 24.7 (decode alone 26.8 -> 18.1); static parameters, 3821 tokens, 27.6 -> 23.5; 16 x 32 of 8101, 3 bit, 135 -> 111;
+// 64 x 32 of 8192, 4 bit, 481 -> 441; 32-token groups, 2 bit, 53.7 -> 36.8 (and 6 % less since the ring is filled by all lanes).  Error against 64 bits of these 5e-5 -> 1e-6 (the fp16
 // products' accumulation truncates; 8192 tokens a warp, N(0,1), 2e-3 -> 1e-5).  Four blocks an SM; five (96 registers, a few spilled)
 // are slower except at 4 bit: 26.4 against 23.9, 422 / 411.
 //
