@@ -249,6 +249,7 @@ __device__ __forceinline__ void qb_pack_matrix(const uint32_t (&pc)[4], int m, u
 struct QbShape {
     int first_token, n_groups;
     unsigned n_items;
+    unsigned none;       // 0, which only the host knows
     int after_edges;     // launched behind the kernel of the same call's ragged ends
 };
 
@@ -555,11 +556,25 @@ quantize_bulk_kernel(Params p, kvsink_cache c, const __grid_constant__ CUtensorM
                 }
             }
         }
-        // every lane has consumed its ldmatrix results: the stage can take the warp's next item, which streams in
-        // while this one is coded from registers
+        // When this item's matrices are in registers the stage can take the warp's next item, which streams in while this one is
+        // coded.  A bulk copy is not kept behind loads that wait in the queue of shared memory, nor by the order of the program alone, so
+        // the copy's condition takes a value that depends on every matrix: the extremes behind the exchange between the lanes, or with static
+        // pairs, where nothing else reads them before they are coded, all registers of the matrices.  Rows of sink tokens may be missing from the
+        // extremes: their codes are 0 whatever the registers hold.
+        // 8 x 32 units of 4096 tokens, us, with the condition and with the copy merely behind the exchange: 2 bit 108.7 and 108.4, 4 bit with 64-token
+        // groups 144.9 and 144.2, 3 bit with 128-token groups 185.4 and 184.6.  A barrier that lane 0 arrives at and waits for instead:
+        // 144, 162, 202; static pairs 136 and now 100 (2 bit), 165 and 160 (3 bit)
         const QbPos nn = qb_advance<G>(nxt, Geo::PAIRED && !(next_id & 1u) ? one : step, sh.n_groups, p.Hkv);
-        __syncwarp();
-        if (lane == 0 && next_id < sh.n_items) qb_issue<G, MODE == 2>(&tm_k, &tm_v, nxt, my_stage, my_full);
+        auto issue_next = [&](uint32_t read) {
+            if (lane == 0 && next_id + (read & sh.none) < sh.n_items) qb_issue<G, MODE == 2>(&tm_k, &tm_v, nxt, my_stage, my_full);
+        };
+        uint32_t read = 0u;
+        __syncwarp();                             // copies of sink rows out of the stage: every lane's
+        if constexpr (MODE == 1) {
+#pragma unroll
+            for (int u = 0; u < 16; ++u) read ^= a[u][0] ^ a[u][1] ^ a[u][2] ^ a[u][3];
+            issue_next(read);
+        }
 
         if (kslab) {
             // the other channels of a token row live in the other half of the register and in the other lanes of the quad
@@ -607,6 +622,18 @@ quantize_bulk_kernel(Params p, kvsink_cache c, const __grid_constant__ CUtensorM
                     mn[s][ab] = qb_hmin2(mn[s][ab], __shfl_xor_sync(0xffffffffu, mn[s][ab], o));
                     mx[s][ab] = qb_hmax2(mx[s][ab], __shfl_xor_sync(0xffffffffu, mx[s][ab], o));
                 }
+        }
+
+        if constexpr (MODE != 1) {
+            constexpr bool few = NS >= 4;         // the exchange left every lane NS / 4 pairs, which depend on all sets
+            if (few && !kslab) {
+#pragma unroll
+                for (int j = 0; j < (few ? NS / 4 : 0); ++j) read ^= mn[j][0];
+            } else {
+#pragma unroll
+                for (int s = 0; s < NS; ++s) read ^= mn[s][0] ^ mn[s][1];
+            }
+            issue_next(read);
         }
 
         // ---- parameters (Eq. 10-11) and thresholds: the eight lanes of a column group share its 4 * NS keys ----
@@ -925,6 +952,7 @@ int launch_bulk(const Params &p, const kvsink_cache &c, const kvsink_static_para
     QbShape shp;
     shp.first_token = first_token;
     shp.n_groups = n_groups;
+    shp.none = 0u;
     shp.after_edges = before.call != nullptr;
     const long n_items = (long)p.B * p.Hkv * n_groups * Geo::IPG;
     if (n_items >= (1L << 30)) return KVSINK_ERR_UNSUPPORTED;

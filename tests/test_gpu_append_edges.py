@@ -186,3 +186,37 @@ def test_flat_chunks_of_many_units(scheme, chunks):
     import test_gpu_pertoken
     wl = TINY.scaled(bits=3, head_dim=128, group=128, n_q_heads=8, n_kv_heads=8, batch=8, seq=sum(chunks), topk=40, pfn_n=1, seed=36000 + chunks[0])
     (test_gpu_calibrated if scheme == "static" else test_gpu_pertoken)._both(wl, chunks=chunks)
+
+
+# A warp of the bulk quantizer takes several items one after the other and asks for the next one while it codes the last: with inputs that
+# are in L2 the next one comes soon, and must not reach the stage before every matrix of the last has left it.  84 MB of inputs, four items a warp and more,
+# half of it taken again and again: the same bytes every time, which are the oracle's
+@pytest.mark.parametrize("scheme,bits,group", [("static", 2, 128), ("static", 2, 64), ("static", 3, 64), ("static", 3, 128), ("static", 4, 64), ("static", 4, 128),
+                                               ("per_token", 2, 64), ("per_token", 3, 128), ("dynamic", 2, 32), ("dynamic", 2, 128), ("dynamic", 3, 64), ("dynamic", 4, 128)])
+def test_many_items_to_a_warp_from_cached_inputs(scheme, bits, group):
+    wl = TINY.scaled(bits=bits, head_dim=128, group=group, n_q_heads=8, n_kv_heads=8, batch=10, seq=2048, topk=40, pfn_n=1, seed=37000 + 10 * group + bits)
+    ocfg, gcfg = configs(wl, max_seq=2048)
+    H = synth.make_hidden(wl, "cuda")
+    K, V = synth.make_kv(wl, 0, "cuda")
+    sinks, listed = kv.predict_sinks(gcfg, H, kv.SinkSet(gcfg)), oracle.predict_sinks(ocfg, np16(H))
+    gc, oc = kv.KVCache(gcfg, sinks, per_token_keys=scheme == "per_token"), oracle.Cache(ocfg, *listed, per_token_keys=scheme == "per_token")
+    if scheme == "static":
+        gp, op = kv.calibrate(gcfg, K[:, :, :500], V[:, :, :500], sinks), oracle.calibrate(ocfg, np16(K[:, :, :500]), np16(V[:, :, :500]), listed[0])
+        append = lambda k, v: kv.quantize_append_calibrated(gcfg, gc, gp, k, v)
+        oracle.quantize_append_calibrated(ocfg, oc, op, np16(K), np16(V))
+    else:
+        one, ref = (kv.quantize_append, oracle.quantize_append) if scheme == "dynamic" else (kv.quantize_append_pertoken, oracle.quantize_append_pertoken)
+        append = lambda k, v: one(gcfg, gc, k, v)
+        ref(ocfg, oc, np16(K), np16(V))
+    append(K, V)
+    for name in ("k_codes", "v_codes", "sink_k", "sink_v") + (() if scheme == "static" else ("k_scale", "k_zero", "v_scale", "v_zero")):
+        assert getattr(gc, name).cpu().numpy().tobytes() == getattr(oc, name).tobytes(), name
+    first = [x.clone() for x in (gc.k_codes, gc.v_codes)]
+    for _ in range(20):
+        gc.k_codes.fill_(0xA5)
+        gc.v_codes.fill_(0xA5)
+        gc.seq_len = 0
+        append(K[:, :, :1024], V[:, :, :1024])          # in L2 by now, which the whole of K, V and the codes would not be
+        append(K[:, :, 1024:], V[:, :, 1024:])
+        assert torch.equal(gc.k_codes, first[0]) and torch.equal(gc.v_codes, first[1])
+    assert kv.read_status(gc) == 0
