@@ -39,7 +39,7 @@ extern "C" {
 
 /* Bits of the device status word (kvsink_cache.status, read with kvsink_read_status). */
 #define KVSINK_STATUS_SINK_MISMATCH 1 /* a token whose mask bit is set was not found in sink_pos */
-#define KVSINK_STATUS_TIMEOUT 2       /* a bounded wait inside a kernel ran out (a bulk copy, a matrix product); the result is invalid */
+#define KVSINK_STATUS_TIMEOUT 2       /* a bounded wait inside a kernel ran out (a bulk copy, a matrix product, another warp's part of a step); the result is invalid */
 #define KVSINK_STATUS_BOUNDS 4        /* a library built with -DKVSINK_DEBUG found an index outside its array and skipped the access */
 
 /* Tokens per packed tile. */

@@ -49,7 +49,8 @@ constexpr int PR_GRID = 148;                    // blocks: one to an SM
 constexpr int PR_ROUNDS = 95;                   // work items of a block at most
 // A zero point up to this size is subtracted from the code in fp16 exactly; farther ones go through an additive term.
 constexpr float PR_NEAR = 1000.f;
-// Limit of a wait: 8 ms and more (a poll comes back after 60 clocks at the earliest); a real wait is for work of the same block, some 10 us.
+// Limit of a wait: 8 ms and more (a poll comes back after 60 clocks at the earliest); a real wait is for a step's work of the same block, some
+// 10 us.  So nothing that goes with the number of sinks stands between two steps.
 // Counted in polls and not in clocks: a look at the clock every 256 polls made the kernel 6 % slower (2661 and 2825 us), since every wait
 // of every role holds a copy of the loop and code is what it has least room for.  No suspend-time hint: with one a poll is twice the
 // instructions, and the waiting warps' polls take the issue slots of the working ones (the chunk above 424000 and 408000 clocks a block).
@@ -99,7 +100,7 @@ struct PromptSmem {
     uint64_t s_full[2][PR_SBUFS], p_full[PR_SBUFS], o_done[PR_SBUFS], o_last[2], q_full[2], drained[2];
     uint32_t tmem;
     int failed;
-    int odd_values;                             // a sink token of the steps so far has a value that is infinite or NaN
+    uint8_t odd[PR_ROUNDS + 1];                 // by work item: a sink token of its steps has a value that is infinite or NaN
 };
 
 // The block holds all 512 columns of TMEM, so its addresses start at 0.  Columns: accumulators, queries of row tile 0 (with those of
@@ -405,6 +406,7 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
             w.n_steps = max(w.n0, w.n1);
         }
         sm.work[tid] = w;
+        sm.odd[tid] = 0;
     }
     if (warp == 16) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&sm.tmem)), "r"(512) : "memory");
@@ -423,7 +425,6 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
             }
             for (int i = 0; i < PR_HDRS; ++i) bar_init(&sm.hdr_full[i], 2);
             sm.failed = 0;
-            sm.odd_values = 0;
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         }
         __syncwarp();
@@ -442,6 +443,8 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
         const uint32_t lanes = (uint32_t)(warp & 3) << 21;                   // this warp's 32 lanes of TMEM
         const uint32_t t_o = lanes + TM_O + 128 * i;
         const float qscale = 1.4426950408889634f * rsqrtf((float)D);
+        // row of a.out and a.lse
+        auto out_row = [&](const Work &w, int r) { const int qt = query_of(r); return (w.b * p.Hq + w.h * p.rep + r - qt * p.rep) * a.T + qt; };
         // The queries of a work item's row tile, four lanes to 64 bytes of a row (a lane to a row of its own took 4000 clocks)
         auto load_queries = [&](const Work &w) {
             if (!(i ? w.n1 : w.n0)) return;
@@ -594,8 +597,7 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
             if (!ok) break;
             items += w.n0 + w.n1;
             hdr0 += w.n_steps;
-            const int unit = w.unit, b = w.b, at = query_of(min(row, n_rows - 1));
-            const int oq = (b * p.Hq + w.h * p.rep + min(row, n_rows - 1) - at * p.rep) * a.T + at;
+            const int oq = out_row(w, min(row, n_rows - 1));
             w = sm.work[round].take();
             load_queries(w);                     // the tile's last scores are there: its queries have been read
             if (steps > 0) {
@@ -631,22 +633,41 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
                     }
                 }
                 if (a.lse && valid) a.lse[oq] = l > 0.f ? (M + log2f(l)) * 0.6931471805599453f : -INFINITY;
-                // values of sink tokens that are infinite or NaN were left out of the products, where they would reach every row of the
-                // tile; only rows that see the token get them
-                __syncwarp();
-                if (valid && *(volatile int *)&sm.odd_values) {
-#pragma unroll 1
-                    for (int y = 0; y < min(c.sink_count[b], p.cap); ++y) {
-                        const int tok = c.sink_pos[(size_t)b * p.cap + y];
-                        if (tok < 0 || tok >= lim || !mask_bit(c.sink_bitmask + (size_t)b * p.mask_words, tok)) continue;
-                        const __half *v = (const __half *)c.sink_v + ((size_t)unit * p.cap + y) * D;
-#pragma unroll 1
-                        for (int ch = 0; ch < D; ++ch)
-                            if (!is_finite(__half2float(v[ch]))) a.out[(size_t)oq * D + ch] += __half2float(v[ch]);
-                    }
-                }
             }
             if (w.n_steps == 0) break;
+        }
+        // Values of sink tokens that are infinite or NaN were left out of the products, where they would reach every row of a tile; only rows
+        // that see the token get them.  This comes behind the block's last item and not behind each: it takes as long as the list of sinks is,
+        // and nobody waits for this warp any more (a wait of the other roles' is bounded by what a step takes).  A lane has four channels; the
+        // sums of the tokens that a row sees go on to the next row, which sees no fewer.
+        __syncwarp();
+#pragma unroll 1
+        for (int round = 0; uniform(sm.work[round].n_steps) > 0; ++round) {
+            if (!uniform(*(volatile uint8_t *)&sm.odd[round])) continue;
+            const Work w = sm.work[round].take();
+            const uint32_t *bm = c.sink_bitmask + (size_t)w.b * p.mask_words;
+            const int32_t *pos = c.sink_pos + (size_t)w.b * p.cap;
+            const uint2 *values = (const uint2 *)((const __half *)c.sink_v + (size_t)w.unit * p.cap * D) + lane;
+            const int n_pos = min(c.sink_count[w.b], p.cap), row0 = w.row0 + 128 * i + 32 * (warp & 3);
+            float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+            int y = 0;
+#pragma unroll 1
+            for (int row = row0; row < min(row0 + 32, w.end); ++row) {
+                const int lim = row_limit(row);
+#pragma unroll 1
+                for (; y < n_pos && pos[y] < lim; ++y) {
+                    if (pos[y] < 0 || !in_bounds(pos[y] < p.max_seq, c.status) || !mask_bit(bm, pos[y])) continue;
+                    const uint2 v = values[(size_t)y * (D / 4)];
+                    const float2 lo = __half22float2(as_half2(v.x)), hi = __half22float2(as_half2(v.y));
+                    if (!is_finite(lo.x)) sum.x += lo.x;
+                    if (!is_finite(lo.y)) sum.y += lo.y;
+                    if (!is_finite(hi.x)) sum.z += hi.x;
+                    if (!is_finite(hi.y)) sum.w += hi.y;
+                }
+                if (is_finite(sum.x) && is_finite(sum.y) && is_finite(sum.z) && is_finite(sum.w)) continue;
+                float4 *to = (float4 *)(a.out + (size_t)out_row(w, row) * D) + lane, o = *to;
+                *to = make_float4(o.x + sum.x, o.y + sum.y, o.z + sum.z, o.w + sum.w);
+            }
         }
     } else if (warp < 16) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
@@ -1025,7 +1046,7 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
                     }
                     top = max3(top, __low2float(large), __high2float(large));
                     rank0 += ns;
-                    if (!keys && __any_sync(0xffffffffu, odd) && lane == 0) *(volatile int *)&sm.odd_values = 1;
+                    if (!keys && __any_sync(0xffffffffu, odd) && lane == 0) *(volatile uint8_t *)&sm.odd[round] = 1;
                 }
                 int e = fit_exponent(warp_top(top));
                 if (keys && tok0 + PR_STEP > n_body && seq_len > n_body) e = min(e, 0);    // fp16 rows of the open group, as they are

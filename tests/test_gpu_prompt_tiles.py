@@ -236,3 +236,77 @@ def test_more_row_blocks_than_the_grid_takes():
         assert (out[:, :, t:t + 8] - small).abs().max() <= 2e-3 + 1e-2 * small.abs().max()
         assert (lse[:, :, t:t + 8] - small_lse).abs().max() <= 2e-3 + 1e-3 * small_lse.abs().max()
     assert kv.read_status(gc) == 0
+
+
+def _many_items(wl, T, pos0, looked_at, shape_keys=None, shape_values=None, strided=False, sink_values=None):
+    """More row blocks than SMs, so that blocks of the grid take several; the oracle has the sequences `looked_at`.  sink_values changes [B, Hkv, slot, D]."""
+    (ocfg, _), gcfg = configs(wl.scaled(batch=1)), configs(wl)[1]
+    g = torch.Generator("cuda").manual_seed(wl.seed)
+    H = torch.randn((wl.batch, wl.seq, wl.hidden), device="cuda", generator=g).half()
+    K, V = (torch.randn((wl.batch, wl.n_kv_heads, wl.seq, 128), device="cuda", generator=g, dtype=torch.float16) for _ in range(2))
+    if shape_keys:
+        shape_keys(K)
+    if shape_values:
+        shape_values(V)
+    gc = kv.KVCache(gcfg, kv.predict_sinks(gcfg, H, kv.SinkSet(gcfg)))
+    kv.quantize_append(gcfg, gc, K, V)
+    if sink_values:
+        sink_values(gc.sink_v.view(wl.batch, wl.n_kv_heads, -1, 128))
+    q = torch.randn((wl.batch, wl.n_q_heads, T, 128), device="cuda", generator=g).half()
+    if strided:
+        q = q.permute(0, 2, 1, 3).contiguous().permute(0, 2, 1, 3)
+    assert kv.prefill_rows(gcfg, T) == 256 and wl.batch * wl.n_kv_heads * -(-T * wl.n_q_heads // wl.n_kv_heads // 256) > 148
+    out, lse = (x.cpu().numpy() for x in kv.prefill_attention(gcfg, gc, q, pos0))
+    assert kv.read_status(gc) == 0
+    top, rows = float(V.abs().max()), gc.sink_v.cpu().numpy().view(np.uint16).reshape(wl.batch, -1)
+    for b in looked_at:
+        oc = oracle.Cache(ocfg, *oracle.predict_sinks(ocfg, np16(H[b:b + 1])))
+        oracle.quantize_append(ocfg, oc, np16(K[b:b + 1]), np16(V[b:b + 1]))
+        oc.sink_v[...] = rows[b].reshape(oc.sink_v.shape)
+        ref, ref_lse = (x[0] for x in oracle.prefill_attention(ocfg, oc, np16(q[b:b + 1]), pos0))
+        fine = np.isfinite(ref)
+        assert np.array_equal(np.isfinite(out[b]), fine) and all(np.array_equal(out[b] == x, ref == x) for x in (np.inf, -np.inf)), f"sequence {b}"
+        assert_close(out[b][fine], ref[fine], f"sequence {b}", atol=2e-3 * max(1.0, top / 6.0))
+        assert np.abs(lse[b] - ref_lse).max() <= 2e-3 + 1e-3 * np.abs(ref_lse).max()
+    return out
+
+
+# 160 row blocks of one unit each: twelve blocks of the grid take two, and units 140 and 155 (heads 4 of sequence 17, 3 of sequence 19) share one.
+# The walk over thousands of sinks for the values that the products leave out must not stand between a block's items, whose waits are bounded
+@pytest.mark.parametrize("b,h", [(17, 4), (19, 3)])
+@pytest.mark.parametrize("bits", [2, 4])
+def test_values_that_are_not_finite_in_one_unit_among_thousands_of_sinks(bits, b, h):
+    wl = TINY.scaled(bits=bits, head_dim=128, group=64, n_q_heads=8, n_kv_heads=8, batch=20, seq=4600, topk=4096, pfn_n=1, seed=38000 + bits)
+
+    def sink_values(v):                            # [sequence, KV head, slot, channel]; the last slots are tokens among the queries'
+        v[b, h, 7, 5], v[b, h, 2000, 5], v[b, h, 1999, 80], v[b, h, 4090, 64] = float("inf"), float("inf"), float("nan"), float("-inf")
+        v[b, h, 4000, 127], v[b, h, 4080, 127] = float("inf"), float("-inf")
+
+    out = _many_items(wl, 256, 4344, (0, 17, 19), sink_values=sink_values)
+    wrong = ~np.isfinite(out)
+    assert wrong[b, h].any() and wrong.sum() == wrong[b, h].sum()
+
+
+# rows of a unit: 400 = 256 + 144 and 280 = 256 + 24 (one row tile), 130
+@pytest.mark.parametrize("bits,group,T,pos0,keys,values,strided", [
+    (2, 64, 100, 70, _far, _far, True), (3, 32, 100, 70, _wide, _far, False), (4, 128, 70, 131, _far, None, True), (3, 64, 70, 0, None, _far, True)])
+def test_ranges_and_strides_with_several_row_blocks_to_a_block(bits, group, T, pos0, keys, values, strided):
+    wl = TINY.scaled(bits=bits, head_dim=128, group=group, n_q_heads=32, n_kv_heads=8, batch=12, seq=pos0 + T, topk=20, pfn_n=1, seed=39000 + bits + T)
+    _many_items(wl, T, pos0, (0, 5, 11), keys, values, strided)
+
+
+# mask bits without an entry in the position list, over several row blocks to a block: against the eight-row blocks, as with one
+@pytest.mark.parametrize("bits", [2, 3, 4])
+def test_mask_bits_without_a_list_entry_with_several_row_blocks_to_a_block(bits):
+    wl = TINY.scaled(bits=bits, head_dim=128, group=64, n_q_heads=32, n_kv_heads=8, batch=12, seq=80, topk=6, pfn_n=1, seed=39500 + bits)
+    gcfg, gc, q = _prompt(wl)
+    listed = set(gc.sinks.pos.cpu().tolist())
+    words = gc.sinks.bitmask.view(wl.batch, -1)
+    for t in (t for t in (2, 31, 40, 63, 64, 79) if t not in listed):
+        words[:, t // 32] |= (1 << t % 32) - (1 << 32 if t % 32 == 31 else 0)
+    assert kv.prefill_rows(gcfg, 80) == 256 and kv.prefill_rows(gcfg, 4) == 8
+    out, lse = kv.prefill_attention(gcfg, gc, q, 0)
+    for t in range(0, 80, 4):
+        small, small_lse = kv.prefill_attention(gcfg, gc, q[:, :, t:t + 4], t)
+        assert_close(out[:, :, t:t + 4].cpu().numpy(), small.cpu().numpy(), f"queries {t}")
+        assert (lse[:, :, t:t + 4] - small_lse).abs().max() <= 2e-3 + 1e-3 * small_lse.abs().max()
