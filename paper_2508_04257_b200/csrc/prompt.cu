@@ -31,7 +31,7 @@
 // 276 and 251; 28 x 32 heads of 165 tokens, 2 bit, 138 and 77; of 335, 3 bit, 276 and 167; 57 x 8 KV heads with four heads each, 1064 tokens,
 // 4 bit, 32-token groups 2366 and 1539; 8 KV heads with eight heads each, 100 queries over 192 tokens 23.3 and 17.0.  The outputs are the same
 // bits.  Relative error of the outputs against 64 bits: 2.6e-6 and 8.2e-6 for the first two.
-#include "common.cuh"
+#include "tile_words.cuh"
 
 namespace kvsink {
 
@@ -50,7 +50,7 @@ constexpr int PR_ROUNDS = 95;                   // work items of a block at most
 // A zero point up to this size is subtracted from the code in fp16 exactly; farther ones go through an additive term.
 constexpr float PR_NEAR = 1000.f;
 // Limit of a wait: 8 ms and more (a poll comes back after 60 clocks at the earliest); a real wait is for a step's work of the same block, some
-// 10 us.  So nothing that goes with the number of sinks stands between two steps.
+// 10 us.  So nothing that goes with the number of sinks stands between two steps (a search in the ascending list of positions goes with its logarithm).
 // Counted in polls and not in clocks: a look at the clock every 256 polls made the kernel 6 % slower (2661 and 2825 us), since every wait
 // of every role holds a copy of the loop and code is what it has least room for.  No suspend-time hint: with one a poll is twice the
 // instructions, and the waiting warps' polls take the issue slots of the working ones (the chunk above 424000 and 408000 clocks a block).
@@ -1017,9 +1017,7 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
                             const int idx = __popc(word & ((1u << lane) - 1u)) + (x ? ns0 : 0), tok = tok0 + 32 * x + lane;
                             int r = rank0 + idx;
                             if (r >= n_pos || pos[r] != tok) {               // mask and list disagree: look for it
-                                r = -1;
-                                for (int y = 0; y < n_pos; ++y)
-                                    if (pos[y] == tok) { r = y; break; }
+                                r = find_slot(pos, n_pos, tok);
                                 miss = r < 0;
                             }
                             sm.rank[role][buf][idx] = r;

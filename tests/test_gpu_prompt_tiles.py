@@ -310,3 +310,24 @@ def test_mask_bits_without_a_list_entry_with_several_row_blocks_to_a_block(bits)
         small, small_lse = kv.prefill_attention(gcfg, gc, q[:, :, t:t + 4], t)
         assert_close(out[:, :, t:t + 4].cpu().numpy(), small.cpu().numpy(), f"queries {t}")
         assert (lse[:, :, t:t + 4] - small_lse).abs().max() <= 2e-3 + 1e-3 * small_lse.abs().max()
+
+
+# a mask bit without an entry ahead of thousands that have one: every sink token behind it has to be looked up, within the other warps' bounded waits
+def test_mask_bit_without_a_list_entry_ahead_of_thousands_of_sinks():
+    wl = TINY.scaled(bits=2, head_dim=128, group=64, n_q_heads=8, n_kv_heads=8, batch=2, seq=4300, topk=4096, pfn_n=0, seed=39900)
+    _, gcfg = configs(wl)
+    g = torch.Generator("cuda").manual_seed(wl.seed)
+    H = torch.randn((2, 4300, wl.hidden), device="cuda", generator=g).half()
+    H[:, :70] = 0                     # none of the sinks
+    K, V = (torch.randn((2, 8, 4300, 128), device="cuda", generator=g, dtype=torch.float16) for _ in range(2))
+    gc = kv.KVCache(gcfg, kv.predict_sinks(gcfg, H, kv.SinkSet(gcfg)))
+    kv.quantize_append(gcfg, gc, K, V)
+    gc.sinks.bitmask.view(2, -1)[:, 0] |= 1 << 3
+    gc.sinks.bitmask.view(2, -1)[:, 2] |= 1 << 1
+    q = torch.randn((2, 8, 1000, 128), device="cuda", generator=g).half()
+    assert kv.prefill_rows(gcfg, 1000) == 256 and kv.prefill_rows(gcfg, 40) == 8
+    out, lse = kv.prefill_attention(gcfg, gc, q, 3300)
+    for t in range(0, 1000, 200):
+        small, small_lse = kv.prefill_attention(gcfg, gc, q[:, :, t:t + 40], 3300 + t)
+        assert_close(out[:, :, t:t + 40].cpu().numpy(), small.cpu().numpy(), f"queries {t}")
+        assert (lse[:, :, t:t + 40] - small_lse).abs().max() <= 2e-3 + 1e-3 * small_lse.abs().max()
