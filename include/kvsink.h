@@ -170,7 +170,7 @@ int kvsink_decode_attention(const kvsink_config *cfg, const kvsink_cache *cache,
  *         multiples of 8).
  *   out   device out, float [B][Hq][T][D].      lse  device out, float [B][Hq][T] or NULL.
  * No workspace: every block of rows (query token, query head) of one KV head streams its own prefix of the cache, 256 rows a block at
- * head size 128 where that is the faster, else eight.
+ * head size 128 where the rows are many enough for it, else eight.
  */
 int kvsink_prefill_attention(const kvsink_config *cfg, const kvsink_cache *cache, const void *q, int32_t T, int32_t q_pos0, int64_t stride_b,
                              int64_t stride_h, int64_t stride_t, float *out, float *lse, void *cuda_stream);

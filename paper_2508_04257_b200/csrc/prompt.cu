@@ -1106,22 +1106,23 @@ int launch(const Params &p, const kvsink_cache &c, const PromptArgs &a, cudaStre
 
 // The kernel for many rows, or the eight-row blocks of the decode kernel, which are faster with few: a block here takes the same time however few of its
 // rows there are (less with one row tile of 128 than with two), one block to an SM; those run four to an SM, each warp on a share of the cache, and slow one
-// another down.  So the line is the number of them on one SM while this kernel does one round of blocks.  Each side of it with 8192 tokens, us (rows x
+// another down.  So the line is the number of them while this kernel does one round of blocks.
+// Speed alone would draw it at 3 of them on an SM (2 bit, one row tile; 4 with two), 2 (3 bit), 2 and 3 (4 bit).  With 8192 tokens, us (rows x
 // units, eight-row blocks on an SM, there and here):
 //   2 bit: one tile   64 x 40,  3,  129 and 177;   96 x 40,  4,  192 and 179;   two tiles  512 x 8, 4,  196 and 252;   192 x 40, 7, 307 and 242
 //   3 bit: one tile  128 x 16,  2,  188 and 192;   64 x 40,  3,  275 and 189;   two tiles  256 x 8, 2,  192 and 248;   384 x 8,  3, 284 and 253
 //   4 bit: one tile  128 x 16,  2,  179 and 186;   96 x 40,  4,  280 and 186;   two tiles  384 x 8, 3,  186 and 249;   512 x 8,  4, 290 and 253
-// With 1000 cached tokens and less this kernel is ahead from somewhat smaller sizes on (2 bit, 512 x 8, 55 and 49; 128 x 40 of a prompt with nothing cached
-// 29 and 11); with several rounds (4 bit, 32 x 320 rows: three) the line is within 3 % (530 and 547).  Near the line, relative error of the outputs
-// against 64 bits, there and here: 8e-6 and 3e-7 for 96 tokens, 7e-5 and 4e-6 for 1023, 2e-4 and 1.4e-5 for 4060 (2 bit, values about zero); with values
-// 40 to 500 from zero and ranges a fiftieth as wide, 1e-6 and 2e-7, 2e-6 and 7e-6, 3e-6 and 2.6e-5: sums in TMEM are rounded downwards at each step.
+// There it lies at 3 bit.  At 2 and 4 bit the eight-row blocks sum the keys' products exactly, in integers, from factors of 30 bits; here keys carry 22 bits, as in
+// the eight-row blocks of 3 bit, and the sums in TMEM are rounded downwards at each product.  So there this kernel has only what lies well beyond:
+// from 1024 and 512 of those blocks a round on.  Relative error against 64 bits, there and here, for prompts between the lines: log-sum-exp 0.7e-7 and
+// 1.8e-7 (3 bit 2e-5 and 1.9e-7); outputs 4e-5 and 1e-6 (3 bit 1.5e-4 and 1e-6) with values about zero; with values 40 to 500 from zero and ranges a
+// fiftieth as wide 1e-6 and 8e-6 behind 1000 tokens, 3e-6 and 3e-5 behind 4000, at every code width.
 bool prompt_takes(const Params &p, int T)
 {
     if (p.D != 128) return false;
-    static const int on_one_sm[3][2] = {{3, 4}, {2, 2}, {2, 3}};
     const int64_t rows = (int64_t)T * p.rep, units = (int64_t)p.B * p.Hkv;
-    const int64_t blocks = (rows + PR_ROWS - 1) / PR_ROWS * units, waves = (blocks + 147) / 148;
-    return rows < (1 << 30) && blocks < (1 << 30) && (rows + 7) / 8 * units > waves * 148 * on_one_sm[p.bits - 2][rows > 128];
+    const int64_t blocks = (rows + PR_ROWS - 1) / PR_ROWS * units, waves = (blocks + 147) / 148, small = (rows + 7) / 8 * units;
+    return rows < (1 << 30) && blocks < (1 << 30) && (p.bits == 3 ? small > waves * 2 * 148 : small >= waves * (p.bits == 2 ? 1024 : 512));
 }
 
 int launch_prompt(const Params &p, const kvsink_cache &c, const __half *q, int T, int q_pos0, int64_t sb, int64_t sh, int64_t stt, float *out,
