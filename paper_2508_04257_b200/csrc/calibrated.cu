@@ -481,19 +481,7 @@ static int launch_tokens(const Params &p, const kvsink_cache &c, const kvsink_st
         return launch_pdl(append_one_flat_kernel<PT>, dim3((unsigned)((units + CO_WARPS - 1) / CO_WARPS)), dim3(32 * CO_WARPS), 0, st, p, c, sp, k_src,
                           v_src, first_token, sb, sh) == cudaSuccess ? KVSINK_OK : KVSINK_ERR_CUDA;
     }
-    if (p.D == 128) {
-        // One launch, whatever the ends.  Group sizes without a bulk form (they have no decode kernel either, codes are all they are for) keep
-        // the launches they had, which are counted: the tokens up to a tile boundary, whole tiles, the rest
-        int at = 0, rc = KVSINK_OK;
-        while (at < n_tokens && rc == KVSINK_OK) {
-            const int lead = (KVSINK_TILE - (first_token + at) % KVSINK_TILE) % KVSINK_TILE, left = n_tokens - at;
-            int n = left;
-            if (p.G != 64 && p.G != 128 && left >= lead + KVSINK_TILE) n = lead > 0 ? lead : left / KVSINK_TILE * KVSINK_TILE;
-            rc = launch_spans<PT>(p, c, sp, k_src, v_src, TokenSpans{{first_token + at, 0}, {n, 0}, {at, 0}, {0, 0}}, sb, sh, stt, st);
-            at += n;
-        }
-        return rc;
-    }
+    if (p.D == 128) return launch_spans<PT>(p, c, sp, k_src, v_src, TokenSpans{{first_token, 0}, {n_tokens, 0}, {0, 0}, {0, 0}}, sb, sh, stt, st);
     const int tiles = (first_token + n_tokens - 1) / KVSINK_TILE - first_token / KVSINK_TILE + 1;
     const dim3 grid(tiles, p.Hkv, p.B);
     return launch_pdl(quantize_calibrated_kernel<PT>, grid, dim3(CQ_THREADS), 0, st, p, c, sp, k_src, v_src, first_token, n_tokens, sb, sh, stt) ==

@@ -98,9 +98,9 @@ def test_inputs_rewritten_in_place_right_before_a_ragged_chunk(bits, group):
             assert torch.equal(a.view(torch.uint8), b.view(torch.uint8)), f"{n}, round {r}"
 
 
-@pytest.mark.parametrize("d,launches", [(64, 1), (128, 3)])
-def test_tokens_before_a_tile_boundary_go_by_themselves_only_where_tiles_have_a_kernel(d, launches):
-    # 100 tokens from position 5 with G = 144 (no whole span): at head size 128 the 11 up to the boundary, five tiles, the last nine
+@pytest.mark.parametrize("d,launches", [(64, 1), (128, 1)])
+def test_a_chunk_without_a_whole_span_is_one_launch(d, launches):
+    # 100 tokens from position 5 with G = 144: 11 up to a tile boundary, five tiles, the last nine
     cfg = kv.Config(1, 2, 2, d, 64, 2, 144, 144, 2, 1, (1,))
     g = torch.Generator("cuda").manual_seed(1)
     K, V = (torch.randn((1, 2, 105, d), device="cuda", generator=g).half() for _ in range(2))
