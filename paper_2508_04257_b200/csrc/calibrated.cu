@@ -5,7 +5,7 @@
 //                 non-sink tokens, then Eq. 10-11
 //   append      : every token is coded on arrival with the fixed pairs (Eq. 8, values outside the calibrated range clamp);
 //                 no key tail, no per-group parameters; sink rows go to the side buffer
-// The same two append kernels serve per-token keys (PT; Section 4.1 "Per-token quantization", Section 5.1's per-token Key and
+// The append kernels of head size 128 serve per-token keys too (PT; Section 4.1 "Per-token quantization", Section 5.1's per-token Key and
 // Value dynamic scheme): keys and values alike get one (scale, zero) per token and channel group, computed on arrival from
 // the token's own extremes (Eq. 10-11) and stored in the cache's parameter arrays, sink tokens (0, 0).
 #include "common.cuh"
@@ -113,18 +113,17 @@ __global__ void calibrate_finish_kernel(Params p, const int *__restrict__ ws, kv
 // Eq. 8 with fixed parameters; scale 0 (nothing was calibrated) gives code 0.
 __device__ __forceinline__ uint32_t code_static(float x, float s, float z, float qmax) { return s == 0.f ? 0u : code_exact(x, s, z, qmax); }
 
-// One block per (tile touched, KV head, sequence): the new tokens' key and value codes are inserted into their tiles
+// Static pairs at head size 64: one block per (tile touched, KV head, sequence).  The new tokens' key and value codes are inserted into their tiles
 // (fields of earlier tokens keep their bits; a tile whose first token arrives is written whole).
 constexpr int CQ_THREADS = 128;
 
-template <bool PT>
 __global__ void __launch_bounds__(CQ_THREADS)
 quantize_calibrated_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *__restrict__ k_src, const __half *__restrict__ v_src,
                            int first_token, int n_tokens, int64_t sb, int64_t sh, int64_t stt)
 {
-    __shared__ uint8_t kcode[KVSINK_TILE * 128], vcode[KVSINK_TILE * 128];
+    constexpr int D = 64;
+    __shared__ uint8_t kcode[KVSINK_TILE * D], vcode[KVSINK_TILE * D];
     __shared__ uint8_t present[KVSINK_TILE];
-    const int D = p.D;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int h = blockIdx.y, b = blockIdx.z;
     const int64_t unit = (int64_t)b * p.Hkv + h;
@@ -136,20 +135,17 @@ quantize_calibrated_kernel(Params p, kvsink_cache c, kvsink_static_params sp, co
     pdl_wait();
     if (!in_bounds(first_token >= 0 && first_token + n_tokens <= p.max_seq && (tile + 1) * KVSINK_TILE <= p.max_seq, c.status)) return;
 
-    const int cpl = D / 32;   // channels per lane (2 or 4)
-    float ks[4], kz[4], vs[4], vz[4];
+    constexpr int cpl = D / 32;   // channels per lane
+    float ks[cpl], kz[cpl], vs[cpl], vz[cpl];
     for (int e = 0; e < cpl; ++e) {
         const int ch = lane * cpl + e;
-        ks[e] = kz[e] = vs[e] = vz[e] = 0.f;
-        if constexpr (!PT) {
-            ks[e] = sp.k_scale[h * D + ch]; kz[e] = sp.k_zero[h * D + ch];
-            vs[e] = sp.v_scale[h * p.NGv + ch / p.Gv]; vz[e] = sp.v_zero[h * p.NGv + ch / p.Gv];
-        }
+        ks[e] = sp.k_scale[h * D + ch]; kz[e] = sp.k_zero[h * D + ch];
+        vs[e] = sp.v_scale[h * p.NGv + ch / p.Gv]; vz[e] = sp.v_zero[h * p.NGv + ch / p.Gv];
     }
     for (int pos = t_lo + warp; pos < t_hi; pos += CQ_THREADS / 32) {
         const int64_t src = b * sb + h * sh + (int64_t)(pos - first_token) * stt;
         const bool sink = mask_bit(bm, pos);
-        __half kx[4], vx[4];
+        __half kx[cpl], vx[cpl];
         for (int e = 0; e < cpl; ++e) { kx[e] = k_src[src + lane * cpl + e]; vx[e] = v_src[src + lane * cpl + e]; }
         if (sink) {
             const int count = min(c.sink_count[b], p.cap);
@@ -160,28 +156,6 @@ quantize_calibrated_kernel(Params p, kvsink_cache c, kvsink_static_params sp, co
                 __half *dk = (__half *)c.sink_k + ((size_t)unit * p.cap + slot) * D;
                 __half *dv = (__half *)c.sink_v + ((size_t)unit * p.cap + slot) * D;
                 for (int e = 0; e < cpl; ++e) { dk[lane * cpl + e] = kx[e]; dv[lane * cpl + e] = vx[e]; }
-            }
-        }
-        if constexpr (PT) {
-            // the token's own parameters: min / max over the lanes of each channel group, keys and values alike
-            float kmn = __half2float(kx[0]), kmx = kmn, vmn = __half2float(vx[0]), vmx = vmn;
-            for (int e = 1; e < cpl; ++e) {
-                kmn = fminf(kmn, __half2float(kx[e])); kmx = fmaxf(kmx, __half2float(kx[e]));
-                vmn = fminf(vmn, __half2float(vx[e])); vmx = fmaxf(vmx, __half2float(vx[e]));
-            }
-            const int lanes_per_group = p.Gv / cpl;
-            for (int o = 1; o < lanes_per_group; o <<= 1) {
-                kmn = fminf(kmn, __shfl_xor_sync(0xffffffffu, kmn, o)); kmx = fmaxf(kmx, __shfl_xor_sync(0xffffffffu, kmx, o));
-                vmn = fminf(vmn, __shfl_xor_sync(0xffffffffu, vmn, o)); vmx = fmaxf(vmx, __shfl_xor_sync(0xffffffffu, vmx, o));
-            }
-            float s0, z0, s1, z1;
-            group_params(!sink, kmn, kmx, qmax, &s0, &z0);
-            group_params(!sink, vmn, vmx, qmax, &s1, &z1);
-            for (int e = 0; e < cpl; ++e) { ks[e] = s0; kz[e] = z0; vs[e] = s1; vz[e] = z1; }
-            if (lane % lanes_per_group == 0) {
-                const size_t o = ((size_t)unit * p.max_seq + pos) * p.NGv + lane / lanes_per_group;
-                c.k_scale[o] = s0; c.k_zero[o] = z0;
-                c.v_scale[o] = s1; c.v_zero[o] = z1;
             }
         }
         for (int e = 0; e < cpl; ++e) {
@@ -209,7 +183,7 @@ quantize_calibrated_kernel(Params p, kvsink_cache c, kvsink_static_params sp, co
 }
 
 // One token per sequence (a decode step's append): one warp per unit codes the key and the value row and sets their fields with
-// word atomics.  The block-per-tile kernel above walks every word of both tiles for one token's fields: a step
+// word atomics.  A block per tile (as above, for any head size then) walks every word of both tiles for one token's fields: a step
 // of a LLaMA2-shaped layer (append and attention) 28.7 us with it, 27.6 with this.
 constexpr int CO_WARPS = 4;
 
@@ -482,10 +456,14 @@ static int launch_tokens(const Params &p, const kvsink_cache &c, const kvsink_st
                           v_src, first_token, sb, sh) == cudaSuccess ? KVSINK_OK : KVSINK_ERR_CUDA;
     }
     if (p.D == 128) return launch_spans<PT>(p, c, sp, k_src, v_src, TokenSpans{{first_token, 0}, {n_tokens, 0}, {0, 0}, {0, 0}}, sb, sh, stt, st);
-    const int tiles = (first_token + n_tokens - 1) / KVSINK_TILE - first_token / KVSINK_TILE + 1;
-    const dim3 grid(tiles, p.Hkv, p.B);
-    return launch_pdl(quantize_calibrated_kernel<PT>, grid, dim3(CQ_THREADS), 0, st, p, c, sp, k_src, v_src, first_token, n_tokens, sb, sh, stt) ==
-                   cudaSuccess ? KVSINK_OK : KVSINK_ERR_CUDA;
+    if constexpr (PT) {
+        return KVSINK_ERR_UNSUPPORTED;      // per-token keys: head size 128 alone
+    } else {
+        const int tiles = (first_token + n_tokens - 1) / KVSINK_TILE - first_token / KVSINK_TILE + 1;
+        const dim3 grid(tiles, p.Hkv, p.B);
+        return launch_pdl(quantize_calibrated_kernel, grid, dim3(CQ_THREADS), 0, st, p, c, sp, k_src, v_src, first_token, n_tokens, sb, sh, stt) ==
+                       cudaSuccess ? KVSINK_OK : KVSINK_ERR_CUDA;
+    }
 }
 
 // Whole G-token spans go to the bulk quantizer where it has a form for the scheme (G only shapes its work items with static parameters); the
