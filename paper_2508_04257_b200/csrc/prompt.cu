@@ -28,7 +28,7 @@
 //
 // One item a block, packed tiles through registers, suspended waits and generic addresses, and now (attention alone, us, in turn on one GPU):
 // 4096 queries over 4096 tokens, 8 sequences of 32 heads, 2 bit, 2661 and 2228; 1003 queries with four heads per KV head over 7403 tokens, 4 bit,
-// 276 and 251; 28 x 32 heads of 165 tokens, 2 bit, 138 and 77; of 335, 3 bit, 276 and 167; 57 x 8 KV heads with four heads each, 1064 tokens,
+// 276 and 251; 28 x 32 heads of 165 tokens, 2 bit, 138 and 77; of 335, 3 bit, 276 and 150; 57 x 8 KV heads with four heads each, 1064 tokens,
 // 4 bit, 32-token groups 2366 and 1539; 8 KV heads with eight heads each, 100 queries over 192 tokens 23.3 and 17.0.  The outputs are the same
 // bits.  Relative error of the outputs against 64 bits: 2.6e-6 and 8.2e-6 for the first two.
 #include "tile_words.cuh"
@@ -431,6 +431,7 @@ __global__ void __launch_bounds__(PR_THREADS, 1) prompt_kernel(Params p, kvsink_
         tc_fence_before();
     }
     __syncthreads();
+    in_bounds(tid == 0 || tid > PR_ROUNDS || sm.work[tid].n1 == 0 || sm.work[tid - 1].n1 > 0, c.status);      // debug builds: the order of the work items
     tc_fence_after();
     pdl_wait();
     pdl_release();

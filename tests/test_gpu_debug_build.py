@@ -49,6 +49,10 @@ for bits, group, hq, hkv, batch, T, pos0, topk in ((2, 128, 16, 16, 8, 64, 0, 3)
                      seed=26000 + bits)
     _check(wl, T, pos0)                  # asserts parity and a zero status word
 _check(TINY.scaled(bits=2, head_dim=128, group=32, n_q_heads=16, n_kv_heads=4, batch=2, seq=300, topk=6, pfn_n=1, seed=26100), 300, 0, _far, _far)
+# several work items to a block, their order among what is checked: the last ones with one row tile, with two
+for bits, group, hq, hkv, batch, T, pos0 in ((2, 128, 16, 16, 12, 300, 0), (3, 64, 32, 8, 12, 100, 70), (4, 64, 8, 4, 40, 130, 50)):
+    wl = TINY.scaled(bits=bits, head_dim=128, group=group, n_q_heads=hq, n_kv_heads=hkv, batch=batch, seq=pos0 + T, topk=5, pfn_n=1, seed=26200 + bits)
+    _check(wl, T, pos0)
 print("debug prompts ok")
 """
 
