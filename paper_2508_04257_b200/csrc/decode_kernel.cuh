@@ -472,15 +472,15 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
 
     // ---- complete key groups of this split: the warps take contiguous, nearly equal ranges of its groups.  A warp's
     //      chunks (CT tiles each) are consecutive in memory and arrive through a ring of NSLOT slots filled
-    //      NSLOT - 1 chunks ahead by lane 0; the key parameters of a group arrive one group ahead through one more slot. ----
+    //      NSLOT - 1 chunks ahead; the key parameters of a group arrive one group ahead through one more slot. ----
     const int g_begin = split * groups_per_split, g_end = min(n_groups, g_begin + groups_per_split);
     const int g_cnt = max(g_end - g_begin, 0);
     const int w_begin = g_begin + (g_cnt * warp) / DEC_WARPS, w_end = g_begin + (g_cnt * (warp + 1)) / DEC_WARPS;
     const int my_groups = w_end - w_begin;
     unsigned char *ring = ring_all + (size_t)warp * Plan::WARP_RING;
     float *kp_ring = (float *)(ring + NSLOT * SLOT_BYTES);           // [scale D | zero D] of the next group to prepare
-    // Every lane keeps the issue bookkeeping (so that addresses and counters stay warp-uniform values); lane 0 alone
-    // issues the copies.  Byte offsets inside the unit's arrays fit 32 bits.
+    // Every lane keeps the issue bookkeeping (so that addresses and counters stay warp-uniform values) and copies its share of a chunk; lane 0
+    // alone issues the parameters' bulk copies.  Byte offsets inside the unit's arrays fit 32 bits.
     const int n_chunks = my_groups * CPG;
     int iss = 0;                                                     // chunks issued so far
     uint32_t iss_kv = (uint32_t)w_begin * TPG * Plan::TILE_BYTES;    // byte offset of the next chunk in the code arrays
@@ -500,6 +500,7 @@ decode_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __half *_
         iss_kv += KV_BYTES;
         iss_sz += SZ_BYTES;
     };
+    // The caller has put the slot's last values through an operation of the whole warp: a bulk copy is not kept behind loads that are queued
     auto issue_params = [&](int gi) {
         if (lane == 0) {
             mbar_expect_tx(pbar, Plan::KP_BYTES);

@@ -273,6 +273,7 @@ decode_one_kernel(Params p, kvsink_cache c, kvsink_static_params sp, const __hal
         iss_kv += KV_BYTES;
         iss_sz += SZ_BYTES;
     };
+    // The caller has put the slot's last values through an operation of the whole warp: a bulk copy is not kept behind loads that are queued
     auto issue_params = [&](int gi) {
         if (lane == 0) {
             mbar_expect_tx(pbar, Plan::KP_BYTES);
